@@ -225,7 +225,7 @@ opattr_status do_attribute(Ctx &c, const opattr_kernels *kern, const opattr_rang
     if (high) {
         for (int i = 0; i < 8; ++i) nd.add<uint32_t>(K);    // names, sort x3, flag/pos, starts, table, hi_op
         nd.add<uint32_t>(radix_hist_elems(K)).add<uint32_t>(scan_scratch_elems(std::max(radix_hist_elems(K), K)));
-        nd.bytes += kernel_order_scratch(K);
+        nd.bytes += time_sort_scratch(K);
     }
     opattr_status st = ensure_arena(c, nd.bytes + 4096);
     if (st) return st;
@@ -263,8 +263,7 @@ opattr_status do_attribute(Ctx &c, const opattr_kernels *kern, const opattr_rang
         if (!k0 || !s0 || !s1 || !s2 || !pos || !ustart || !table || !hi_op || !hist || !part) return OPATTR_E_OOM;
         uint32_t *korder = nullptr;
         if (!k_sorted) {
-            korder = kernel_time_order(c, a, kern->stream, kern->start_ns, K);
-            if (!korder) return OPATTR_E_OOM;
+            if ((st = kernel_time_order(c, a, kern->stream, kern->start_ns, K, &korder))) return st;
         }
         // names in time order, sorted stably: each name's launches in one run
         launch(c, "attr_names", k_gather_names, dim3(gK), dim3(256), 0, kern->name_id, (const uint32_t *)korder, K,

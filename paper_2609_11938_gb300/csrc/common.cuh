@@ -32,6 +32,7 @@ enum FlagBit : unsigned {
     F_OP_DUP = 16u,       // two operator ranges share an op id
     F_AGG_MISS = 32u,     // the owned-range aggregation missed kernels
     F_IDX_NOT_ID = 64u,   // some kernel's ncu row index is neither its own index nor -1
+    F_BUCKETS = 256u,     // times too crowded for the bucketed time sort
 };
 enum CountSlot {
     C_NAMES_MISMATCH = 0,

@@ -631,7 +631,7 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     nd.add<uint32_t>(K).add<uint32_t>(nt_max).add<int2>(nt_max * 32);
     const bool keep_order = c.in_join && K > 0;       // a join keeps the time order for its matching
     if (keep_order) nd.add<uint32_t>(K);
-    size_t need = nd.bytes + kernel_order_scratch(K) + 4096;
+    size_t need = nd.bytes + time_sort_scratch(K) + 4096;
     c.spec_ran = false;
     opattr_status st = ensure_arena(c, need);
     if (st) return st;
@@ -753,8 +753,9 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     uint32_t *korder = nullptr;
     if (!k_sorted && K > 0) {
         // keyed by the compact ids of the streams with kernels
-        korder = kernel_time_order(c, a, kern->stream, kern->start_ns, K, d_scmap, bits_for((uint64_t)(nks - 1)));
-        if (!korder) return OPATTR_E_OOM;
+        if ((st = kernel_time_order(c, a, kern->stream, kern->start_ns, K, &korder, d_scmap,
+                                    bits_for((uint64_t)(nks - 1)))))
+            return st;
         if (kept_order) {
             cudaMemcpyAsync(kept_order, korder, sizeof(uint32_t) * K, cudaMemcpyDeviceToDevice, c.stream);
             c.join_korder = kept_order;

@@ -452,7 +452,7 @@ opattr_status do_match(Ctx &c, const opattr_kernels *kern, const opattr_ncu *ncu
     for (int i = 0; i < 4; ++i) nd.add<uint32_t>(M);                 // ncu sort
     nd.add<uint32_t>(radix_hist_elems(NX)).add<uint32_t>(scan_scratch_elems(std::max(radix_hist_elems(NX), NX)));
     nd.add<unsigned long long>(4);
-    size_t need = nd.bytes + kernel_order_scratch(K) + 4096;
+    size_t need = nd.bytes + time_sort_scratch(K) + 4096;
     opattr_status st = ensure_arena(c, need);
     if (st) return st;
     Arena a(c);
@@ -521,8 +521,8 @@ opattr_status do_match(Ctx &c, const opattr_kernels *kern, const opattr_ncu *ncu
     if (K > 0) launch(c, "fill_match", k_fill_match, dim3(gK), dim3(256), 0, out_idx, out_kind, K);
     uint32_t *korder = nullptr;
     if (!k_sorted && K > 0) {
-        korder = known_unsorted ? c.join_korder : kernel_time_order(c, a, kern->stream, kern->start_ns, K);
-        if (!korder) return OPATTR_E_OOM;
+        if (known_unsorted) korder = c.join_korder;
+        else if ((st = kernel_time_order(c, a, kern->stream, kern->start_ns, K, &korder))) return st;
     }
     // rk[j] = kernel index of the j-th replayed kernel in time order
     int64_t nrep = K;

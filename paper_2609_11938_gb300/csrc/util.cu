@@ -1,4 +1,6 @@
 // util.cu -- kernel time-order check and permutation.
+#include <algorithm>
+
 #include "sort.cuh"
 #include "util.cuh"
 
@@ -120,39 +122,211 @@ void check_kernel_order(Ctx &c, const uint8_t *stream, const int64_t *start, int
            dim3(CHK_THREADS), 0, stream, start, n, vec, c.d_status, stream_hist, tile_hist);
 }
 
-__global__ void k_time_keys(const uint8_t *__restrict__ stream, const int64_t *__restrict__ start, int64_t n,
-                            long long tmin, const uint8_t *__restrict__ scmap, int sbits,
-                            uint64_t *__restrict__ keys) {
+// ------------------------------------------------------------------ time sort
+// Records sorted by a time key, ties by index: the key's high bits split the
+// records over buckets of up to BK_TARGET on average (a count, a scan of the
+// counts, a scatter in any order), then a block sorts each bucket in shared
+// memory by spreading it over BK_BINS bins of the bucket's span and sorting
+// every bin, a few records each, by key and index.  Two reads and two writes of
+// 8 bytes per record, where the radix sort makes a pass of 24 bytes per eight
+// key bits.  Times crowd when a trace has long gaps or many equal times: a
+// bucket above BK_CAP records or a bin above BK_BIN_MAX sets F_BUCKETS, and the
+// radix sort does the whole again.
+//
+// 6M kernel records in no order: 16 us to count, 77 to scatter (bound by the
+// scattered 8-byte writes), 90 to sort the buckets (shared-memory latency),
+// against 115 us for each of five radix passes.
+constexpr int BK_THREADS = 512, BK_ITEMS = 16, BK_CAP = BK_THREADS * BK_ITEMS, BK_BIN_BITS = 12,
+              BK_BINS = 1 << BK_BIN_BITS;
+constexpr int BK_TARGET = 3072;
+constexpr int BK_BIN_MAX = 64;
+constexpr int64_t BK_MAX = 32 * 1024;        // buckets: their counts fit a block's shared memory and one block's scan
+
+// Each block counts an equal share of the records in shared memory (global
+// counters take few, coalesced additions: single ones ran at 50 a nanosecond).
+template <typename Key>
+__global__ void __launch_bounds__(BK_THREADS) k_bucket_count(Key key, int64_t n, int shift, int nb,
+                                                             uint32_t *__restrict__ cnt) {
     pdl_wait();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned s = scmap ? scmap[stream[i]] : stream[i];
-        keys[i] = ((uint64_t)(start[i] - tmin) << sbits) | s;
+    extern __shared__ uint32_t bk[];
+    for (int i = threadIdx.x; i < nb; i += BK_THREADS) bk[i] = 0;
+    __syncthreads();
+    const int64_t share = (n + gridDim.x - 1) / gridDim.x, i0 = share * blockIdx.x;
+    const int64_t i1 = i0 + share < n ? i0 + share : n;
+#pragma unroll 4
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += BK_THREADS) atomicAdd(&bk[key(i) >> shift], 1u);
+    __syncthreads();
+    for (int i = threadIdx.x; i < nb; i += BK_THREADS)
+        if (bk[i]) atomicAdd(&cnt[i], bk[i]);
+}
+// Bucket b fills [off[b], off[b + 1]): entries (key below `shift`) << 32 | i;
+// leaves off[b] at the bucket's end.  Same shares: counted again, room taken in
+// every bucket at once, then handed out.
+template <typename Key>
+__global__ void __launch_bounds__(BK_THREADS) k_bucket_scatter(Key key, int64_t n, int shift, int nb,
+                                                               uint32_t *__restrict__ off,
+                                                               uint64_t *__restrict__ out) {
+    pdl_wait();
+    extern __shared__ uint32_t bk[];
+    for (int i = threadIdx.x; i < nb; i += BK_THREADS) bk[i] = 0;
+    __syncthreads();
+    const int64_t share = (n + gridDim.x - 1) / gridDim.x, i0 = share * blockIdx.x;
+    const int64_t i1 = i0 + share < n ? i0 + share : n;
+#pragma unroll 4
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += BK_THREADS) atomicAdd(&bk[key(i) >> shift], 1u);
+    __syncthreads();
+    for (int i = threadIdx.x; i < nb; i += BK_THREADS)
+        if (bk[i]) bk[i] = atomicAdd(&off[i], bk[i]);
+    __syncthreads();
+    const uint64_t low = (1ull << shift) - 1;
+#pragma unroll 4
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += BK_THREADS) {
+        const uint64_t k = key(i);
+        out[atomicAdd(&bk[k >> shift], 1u)] = (k & low) << 32 | (uint32_t)i;
     }
 }
+__global__ void __launch_bounds__(BK_THREADS) k_bucket_sort(const uint64_t *__restrict__ in,
+                                                            const uint32_t *__restrict__ end, int shift,
+                                                            uint64_t *__restrict__ keys, uint32_t *__restrict__ perm,
+                                                            DevStatus *st) {
+    pdl_wait();
+    extern __shared__ __align__(16) unsigned char bk_smem[];
+    uint64_t *buf = reinterpret_cast<uint64_t *>(bk_smem);              // [BK_CAP]
+    uint32_t *bin = reinterpret_cast<uint32_t *>(buf + BK_CAP);         // [BK_BINS]
+    __shared__ uint32_t wbuf[33];
+    const int64_t b = blockIdx.x;
+    const uint32_t s0 = b ? end[b - 1] : 0u, m = end[b] - s0;
+    if (m == 0) return;
+    if (m > (uint32_t)BK_CAP) {
+        if (threadIdx.x == 0) set_flag(st, F_BUCKETS);
+        return;
+    }
+    constexpr int PER = BK_BINS / BK_THREADS;
+    for (int i = threadIdx.x; i < BK_BINS; i += BK_THREADS) bin[i] = 0;
+    __syncthreads();
+    // bins by the bits below the bucket's: the top BK_BIN_BITS of them
+    const int down = 32 + (shift > BK_BIN_BITS ? shift - BK_BIN_BITS : 0);
+    uint64_t v[BK_ITEMS];
+    uint32_t r[BK_ITEMS];
+#pragma unroll
+    for (int i = 0; i < BK_ITEMS; ++i) {
+        const uint32_t j = i * BK_THREADS + threadIdx.x;
+        if (j >= m) continue;
+        v[i] = in[s0 + j];
+        r[i] = atomicAdd(&bin[v[i] >> down], 1u);
+    }
+    __syncthreads();
+    uint32_t c[PER], sum = 0;
+    bool full = false;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        c[q] = bin[threadIdx.x * PER + q];
+        full |= c[q] > (uint32_t)BK_BIN_MAX;
+        sum += c[q];
+    }
+    uint32_t ex = block_exclusive_scan<uint32_t>(sum, wbuf, (uint32_t *)nullptr);
+    const uint32_t first = ex;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        bin[threadIdx.x * PER + q] = ex;
+        ex += c[q];
+    }
+    if (__syncthreads_or(full)) {
+        if (threadIdx.x == 0) set_flag(st, F_BUCKETS);
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < BK_ITEMS; ++i)
+        if (i * BK_THREADS + threadIdx.x < m) buf[bin[v[i] >> down] + r[i]] = v[i];
+    __syncthreads();
+    // each thread's bins, one after another: insertion sort (unique entries)
+    for (uint32_t q = 0, a = first; q < (uint32_t)PER; ++q) {
+        const uint32_t z = q + 1 < (uint32_t)PER ? bin[threadIdx.x * PER + q + 1] : ex;
+        for (uint32_t i = a + 1; i < z; ++i) {
+            const uint64_t x = buf[i];
+            uint32_t j = i;
+            for (; j > a && buf[j - 1] > x; --j) buf[j] = buf[j - 1];
+            buf[j] = x;
+        }
+        a = z;
+    }
+    __syncthreads();
+    for (uint32_t j = threadIdx.x; j < m; j += BK_THREADS) {
+        const uint64_t x = buf[j];
+        keys[s0 + j] = (uint64_t)b << shift | x >> 32;
+        perm[s0 + j] = (uint32_t)x;
+    }
+}
+template <typename Key>
+__global__ void k_write_keys(Key key, int64_t n, uint64_t *__restrict__ keys) {
+    pdl_wait();
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        keys[i] = key(i);
+}
 
-size_t kernel_order_scratch(int64_t n) {
+size_t time_sort_scratch(int64_t n) {
     Need nd;
     nd.add<uint64_t>(n).add<uint64_t>(n).add<uint32_t>(n).add<uint32_t>(n);
-    nd.add<uint32_t>(radix_hist_elems(n)).add<uint32_t>(scan_scratch_elems(radix_hist_elems(n)));
+    nd.add<uint32_t>(std::max<int64_t>(radix_hist_elems(n), BK_MAX + 1));
+    nd.add<uint32_t>(scan_scratch_elems(std::max<int64_t>(radix_hist_elems(n), BK_MAX + 1)));
     return nd.bytes;
 }
 
-uint32_t *kernel_time_order(Ctx &c, Arena &a, const uint8_t *stream, const int64_t *start, int64_t n,
-                            const uint8_t *scmap, int stream_bits) {
+template <typename Key>
+static opattr_status time_sort(Ctx &c, Arena &a, Key key, int64_t n, uint64_t top, uint64_t **keys, uint32_t **perm) {
+    const int64_t hist_n = std::max<int64_t>(radix_hist_elems(n), BK_MAX + 1);
     uint64_t *k0 = a.take<uint64_t>(n), *k1 = a.take<uint64_t>(n);
     uint32_t *v0 = a.take<uint32_t>(n), *v1 = a.take<uint32_t>(n);
-    uint32_t *hist = a.take<uint32_t>(radix_hist_elems(n));
-    uint32_t *part = a.take<uint32_t>(scan_scratch_elems(radix_hist_elems(n)));
-    if (!k0 || !k1 || !v0 || !v1 || !hist || !part) return nullptr;
-    long long tmin = c.h_status->mm[MM_KSTART_MIN], tmax = c.h_status->mm[MM_KSTART_MAX];
+    uint32_t *hist = a.take<uint32_t>(hist_n), *part = a.take<uint32_t>(scan_scratch_elems(hist_n));
+    if (!k0 || !k1 || !v0 || !v1 || !hist || !part) return OPATTR_E_OOM;
+    // widest buckets of BK_TARGET records on average whose span fits the entries' 32 bits
+    int shift = 32;
+    while (shift > 0 && (int64_t)(top >> shift) + 1 < (n + BK_TARGET - 1) / BK_TARGET) --shift;
+    const int64_t nb = (int64_t)(top >> shift) + 1;
+    if (c.host_mapped && nb <= BK_MAX) {
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device);
+        const size_t smem = sizeof(uint32_t) * nb, sort_smem = sizeof(uint64_t) * BK_CAP + sizeof(uint32_t) * BK_BINS;
+        const dim3 g(grid_for(n, BK_THREADS * 8, (smem > 64 * 1024 ? 1 : 3) * std::max(1, sms)));
+        cudaFuncSetAttribute(k_bucket_count<Key>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(4 * BK_MAX));
+        cudaFuncSetAttribute(k_bucket_scatter<Key>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(4 * BK_MAX));
+        cudaFuncSetAttribute(k_bucket_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem);
+        cudaMemsetAsync(hist, 0, sizeof(uint32_t) * nb, c.stream);
+        launch(c, "bucket_count", k_bucket_count<Key>, g, dim3(BK_THREADS), smem, key, n, shift, (int)nb, hist);
+        scan_exclusive_u32(c, hist, hist, nb, part, nullptr);
+        launch(c, "bucket_scatter", k_bucket_scatter<Key>, g, dim3(BK_THREADS), smem, key, n, shift, (int)nb, hist, k0);
+        launch(c, "bucket_sort", k_bucket_sort, dim3((unsigned)nb), dim3(BK_THREADS), sort_smem, (const uint64_t *)k0,
+               (const uint32_t *)hist, shift, k1, v1, c.d_status);
+        opattr_status st = read_status(c);
+        if (st) return st;
+        *keys = k1;
+        *perm = v1;
+        if (!(c.h_status->flags & F_BUCKETS)) return OPATTR_OK;
+    }
+    launch(c, "time_keys", k_write_keys<Key>, dim3(grid_for(n, 256, 65535)), dim3(256), 0, key, n, k0);
+    radix_sort_pairs<uint64_t>(c, k0, v0, k1, v1, n, bits_for(top), true, hist, part, keys, perm);
+    return OPATTR_OK;
+}
+
+struct KernelTimeKey {
+    const int64_t *start;
+    const uint8_t *stream, *scmap;      // scmap may be NULL
+    long long tmin;
+    int sbits;
+    __device__ __forceinline__ uint64_t operator()(int64_t i) const {
+        const unsigned s = stream[i];
+        return ((uint64_t)(start[i] - tmin) << sbits) | (scmap ? scmap[s] : s);
+    }
+};
+opattr_status kernel_time_order(Ctx &c, Arena &a, const uint8_t *stream, const int64_t *start, int64_t n,
+                                uint32_t **order, const uint8_t *scmap, int stream_bits, uint64_t **keys) {
+    const long long tmin = c.h_status->mm[MM_KSTART_MIN], tmax = c.h_status->mm[MM_KSTART_MAX];
     const int sbits = scmap ? stream_bits : 8;
-    launch(c, "time_keys", k_time_keys, dim3(grid_for(n, 256, 65535)), dim3(256), 0, stream, start, n, tmin, scmap,
-           sbits, k0);
-    uint64_t *ko;
-    uint32_t *vo;
-    radix_sort_pairs<uint64_t>(c, k0, v0, k1, v1, n, bits_for((uint64_t)(tmax - tmin)) + sbits, true, hist, part,
-                               &ko, &vo);
-    return vo;
+    uint64_t *k = nullptr;
+    const opattr_status st = time_sort(c, a, KernelTimeKey{start, stream, scmap, tmin, sbits}, n,
+                                       ((uint64_t)(tmax - tmin) << sbits) | ((1ull << sbits) - 1), &k, order);
+    if (keys) *keys = k;
+    return st;
 }
 
 }  // namespace opattr

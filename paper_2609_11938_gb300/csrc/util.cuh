@@ -14,17 +14,18 @@ namespace opattr {
 void check_kernel_order(Ctx &c, const uint8_t *stream, const int64_t *start, int64_t n,
                         uint32_t *stream_hist = nullptr, uint32_t *tile_hist = nullptr);
 
-// Scratch (bytes) of kernel_time_order for n kernels.
-size_t kernel_order_scratch(int64_t n);
+// Scratch (bytes) of a time sort of n records (kernel_time_order).
+size_t time_sort_scratch(int64_t n);
 
-// Permutation of kernel indices into time order (start, stream, index) by a
-// stable radix sort of ((start - min_start) << sbits | stream).  Needs the
-// min / max from check_kernel_order in c.h_status.  With scmap (device,
-// [256]: increasing compact ids of the streams that have kernels) the key
-// holds the compact id in stream_bits bits instead of the id in 8, which
-// saves a pass when the span and the stream count allow.  Returns a device
-// array of n indices carved from `a`, or NULL on arena exhaustion.
-uint32_t *kernel_time_order(Ctx &c, struct Arena &a, const uint8_t *stream, const int64_t *start, int64_t n,
-                            const uint8_t *scmap = nullptr, int stream_bits = 8);
+// Permutation of kernel indices into time order (start, stream, index): sorted
+// by (start - min_start) << sbits | stream.  Needs the min / max from
+// check_kernel_order in c.h_status.  With scmap (device, [256]: increasing
+// compact ids of the streams that have kernels) the key holds the compact id
+// in stream_bits bits instead of the id in 8.  *order receives a device array
+// of n indices carved from `a`, *keys (if given) the sorted keys.  May wait on
+// the stream (and reads the status block then).
+opattr_status kernel_time_order(Ctx &c, struct Arena &a, const uint8_t *stream, const int64_t *start, int64_t n,
+                                uint32_t **order, const uint8_t *scmap = nullptr, int stream_bits = 8,
+                                uint64_t **keys = nullptr);
 
 }  // namespace opattr
