@@ -312,6 +312,13 @@ __device__ __forceinline__ int32_t range_of_t(const int32_t *rok, const uint32_t
     return rok[k];
 }
 
+// Within a join whose enclosure's verdict is still to be read (pending): the
+// enclosure found records out of order, more levels than its layout holds or
+// an error, and wrote nothing to aggregate.
+__device__ __forceinline__ bool stopped(const DevStatus *st) {
+    return (st->err & (ERR_INVALID | ERR_DEPTH)) || (st->flags & (F_K_UNSORTED | F_R_UNSORTED | F_LEVELS_MANY));
+}
+
 // ------------------------------------------------------------------ count
 // Per kernel: duration >= 0, range index in [-1, R), an attributed range is
 // an operator below n_ops, row index in [-1, M).  Totals: all / attributed
@@ -333,8 +340,10 @@ template <bool DIRECT>
 __global__ void __launch_bounds__(256, 5) k_agg_count(const int64_t *__restrict__ dur, const int32_t *__restrict__ rok,
                             const int32_t *__restrict__ nidx, const uint32_t *__restrict__ r_op, int64_t K, int64_t R,
                             int64_t M, int64_t n_ops, uint32_t *__restrict__ cnt, uint32_t *__restrict__ rank,
-                            int64_t run, int ident_rows, unsigned *__restrict__ nonident, DevStatus *st) {
+                            int64_t run, int ident_rows, unsigned *__restrict__ nonident, int pending,
+                            DevStatus *st) {
     pdl_wait();
+    if (pending && stopped(st)) return;
     const unsigned lane = lane_id(), lt = lanemask_lt();
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
     const int64_t nwarps = (int64_t)gridDim.x * blockDim.x / 32;
@@ -400,8 +409,9 @@ __global__ void __launch_bounds__(256, 5) k_agg_count(const int64_t *__restrict_
 template <bool DIRECT>
 __global__ void k_agg_place(const int32_t *__restrict__ rok, const uint32_t *__restrict__ r_op, int64_t K, int64_t R,
                             int64_t n_ops, const uint32_t *__restrict__ off, const uint32_t *__restrict__ rank,
-                            uint32_t *__restrict__ list) {
+                            uint32_t *__restrict__ list, int pending, const DevStatus *st) {
     pdl_wait();
+    if (pending && stopped(st)) return;
     constexpr int U = 4;                    // kernels per thread per round, loads issued together
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t k0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k0 < K; k0 += stride * U) {
@@ -579,8 +589,9 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 __global__ void __launch_bounds__(AG_THREADS, 5) k_agg_ops(const uint32_t *__restrict__ off, uint32_t *list,
-                                                          AggIn A) {
+                                                          AggIn A, int pending, const DevStatus *st) {
     pdl_wait();
+    if (pending && stopped(st)) return;
     extern __shared__ __align__(16) unsigned char ag_smem[];
     OpsWarp &W = reinterpret_cast<OpsWarp *>(ag_smem)[threadIdx.x / 32];
     const unsigned lane = lane_id();
@@ -997,8 +1008,8 @@ __global__ void __launch_bounds__(FIN_THREADS) k_agg_long_ops(const uint32_t *__
 
 // Blocks of the ops pass: what stays resident, fewer for few ops.
 static unsigned ops_grid(Ctx &c, int64_t O) {
-    int sms = 0, per_sm = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device);
+    const int sms = sm_count(c);
+    int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_agg_ops, AG_THREADS, AG_SMEM);
     cudaGetLastError();
     const int64_t resident = (int64_t)std::max(1, sms) * std::max(1, per_sm);
@@ -1030,9 +1041,6 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
     opattr_status st = ensure_arena(c, nd.bytes + 4096);
     if (st) return st;
     Arena a(c);
-    // with the enclosure's verdict pending (a join) the status block keeps it:
-    // the enclosure's reset left the aggregation's slots at zero
-    if (!c.enclose_pending && (st = reset_status(c))) return st;
     uint32_t *cnt = a.take<uint32_t>(O + 1), *off = a.take<uint32_t>(O + 1);
     // tmp holds each kernel's slot among its op's kernels until the list is
     // placed, then serves the segment sorts
@@ -1046,16 +1054,16 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
     uint32_t *npc = a.take<uint32_t>(O + 1);
     Acc *partials = a.take<Acc>(K / AG_PIECE + (K / (AG_SHORT_MAX + 1)) + 1);
     if (!npc || !partials) return OPATTR_E_OOM;
-    cudaMemsetAsync(ctr, 0, 3 * sizeof(unsigned), c.stream);
     uint32_t *part = a.take<uint32_t>(scan_scratch_elems(std::max<int64_t>(O + 1, radix_hist_elems(K))));
     uint32_t *hidx = a.take<uint32_t>(O + 1), *hhist = a.take<uint32_t>(radix_hist_elems(K));
     uint32_t *info = a.take<uint32_t>(8), *hop = a.take<uint32_t>(O + 1);
     if (!hidx || !hhist || !info || !hop) return OPATTR_E_OOM;
     if (!cnt || !off || !list || !tmp || !longs || !nlong || !part || !nonident || !dirty) return OPATTR_E_OOM;
-    cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * (O + 1), c.stream);
-    cudaMemsetAsync(nonident, 0, sizeof(unsigned), c.stream);
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device);
+    // with the enclosure's verdict pending (a join) the status block keeps it:
+    // the enclosure's reset left the aggregation's slots at zero
+    const ZeroRun zr[3] = {{cnt, O + 1}, {ctr, 3}, {nonident, 1}};
+    if ((st = c.enclose_pending ? zero_runs(c, 3, zr) : reset_status(c, 3, zr))) return st;
+    const int sms = sm_count(c);
     // runs long enough to keep most segments in one warp, short enough that
     // the grid is one wave of resident warps (five blocks of eight per SM)
     const int64_t warps = (int64_t)std::max(1, sms) * 40;
@@ -1063,7 +1071,7 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
     if (K > 0)
         launch(c, "agg_count", rok ? k_agg_count<false> : k_agg_count<true>,
                dim3(grid_for(K, 256 / 32 * run, 65535)), dim3(256), 0, kern->dur_ns, rok, nidx, rng->op_id, K, R, M,
-               O, cnt, tmp, run, (int)(c.in_join && c.rows_identity), nonident, c.d_status);
+               O, cnt, tmp, run, (int)(c.in_join && c.rows_identity), nonident, (int)c.enclose_pending, c.d_status);
     AggIn in;
     in.dur = kern->dur_ns;
     in.ncu_idx = nidx;
@@ -1082,20 +1090,21 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
         if (K > 0)
             launch(c, "agg_place", rok ? k_agg_place<false> : k_agg_place<true>,
                    dim3(grid_for(K, 256 * 4, REDUCE_GRID)), dim3(256), 0, rok, rng->op_id, K, R, O,
-                   (const uint32_t *)off, (const uint32_t *)tmp, list);
+                   (const uint32_t *)off, (const uint32_t *)tmp, list, (int)c.enclose_pending,
+                   (const DevStatus *)c.d_status);
         static unsigned attr_done = 0;
         if (c.device < 32 && !(attr_done & (1u << c.device))) {
             cudaFuncSetAttribute(k_agg_ops, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AG_SMEM);
             attr_done |= 1u << c.device;
         }
         launch(c, "agg_ops", k_agg_ops, dim3(ops_grid(c, O)), dim3(AG_THREADS), AG_SMEM,
-               (const uint32_t *)off, list, in);
+               (const uint32_t *)off, list, in, (int)c.enclose_pending, (const DevStatus *)c.d_status);
         // the ops the pass left: listed with a null or infinite value (redone
         // by k_agg_careful), long ones (the pieces pass); both
         // counts come back with the status
-        const SmallCopy counts{c.h_levels, ctr + 1, 2 * sizeof(uint32_t)};
+        const SmallCopy counts{c.h_small, ctr + 1, 2 * sizeof(uint32_t)};
         if ((st = read_status(c, 1, &counts))) return st;
-        const uint32_t n_dirty = c.h_levels[0], n_long = c.h_levels[1];
+        const uint32_t n_dirty = c.h_small[0], n_long = c.h_small[1];
         status_fresh = n_dirty == 0 && n_long == 0;
         if (n_dirty > 0)
             launch(c, "agg_careful", k_agg_careful, dim3(std::max(1, sms)), dim3(128), 0, (const uint32_t *)off, list,
@@ -1104,11 +1113,11 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
         if (n_long > 0) {
             launch(c, "agg_piece_offsets", k_agg_piece_offsets, dim3(1), dim3(1024), 0, (const uint32_t *)off,
                    (const uint32_t *)longs, (const unsigned *)nlong, 0u, npc, info, hop);
-            const SmallCopy pinfo{c.h_levels, info, 5 * sizeof(uint32_t)};
+            const SmallCopy pinfo{c.h_small, info, 5 * sizeof(uint32_t)};
             if ((st = read_status(c, 1, &pinfo))) return st;
-            pieces = c.h_levels[1];
-            longest = c.h_levels[2];
-            n_huge = c.h_levels[4];
+            pieces = c.h_small[1];
+            longest = c.h_small[2];
+            n_huge = c.h_small[4];
         }
         if (pieces > 0) {
             if (n_huge <= (uint32_t)RADIX_BINS && longest > AG_BLOCK_SORT_MAX && K > 0) {

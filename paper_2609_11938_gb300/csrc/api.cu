@@ -88,24 +88,13 @@ opattr_status ensure_arena(Ctx &c, size_t bytes) {
     return OPATTR_OK;
 }
 
-opattr_status ensure_side(Ctx &c) {
-    if (c.side) return OPATTR_OK;
-    cudaStream_t s = nullptr;
-    cudaEvent_t e[3] = {nullptr, nullptr, nullptr};
-    bool ok = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
-    for (int i = 0; i < 3 && ok; ++i) ok = cudaEventCreateWithFlags(&e[i], cudaEventDisableTiming) == cudaSuccess;
-    if (!ok) {
+int sm_count(Ctx &c) {
+    if (c.sms == 0) {
+        cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, c.device);
         cudaGetLastError();
-        for (cudaEvent_t x : e)
-            if (x) cudaEventDestroy(x);
-        if (s) cudaStreamDestroy(s);
-        return OPATTR_E_CUDA;
+        if (c.sms < 1) c.sms = 1;
     }
-    c.side = s;
-    c.ev_fork = e[0];
-    c.ev_join = e[1];
-    c.ev_join2 = e[2];
-    return OPATTR_OK;
+    return c.sms;
 }
 
 // Up to SMALL_COPIES transfers in one launch, each between mapped pinned host
@@ -167,8 +156,72 @@ opattr_status copy_small(Ctx &c, void *dst, const void *src, size_t bytes, cudaM
     return copy_small_n(c, 1, &cp, kind);
 }
 
-opattr_status reset_status(Ctx &c) {
-    return copy_small(c, c.d_status, c.h_init, sizeof(DevStatus), cudaMemcpyHostToDevice);
+// Zeroes up to ZERO_RUNS runs of words and, with st, resets the status block:
+// one launch where a copy and several memsets would each be one.
+constexpr int ZERO_RUNS = 4;
+struct ZeroRuns {
+    uint32_t *p[ZERO_RUNS];
+    long long n[ZERO_RUNS];
+    int count;
+};
+__global__ void k_reset(DevStatus *st, ZeroRuns z) {
+    pdl_wait();
+    const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    for (int q = 0; q < z.count; ++q) {
+        uint32_t *p = z.p[q];
+        const long long n = z.n[q], n4 = n / 4;
+        if ((reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+            for (long long i = t0; i < n4; i += step) reinterpret_cast<uint4 *>(p)[i] = make_uint4(0, 0, 0, 0);
+            for (long long i = 4 * n4 + t0; i < n; i += step) p[i] = 0;
+        } else {
+            for (long long i = t0; i < n; i += step) p[i] = 0;
+        }
+    }
+    if (!st || blockIdx.x != 0) return;
+    if (threadIdx.x < C_NSLOTS) st->cnt[threadIdx.x] = 0;
+    if (threadIdx.x < MM_NSLOTS)
+        st->mm[threadIdx.x] = threadIdx.x == MM_KSTART_MIN || threadIdx.x == MM_RSTART_MIN   ? LLONG_MAX
+                              : threadIdx.x == MM_KSTART_MAX || threadIdx.x == MM_REND_MAX ? LLONG_MIN
+                                                                                           : 0;
+    if (threadIdx.x < 8) st->kstreams[threadIdx.x] = 0;
+    if (threadIdx.x == 0) st->err = st->flags = st->nlevels = st->pad = 0;
+}
+
+static opattr_status launch_reset(Ctx &c, DevStatus *st, int n, const ZeroRun *z) {
+    if (n < 0 || n > ZERO_RUNS) return OPATTR_E_INVALID_ARG;
+    ZeroRuns a{};
+    int64_t most = 1;
+    for (int q = 0; q < n; ++q) {
+        if (z[q].words <= 0) continue;
+        a.p[a.count] = static_cast<uint32_t *>(z[q].p);
+        a.n[a.count++] = z[q].words;
+        most = std::max(most, z[q].words);
+    }
+    launch(c, "reset", k_reset, dim3(grid_for(most, 256 * 16, REDUCE_GRID)), dim3(256), 0, st, a);
+    return c.last_error == cudaSuccess ? OPATTR_OK : cuda_status(c, c.last_error);
+}
+opattr_status zero_runs(Ctx &c, int n, const ZeroRun *z) { return launch_reset(c, nullptr, n, z); }
+opattr_status reset_status(Ctx &c, int n, const ZeroRun *z) { return launch_reset(c, c.d_status, n, z); }
+
+opattr_status post_status(Ctx &c, int n_extra, const SmallCopy *extra) {
+    if (c.last_error != cudaSuccess) return cuda_status(c, c.last_error);
+    if (n_extra < 0 || n_extra > SMALL_COPIES - 1) return OPATTR_E_INVALID_ARG;
+    SmallCopy cp[SMALL_COPIES];
+    int n = 0;
+    cp[n++] = SmallCopy{c.h_status, c.d_status, sizeof(DevStatus)};
+    for (int q = 0; q < n_extra; ++q) cp[n++] = extra[q];
+    opattr_status st = copy_small_n(c, n, cp, cudaMemcpyDeviceToHost);
+    if (st) return st;
+    if (!c.ev_status && cudaEventCreateWithFlags(&c.ev_status, cudaEventDisableTiming) != cudaSuccess) {
+        c.ev_status = nullptr;
+        return cuda_status(c, cudaGetLastError());
+    }
+    const cudaError_t e = cudaEventRecord(c.ev_status, c.stream);
+    return e == cudaSuccess ? OPATTR_OK : cuda_status(c, e);
+}
+opattr_status await_status(Ctx &c) {
+    const cudaError_t e = cudaEventSynchronize(c.ev_status);
+    return e == cudaSuccess ? OPATTR_OK : cuda_status(c, e);
 }
 
 opattr_status read_status(Ctx &c, int n_extra, const SmallCopy *extra) {
@@ -278,15 +331,13 @@ opattr_status opattr_create(opattr_ctx **out, int device, void *cuda_stream, con
     c.cfg = conf;
     bool fail = cudaMalloc(&c.d_status, sizeof(DevStatus)) != cudaSuccess;
     fail = fail || cudaMallocHost(&c.h_status, sizeof(DevStatus)) != cudaSuccess;
-    fail = fail || cudaMallocHost(&c.h_init, sizeof(DevStatus)) != cudaSuccess;
-    fail = fail || cudaMallocHost(&c.h_levels, sizeof(uint32_t) * (N_LEVELS + 1 + 256)) != cudaSuccess;
+    fail = fail || cudaMallocHost(&c.h_small, sizeof(uint32_t) * SMALL_WORDS) != cudaSuccess;
     fail = fail || cudaMallocHost(&c.h_stage, STAGE_BYTES) != cudaSuccess;
     if (fail) {
         cudaGetLastError();
         if (c.d_status) cudaFree(c.d_status);
         if (c.h_status) cudaFreeHost(c.h_status);
-        if (c.h_init) cudaFreeHost(c.h_init);
-        if (c.h_levels) cudaFreeHost(c.h_levels);
+        if (c.h_small) cudaFreeHost(c.h_small);
         if (c.h_stage) cudaFreeHost(c.h_stage);
         delete x;
         return OPATTR_E_OOM;
@@ -294,26 +345,14 @@ opattr_status opattr_create(opattr_ctx **out, int device, void *cuda_stream, con
     // the pinned buffers are moved by small kernels when the device sees them
     // at their host addresses (unified addressing), by cudaMemcpyAsync if not
     bool mapped = true;
-    for (void *h : {(void *)c.h_status, (void *)c.h_init, (void *)c.h_levels, (void *)c.h_stage}) {
+    for (void *h : {(void *)c.h_status, (void *)c.h_small, (void *)c.h_stage}) {
         void *dp = nullptr;
         mapped = mapped && cudaHostGetDevicePointer(&dp, h, 0) == cudaSuccess && dp == h;
     }
     cudaGetLastError();
     c.host_mapped = mapped;
-    memset(c.h_init, 0, sizeof(DevStatus));
-    c.h_init->mm[MM_KSTART_MIN] = LLONG_MAX;
-    c.h_init->mm[MM_KSTART_MAX] = LLONG_MIN;
-    c.h_init->mm[MM_RSTART_MIN] = LLONG_MAX;
-    c.h_init->mm[MM_REND_MAX] = LLONG_MIN;
-    *c.h_status = *c.h_init;
+    memset(c.h_status, 0, sizeof(DevStatus));
     *out = x;
-    return OPATTR_OK;
-}
-
-// The enclosure's error bits as a status (the order of do_enclose's checks).
-static opattr_status status_from_enclose_err(unsigned err) {
-    if (err & ERR_DEPTH) return OPATTR_E_DEPTH;
-    if (err & ERR_NOT_NESTED) return OPATTR_E_NOT_NESTED;
     return OPATTR_OK;
 }
 
@@ -388,7 +427,7 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
             c.enclose_pending = false;
         }
     } scope(c);
-    // the matching's identity pairing may run beside the enclosure: rows one
+    // the matching's identity pairing may run within the enclosure: rows one
     // for one with the kernels, no layer deduplication, no per-stream rows;
     // then the enclosure's last status read can wait for the aggregation's
     const bool spec = !dedup && !ncu->stream && kernels->n > 0 && kernels->n == ncu->n && kernels->name_id &&
@@ -427,8 +466,14 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
                 const opattr_status s2 = read_status(c);
                 if (s2 < 0) return s2;
             }
-            if (c.h_status->flags & F_LEVEL_FIXUP) continue;          // redone without deferring
-            if (c.h_status->err & (ERR_NOT_NESTED | ERR_DEPTH)) return status_from_enclose_err(c.h_status->err);
+            // redone without deferring
+            if (c.h_status->flags & (F_LEVEL_FIXUP | F_K_UNSORTED | F_R_UNSORTED | F_LEVELS_MANY)) continue;
+            // the enclosure's error before the aggregation's (nesting is only
+            // judged when the range records passed their checks)
+            DevStatus H = *c.h_status;
+            if (H.err & ERR_NOT_NESTED) H.err &= ~ERR_INVALID;
+            const opattr_status ve = enclose_verdict(H, kernels->n);
+            if (ve < 0) return ve;
             if (st >= 0 && (c.h_status->flags & F_NAMES_DIFFER)) {
                 // the names disagree: the matching and the aggregation proper
                 c.order_from_enclose = true;
@@ -483,21 +528,14 @@ void opattr_destroy(opattr_ctx *ctx) {
         if (c.arena) cudaFree(c.arena);
         if (c.d_status) cudaFree(c.d_status);
         if (c.h_status) cudaFreeHost(c.h_status);
-        if (c.h_init) cudaFreeHost(c.h_init);
-        if (c.h_levels) cudaFreeHost(c.h_levels);
+        if (c.h_small) cudaFreeHost(c.h_small);
         if (c.h_stage) cudaFreeHost(c.h_stage);
+        if (c.ev_status) cudaEventDestroy(c.ev_status);
         for (auto &p : c.pending) {
             cudaEventDestroy(p.second.first);
             cudaEventDestroy(p.second.second);
         }
         for (cudaEvent_t e : c.event_pool) cudaEventDestroy(e);
-        if (c.side) {
-            cudaStreamSynchronize(c.side);
-            cudaEventDestroy(c.ev_fork);
-            cudaEventDestroy(c.ev_join);
-            cudaEventDestroy(c.ev_join2);
-            cudaStreamDestroy(c.side);
-        }
         cudaGetLastError();
     }
     delete ctx;

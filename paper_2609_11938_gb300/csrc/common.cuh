@@ -32,7 +32,7 @@ enum FlagBit : unsigned {
     F_OP_DUP = 16u,       // two operator ranges share an op id
     F_AGG_MISS = 32u,     // the owned-range aggregation missed kernels
     F_IDX_NOT_ID = 64u,   // some kernel's ncu row index is neither its own index nor -1
-    F_BUCKETS = 256u,     // times too crowded for the bucketed time sort
+    F_LEVELS_MANY = 128u, // more range levels than the enclosure's common layout holds
 };
 enum CountSlot {
     C_NAMES_MISMATCH = 0,
@@ -61,6 +61,9 @@ struct DevStatus {
     unsigned int flags;
     unsigned long long cnt[C_NSLOTS];
     long long mm[MM_NSLOTS];
+    unsigned int kstreams[8];    // streams with kernels, one bit each (the enclosure's checks)
+    unsigned int nlevels;        // range levels present (the enclosure)
+    unsigned int pad;
 };
 
 // ------------------------------------------------------------------ context
@@ -71,16 +74,14 @@ struct TimingSlot {
 };
 
 constexpr int N_LEVELS = 256 * 32;   // (stream, depth) levels of the enclosure
-constexpr size_t STAGE_BYTES = 32768;  // pinned staging of host-built tables (one copy per call)
+constexpr size_t STAGE_BYTES = 1024;   // pinned staging of host-built tables
+constexpr int SMALL_WORDS = 512;
 
 struct Ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
-    // a second stream for independent chains of one call (the enclosure's
-    // level lists beside its stream partition), with the events that fork
-    // from and join back into `stream`; created on first use
-    cudaStream_t side = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
+    int sms = 0;                     // multiprocessors of the device (sm_count)
+    cudaEvent_t ev_status = nullptr; // a status copy under way (post_status); created on first use
     opattr_config cfg{};
     bool broken = false;
     // scratch arena (bump allocation, reset per call)
@@ -90,12 +91,9 @@ struct Ctx {
     // status block
     DevStatus *d_status = nullptr;
     DevStatus *h_status = nullptr;   // pinned mirror
-    DevStatus *h_init = nullptr;     // pinned reset template
-    uint32_t *h_levels = nullptr;    // pinned host copy of the enclosure's level offsets [N_LEVELS + 1] and
-                                     // kernels per stream [256];
-                                     // the aggregation reuses it for a few values read mid-call
+    uint32_t *h_small = nullptr;     // pinned room for a few values read mid-call [SMALL_WORDS]
     unsigned char *h_stage = nullptr; // pinned staging for small host-built tables [STAGE_BYTES]
-    bool host_mapped = false;        // the four pinned buffers above are addressable from the device as they are
+    bool host_mapped = false;        // the three pinned buffers above are addressable from the device as they are
     // kernel time order as the last enclosure found it (-1 unknown, 0 / 1),
     // and whether the matching may take it instead of checking again (join)
     int enclose_k_sorted = -1;
@@ -108,9 +106,9 @@ struct Ctx {
     size_t arena_keep = 0;
     // launch accounting
     // within a join: the matching's identity pairing (rows equal to the
-    // kernels in time order), launched beside the enclosure when spec_k > 0;
-    // spec_ran: it ran in the enclosure's last attempt, its verdict in the
-    // status the enclosure read last
+    // kernels in time order), done by the enclosure's checking pass when
+    // spec_k > 0; spec_ran: it was, its verdict in the status the enclosure
+    // read last
     const uint32_t *spec_kname = nullptr, *spec_nname = nullptr;
     int32_t *spec_idx = nullptr;
     uint8_t *spec_kind = nullptr;
@@ -157,27 +155,10 @@ struct Need {
 };
 
 opattr_status ensure_arena(Ctx &c, size_t bytes);
-opattr_status ensure_side(Ctx &c);       // the side stream and its events
-// Algorithm 1's identity pairing on c.stream (match.cu): kernel j's row is
-// row j, F_NAMES_DIFFER set where the names disagree
-void launch_identity_match(Ctx &c, const uint32_t *kname, const uint32_t *nname, int64_t K, int32_t *out_idx,
-                           uint8_t *out_kind);
-
-// Launches and async copies within the scope go to stream s (c.stream is
-// swapped and restored).
-struct OnStream {
-    Ctx &c;
-    cudaStream_t prev;
-    OnStream(Ctx &ctx, cudaStream_t s) : c(ctx), prev(ctx.stream) { c.stream = s; }
-    ~OnStream() { c.stream = prev; }
-    OnStream(const OnStream &) = delete;
-    OnStream &operator=(const OnStream &) = delete;
-};
-// `to` waits for the work issued to `from` so far (through event e).
-inline void stream_after(cudaStream_t to, cudaStream_t from, cudaEvent_t e) {
-    cudaEventRecord(e, from);
-    cudaStreamWaitEvent(to, e, 0);
-}
+int sm_count(Ctx &c);
+// The status of an enclosure that read `H` (a NOT_NESTED found beside
+// F_LEVEL_FIXUP does not count: the run on sorted ranges decides).
+opattr_status enclose_verdict(const DevStatus &H, int64_t K);
 // A small transfer between the context's pinned host buffers and device
 // memory, on c.stream.  When those buffers are mapped into the device's
 // address space (opattr_create checks), a small kernel moves the bytes through
@@ -192,7 +173,19 @@ struct SmallCopy {
 };
 // Several such transfers of one direction, four to a launch.
 opattr_status copy_small_n(Ctx &c, int count, const SmallCopy *cp, cudaMemcpyKind kind);
-opattr_status reset_status(Ctx &c);
+// Words to be zeroed, up to four runs in one launch; with reset_status in the
+// launch that resets the status block.
+struct ZeroRun {
+    void *p;
+    int64_t words;
+};
+opattr_status zero_runs(Ctx &c, int n, const ZeroRun *z);
+opattr_status reset_status(Ctx &c, int n = 0, const ZeroRun *z = nullptr);
+// The status block sent to the host without waiting (with up to three more
+// transfers in the launch), and the wait for it alone: work queued after
+// post_status goes on meanwhile.
+opattr_status post_status(Ctx &c, int n_extra = 0, const SmallCopy *extra = nullptr);
+opattr_status await_status(Ctx &c);
 // The status block back to the host (with up to three more device->host
 // transfers in the same launch), then a stream synchronize.
 opattr_status read_status(Ctx &c, int n_extra = 0, const SmallCopy *extra = nullptr);

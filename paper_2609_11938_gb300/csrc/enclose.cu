@@ -1,22 +1,25 @@
 // enclose.cu -- Algorithm 2 (NVTX enclosure attribution, Sec. 3.5) on the GPU.
 //
-// Data layout.  Ranges are regrouped into per-(stream, depth) level lists,
-// each in (start, end, index) order: lvl_start / lvl_end (i64) and lvl_info
-// (u32: range index in the low 30 bits, kind in the top 2: 0 operator,
-// 1 non-op, 2 structural).  lvl_off[level] gives the list bounds, level =
-// stream * 32 + depth.  Within a level ranges are disjoint or touching, so
-// "the last range with start <= T" is the only one that can contain T.
-//
-// Kernels are answered stream by stream, in tiles of consecutive kernels of
-// one stream (the per-stream tiles section below).  A window table bounds,
-// per tile and depth, the ranges the tile can hit; the enclosure kernel
-// stages those windows in shared memory as 32-bit times relative to the
-// tile's first kernel and sweeps the tile's kernels in time order, walking
-// depths outward-in (0, 1, ...) until a depth has no containing range.  The
-// walk state needs no stack: a structural range resets the collection
-// (everything above it is beyond the cut); an operator becomes the innermost
-// answer and counts; a non-op range is passed over.
+// Kernels in time order and ranges in start order are walked together, as one
+// merged sequence of events in which a range comes before the kernels that
+// start no earlier.  The sequence is cut into tiles of equal length, runs of
+// tiles into parts, one block each; a block needs, besides its own events, only
+// the last range before it on every level (stream, depth), because within a
+// level ranges are disjoint or touching, so "the last range with start <= T"
+// is the only one that can contain T.  Three launches, no host decision
+// between them:
+//   enc_parts  checks kernel and range records (order, intervals, depths);
+//              each tile's place in the merged sequence, and the last range of
+//              every level inside each part
+//   enc_carry  those, made a running maximum over the parts (many parts only)
+//   enclose    the parts, tile by tile: parents, chains and laminar checks of
+//              the tile's ranges in shared memory, then its kernels
+// Nothing is regrouped in device memory: kernels and ranges are read where
+// they lie, in order, and results are written in order.  Records out of order
+// are found by enc_parts (the other two then leave at once), sorted, and the
+// last two run again on the sorted view.
 #include <algorithm>
+#include <type_traits>
 
 #include "sort.cuh"
 #include "util.cuh"
@@ -25,588 +28,915 @@ namespace opattr {
 
 constexpr int LEVELS = N_LEVELS;
 constexpr uint32_t KIND_OP = 0, KIND_NONOP = 1, KIND_STRUCT = 2;
+constexpr uint32_t POS_MASK = 0x3FFFFFFFu;
 
 __device__ __forceinline__ uint32_t kind_of(uint32_t op) {
     return op == OPATTR_OP_STRUCTURAL ? KIND_STRUCT : (op == OPATTR_OP_NONOP ? KIND_NONOP : KIND_OP);
 }
 
-// ------------------------------------------------------------------ range checks
-// end >= start, depth <= 31, start order of the array, min start / max end,
-// and a histogram of level keys (per block in shared memory, flushed with
-// one global atomic per non-empty bin).
-constexpr int RCHK_THREADS = 256;
-constexpr int RCHK_ITEMS = 16;
-__global__ void __launch_bounds__(RCHK_THREADS) k_check_ranges(const uint8_t *__restrict__ stream,
-                                                               const int64_t *__restrict__ start,
-                                                               const int64_t *__restrict__ end,
-                                                               const uint8_t *__restrict__ depth, int64_t n,
-                                                               uint32_t *__restrict__ level_hist, DevStatus *st) {
-    pdl_wait();
-    __shared__ uint32_t h[LEVELS];
-    __shared__ int flags;
-    __shared__ long long smin, smax;
-    for (int i = threadIdx.x; i < LEVELS; i += RCHK_THREADS) h[i] = 0;
-    if (threadIdx.x == 0) { flags = 0; smin = LLONG_MAX; smax = LLONG_MIN; }
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * RCHK_THREADS * RCHK_ITEMS;
-    long long mn = LLONG_MAX, mx = LLONG_MIN;
-    int f = 0;
-    constexpr int B = 4;                    // items per batch, loads issued together
-    for (int it0 = 0; it0 < RCHK_ITEMS; it0 += B) {
-        long long sv[B], ev[B], nv[B];
-        unsigned dv[B], stv[B];
-#pragma unroll
-        for (int u = 0; u < B; ++u) {
-            const int64_t i = base + (it0 + u) * RCHK_THREADS + threadIdx.x;
-            const bool in = i < n;
-            sv[u] = in ? start[i] : 0;
-            ev[u] = in ? end[i] : 0;
-            nv[u] = i + 1 < n ? start[i + 1] : LLONG_MAX;
-            dv[u] = in ? depth[i] : 0u;
-            stv[u] = in ? stream[i] : 0u;
-        }
-#pragma unroll
-        for (int u = 0; u < B; ++u) {
-            const int64_t i = base + (it0 + u) * RCHK_THREADS + threadIdx.x;
-            if (i >= n) continue;
-            if (ev[u] < sv[u]) f |= 1;
-            if (dv[u] >= OPATTR_MAX_DEPTH) f |= 2;
-            if (nv[u] < sv[u]) f |= 4;
-            mn = sv[u] < mn ? sv[u] : mn;
-            mx = ev[u] > mx ? ev[u] : mx;
-            if (dv[u] < OPATTR_MAX_DEPTH) atomicAdd(&h[stv[u] * 32 + dv[u]], 1u);
-        }
-    }
-    if (f) atomicOr(&flags, f);
-    atomicMin(&smin, mn);
-    atomicMax(&smax, mx);
-    __syncthreads();
-    for (int i = threadIdx.x; i < LEVELS; i += RCHK_THREADS)
-        if (h[i]) atomicAdd(&level_hist[i], h[i]);
-    if (threadIdx.x == 0) {
-        if (flags & 1) set_err(st, ERR_INVALID);
-        if (flags & 2) set_err(st, ERR_DEPTH);
-        if (flags & 4) set_flag(st, F_R_UNSORTED);
-        atomicMin(&st->mm[MM_RSTART_MIN], smin);
-        atomicMax(&st->mm[MM_REND_MAX], smax);
-    }
-}
-
-// ------------------------------------------------------------------ level lists
-__global__ void k_level_keys(const uint8_t *__restrict__ stream, const uint8_t *__restrict__ depth,
-                             const uint32_t *__restrict__ perm, int64_t n, uint32_t *__restrict__ keys) {
-    pdl_wait();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t r = perm ? perm[i] : i;
-        keys[i] = (uint32_t)stream[r] * 32u + depth[r];
-    }
-}
-// The level lists' order key of range i: its start, then 0 for a
-// zero-length range and 1 for a longer one.  Within a level of laminar
-// ranges two ranges share a start only if all but the last of them have
-// zero length, so a stable sort on this key puts every level in (start,
-// end, index) order -- the order of Algorithm 2's one representative per
-// depth -- in one sort; two longer ranges sharing a start in one level are
-// out of that order only when they overlap, which the validation reports.
-__global__ void k_range_start_key(const int64_t *__restrict__ start, const int64_t *__restrict__ end, int64_t n,
-                                  long long tmin, uint64_t *__restrict__ keys) {
-    pdl_wait();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        keys[i] = ((uint64_t)(start[i] - tmin) << 1) | (end[i] > start[i] ? 1u : 0u);
-}
-__global__ void k_level_gather(const int64_t *__restrict__ start, const int64_t *__restrict__ end,
-                               const uint32_t *__restrict__ op, const uint32_t *__restrict__ perm, int64_t n,
-                               int64_t *__restrict__ ls, int64_t *__restrict__ le, uint32_t *__restrict__ li) {
-    pdl_wait();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t r = perm[i];
-        ls[i] = start[r];
-        le[i] = end[r];
-        li[i] = r | (kind_of(op[r]) << 30);
-    }
-}
-
-// The same partition in one counting pass when at most 256 levels are
-// present: range i's digit is its compact level id (levels numbered in
-// (stream, depth) order, so a stable partition by compact id is the stable
-// sort by level key), and k_level_place writes each range's level-list
-// entry in place of the key sort and the gather.
-struct LevelDigit {
-    const uint8_t *stream, *depth;
-    const uint8_t *cmap;        // [LEVELS] compact id of each present level
-    const uint32_t *perm;       // NULL = array order
-    __device__ __forceinline__ unsigned operator()(int64_t i) const {
-        const uint32_t r = perm ? perm[i] : (uint32_t)i;
-        return cmap[stream[r] * 32u + depth[r]];
-    }
-};
-// The placing pass: the digit-rank of the tile's ranges gives each its
-// place in the tile sorted by compact level; the range's tile index is
-// staged there in shared memory, then each level's run of the tile goes out
-// to consecutive addresses (one coalesced write per run instead of one
-// scattered write per range), the range fields read back from the tile just
-// loaded (L1 / L2).  Same tiles as digit_offsets.
-struct PlaceSmem {
-    uint16_t lidx[RADIX_TILE];
-    uint8_t dig[RADIX_TILE];
-    uint32_t wcnt[(RADIX_THREADS / 32) * RADIX_BINS];
-    uint32_t dstart[RADIX_BINS];
-    uint32_t gbase[RADIX_BINS];
-    uint32_t wbuf[33];
-};
-__global__ void __launch_bounds__(RADIX_THREADS) k_level_place(LevelDigit digit, const int64_t *__restrict__ start,
-                                                               const int64_t *__restrict__ end,
-                                                               const uint32_t *__restrict__ op, int64_t n,
-                                                               const uint32_t *__restrict__ offs, int64_t ntiles,
-                                                               int64_t *__restrict__ ls, int64_t *__restrict__ le,
-                                                               uint32_t *__restrict__ li) {
-    pdl_wait();
-    __shared__ PlaceSmem S;
-    const unsigned w = threadIdx.x >> 5, lane = lane_id();
-    for (int i = threadIdx.x; i < (RADIX_THREADS / 32) * RADIX_BINS; i += RADIX_THREADS) S.wcnt[i] = 0;
-    __syncthreads();
-    const int64_t tile0 = (int64_t)blockIdx.x * RADIX_TILE;
-    const int64_t base = tile0 + w * (RADIX_TILE / 8);
-    unsigned dg[RADIX_ITEMS];
-    uint32_t rank[RADIX_ITEMS];
-    const unsigned lt = lanemask_lt();
-    unsigned peers[RADIX_ITEMS];
-#pragma unroll
-    for (int it = 0; it < RADIX_ITEMS; ++it) {        // digits and peer groups first: independent
-        const int64_t i = base + it * 32 + lane;
-        const unsigned d = i < n ? digit(i) : (unsigned)RADIX_BINS;
-        peers[it] = warp_peers8(d, d < RADIX_BINS);
-        dg[it] = d;
-    }
-#pragma unroll
-    for (int it = 0; it < RADIX_ITEMS; ++it) {
-        const unsigned d = dg[it];
-        const unsigned before = d < RADIX_BINS ? S.wcnt[w * RADIX_BINS + d] : 0u;
-        __syncwarp();
-        if (d < RADIX_BINS && (peers[it] & lt) == 0) S.wcnt[w * RADIX_BINS + d] = before + __popc(peers[it]);
-        __syncwarp();
-        rank[it] = before + __popc(peers[it] & lt);
-    }
-    __syncthreads();
-    uint32_t tot;
-    {
-        // RADIX_THREADS == RADIX_BINS: thread d owns digit d
-        const unsigned d = threadIdx.x;
-        uint32_t sum = 0;
-#pragma unroll
-        for (int q = 0; q < RADIX_THREADS / 32; ++q) {
-            const uint32_t x = S.wcnt[q * RADIX_BINS + d];
-            S.wcnt[q * RADIX_BINS + d] = sum;
-            sum += x;
-        }
-        tot = sum;
-    }
-    const uint32_t ds = block_exclusive_scan<uint32_t>(tot, S.wbuf, (uint32_t *)nullptr);
-    S.dstart[threadIdx.x] = ds;
-    S.gbase[threadIdx.x] = offs[(int64_t)threadIdx.x * ntiles + blockIdx.x];
-    __syncthreads();
-#pragma unroll
-    for (int it = 0; it < RADIX_ITEMS; ++it) {
-        const int64_t i = base + it * 32 + lane;
-        const unsigned d = dg[it];
-        if (d < RADIX_BINS) {
-            const uint32_t p = S.dstart[d] + S.wcnt[w * RADIX_BINS + d] + rank[it];
-            S.lidx[p] = (uint16_t)(i - tile0);
-            S.dig[p] = (uint8_t)d;
-        }
-    }
-    __syncthreads();
-    const int cnt = (int)(n - tile0 < RADIX_TILE ? n - tile0 : RADIX_TILE);
-    constexpr int U = 4;                    // entries per thread per round, loads issued together
-    for (int j0 = threadIdx.x; j0 < cnt; j0 += RADIX_THREADS * U) {
-        uint32_t r[U];
-        long long sv[U], ev[U];
-        uint32_t ov[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int j = j0 + u * RADIX_THREADS;
-            const int64_t i = tile0 + (j < cnt ? S.lidx[j] : 0);
-            r[u] = digit.perm ? digit.perm[i] : (uint32_t)i;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            sv[u] = start[r[u]];
-            ev[u] = end[r[u]];
-            ov[u] = op[r[u]];
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int j = j0 + u * RADIX_THREADS;
-            if (j >= cnt) continue;
-            const unsigned d = S.dig[j];
-            const int64_t o = (int64_t)S.gbase[d] + (j - S.dstart[d]);
-            ls[o] = sv[u];
-            le[o] = ev[u];
-            li[o] = r[u] | (kind_of(ov[u]) << 30);
-        }
-    }
-}
-
-// Laminar checks over level positions: adjacent pairs of a level, and the
-// parent of every range at depth > 0 (the last range of level (s, d-1) that
-// starts no later; it must end no earlier).  A thread takes VL_PER
-// consecutive positions: starts do not decrease along a level, so the parent
-// is searched once and then followed forward.
-constexpr int VL_PER = 8;
-__global__ void k_validate_levels(const uint8_t *__restrict__ stream, const uint8_t *__restrict__ depth,
-                                  const int64_t *__restrict__ ls, const int64_t *__restrict__ le,
-                                  const uint32_t *__restrict__ li, const uint32_t *__restrict__ lvl_off, int64_t n,
-                                  DevStatus *st) {
-    pdl_wait();
-    bool err = false, fix = false;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x * VL_PER;
-    for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * VL_PER; i0 < n; i0 += stride) {
-        const int64_t i1 = i0 + VL_PER < n ? i0 + VL_PER : n;
-        int64_t lend = -1, plo = 0, phi = 0, pp = 0;
-        uint32_t d = 0;
-        bool have_parent = false;
-        long long a = ls[i0], b = le[i0];
-        for (int64_t i = i0; i < i1; ++i) {
-            if (i >= lend) {                     // the level of position i
-                const uint32_t r = li[i] & 0x3FFFFFFFu;
-                const uint32_t L = (uint32_t)stream[r] * 32u + depth[r];
-                d = depth[r];
-                lend = lvl_off[L + 1];
-                if (d > 0) { plo = lvl_off[L - 1]; phi = lvl_off[L]; }
-                have_parent = false;
-            }
-            long long a2 = 0, b2 = 0;
-            if (i + 1 < n) { a2 = ls[i + 1]; b2 = le[i + 1]; }
-            if (i + 1 < lend) {
-                if (a2 == a && b2 < b) fix = true;
-                else if (b > a2) err = true;
-            }
-            if (d > 0) {
-                if (!have_parent) {              // last parent-level position with start <= a
-                    int64_t x = plo, y = phi;
-                    while (x < y) {
-                        const int64_t m = (x + y) >> 1;
-                        if (ls[m] <= a) x = m + 1; else y = m;
-                    }
-                    pp = x - 1;
-                    have_parent = true;
-                } else {
-                    while (pp + 1 < phi && ls[pp + 1] <= a) ++pp;
-                }
-                if (pp < plo || le[pp] < b) err = true;
-            }
-            a = a2;
-            b = b2;
-        }
-    }
-    if (__any_sync(0xffffffffu, fix) && lane_id() == 0) set_flag(st, F_LEVEL_FIXUP);
-    if (__any_sync(0xffffffffu, err) && lane_id() == 0) set_err(st, ERR_NOT_NESTED);
-}
-
-// ------------------------------------------------------------------ per-stream tiles
-// The enclosure answers kernels stream by stream.  psk holds every kernel
-// index regrouped by stream: a stable partition of the time-ordered kernels,
-// so each stream's kernels are in time order, streams one after another
-// (stream s from koff[s]).  Each stream's run is cut into tiles of EN_TILE
-// kernels; tile r of stream s has the stream-major index u = toff[s] + r.
-// Tiles are launched round-robin over the streams (tile r of every stream
-// before tile r + 1 of any), so the tiles in flight cover one window of time
-// and their gathers of start times and scattered result writes share sectors
-// in L2.
-constexpr int EN_THREADS = 128;
-constexpr int EN_PER = 16;                        // consecutive kernels one thread sweeps
-constexpr int EN_TILE = EN_THREADS * EN_PER;      // kernels of one stream per tile
-constexpr int EN_WIN = 3072;                      // staged range entries per tile
-constexpr int EN_RD = 8;                          // depths whose sweep state stays in registers
-
-// The stream of the kernel at time position i (as its compact id: streams
-// with kernels numbered in order), and its place in psk.
-struct TimeStreamDigit {
-    const uint8_t *stream;
-    const uint32_t *korder;     // time order, NULL = array order
-    const uint8_t *scmap;       // [256] compact id of a stream with kernels
-    __device__ __forceinline__ unsigned operator()(int64_t i) const {
-        return scmap[stream[korder ? korder[i] : (uint32_t)i]];
-    }
-};
-// The stream of kernel i in array order (the kernels in time order).
-struct ArrayStreamDigit {
-    const uint8_t *stream;
-    __device__ __forceinline__ unsigned operator()(int64_t i) const { return stream[i]; }
-};
-struct PlaceByStream {
-    const uint32_t *korder;
-    uint32_t *psk;
-    __device__ __forceinline__ unsigned operator()(int64_t i, uint32_t dest, unsigned) const {
-        psk[dest] = korder ? korder[i] : (uint32_t)i;
-        return 0u;
-    }
-    __device__ __forceinline__ void done(unsigned) const {}
-};
-
-// Window of every (tile, depth): P[u * 32 + d] = (last position of level
-// (s, d) with start <= the tile's first time, last position with start <= its
-// last time), relative to the level's start, -1 for none.  Lane d of a warp
-// takes depth d of one tile.  The warp also places the tile in the launch
-// order: tile u = toff[s] + r goes to
-//   sum over streams q of min(tiles of q, r)  +  #{q < s : tiles of q > r},
-// tinfo[position] = s | r << 8.
-__global__ void k_stream_windows(const int64_t *__restrict__ ls, const uint32_t *__restrict__ lvl_off,
-                                 const uint8_t *__restrict__ ndep, const uint32_t *__restrict__ toff,
-                                 const uint32_t *__restrict__ koff, const uint32_t *__restrict__ kcnt,
-                                 const uint32_t *__restrict__ psk, const int64_t *__restrict__ k_start, int64_t nt,
-                                 int2 *__restrict__ P, uint32_t *__restrict__ tinfo) {
-    pdl_wait();
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nt * 32; q += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t u = q >> 5;
-        const int d = (int)(q & 31);
-        int lo = 0, hi = 256;
-        while (hi - lo > 1) {
-            const int m = (lo + hi) >> 1;
-            if (toff[m] <= (uint32_t)u) lo = m; else hi = m;
-        }
-        const int sid = lo;
-        {
-            // the tile's launch position: each lane adds the terms of eight streams
-            const uint32_t r = (uint32_t)u - toff[sid];
-            uint32_t p = 0;
-            for (int qs = d; qs < 256; qs += 32) {
-                const uint32_t c = toff[qs + 1] - toff[qs];
-                p += (c < r ? c : r) + (qs < sid && c > r ? 1u : 0u);
-            }
-            p = warp_sum<uint32_t>(p);
-            if (d == 0) tinfo[p] = (uint32_t)sid | (r << 8);
-        }
-        if (d >= ndep[sid]) continue;
-        const int64_t pos0 = (u - toff[sid]) * (int64_t)EN_TILE;
-        const int64_t cnt = (int64_t)kcnt[sid] - pos0 < EN_TILE ? (int64_t)kcnt[sid] - pos0 : EN_TILE;
-        const long long tf = k_start[psk[koff[sid] + pos0]], tl = k_start[psk[koff[sid] + pos0 + cnt - 1]];
-        const int64_t L0 = lvl_off[sid * 32 + d], L1 = lvl_off[sid * 32 + d + 1];
-        int64_t x = L0, y = L1;                    // first position with start > tf
-        while (x < y) {
-            const int64_t m = (x + y) >> 1;
-            if (ls[m] <= tf) x = m + 1; else y = m;
-        }
-        const int64_t a = x;
-        y = L1;                                    // first position with start > tl (at or after a)
-        while (x < y) {
-            const int64_t m = (x + y) >> 1;
-            if (ls[m] <= tl) x = m + 1; else y = m;
-        }
-        P[q] = make_int2((int)(a - L0 - 1), (int)(x - L0 - 1));
-    }
-}
-
-struct EncArgs {
+// Kernels in time order, ranges in start order: the caller's arrays, or the
+// sorted view of records out of order (kernels as the sorted time keys,
+// ranges as sorted copies; korder / perm give the caller's indices).
+struct EncView {
     const int64_t *k_start;
-    const uint32_t *psk, *tinfo, *toff, *koff, *kcnt;
-    const uint8_t *ndep;
-    const int64_t *ls, *le;
-    const uint32_t *li;
-    const uint32_t *lvl_off;    // [LEVELS + 1]
-    const int2 *P;              // [tiles * 32]
-    int32_t *out_range;
-    uint8_t *out_nop;
+    const uint8_t *k_stream;
+    const uint64_t *k_key;       // (start - k_tmin) << k_sbits | compact stream id, or NULL
+    long long k_tmin;
+    int k_sbits;
+    const uint8_t *k_unmap;      // stream of each compact id
+    const uint32_t *korder;      // NULL = array order
+    int64_t K;
+    const int64_t *r_start, *r_end;
+    const uint8_t *r_stream, *r_depth;
+    const uint32_t *r_op;
+    const uint32_t *perm;        // NULL = array order
+    int64_t R;
+
+    template <bool KEYS>
+    __device__ __forceinline__ long long time(int64_t i) const {
+        return KEYS ? k_tmin + (long long)(k_key[i] >> k_sbits) : k_start[i];
+    }
+    template <bool KEYS>
+    __device__ __forceinline__ unsigned stream(int64_t i) const {
+        return KEYS ? k_unmap[(unsigned)k_key[i] & ((1u << k_sbits) - 1u)] : k_stream[i];
+    }
 };
 
-struct EncSmem {
-    uint32_t ws[EN_WIN];        // staged start, relative to the tile's first time (+1, clamped)
-    uint32_t we[EN_WIN];        // staged end, same encoding
-    uint32_t wi[EN_WIN];        // staged lvl_info
-    int woff[32], wcnt[32];     // per depth: first staged entry and count
-    int wlev[32];               // per depth: level position of the window's first entry
-    int nwin;
+// ------------------------------------------------------------------ parts
+// The merged events of tile i of n: [tile_event(i), tile_event(i + 1)).
+// Part b of the tiles' parts is tiles [b * tp, (b + 1) * tp).
+__device__ __forceinline__ int64_t tile_event(int64_t i, int64_t n, int64_t events) {
+    return (int64_t)((unsigned long long)events * (unsigned long long)i / (unsigned long long)n);   // below 2^52
+}
+
+// Ranges among the first d merged events, by one warp: 32 probes a round.  A
+// range precedes the kernels that start no earlier.  Ends in [0, R] whatever
+// the order of the records.
+template <bool KEYS>
+__device__ __forceinline__ int64_t ranges_before(const EncView &V, int64_t d) {
+    int64_t lo = d > V.K ? d - V.K : 0, hi = d < V.R ? d : V.R;
+    const unsigned lane = lane_id();
+    while (lo < hi) {
+        const int64_t step = (hi - lo + 31) >> 5;
+        const int64_t p = lo + (int64_t)lane * step;
+        const bool before = p < hi && V.r_start[p] <= V.time<KEYS>(d - p - 1);
+        const unsigned m = ~__ballot_sync(0xffffffffu, before);
+        const int c = m ? __ffs(m) - 1 : 32;          // lanes 0 .. c - 1 lie before
+        if (c == 0) return lo;
+        const int64_t nh = lo + (int64_t)c * step;
+        lo = lo + (int64_t)(c - 1) * step + 1;
+        hi = nh < hi ? nh : hi;
+    }
+    return lo;
+}
+
+// What enc_parts checks and, within a join, the matching's identity pairing
+// (row j for kernel j), written in the same pass over the kernels.
+struct EncCheck {
+    const uint32_t *kname, *nname;       // NULL: no pairing
+    int32_t *idx;
+    uint8_t *kind;                       // may be NULL
+    int vec;                             // kernel arrays aligned for 16-byte accesses
+    int pair_vec;                        // the pairing's arrays too
 };
 
-__device__ __forceinline__ uint32_t rel32(long long x, long long base) {
-    long long v = x - base + 1;
-    return v <= 0 ? 0u : (v >= 0xFFFFFFFFll ? 0xFFFFFFFFu : (uint32_t)v);
-}
-
-// Algorithm 2's walk over one depth's representative, outward-in: a
-// structural range resets the collection (everything above it is beyond the
-// cut), an operator becomes the innermost answer and counts, a non-op range
-// is passed over.
-__device__ __forceinline__ void walk_step(uint32_t info, int32_t &ans, int &nop) {
-    const uint32_t kind = info >> 30;
-    if (kind == KIND_STRUCT) { ans = -1; nop = 0; }
-    else if (kind == KIND_OP) { ans = (int32_t)(info & 0x3FFFFFFFu); nop++; }
-}
-
-// One tile of one stream.  Thread t sweeps the tile's kernels
-// [t * EN_PER, (t + 1) * EN_PER) in time order, keeping per depth (the first
-// EN_RD in registers) the last staged range starting at or before the
-// current kernel: its position, end and info, and the next range's start.  A
-// depth is searched once at the thread's first kernel and afterwards moves
-// only when the next start is passed, so a kernel usually costs one
-// comparison per depth.  The walk over the tracked depths runs for every
-// kernel without branches (threads of a warp stay together; redoing it only
-// when something changed saves less than the divergence costs); deeper
-// levels are searched when the walk reaches them.  A tile whose windows outgrow the
-// staging, or whose kernels span 2^32 ns or more (relative times no longer
-// fit), searches the global level lists instead.
-__global__ void __launch_bounds__(EN_THREADS) k_enclose(EncArgs A) {
+constexpr int EP_THREADS = 256;
+constexpr int EP_G = 8;                  // consecutive kernels of a thread
+// One block per part of tp tiles.  With CHECK it also verifies an equal share of the
+// records as they lie: kernel order (start, stream), range intervals, depths
+// and start order, the smallest and largest times, the streams with kernels
+// and the depths present on every stream.  Then the tiles' bounds in the
+// merged sequence (tile_r: ranges before each tile) and, in shared memory, the
+// last range of every level among the part's ranges, written as a row of `rows`
+// up to the highest level present (row_len; position + 1, 0 for none).
+//
+// Bound by HBM: 9 bytes per kernel and 18 per range (21 more per kernel with
+// the pairing), each read once.
+template <bool CHECK, bool KEYS>
+__global__ void __launch_bounds__(EP_THREADS) k_enc_parts(EncView V, EncCheck C, int64_t parts, int tp,
+                                                          uint32_t *__restrict__ tile_r, uint32_t *__restrict__ rows,
+                                                          uint32_t *__restrict__ row_len,
+                                                          uint32_t *__restrict__ lvlmask, DevStatus *st) {
     pdl_wait();
-    __shared__ EncSmem S;
-    const uint32_t info = A.tinfo[blockIdx.x];
-    const int sid = (int)(info & 0xFFu);
-    const uint32_t r = info >> 8;
-    const int64_t u = A.toff[sid] + r;
-    const int64_t pos0 = (int64_t)r * EN_TILE;
-    const int cnt = (int)((int64_t)A.kcnt[sid] - pos0 < EN_TILE ? (int64_t)A.kcnt[sid] - pos0 : EN_TILE);
-    const uint32_t *tk = A.psk + A.koff[sid] + pos0;         // the tile's kernels in time order
-    const int nd = A.ndep[sid];
-    const long long tbase = A.k_start[tk[0]], tlast = A.k_start[tk[cnt - 1]];
-    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
-    if (warp == 0) {
-        const int d = (int)lane;
-        int c = 0, first = 0;
-        if (d < nd) {
-            const int2 w = A.P[u * 32 + d];
-            first = w.x < 0 ? 0 : w.x;
-            c = w.y < 0 ? 0 : w.y - first + 1;
+    __shared__ uint32_t last[LEVELS];
+    __shared__ uint32_t dmask[256];
+    __shared__ uint8_t kseen[256];
+    __shared__ int flags_s;
+    __shared__ long long mm_s[4];
+    __shared__ int64_t bound[2];
+    __shared__ uint32_t top_s;
+    const int tid = threadIdx.x;
+    const int64_t b = blockIdx.x;
+    const unsigned lane = lane_id(), warp = tid >> 5;
+    for (int i = tid; i < LEVELS; i += EP_THREADS) last[i] = 0;
+    if (CHECK) {
+        for (int i = tid; i < 256; i += EP_THREADS) {
+            dmask[i] = 0;
+            kseen[i] = 0;
         }
-        const int incl = warp_inclusive_scan(c);
-        S.woff[d] = incl - c;
-        S.wcnt[d] = c;
-        S.wlev[d] = (d < nd ? (int)A.lvl_off[sid * 32 + d] : 0) + first;
-        if (d == 31) S.nwin = incl;
+        if (tid == 0) {
+            flags_s = 0;
+            mm_s[0] = mm_s[2] = LLONG_MAX;
+            mm_s[1] = mm_s[3] = LLONG_MIN;
+        }
     }
+    if (tid == 0) top_s = 0;
     __syncthreads();
-    const bool slow = S.nwin > EN_WIN || (tlast - tbase) >= 0xFFFFFFF0ll;
-    if (slow) {
-        // global searches inside each depth's window
-        for (int j = threadIdx.x; j < cnt; j += EN_THREADS) {
-            const uint32_t k = tk[j];
-            const long long T = A.k_start[k];
-            int32_t ans = -1;
-            int nop = 0;
-            for (int d = 0; d < nd; ++d) {
-                int64_t x = S.wlev[d], y = x + S.wcnt[d];
-                const int64_t o = x;
-                while (x < y) {
-                    const int64_t m = (x + y) >> 1;
-                    if (A.ls[m] <= T) x = m + 1; else y = m;
+    if (CHECK) {
+        enum { U_KERN = 1, U_RANGE = 2, BAD_END = 4, BAD_DEPTH = 8, NAMES = 16 };
+        int f = 0;
+        long long kmn = LLONG_MAX, kmx = LLONG_MIN, rmn = LLONG_MAX, rmx = LLONG_MIN;
+        const int64_t kshare = ((V.K + parts - 1) / parts + EP_G - 1) / EP_G * EP_G;
+        const int64_t kb = b * kshare, ke = kb + kshare < V.K ? kb + kshare : V.K;
+        for (int64_t i0 = kb + (int64_t)tid * EP_G; i0 < ke; i0 += EP_THREADS * EP_G) {
+            long long t[EP_G + 1];
+            unsigned s[EP_G + 1];
+            const bool whole = i0 + EP_G <= V.K;
+            if (C.vec && whole) {
+                const longlong2 *p = reinterpret_cast<const longlong2 *>(V.k_start + i0);
+#pragma unroll
+                for (int q = 0; q < EP_G / 2; ++q) {
+                    const longlong2 x = p[q];
+                    t[2 * q] = x.x;
+                    t[2 * q + 1] = x.y;
                 }
-                if (x == o || A.le[x - 1] < T) break;
-                walk_step(A.li[x - 1], ans, nop);
-            }
-            A.out_range[k] = ans;
-            if (A.out_nop) A.out_nop[k] = (uint8_t)nop;
-        }
-        return;
-    }
-    // stage the windows: one warp per depth, each depth's entries contiguous
-    for (int d = (int)warp; d < nd; d += EN_THREADS / 32) {
-        const int c = S.wcnt[d], o = S.woff[d];
-        const int64_t g0 = S.wlev[d];
-        for (int e = (int)lane; e < c; e += 32) {
-            S.ws[o + e] = rel32(A.ls[g0 + e], tbase);
-            S.we[o + e] = rel32(A.le[g0 + e], tbase);
-            S.wi[o + e] = A.li[g0 + e];
-        }
-    }
-    __syncthreads();
-    constexpr uint32_t NONE_T = 0xFFFFFFFFu;
-    const int j0 = (int)threadIdx.x * EN_PER;
-    const int j1 = j0 + EN_PER < cnt ? j0 + EN_PER : cnt;
-    if (j0 >= j1) return;
-    int pos[EN_RD];                               // window position of the depth's range, -1 none
-    uint32_t nxt[EN_RD], cend[EN_RD], cinf[EN_RD]; // next start; end and info of the range
-    constexpr int B = 4;                          // kernels loaded per batch
-    uint32_t kb[B];
-    long long tb[B];
-    auto load_batch = [&](int jb) {
+                const uint2 w = *reinterpret_cast<const uint2 *>(V.k_stream + i0);
 #pragma unroll
-        for (int v = 0; v < B; ++v) kb[v] = tk[jb + v < j1 ? jb + v : j0];
-#pragma unroll
-        for (int v = 0; v < B; ++v) tb[v] = A.k_start[kb[v]];
-    };
-    load_batch(j0);
-    for (int jb = j0; jb < j1; jb += B) {
-        uint32_t kc[B], tc[B];
-#pragma unroll
-        for (int v = 0; v < B; ++v) { kc[v] = kb[v]; tc[v] = rel32(tb[v], tbase); }
-        if (jb + B < j1) load_batch(jb + B);      // the next batch in flight during this one
-#pragma unroll
-        for (int v = 0; v < B; ++v) {
-            const int j = jb + v;
-            if (j >= j1) break;
-            const uint32_t T = tc[v];
-            if (j == j0) {
-#pragma unroll
-                for (int d = 0; d < EN_RD; ++d) {
-                    const int c = d < nd ? S.wcnt[d] : 0, o = d < nd ? S.woff[d] : 0;
-                    int x = o, y = o + c;         // last window position with start <= T
-                    while (x < y) {
-                        const int m = (x + y) >> 1;
-                        if (S.ws[m] <= T) x = m + 1; else y = m;
-                    }
-                    const int p = x - o - 1;
-                    pos[d] = p;
-                    nxt[d] = p + 1 < c ? S.ws[o + p + 1] : NONE_T;
-                    cend[d] = p >= 0 ? S.we[o + p] : 0u;
-                    cinf[d] = p >= 0 ? S.wi[o + p] : 0u;
+                for (int u = 0; u < 4; ++u) {
+                    s[u] = (w.x >> (8 * u)) & 0xFFu;
+                    s[4 + u] = (w.y >> (8 * u)) & 0xFFu;
                 }
             } else {
 #pragma unroll
-                for (int d = 0; d < EN_RD; ++d) {
-                    if (nxt[d] <= T) {            // a later range of this depth starts by T
-                        const int c = S.wcnt[d], o = S.woff[d];
-                        int p = pos[d] + 1;
-                        while (p + 1 < c && S.ws[o + p + 1] <= T) ++p;
-                        pos[d] = p;
-                        nxt[d] = p + 1 < c ? S.ws[o + p + 1] : NONE_T;
-                        cend[d] = S.we[o + p];
-                        cinf[d] = S.wi[o + p];
-                    }
+                for (int u = 0; u < EP_G; ++u) {
+                    t[u] = i0 + u < V.K ? V.k_start[i0 + u] : LLONG_MAX;
+                    s[u] = i0 + u < V.K ? V.k_stream[i0 + u] : 255u;
                 }
             }
-            // the walk over the tracked depths, every kernel, without branches
-            int32_t ans = -1;
-            int nop = 0;
-            bool alive = true;
+            t[EP_G] = i0 + EP_G < V.K ? V.k_start[i0 + EP_G] : LLONG_MAX;
+            s[EP_G] = i0 + EP_G < V.K ? V.k_stream[i0 + EP_G] : 255u;
+            if (C.kname) {
+                if (C.pair_vec && whole) {
+                    uint4 x[2], y[2];
 #pragma unroll
-            for (int d = 0; d < EN_RD; ++d) {
-                alive = alive && d < nd && pos[d] >= 0 && cend[d] >= T;
-                const uint32_t kind = cinf[d] >> 30;
-                const bool st_d = alive && kind == KIND_STRUCT, op_d = alive && kind == KIND_OP;
-                ans = st_d ? -1 : (op_d ? (int32_t)(cinf[d] & 0x3FFFFFFFu) : ans);
-                nop = st_d ? 0 : nop + (op_d ? 1 : 0);
-            }
-            if (alive && nd > EN_RD) {
-                for (int d = EN_RD; d < nd; ++d) {   // deeper levels: one search each
-                    const int c = S.wcnt[d], o = S.woff[d];
-                    int x = o, y = o + c;
-                    while (x < y) {
-                        const int m = (x + y) >> 1;
-                        if (S.ws[m] <= T) x = m + 1; else y = m;
+                    for (int q = 0; q < 2; ++q) {
+                        x[q] = *reinterpret_cast<const uint4 *>(C.kname + i0 + 4 * q);
+                        y[q] = *reinterpret_cast<const uint4 *>(C.nname + i0 + 4 * q);
                     }
-                    if (x == o || S.we[x - 1] < T) break;
-                    walk_step(S.wi[x - 1], ans, nop);
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        if ((x[q].x != y[q].x) | (x[q].y != y[q].y) | (x[q].z != y[q].z) | (x[q].w != y[q].w)) f |= NAMES;
+                        const int32_t j = (int32_t)(i0 + 4 * q);
+                        *reinterpret_cast<int4 *>(C.idx + j) = make_int4(j, j + 1, j + 2, j + 3);
+                    }
+                    if (C.kind) *reinterpret_cast<uint2 *>(C.kind + i0) = make_uint2(0x01010101u, 0x01010101u);
+                } else {
+                    for (int u = 0; u < EP_G && i0 + u < V.K; ++u) {
+                        if (C.kname[i0 + u] != C.nname[i0 + u]) f |= NAMES;
+                        C.idx[i0 + u] = (int32_t)(i0 + u);
+                        if (C.kind) C.kind[i0 + u] = 1;
+                    }
                 }
             }
-            A.out_range[kc[v]] = ans;
-            if (A.out_nop) A.out_nop[kc[v]] = (uint8_t)nop;
+#pragma unroll
+            for (int u = 0; u < EP_G; ++u) {
+                if (i0 + u >= V.K) break;
+                kmn = t[u] < kmn ? t[u] : kmn;
+                kmx = t[u] > kmx ? t[u] : kmx;
+                if (i0 + u + 1 < V.K && (t[u + 1] < t[u] || (t[u + 1] == t[u] && s[u + 1] < s[u]))) f |= U_KERN;
+                kseen[s[u]] = 1;
+            }
         }
+        const int64_t rshare = (V.R + parts - 1) / parts;
+        const int64_t rb = b * rshare, re = rb + rshare < V.R ? rb + rshare : V.R;
+        constexpr int B = 4;             // ranges of a thread, loads issued together
+        for (int64_t j0 = rb + tid; j0 < re; j0 += EP_THREADS * B) {
+            long long sv[B], ev[B], nv[B];
+            unsigned dv[B], tv[B];
+#pragma unroll
+            for (int u = 0; u < B; ++u) {
+                const int64_t i = j0 + u * EP_THREADS;
+                const bool in = i < re;
+                sv[u] = in ? V.r_start[i] : 0;
+                ev[u] = in ? V.r_end[i] : 0;
+                nv[u] = in && i + 1 < V.R ? V.r_start[i + 1] : LLONG_MAX;
+                dv[u] = in ? V.r_depth[i] : 0u;
+                tv[u] = in ? V.r_stream[i] : 0u;
+            }
+#pragma unroll
+            for (int u = 0; u < B; ++u) {
+                if (j0 + u * EP_THREADS >= re) break;
+                if (ev[u] < sv[u]) f |= BAD_END;
+                if (dv[u] >= OPATTR_MAX_DEPTH) f |= BAD_DEPTH;
+                if (nv[u] < sv[u]) f |= U_RANGE;
+                rmn = sv[u] < rmn ? sv[u] : rmn;
+                rmx = ev[u] > rmx ? ev[u] : rmx;
+                if (dv[u] < OPATTR_MAX_DEPTH && !((dmask[tv[u]] >> dv[u]) & 1u)) atomicOr(&dmask[tv[u]], 1u << dv[u]);
+            }
+        }
+        f = (int)__reduce_or_sync(0xffffffffu, (unsigned)f);
+        if (lane == 0 && f) atomicOr(&flags_s, f);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const long long a0 = __shfl_xor_sync(0xffffffffu, kmn, o), a1 = __shfl_xor_sync(0xffffffffu, kmx, o);
+            const long long a2 = __shfl_xor_sync(0xffffffffu, rmn, o), a3 = __shfl_xor_sync(0xffffffffu, rmx, o);
+            kmn = a0 < kmn ? a0 : kmn;
+            kmx = a1 > kmx ? a1 : kmx;
+            rmn = a2 < rmn ? a2 : rmn;
+            rmx = a3 > rmx ? a3 : rmx;
+        }
+        if (lane == 0) {
+            atomicMin(&mm_s[0], kmn);
+            atomicMax(&mm_s[1], kmx);
+            atomicMin(&mm_s[2], rmn);
+            atomicMax(&mm_s[3], rmx);
+        }
+        __syncthreads();
+        if (tid < 256) {
+            const uint32_t m = dmask[tid];
+            if (m) atomicOr(&lvlmask[tid], m);
+            const unsigned w = __ballot_sync(0xffffffffu, kseen[tid] != 0);
+            if (lane == 0 && w) atomicOr(&st->kstreams[warp], w);
+        }
+        if (tid == 0) {
+            if (flags_s & BAD_END) set_err(st, ERR_INVALID);
+            if (flags_s & BAD_DEPTH) set_err(st, ERR_DEPTH);
+            const unsigned fl = ((flags_s & U_KERN) ? F_K_UNSORTED : 0u) | ((flags_s & U_RANGE) ? F_R_UNSORTED : 0u) |
+                                ((flags_s & NAMES) ? F_NAMES_DIFFER : 0u);
+            if (fl) set_flag(st, fl);
+            if (kb < ke) {
+                atomicMin(&st->mm[MM_KSTART_MIN], mm_s[0]);
+                atomicMax(&st->mm[MM_KSTART_MAX], mm_s[1]);
+            }
+            if (rb < re) {
+                atomicMin(&st->mm[MM_RSTART_MIN], mm_s[2]);
+                atomicMax(&st->mm[MM_REND_MAX], mm_s[3]);
+            }
+        }
+    }
+    // the part's tiles and ranges
+    const int64_t nt = parts * tp, t0 = b * tp;
+    for (int q = (int)warp; q <= tp; q += EP_THREADS / 32) {
+        const int64_t r = ranges_before<KEYS>(V, tile_event(t0 + q, nt, V.K + V.R));
+        if (lane != 0) continue;
+        if (q < tp || t0 + q == nt) tile_r[t0 + q] = (uint32_t)r;
+        if (q == 0) bound[0] = r;
+        if (q == tp) bound[1] = r;
+    }
+    __syncthreads();
+    const int64_t r0 = bound[0];
+    // (records out of order, whose bounds mean nothing: no more than a part's worth)
+    const int64_t most = r0 + tile_event(t0 + tp, nt, V.K + V.R) - tile_event(t0, nt, V.K + V.R);
+    const int64_t r1 = bound[1] < most ? bound[1] : most;
+    uint32_t top = 0;
+    for (int64_t i = r0 + tid; i < r1; i += EP_THREADS) {
+        const unsigned d = V.r_depth[i];
+        if (d >= OPATTR_MAX_DEPTH) continue;
+        const unsigned l = (unsigned)V.r_stream[i] * 32u + d;
+        atomicMax(&last[l], (uint32_t)i + 1u);
+        top = l + 1 > top ? l + 1 : top;
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (lane == 0 && top) atomicMax(&top_s, top);
+    __syncthreads();
+    const uint32_t n = top_s;
+    for (uint32_t i = tid; i < n; i += EP_THREADS) rows[b * LEVELS + i] = last[i];
+    if (tid == 0) row_len[b] = n;
+}
+
+// Rows of the parts' last ranges to rows of the last range before each part:
+// a running maximum down every column.  One block per stream: lane d of a
+// warp takes depth d, each of the 32 warps an equal run of the parts.
+__global__ void __launch_bounds__(1024) k_enc_carry(uint32_t *__restrict__ rows, const uint32_t *__restrict__ row_len,
+                                                    int64_t parts, const uint32_t *__restrict__ lvlmask) {
+    pdl_wait();
+    if (lvlmask[blockIdx.x] == 0) return;
+    __shared__ uint32_t seg[32][33];
+    const unsigned lane = lane_id(), w = threadIdx.x >> 5;
+    const uint32_t l = blockIdx.x * 32u + lane;
+    const int64_t per = (parts + 31) / 32;
+    const int64_t b0 = w * per, b1 = b0 + per < parts ? b0 + per : parts;
+    uint32_t m = 0;
+#pragma unroll 8
+    for (int64_t b = b0; b < b1; ++b) {
+        const uint32_t v = l < row_len[b] ? rows[b * LEVELS + l] : 0u;
+        m = v > m ? v : m;
+    }
+    seg[w][lane] = m;
+    __syncthreads();
+    m = 0;
+    for (unsigned q = 0; q < w; ++q) m = seg[q][lane] > m ? seg[q][lane] : m;
+#pragma unroll 8
+    for (int64_t b = b0; b < b1; ++b) {
+        const uint32_t v = l < row_len[b] ? rows[b * LEVELS + l] : 0u;
+        rows[b * LEVELS + l] = m;
+        m = v > m ? v : m;
     }
 }
 
-__global__ void k_fill_unattributed(int32_t *out_range, uint8_t *out_nop, int64_t n) {
+// ------------------------------------------------------------------ enclosure
+// Shared memory of a tile: entries 0 .. SR - 1 are its ranges in order, entry
+// SR + l the range open on level l when the tile begins (alive bits in amask).
+// Levels of a stream are consecutive, depth by depth; 16-bit indices name
+// entries, E_NONE none.
+constexpr unsigned E_NONE = 0xFFFFu;
+constexpr unsigned D_DEPTH = 31u, D_MIXED = 32u;     // bits of `dep`
+template <int THREADS_, int BLOCKS_, int RW_, int RPT_>
+struct EncTile {
+    static constexpr int THREADS = THREADS_, BLOCKS = BLOCKS_, RW = RW_, RPT = RPT_;
+    static constexpr int SR = RW * 32 * RPT;         // ranges of a step at most
+    static constexpr int WORDS = SR / 32;
+    uint32_t *ss, *se, *si;      // start, end (relative), position | kind << 30
+    uint32_t *re;                // end of the outermost ancestor
+    uint32_t *amask;             // [ns] depths with an open range, per compact stream
+    uint32_t *smask;             // [ns][WORDS] the stream's ranges among the tile's, one bit each
+    uint16_t *par, *prev, *best; // parent; the entry before on the stream; where the climb begins (below)
+    uint16_t *va;                // innermost operator of the entry's chain
+    uint16_t *last;              // [RW + 1][nl] last range of each level in a warp's run, index + 1; then in
+                                 // the runs before it, and at last in all
+    uint16_t *swords;            // [ns] which words of smask are not empty
+    uint16_t *dopen;             // [ns] deepest open range, E_NONE none
+    uint16_t *cbase;             // [256] first level of a stream
+    uint16_t *scid;              // [256] compact id of a stream (streams with levels, in order), E_NONE none
+    uint8_t *dep, *vn;           // depth | D_MIXED; operators in the chain
+    uint8_t *sid;                // compact stream
+    uint8_t *ndep;               // [256] levels of a stream
+    uint8_t *slist;              // [256] the stream of a compact id
+    __device__ __forceinline__ EncTile(unsigned char *p, int nl, int ns) {
+        const int cap = SR + nl;
+        auto take = [&](size_t n) { unsigned char *q = p; p += n; return q; };
+        ss = reinterpret_cast<uint32_t *>(take((size_t)cap * 4));
+        se = reinterpret_cast<uint32_t *>(take((size_t)cap * 4));
+        si = reinterpret_cast<uint32_t *>(take((size_t)cap * 4));
+        re = reinterpret_cast<uint32_t *>(take((size_t)cap * 4));
+        amask = reinterpret_cast<uint32_t *>(take((size_t)ns * 4));
+        smask = reinterpret_cast<uint32_t *>(take((size_t)ns * WORDS * 4));
+        par = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
+        prev = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
+        best = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
+        va = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
+        last = reinterpret_cast<uint16_t *>(take((size_t)(RW + 1) * nl * 2));
+        swords = reinterpret_cast<uint16_t *>(take((size_t)ns * 2));
+        dopen = reinterpret_cast<uint16_t *>(take((size_t)ns * 2));
+        cbase = reinterpret_cast<uint16_t *>(take(512));
+        scid = reinterpret_cast<uint16_t *>(take(512));
+        dep = take(cap);
+        vn = take(cap);
+        sid = take(cap);
+        ndep = take(256);
+        slist = take(256);
+    }
+    static size_t smem(int nl, int ns) {
+        return (size_t)(SR + nl) * 27 + (size_t)(RW + 1) * nl * 2 + (size_t)ns * (4 + 4 * WORDS + 4) + 1024 + 512;
+    }
+};
+using EncTileA = EncTile<256, 4, 8, 2>;
+using EncTileB = EncTile<512, 2, 4, 4>;
+constexpr int EN_LEVELS_A = 512, EN_STREAMS_A = 64;      // levels and streams of the common layout
+constexpr int EN_LEVELS_B = 2048;                        // of the wide one: 64 streams of every depth
+constexpr int64_t EN_TILE = 2048, EN_TILE_MIN = 512;     // events of a tile; of a part's one tile in small traces
+constexpr int64_t EN_EARLY = 1 << 20;                    // events from which a join looks at the checks before the end
+constexpr uint32_t EN_SPAN = 0xFFFFFFF0u;                // a step's times fit 32 bits relative to its first
+
+// One block per part, tile by tile; a tile with more ranges than SR, or whose
+// times span 2^32 ns, is taken in steps.  A step's ranges, and the ranges open
+// when it begins, lie in shared memory (times relative to its first event, 32
+// bits), and once per range this is worked out:
+//   parent  the last range of the level above that starts no later
+//   chain   Algorithm 2's result for the range and its ancestors: walking
+//           outward to the first structural range, the innermost operator
+//           and the number of operators
+//   best    of the ranges of the stream up to this one the latest-starting
+//           that has a length, the deepest of those with its start: whatever
+//           contains a time after this entry's start and before the stream's
+//           next one is `best` or an ancestor of it
+// A kernel then takes the last range of its stream that starts by it (the
+// step's ranges before the kernel are counted along the warp's kernels, the
+// stream's last one among them found by its bit mask), climbs from its `best`
+// past the ranges that have ended, and has its answer in the chain found
+// there.  A kernel that starts with that range takes the range's own chain,
+// unless another range of the stream starts or ends at that instant (D_MIXED):
+// then the last range of each level up to the instant stands for its level,
+// and the chain is walked along those (closed intervals).
+//
+// The laminar checks ride along: each range against its predecessor in its
+// level, and against its parent (equal starts in array order included; where
+// those go on past the loaded ranges, F_LEVEL_FIXUP asks for a run on ranges
+// sorted so that parents come first).  F_LEVEL_FIXUP also reports equal starts
+// of a level out of (start, end) order.  With `final` both are errors.
+// Ranges that are not laminar give wrong answers but no stray access: parents
+// lie one level up, so every climb and walk ends within 32 steps.
+//
+// Bound by issue (2.4 instructions a cycle) and by the shared-memory chains of
+// the links, not by HBM: 490 us for 20M kernels and 5.1M ranges on 16 streams,
+// 17 us for 2,000.  The level lists, stream partition, windows and per-stream
+// tiles it replaces took 436 us in their largest kernel and another 300 us in
+// eight more launches (partly side by side) for the same trace, two host waits
+// and 60 us for the small one.  Also measured: one search per depth and kernel
+// in level lists of the tile (1,170 us), entries grouped by stream with a
+// search per kernel (696 us).
+//
+// blockIdx.y is a group of 2^gshift consecutive stream ids: the block leaves
+// the other groups' kernels and ranges alone (traces with more levels than the
+// wide layout holds; else one group of all 256).
+template <typename TL, bool KEYS, bool GROUPS>
+__global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
+    k_enclose(EncView V, int64_t parts, int tp, const uint32_t *__restrict__ tile_r,
+              const uint32_t *__restrict__ rows, const uint32_t *__restrict__ row_len, int carried,
+              const uint32_t *__restrict__ lvlmask, int nlcap, int nscap, int gshift, unsigned leave_on, int final,
+              int32_t *__restrict__ out_range, uint8_t *__restrict__ out_nop, DevStatus *st) {
     pdl_wait();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        out_range[i] = -1;
-        if (out_nop) out_nop[i] = 0;
+    constexpr int THREADS = TL::THREADS, WARPS = THREADS / 32, RW = TL::RW, RPT = TL::RPT, SR = TL::SR,
+                  WORDS = TL::WORDS;
+    static_assert(THREADS >= 256, "a thread per stream");
+    static_assert(WORDS <= 16, "words of a stream's mask");
+    if ((st->err & (ERR_INVALID | ERR_DEPTH)) || (st->flags & leave_on)) return;
+    extern __shared__ __align__(16) unsigned char en_smem[];
+    const TL S(en_smem, nlcap, nscap);
+    __shared__ uint32_t wbuf[33];
+    __shared__ int taken[2];
+    const int tid = threadIdx.x;
+    const unsigned lane = lane_id(), warp = tid >> 5, lt = lanemask_lt();
+    const int64_t b = blockIdx.x;
+    const unsigned grp = blockIdx.y;
+    auto mine = [&](unsigned s) { return !GROUPS || (s >> gshift) == grp; };
+    // levels present: depths 0 .. ndep - 1 of each stream (a depth below a gap
+    // has no parent level: its ranges are not nested)
+    int nl, ns;
+    {
+        uint32_t n = 0;
+        if (tid < 256 && mine(tid)) {
+            const uint32_t m = lvlmask[tid];
+            n = m == 0xFFFFFFFFu ? 32u : (uint32_t)__ffs(~m) - 1u;
+        }
+        uint32_t tot;
+        const uint32_t ex = block_exclusive_scan<uint32_t>(n | (n ? 1u << 16 : 0u), wbuf, &tot);
+        nl = (int)(tot & 0xFFFFu);
+        ns = (int)(tot >> 16);
+        if (nl > nlcap || ns > nscap) {
+            if (b == 0 && tid == 0) {
+                atomicMax(&st->nlevels, (unsigned)nl);
+                set_flag(st, F_LEVELS_MANY);
+            }
+            return;
+        }
+        if (tid < 256) {
+            S.cbase[tid] = (uint16_t)(ex & 0xFFFFu);
+            S.ndep[tid] = (uint8_t)n;
+            S.scid[tid] = n ? (uint16_t)(ex >> 16) : (uint16_t)E_NONE;
+            if (n) {
+                S.slist[ex >> 16] = (uint8_t)tid;
+                S.amask[ex >> 16] = 0;
+            }
+        }
+    }
+    const int64_t nt = parts * tp, events = V.K + V.R;
+    int64_t r = tile_r[b * tp];
+    int64_t k = tile_event(b * tp, nt, events) - r;
+    __syncthreads();
+    // the earliest event at or after (k, r): what has ended before it is over
+    auto first_time = [&](int64_t kk, int64_t rr) {
+        const long long t = kk < V.K ? V.time<KEYS>(kk) : LLONG_MAX, a = rr < V.R ? V.r_start[rr] : LLONG_MAX;
+        return t < a ? t : a;
+    };
+    long long base = first_time(k, r);
+    auto rel = [&](long long x) -> uint32_t {
+        const unsigned long long v = (unsigned long long)x - (unsigned long long)base;
+        return x < base ? 0u : (v >= 0xFFFFFFFEull ? 0xFFFFFFFFu : (uint32_t)v + 1u);
+    };
+    for (int l = tid; l < LEVELS; l += THREADS) {
+        const int s = l >> 5, d = l & 31;
+        if (d >= S.ndep[s]) continue;
+        uint32_t v = 0;
+        if (carried) v = rows[b * LEVELS + l];
+        else
+            for (int64_t q = 0; q < b; ++q) {
+                const uint32_t x = (uint32_t)l < row_len[q] ? rows[q * LEVELS + l] : 0u;
+                v = x > v ? x : v;
+            }
+        if (v == 0) continue;
+        const long long z = V.r_end[v - 1];
+        if (z < base) continue;
+        const int e = SR + S.cbase[s] + d;
+        S.ss[e] = rel(V.r_start[v - 1]);
+        S.se[e] = rel(z);
+        S.si[e] = (v - 1) | kind_of(V.r_op[v - 1]) << 30;
+        S.dep[e] = (uint8_t)(d | D_MIXED);
+        atomicOr(&S.amask[S.scid[s]], 1u << d);
+    }
+    bool err = false, fix = false;
+    __syncthreads();
+    for (int64_t t = b * tp; t < (b + 1) * tp; ++t) {
+        const int64_t r1 = tile_r[t + 1], k1 = tile_event(t + 1, nt, events) - r1;
+        while (k < k1 || r < r1) {
+            int nr = (int)(r1 - r < SR ? r1 - r : SR), nk = (int)(k1 - k);
+            // ---- the step: the whole tile, or up to the first event that
+            // must wait (a kernel that starts no earlier than a range not
+            // loaded; 2^32 ns)
+            auto near = [&](long long x) { return (unsigned long long)x - (unsigned long long)base < EN_SPAN; };
+            bool whole = r1 - r <= SR;
+            if (nk > 0) whole = whole && near(V.time<KEYS>(k + nk - 1));
+            if (nr > 0) whole = whole && near(V.r_start[r + nr - 1]);
+            if (!whole) {
+                // by two warps, 32 probes a round
+                if (warp < 2) {
+                    const bool more = r + nr < r1;
+                    const long long next = more ? V.r_start[r + nr] : 0;
+                    int lo = 0, hi = warp == 0 ? nk : nr;
+                    while (lo < hi) {
+                        const int step = (hi - lo + 31) >> 5, p = lo + (int)lane * step;
+                        bool ok = false;
+                        if (p < hi) {
+                            const long long x = warp == 0 ? V.time<KEYS>(k + p) : V.r_start[r + p];
+                            ok = near(x) && !(warp == 0 && more && x >= next);
+                        }
+                        const unsigned m = ~__ballot_sync(0xffffffffu, ok);
+                        const int c = m ? __ffs(m) - 1 : 32;
+                        if (c == 0) break;
+                        const int nh = lo + c * step;
+                        lo += (c - 1) * step + 1;
+                        hi = nh < hi ? nh : hi;
+                    }
+                    if (lane == 0) taken[warp] = lo;
+                }
+                __syncthreads();
+                nk = taken[0];
+                nr = taken[1];
+                if (nk == 0 && nr == 0) {                                // cannot happen on ordered records
+                    if (tid == 0) set_err(st, ERR_INVALID);
+                    return;
+                }
+                // kernels before every range that is taken later: with kernels
+                // left over, ranges only while they start by the last one taken
+                // or no kernel is (all those left start after them)
+            }
+            const bool more = r + nr < V.R;                              // ranges past this step's
+            const long long next = more ? V.r_start[r + nr] : 0;
+            // times of this step as 32 bits: exact for its events
+            auto rel_near = [&](long long x) { return (uint32_t)x - (uint32_t)base + 1u; };
+            // ---- ranges, 32 at a time: the stream's and the level's earlier
+            // ranges in the warp's run by lane masks, before it by tables
+            uint32_t lk[RPT], pk[RPT];               // the level's range before | level << 16; parent | prev on stream << 16
+            if (warp < RW) {
+                uint16_t *wl = S.last + warp * nlcap;
+                for (int l = (int)lane; l < nl; l += 32) wl[l] = 0;
+                for (int q = (int)lane; q < ns; q += 32)
+#pragma unroll
+                    for (int i = 0; i < RPT; ++i) S.smask[q * WORDS + warp * RPT + i] = 0;
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) {
+                    const int e = (int)warp * 32 * RPT + i * 32 + (int)lane;
+                    if (e - (int)lane >= nr) {
+                        lk[i] = 0xFFFFu << 16;
+                        continue;
+                    }
+                    const bool in = e < nr;
+                    const int64_t p = r + (in ? e : 0);
+                    const long long a = in ? V.r_start[p] : 0, z = in ? V.r_end[p] : 0;
+                    const unsigned s = in ? V.r_stream[p] : 0u, d = in ? V.r_depth[p] : 0u;
+                    const uint32_t op = in ? V.r_op[p] : 0u;
+                    const bool lvl = in && d < S.ndep[s];
+                    err |= in && !lvl && mine(s);
+                    const unsigned q = lvl ? S.scid[s] : 256u;
+                    const unsigned c = lvl ? S.cbase[s] + d : 0u;
+                    const unsigned ps = __match_any_sync(0xffffffffu, q);
+                    unsigned pl = ps, pp = ps;       // lanes of the level, of the level above
+#pragma unroll
+                    for (int bit = 0; bit < 5; ++bit) {
+                        const unsigned x = __ballot_sync(0xffffffffu, (d >> bit) & 1u);
+                        pl &= (d >> bit) & 1u ? x : ~x;
+                        pp &= ((d - 1u) >> bit) & 1u ? x : ~x;
+                    }
+                    lk[i] = pk[i] = 0;
+                    if (lvl) {
+                        const unsigned at = (unsigned)e - lane;
+                        const unsigned ml = pl & lt, mp = d ? pp & lt : 0u, ms = ps & lt;
+                        unsigned u;
+                        u = ml ? at + 31u - __clz(ml) + 1u : wl[c];                      // index + 1, 0 not here
+                        lk[i] = u | c << 16;
+                        u = mp ? at + 31u - __clz(mp) + 1u : (d ? wl[c - 1] : 0u);
+                        pk[i] = u | (ms ? at + 31u - __clz(ms) + 1u : 0u) << 16;
+                        S.ss[e] = rel_near(a);
+                        S.se[e] = rel(z);
+                        S.si[e] = (uint32_t)p | kind_of(op) << 30;
+                        S.dep[e] = (uint8_t)d;
+                        S.sid[e] = (uint8_t)q;
+                    } else if (in) {                 // another group's, or below a gap: on no stream's chain
+                        S.ss[e] = rel_near(a);
+                        S.se[e] = 0;
+                        S.si[e] = KIND_STRUCT << 30;
+                        S.dep[e] = (uint8_t)(D_DEPTH | D_MIXED);
+                        S.sid[e] = 255;
+                        S.par[e] = S.prev[e] = (uint16_t)E_NONE;
+                    }
+                    __syncwarp();
+                    if (lvl) {
+                        if ((pl >> lane) == 1u) wl[c] = (uint16_t)(e + 1);               // the level's last of the 32
+                        if ((ps & lt) == 0) S.smask[q * WORDS + warp * RPT + i] = ps;
+                    }
+                    if (!lvl) lk[i] = 0xFFFFu << 16;
+                    __syncwarp();
+                }
+            }
+            __syncthreads();
+            // ---- links, and the laminar checks.  Relative times are exact
+            // below 2^32 - 1; two clamped ends are compared as they are.
+            for (int l = tid; l < nl; l += THREADS) {
+                uint32_t u = 0;
+#pragma unroll
+                for (int w = 0; w < RW; ++w) {
+                    const uint32_t x = S.last[w * nlcap + l];
+                    S.last[w * nlcap + l] = (uint16_t)u;
+                    u = x ? x : u;
+                }
+                S.last[RW * nlcap + l] = (uint16_t)u;
+            }
+            for (int q = THREADS - 1 - tid; q < ns; q += THREADS) {
+                unsigned m = 0;
+#pragma unroll
+                for (int w = 0; w < WORDS; ++w) m |= (S.smask[q * WORDS + w] ? 1u : 0u) << w;
+                S.swords[q] = (uint16_t)m;
+                const uint32_t o = S.amask[q];
+                S.dopen[q] = o ? (uint16_t)(SR + S.cbase[S.slist[q]] + 31 - __clz(o)) : (uint16_t)E_NONE;
+            }
+            __syncthreads();
+            if (warp < RW) {
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) {
+                    const uint32_t c = lk[i] >> 16;
+                    if (c == 0xFFFFu) continue;
+                    const uint32_t e = warp * 32 * RPT + i * 32 + lane;
+                    const unsigned q = S.sid[e], d = S.dep[e] & D_DEPTH, am = S.amask[q];
+                    const uint32_t a = S.ss[e];
+                    auto earlier = [&](uint32_t u, uint32_t l, unsigned depth) -> uint32_t {
+                        if (u == 0) u = S.last[warp * nlcap + l];
+                        return u ? u - 1 : ((am >> depth) & 1u ? (uint32_t)SR + l : (uint32_t)E_NONE);
+                    };
+                    const uint32_t y = earlier(lk[i] & 0xFFFFu, c, d);
+                    uint32_t p = d ? earlier(pk[i] & 0xFFFFu, c - 1, d - 1) : (uint32_t)E_NONE;
+                    uint32_t x = pk[i] >> 16;                                            // before it on the stream
+                    if (x) --x;
+                    else {
+                        const unsigned h = S.swords[q] & ((1u << (warp * RPT + i)) - 1u);
+                        const unsigned w = 31 - __clz(h);
+                        x = h ? w * 32 + 31 - __clz(S.smask[q * WORDS + w]) : (uint32_t)S.dopen[q];
+                    }
+                    bool mixed = x != E_NONE && S.ss[x] == a;
+                    for (int f = (int)e + 1; f < nr && S.ss[f] == a; ++f) {              // equal starts further on
+                        if (S.sid[f] != q) continue;
+                        mixed = true;
+                        if (d && (S.dep[f] & D_DEPTH) == d - 1) p = f;
+                    }
+                    auto end_of = [&](uint32_t w) { return V.r_end[S.si[w] & POS_MASK]; };
+                    auto ends_before = [&](uint32_t w, uint32_t v) {                     // entry w ends before entry v
+                        const uint32_t f = S.se[w], g = S.se[v];
+                        return f == 0xFFFFFFFFu && g == 0xFFFFFFFFu ? end_of(w) < end_of(v) : f < g;
+                    };
+                    if (y != E_NONE) {
+                        if (S.ss[y] == a && ends_before(e, y)) fix = true;               // starts with it, ends before it
+                        else if (S.se[y] > a) err = true;
+                        mixed |= S.se[y] == a;
+                    }
+                    if (d && (p == E_NONE || ends_before(p, e))) {
+                        if (more && !final && next == V.r_start[r + e]) fix = true;
+                        else err = true;
+                    }
+                    S.par[e] = (uint16_t)p;
+                    S.prev[e] = (uint16_t)x;
+                    if (mixed) S.dep[e] = (uint8_t)(d | D_MIXED);
+                }
+            }
+            for (int q = (int)warp; q < ns; q += WARPS) {                                // a warp per stream, a lane per depth
+                const uint32_t m = S.amask[q];
+                if (!((m >> lane) & 1u)) continue;
+                const uint32_t e = (uint32_t)SR + S.cbase[S.slist[q]] + lane;
+                S.par[e] = lane > 0 && ((m >> (lane - 1)) & 1u) ? (uint16_t)(e - 1) : (uint16_t)E_NONE;
+                S.prev[e] = m & lt ? (uint16_t)(e - lane + 31u - __clz(m & lt)) : (uint16_t)E_NONE;
+            }
+            __syncthreads();
+            // ---- chains and `best`
+            auto best_of = [&](uint32_t e) -> uint32_t {
+                while (e != E_NONE && S.ss[e] >= S.se[e]) e = S.prev[e];                 // zero length
+                if (e == E_NONE) return e;
+                uint32_t w = e;
+                const uint32_t a = S.ss[e];
+                for (uint32_t x = S.prev[e]; x != E_NONE && S.ss[x] == a; x = S.prev[x])
+                    if (S.se[x] > a && (S.dep[x] & D_DEPTH) > (S.dep[w] & D_DEPTH)) w = x;
+                return w;
+            };
+            auto chain = [&](uint32_t e) {
+                uint32_t ans = E_NONE, n = 0, top = e;
+                bool on = true;
+                for (uint32_t x = e; x != E_NONE; x = S.par[x]) {
+                    const uint32_t kind = S.si[x] >> 30;
+                    on = on && kind != KIND_STRUCT;
+                    if (on && kind == KIND_OP && n++ == 0) ans = x;
+                    top = x;
+                }
+                S.va[e] = (uint16_t)ans;
+                S.vn[e] = (uint8_t)n;
+                S.re[e] = S.se[top];
+                S.best[e] = (uint16_t)best_of(e);
+            };
+            for (int e = tid; e < nr; e += THREADS) chain(e);
+            for (int q = (int)warp; q < ns; q += WARPS)
+                if ((S.amask[q] >> lane) & 1u) chain((uint32_t)SR + S.cbase[S.slist[q]] + lane);
+            __syncthreads();
+            // ---- the kernels: each warp an equal run, 32 at a time
+            {
+                const int per = (nk + 32 * WARPS - 1) / (32 * WARPS) * 32;
+                const int j0 = (int)warp * per, j1 = j0 + per < nk ? j0 + per : nk;
+                int q0 = 0;                                                              // ranges before the run
+                long long t_n = 0;
+                unsigned s_n = 0;
+                if (j0 < j1) {
+                    if (j0 + (int)lane < j1) {
+                        t_n = V.time<KEYS>(k + j0 + lane);
+                        s_n = V.stream<KEYS>(k + j0 + lane);
+                    }
+                    const uint32_t T0 = __shfl_sync(0xffffffffu, rel_near(t_n), 0);
+                    int hi = nr;
+                    while (q0 < hi) {
+                        const int m = (q0 + hi) >> 1;
+                        if (S.ss[m] <= T0) q0 = m + 1; else hi = m;
+                    }
+                }
+                for (int j = j0; j < j1; j += 32) {
+                    const bool in = j + (int)lane < j1;
+                    const uint32_t T = rel_near(t_n);
+                    const unsigned s = s_n;
+                    const int64_t kk = k + j + (int)lane;
+                    if (j + 32 + (int)lane < j1) {
+                        t_n = V.time<KEYS>(kk + 32);
+                        s_n = V.stream<KEYS>(kk + 32);
+                    }
+                    // ranges that start by each kernel: those by the last one
+                    // first, then each lane's share of them
+                    const int top = j1 - j < 32 ? j1 - j - 1 : 31;
+                    const uint32_t Tm = __shfl_sync(0xffffffffu, T, top);
+                    int qn = q0;
+                    for (;;) {
+                        const uint32_t v = q0 + (int)lane < nr ? S.ss[q0 + lane] : 0xFFFFFFFFu;
+                        const int c = __popc(__ballot_sync(0xffffffffu, v <= Tm));
+                        for (int i = 0; i < c; ++i) qn += __shfl_sync(0xffffffffu, v, i) <= T ? 1 : 0;
+                        q0 += c;
+                        if (c < 32) break;
+                    }
+                    if (!in || !mine(s)) continue;
+                    uint32_t ans = E_NONE;
+                    unsigned n = 0;
+                    const unsigned q = S.scid[s];
+                    if (q != E_NONE) {
+                        uint32_t x, m = 0;                                               // the stream's last one
+                        unsigned w = (unsigned)qn >> 5;
+                        if (w < WORDS) m = S.smask[q * WORDS + w] & ((1u << (qn & 31)) - 1u);
+                        if (m == 0) {
+                            const unsigned h = S.swords[q] & ((1u << w) - 1u);
+                            w = 31 - __clz(h);
+                            if (h) m = S.smask[q * WORDS + w];
+                        }
+                        x = m ? w * 32 + 31 - __clz(m) : (uint32_t)S.dopen[q];
+                        if (x != E_NONE) {
+                            const bool at_start = S.ss[x] == T;
+                            if (!at_start || !(S.dep[x] & D_MIXED)) {
+                                if (!at_start) x = S.best[x];
+                                if (x != E_NONE && S.re[x] >= T) {
+                                    while (S.se[x] < T) x = S.par[x];
+                                    ans = S.va[x];
+                                    n = S.vn[x];
+                                }
+                            } else {
+                                // ranges that start at T stand in for the older ones of their
+                                // levels, beside older ones of other levels that end at T
+                                const uint32_t e = x;
+                                uint32_t z = e, g = e, at = 1u << (S.dep[e] & D_DEPTH);  // deepest (last) at T; first; depths
+                                for (uint32_t f = S.prev[e]; f != E_NONE && S.ss[f] == T; f = S.prev[f]) {
+                                    g = f;
+                                    at |= 1u << (S.dep[f] & D_DEPTH);
+                                    if ((S.dep[f] & D_DEPTH) > (S.dep[z] & D_DEPTH)) z = f;
+                                }
+                                x = best_of(S.prev[g]);                                  // open before T
+                                while (x != E_NONE && S.se[x] < T) x = S.par[x];
+                                if (x == E_NONE || (S.dep[x] & D_DEPTH) <= (S.dep[z] & D_DEPTH)) x = z;
+                                while (x != E_NONE) {
+                                    const uint32_t kind = S.si[x] >> 30, d = S.dep[x] & D_DEPTH;
+                                    if (kind == KIND_STRUCT) break;
+                                    if (kind == KIND_OP && n++ == 0) ans = x;
+                                    x = S.par[x];
+                                    if (x != E_NONE && ((at >> (d - 1)) & 1u))           // the last of this depth at T
+                                        for (x = e; (S.dep[x] & D_DEPTH) != d - 1;) x = S.prev[x];
+                                }
+                            }
+                        }
+                    }
+                    const int64_t o = V.korder ? V.korder[kk] : kk;
+                    int32_t range = -1;
+                    if (ans != E_NONE) {
+                        const uint32_t p = S.si[ans] & POS_MASK;
+                        range = (int32_t)(V.perm ? V.perm[p] : p);
+                    }
+                    out_range[o] = range;
+                    if (out_nop) out_nop[o] = (uint8_t)n;
+                }
+            }
+            __syncthreads();
+            // ---- the range each level carries on: its last one, unless it is over
+            k += nk;
+            r += nr;
+            const long long nbase = first_time(k, r);
+            const unsigned long long shift = (unsigned long long)nbase - (unsigned long long)base;
+            for (int q = (int)warp; q < ns; q += WARPS) {
+                const unsigned s = S.slist[q];
+                bool live = false;
+                if ((int)lane < S.ndep[s]) {
+                    const uint32_t l = S.cbase[s] + lane;
+                    const uint32_t u = S.last[RW * nlcap + l];
+                    const uint32_t e = SR + l, f = u ? u - 1 : e;
+                    if (u || ((S.amask[q] >> lane) & 1u)) {
+                        const uint32_t a = S.ss[f], z = S.se[f], i = S.si[f];
+                        // times relative to the next step
+                        uint32_t z2;
+                        if (z == 0xFFFFFFFFu) {
+                            const long long end = V.r_end[i & POS_MASK];
+                            const unsigned long long v = (unsigned long long)end - (unsigned long long)nbase;
+                            z2 = end < nbase ? 0u : (v >= 0xFFFFFFFEull ? 0xFFFFFFFFu : (uint32_t)v + 1u);
+                        } else {
+                            z2 = (unsigned long long)z > shift ? z - (uint32_t)shift : 0u;
+                        }
+                        live = z2 > 0;
+                        S.ss[e] = (unsigned long long)a > shift ? a - (uint32_t)shift : 0u;
+                        S.se[e] = z2;
+                        S.si[e] = i;
+                        S.dep[e] = (uint8_t)(lane | D_MIXED);
+                    }
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, live);
+                if (lane == 0) S.amask[q] = m;
+            }
+            base = nbase;
+            __syncthreads();
+        }
+    }
+    if (final && fix) {
+        err = true;
+        fix = false;
+    }
+    if (__any_sync(0xffffffffu, fix) && lane == 0) set_flag(st, F_LEVEL_FIXUP);
+    if (__any_sync(0xffffffffu, err) && lane == 0) set_err(st, ERR_NOT_NESTED);
+}
+
+// ------------------------------------------------------------------ sorted views
+// Range records in the order of the sorted keys (which hold the starts).
+__global__ void k_range_gather(EncView V, const uint64_t *__restrict__ key, int shift, long long tmin,
+                               const uint32_t *__restrict__ perm, int64_t *__restrict__ start,
+                               int64_t *__restrict__ end, uint8_t *__restrict__ stream, uint8_t *__restrict__ depth,
+                               uint32_t *__restrict__ op) {
+    pdl_wait();
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < V.R; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t r = perm[i];
+        start[i] = tmin + (long long)(key[i] >> shift);
+        end[i] = V.r_end[r];
+        stream[i] = V.r_stream[r];
+        depth[i] = V.r_depth[r];
+        op[i] = V.r_op[r];
     }
 }
 
 // ------------------------------------------------------------------ host
-static opattr_status status_from_err(unsigned err) {
-    if (err & ERR_INVALID) return OPATTR_E_INVALID_ARG;
-    if (err & ERR_DEPTH) return OPATTR_E_DEPTH;
-    if (err & ERR_NOT_NESTED) return OPATTR_E_NOT_NESTED;
-    if (err & ERR_TIMEOUT) return OPATTR_E_TIMEOUT;
+opattr_status enclose_verdict(const DevStatus &H, int64_t K) {
+    if (H.err & ERR_INVALID) return OPATTR_E_INVALID_ARG;
+    if (H.err & ERR_DEPTH) return OPATTR_E_DEPTH;
+    if (K > 0 && (H.mm[MM_KSTART_MAX] - H.mm[MM_KSTART_MIN]) >= (1ll << 55)) return OPATTR_E_INVALID_ARG;
+    if (H.err & ERR_NOT_NESTED) return OPATTR_E_NOT_NESTED;
+    if (H.err & ERR_TIMEOUT) return OPATTR_E_TIMEOUT;
     return OPATTR_OK;
+}
+
+// The enclosure launches on view V: the parts (already there after the
+// checking pass on V itself), the carried ranges, the tiles.
+struct EncBufs {
+    int64_t parts;
+    int tp;                      // tiles of a part
+    uint32_t *tile_r, *rows, *row_len, *lvlmask;
+};
+constexpr int64_t EN_DIRECT_PARTS = 32;          // up to this many: a block scans the rows before its own itself
+template <typename TL, bool KEYS, bool GROUPS = false>
+static void launch_tiles(Ctx &c, const EncView &V, const EncBufs &B, int nl, int groups, unsigned leave_on,
+                         bool final, int32_t *out_range, uint8_t *out_nop) {
+    const int ns = std::is_same<TL, EncTileA>::value ? EN_STREAMS_A : 256;
+    const size_t smem = TL::smem(nl, ns);
+    if (smem > 48 * 1024)
+        cudaFuncSetAttribute(k_enclose<TL, KEYS, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    launch(c, "enclose", k_enclose<TL, KEYS, GROUPS>, dim3((unsigned)B.parts, (unsigned)groups), dim3(TL::THREADS), smem, V,
+           B.parts, B.tp, (const uint32_t *)B.tile_r, (const uint32_t *)B.rows, (const uint32_t *)B.row_len,
+           (int)(B.parts > EN_DIRECT_PARTS), (const uint32_t *)B.lvlmask, nl, ns, groups > 1 ? 6 : 8, leave_on, (int)final,
+           out_range, out_nop, c.d_status);
+}
+static void launch_carry(Ctx &c, const EncBufs &B) {
+    if (B.parts > EN_DIRECT_PARTS)
+        launch(c, "enc_carry", k_enc_carry, dim3(256), dim3(1024), 0, B.rows, (const uint32_t *)B.row_len, B.parts,
+               (const uint32_t *)B.lvlmask);
 }
 
 opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges *rng, int32_t *out_range,
@@ -617,268 +947,200 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     if (R > 0 && (!rng->stream || !rng->start_ns || !rng->end_ns || !rng->depth || !rng->op_id))
         return OPATTR_E_INVALID_ARG;
 
-    // scratch: range sort (u64 keys x2, values x2), level arrays, tables,
-    // kernel order, the stream partition of the kernels and its tile tables
-    const int64_t nt_max = (K + EN_TILE - 1) / EN_TILE + 256;
+    EncBufs B{};
+    B.parts = std::max<int64_t>(1, std::min<int64_t>((K + R + EN_TILE_MIN - 1) / EN_TILE_MIN,
+                                                     (int64_t)sm_count(c) * EncTileA::BLOCKS));
+    B.tp = (int)std::max<int64_t>(1, (K + R + B.parts * EN_TILE - 1) / (B.parts * EN_TILE));
+    const int64_t tiles = B.parts * B.tp;
     Need nd;
-    nd.add<uint32_t>(LEVELS + 1 + 256).add<uint32_t>(LEVELS + 1).add<uint32_t>(radix_hist_elems(K));
-    nd.add<uint64_t>(R).add<uint64_t>(R).add<uint32_t>(R).add<uint32_t>(R);
-    const int64_t hist_n = std::max(radix_hist_elems(R), radix_hist_elems(K));
-    const int64_t part_n = std::max<int64_t>(scan_scratch_elems(hist_n), scan_scratch_elems(LEVELS + 1));
-    nd.add<uint32_t>(hist_n).add<uint32_t>(part_n).add<uint32_t>(hist_n).add<uint32_t>(part_n);
-    nd.add<int64_t>(R).add<int64_t>(R).add<uint32_t>(R);
-    nd.add<unsigned char>(STAGE_BYTES);
-    nd.add<uint32_t>(K).add<uint32_t>(nt_max).add<int2>(nt_max * 32);
+    nd.add<uint32_t>(tiles + 1).add<uint32_t>(B.parts).add<uint32_t>(B.parts * LEVELS).add<uint32_t>(256);
     const bool keep_order = c.in_join && K > 0;       // a join keeps the time order for its matching
     if (keep_order) nd.add<uint32_t>(K);
-    size_t need = nd.bytes + time_sort_scratch(K) + 4096;
-    c.spec_ran = false;
-    opattr_status st = ensure_arena(c, need);
+    opattr_status st = ensure_arena(c, nd.bytes + 4096);
     if (st) return st;
-    if ((st = ensure_side(c))) return st;
     Arena a(c);
     uint32_t *kept_order = keep_order ? a.take<uint32_t>(K) : nullptr;     // first: the start of the arena
-    if ((st = reset_status(c))) return st;
+    B.lvlmask = a.take<uint32_t>(256);
+    B.tile_r = a.take<uint32_t>(tiles + 1);
+    B.row_len = a.take<uint32_t>(B.parts);
+    B.rows = a.take<uint32_t>(B.parts * LEVELS);
+    if (!B.lvlmask || !B.tile_r || !B.row_len || !B.rows) return OPATTR_E_OOM;
+    const ZeroRun z{B.lvlmask, 256};
+    if ((st = reset_status(c, 1, &z))) return st;
 
-    // level histogram [LEVELS] and kernels per stream [256], zeroed together
-    uint32_t *level_hist = a.take<uint32_t>(LEVELS + 1 + 256);
-    uint32_t *kstream = level_hist + LEVELS + 1;
-    uint32_t *lvl_off = a.take<uint32_t>(LEVELS + 1);
-    uint32_t *part = a.take<uint32_t>(part_n), *part2 = a.take<uint32_t>(part_n);
-    uint32_t *ktile = a.take<uint32_t>(radix_hist_elems(K));     // per tile, kernels of each stream
-    if (!level_hist || !lvl_off || !part || !part2 || !ktile) return OPATTR_E_OOM;
-    cudaMemsetAsync(level_hist, 0, sizeof(uint32_t) * (LEVELS + 1 + 256), c.stream);
-    // the ranges' checks and level histogram on the side stream, beside the
-    // kernels' order check; the level offsets and the stream counts come back
-    // with the status: one synchronisation for all
-    stream_after(c.side, c.stream, c.ev_fork);
-    {
-        OnStream on(c, c.side);
-        if (R > 0)
-            launch(c, "check_ranges", k_check_ranges, dim3(grid_for(R, RCHK_THREADS * RCHK_ITEMS)),
-                   dim3(RCHK_THREADS), 0, rng->stream, rng->start_ns, rng->end_ns, rng->depth, R, level_hist,
-                   c.d_status);
-        scan_exclusive_u32(c, level_hist, lvl_off, LEVELS + 1, part2, nullptr);
+    EncView V{};
+    V.k_start = kern->start_ns;
+    V.k_stream = kern->stream;
+    V.K = K;
+    V.r_start = rng->start_ns;
+    V.r_end = rng->end_ns;
+    V.r_stream = rng->stream;
+    V.r_depth = rng->depth;
+    V.r_op = rng->op_id;
+    V.R = R;
+    auto al = [](const void *p, uintptr_t n) { return (reinterpret_cast<uintptr_t>(p) & (n - 1)) == 0; };
+    EncCheck C{};
+    C.vec = al(kern->start_ns, 16) && al(kern->stream, 8);
+    c.spec_ran = c.spec_k > 0;
+    if (c.spec_ran) {
+        C.kname = c.spec_kname;
+        C.nname = c.spec_nname;
+        C.idx = c.spec_idx;
+        C.kind = c.spec_kind;
+        C.pair_vec = al(C.kname, 16) && al(C.nname, 16) && al(C.idx, 16) && al(C.kind, 8);
     }
-    check_kernel_order(c, kern->stream, kern->start_ns, K, kstream, ktile);
-    stream_after(c.stream, c.side, c.ev_join);
-    {
-        // the level offsets and the stream counts come back with the status
-        const SmallCopy back[2] = {{c.h_levels, lvl_off, sizeof(uint32_t) * (LEVELS + 1)},
-                                   {c.h_levels + LEVELS + 1, kstream, sizeof(uint32_t) * 256}};
-        if ((st = read_status(c, 2, back))) return st;
-    }
-    if ((st = status_from_err(c.h_status->err))) return st;
-    const bool k_sorted = !(c.h_status->flags & F_K_UNSORTED);
-    const bool r_sorted = !(c.h_status->flags & F_R_UNSORTED);
-    c.enclose_k_sorted = k_sorted ? 1 : 0;
-    const long long rmin = c.h_status->mm[MM_RSTART_MIN], rmax = c.h_status->mm[MM_REND_MAX];
-    const long long kmin = c.h_status->mm[MM_KSTART_MIN], kmax = c.h_status->mm[MM_KSTART_MAX];
-    if (K > 0 && (kmax - kmin) >= (1ll << 55)) return OPATTR_E_INVALID_ARG;
-
-    if (R == 0) {
-        if (K > 0)
-            launch(c, "fill_unattributed", k_fill_unattributed, dim3(grid_for(K, 256, 65535)), dim3(256), 0, out_range,
-                   out_nop, K);
-        return read_status(c);
-    }
-
-    // ---- host-built tables, sent with one copy from pinned staging: level of
-    // each compact level (u16 [LEVELS]), first compact level of a stream
-    // (u16 [256]), levels of a stream (u8 [256]), compact id of a level
-    // (u8 [LEVELS], at most 256 levels), and per stream its first place in
-    // the stream partition, its kernels and its first tile (u32 [256],
-    // [256], [257])
-    constexpr size_t ST_LOC = 0, ST_CBASE = ST_LOC + 2 * LEVELS, ST_NDEP = ST_CBASE + 2 * 256,
-                     ST_CMAP = ST_NDEP + 256, ST_KOFF = ST_CMAP + LEVELS, ST_KCNT = ST_KOFF + 4 * 256,
-                     ST_TOFF = ST_KCNT + 4 * 256, ST_SCMAP = ST_TOFF + 4 * 257, ST_END = ST_SCMAP + 256;
-    static_assert(ST_END <= STAGE_BYTES, "staging too small");
-    const uint32_t *off = c.h_levels;
-    const uint32_t *kcnt_h = c.h_levels + LEVELS + 1;
-    uint16_t *level_of_compact = reinterpret_cast<uint16_t *>(c.h_stage + ST_LOC);
-    uint16_t *cbase = reinterpret_cast<uint16_t *>(c.h_stage + ST_CBASE);
-    uint8_t *ndep = c.h_stage + ST_NDEP;
-    uint8_t *cmap = c.h_stage + ST_CMAP;
-    uint32_t *koff_h = reinterpret_cast<uint32_t *>(c.h_stage + ST_KOFF);
-    uint32_t *kcnt_s = reinterpret_cast<uint32_t *>(c.h_stage + ST_KCNT);
-    uint32_t *toff_h = reinterpret_cast<uint32_t *>(c.h_stage + ST_TOFF);
-    uint8_t *scmap = c.h_stage + ST_SCMAP;
-    int nl = 0;
-    for (int s = 0; s < 256; ++s) {
-        cbase[s] = (uint16_t)nl;
-        int n = 0;
-        while (n < 32 && off[s * 32 + n + 1] > off[s * 32 + n]) {
-            level_of_compact[nl++] = (uint16_t)(s * 32 + n);
-            n++;
+    launch(c, "enc_parts", k_enc_parts<true, false>, dim3((unsigned)B.parts), dim3(EP_THREADS), 0, V, C, B.parts,
+           B.tp, B.tile_r, B.rows, B.row_len, B.lvlmask, c.d_status);
+    // a large join looks at the checks' verdict while the rest runs on the
+    // taking that the records are in order; a small one reads it once, at its end
+    const bool early = c.defer_status && K + R >= EN_EARLY;
+    const SmallCopy masks{c.h_small, B.lvlmask, 256 * sizeof(uint32_t)};
+    if (early && (st = post_status(c, 1, &masks))) return st;
+    launch_carry(c, B);
+    launch_tiles<EncTileA, false>(c, V, B, EN_LEVELS_A, 1, F_K_UNSORTED | F_R_UNSORTED, false, out_range, out_nop);
+    if (c.defer_status) {
+        bool usual = true;
+        if (early) {
+            if ((st = await_status(c))) return st;
+            int levels = 0, streams = 0;
+            for (int s = 0; s < 256; ++s) {
+                levels += __builtin_popcount(c.h_small[s]);
+                streams += c.h_small[s] != 0;
+            }
+            usual = !(c.h_status->flags & (F_K_UNSORTED | F_R_UNSORTED)) && levels <= EN_LEVELS_A &&
+                    streams <= EN_STREAMS_A;
         }
-        ndep[s] = (uint8_t)n;
+        if (usual) {
+            // the rest of the verdict comes with the aggregation's status, which the join checks
+            c.enclose_k_sorted = 1;
+            c.enclose_pending = true;
+            return OPATTR_OK;
+        }
     }
-    memset(cmap, 0, LEVELS);
-    for (int l = 0; l < nl && l < 256; ++l) cmap[level_of_compact[l]] = (uint8_t)l;
-    uint32_t kacc = 0, tacc = 0;
+    if ((st = read_status(c))) return st;
+    bool k_sorted = !(c.h_status->flags & F_K_UNSORTED), r_sorted = !(c.h_status->flags & F_R_UNSORTED);
+    c.enclose_k_sorted = k_sorted ? 1 : 0;
+    const bool many = (c.h_status->flags & F_LEVELS_MANY) != 0;
+    const bool fixup = (c.h_status->flags & F_LEVEL_FIXUP) != 0;
+    if ((st = enclose_verdict(*c.h_status, K)) && !(fixup && st == OPATTR_E_NOT_NESTED)) return st;
+    if (k_sorted && r_sorted && !many && !fixup) return OPATTR_OK;
+
+    // ---- records out of order, ranges of one level that share a start and are
+    // out of (start, end) order, or more levels than the common layout holds:
+    // the tiles again, on the sorted view, with room for every level
+    const unsigned names_differ = c.h_status->flags & F_NAMES_DIFFER;   // the pairing's verdict stays
+    const long long rmin = c.h_status->mm[MM_RSTART_MIN], rmax = c.h_status->mm[MM_REND_MAX];
+    const long long kmin = c.h_status->mm[MM_KSTART_MIN];
+    const unsigned levels = c.h_status->nlevels;
     int nks = 0;                                  // streams with kernels
-    for (int s = 0; s < 256; ++s) {
-        scmap[s] = (uint8_t)nks;
-        nks += kcnt_h[s] > 0;
-        koff_h[s] = kacc;
-        kcnt_s[s] = kcnt_h[s];
-        toff_h[s] = tacc;
-        kacc += kcnt_h[s];
-        tacc += (kcnt_h[s] + EN_TILE - 1) / EN_TILE;
+    uint8_t *scmap = c.h_stage, *unmap = c.h_stage + 256;
+    memset(c.h_stage, 0, 512);
+    for (int s = 0; s < 256; ++s)
+        if ((c.h_status->kstreams[s >> 5] >> (s & 31)) & 1u) {
+            scmap[s] = (uint8_t)nks;
+            unmap[nks++] = (uint8_t)s;
+        }
+    size_t more = 0;
+    if (!k_sorted) more += time_sort_scratch(K) + 512 + 4096;
+    {
+        Need n2;
+        n2.add<int64_t>(R).add<int64_t>(R).add<uint8_t>(R).add<uint8_t>(R).add<uint32_t>(R);
+        more += n2.bytes + time_sort_scratch(R) + 4096;
     }
-    toff_h[256] = tacc;
-    const int64_t NT = tacc;
-
-    uint64_t *rk0 = a.take<uint64_t>(R), *rk1 = a.take<uint64_t>(R);
-    uint32_t *rv0 = a.take<uint32_t>(R), *rv1 = a.take<uint32_t>(R);
-    uint32_t *hist = a.take<uint32_t>(hist_n), *hist2 = a.take<uint32_t>(hist_n);
-    int64_t *ls = a.take<int64_t>(R), *le = a.take<int64_t>(R);
-    uint32_t *li = a.take<uint32_t>(R);
-    unsigned char *d_stage = a.take<unsigned char>(ST_END);
-    uint32_t *psk = a.take<uint32_t>(K), *tinfo = a.take<uint32_t>(NT);
-    int2 *P = a.take<int2>(NT * 32);
-    if (!rk0 || !rk1 || !rv0 || !rv1 || !hist || !hist2 || !ls || !le || !li || !d_stage || !psk || !tinfo || !P)
-        return OPATTR_E_OOM;
-    const uint8_t *d_ndep = d_stage + ST_NDEP;
-    const uint8_t *d_cmap = d_stage + ST_CMAP;
-    const uint32_t *d_koff = reinterpret_cast<const uint32_t *>(d_stage + ST_KOFF);
-    const uint32_t *d_kcnt = reinterpret_cast<const uint32_t *>(d_stage + ST_KCNT);
-    const uint32_t *d_toff = reinterpret_cast<const uint32_t *>(d_stage + ST_TOFF);
-    const uint8_t *d_scmap = d_stage + ST_SCMAP;
-    if ((st = copy_small(c, d_stage, c.h_stage, ST_END, cudaMemcpyHostToDevice))) return st;
-    // the level lists (below) may start on the side stream from here
-    stream_after(c.side, c.stream, c.ev_fork);
-
-    // ---- kernel time order, then the kernels partitioned by stream
-    uint32_t *korder = nullptr;
+    // growing the arena keeps the prefix taken so far
+    c.arena_keep = (c.arena_used + 255) & ~(size_t)255;
+    {
+        const char *before = c.arena;
+        st = ensure_arena(c, more);
+        c.arena_keep = 0;
+        if (st) return st;
+        const ptrdiff_t moved = c.arena - before;
+        auto shift = [&](uint32_t *&p) { if (p) p = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(p) + moved); };
+        shift(kept_order);
+        shift(B.lvlmask);
+        shift(B.tile_r);
+        shift(B.row_len);
+        shift(B.rows);
+    }
     if (!k_sorted && K > 0) {
+        unsigned char *d_map = a.take<unsigned char>(512);
+        if (!d_map) return OPATTR_E_OOM;
+        if ((st = copy_small(c, d_map, c.h_stage, 512, cudaMemcpyHostToDevice))) return st;
         // keyed by the compact ids of the streams with kernels
-        if ((st = kernel_time_order(c, a, kern->stream, kern->start_ns, K, &korder, d_scmap,
-                                    bits_for((uint64_t)(nks - 1)))))
-            return st;
+        const int sbits = bits_for((uint64_t)(nks - 1));
+        uint64_t *keys = nullptr;
+        uint32_t *korder = nullptr;
+        if ((st = kernel_time_order(c, a, kern->stream, kern->start_ns, K, &korder, d_map, sbits, &keys))) return st;
+        V.k_key = keys;
+        V.k_tmin = kmin;
+        V.k_sbits = sbits;
+        V.k_unmap = d_map + 256;
+        V.korder = korder;
         if (kept_order) {
             cudaMemcpyAsync(kept_order, korder, sizeof(uint32_t) * K, cudaMemcpyDeviceToDevice, c.stream);
             c.join_korder = kept_order;
             c.arena_keep = (sizeof(uint32_t) * (size_t)K + 255) & ~(size_t)255;
         }
     }
-    if (K > 0 && nl > 0 && k_sorted) {
-        // in time order already: the order check's tile counts are the
-        // partition's histogram (stream ids as digits)
-        // (rows past the last stream with kernels hold only zeros: not scanned)
-        const int64_t ntk = (K + RADIX_TILE - 1) / RADIX_TILE;
-        int rows = 0;
-        for (int q = 0; q < 256; ++q)
-            if (kcnt_h[q] > 0) rows = q + 1;
-        scan_exclusive_u32(c, ktile, hist, ntk * rows, part, nullptr);
-        digit_rank(c, "stream_place", ArrayStreamDigit{kern->stream}, K, hist, PlaceByStream{nullptr, psk});
-    } else if (K > 0 && nl > 0) {
-        const TimeStreamDigit dg{kern->stream, korder, d_scmap};
-        const uint32_t *offs = digit_offsets(c, dg, K, hist, part, nks);
-        digit_rank(c, "stream_place", dg, K, offs, PlaceByStream{korder, psk});
-    }
-
-    // ---- level lists, their validation, the windows and the enclosure, without
-    // a synchronisation in between: a failed validation is reported at the end
-    // (the enclosure reads only positions found by searches inside the level
-    // lists, so non-laminar ranges give wrong answers but no stray access).
-    // If ranges with equal starts were not in (start, end, index) order within
-    // a level, the whole pass runs again on fully sorted ranges.  The level
-    // lists and their validation run on the side stream, beside the stream
-    // partition (their own scratch: hist2, part2); the windows wait for the
-    // lists, the status read for the validation.
-    const unsigned g = grid_for(R, 256, 65535);
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        const bool full_sort = !r_sorted || attempt > 0;
-        if (attempt > 0) stream_after(c.side, c.stream, c.ev_fork);
-        {
-            OnStream on(c, c.side);
-            uint32_t *perm = nullptr;     // range indices in the order of the level sort
-            if (full_sort) {
-                // (start, end, index) order within every level of laminar
-                // ranges: one stable sort on (start, longer than zero)
-                uint64_t *ko;
-                const int bits = bits_for((uint64_t)(rmax - rmin)) + 1;
-                launch(c, "range_time_key", k_range_start_key, dim3(g), dim3(256), 0, rng->start_ns, rng->end_ns, R,
-                       rmin, rk0);
-                radix_sort_pairs<uint64_t>(c, rk0, rv0, rk1, rv1, R, bits, true, hist2, part2, &ko, &perm);
-            }
-            if (nl <= 256) {
-                // stable partition by compact level id, ranges written in place
-                const LevelDigit dg{rng->stream, rng->depth, d_cmap, perm};
-                const uint32_t *offs = digit_offsets(c, dg, R, hist2, part2, nl);
-                const int64_t ntiles = (R + RADIX_TILE - 1) / RADIX_TILE;
-                launch(c, "level_place", k_level_place, dim3((unsigned)ntiles), dim3(RADIX_THREADS), 0, dg,
-                       rng->start_ns, rng->end_ns, rng->op_id, R, offs, ntiles, ls, le, li);
-            } else {
-                // stable partition by level key (13 bits)
-                uint32_t *lk0 = reinterpret_cast<uint32_t *>(rk0), *lk1 = reinterpret_cast<uint32_t *>(rk1);
-                uint32_t *va = perm ? perm : rv0;
-                uint32_t *vb = perm == rv0 ? rv1 : (perm == rv1 ? rv0 : rv1);
-                launch(c, "level_keys", k_level_keys, dim3(g), dim3(256), 0, rng->stream, rng->depth,
-                       (const uint32_t *)perm, R, lk0);
-                uint32_t *ko32, *lperm;
-                radix_sort_pairs<uint32_t>(c, lk0, va, lk1, vb, R, 13, perm == nullptr, hist2, part2, &ko32, &lperm);
-                launch(c, "level_gather", k_level_gather, dim3(g), dim3(256), 0, rng->start_ns, rng->end_ns,
-                       rng->op_id, (const uint32_t *)lperm, R, ls, le, li);
-            }
-            cudaEventRecord(c.ev_join, c.side);           // the level lists are in place
-            launch(c, "validate_levels", k_validate_levels, dim3(grid_for(R, 256 * VL_PER, 65535)), dim3(256), 0,
-                   rng->stream, rng->depth, (const int64_t *)ls, (const int64_t *)le, (const uint32_t *)li,
-                   (const uint32_t *)lvl_off, R, c.d_status);
-            // within a join: the matching's identity pairing, beside the enclosure
-            if (c.spec_k > 0) {
-                launch_identity_match(c, c.spec_kname, c.spec_nname, c.spec_k, c.spec_idx, c.spec_kind);
-                c.spec_ran = true;
-            }
-            cudaEventRecord(c.ev_join2, c.side);          // and checked
+    const EncView raw = V;
+    int64_t *gs = a.take<int64_t>(R), *ge = a.take<int64_t>(R);
+    uint8_t *gt = a.take<uint8_t>(R), *gd = a.take<uint8_t>(R);
+    uint32_t *go = a.take<uint32_t>(R);
+    if (!gs || !ge || !gt || !gd || !go) return OPATTR_E_OOM;
+    // ranges sorted so that parents come first: their verdict is final
+    bool sort_ranges = !r_sorted || fixup, sorted = false;
+    bool have_parts = k_sorted && !sort_ranges;       // (too many levels only: the checking pass's parts stand)
+    int nl = many ? (int)levels : EN_LEVELS_A;
+    bool wide = many;
+    for (int attempt = 0; attempt < 4; ++attempt) {
+        if (sort_ranges && R > 0) {
+            uint64_t *ko = nullptr;
+            uint32_t *perm = nullptr;
+            if ((st = range_time_order(c, a, rng->start_ns, rng->end_ns, rng->depth, R, rmin, rmax, &perm, &ko)))
+                return st;
+            launch(c, "range_gather", k_range_gather, dim3(grid_for(R, 256, 65535)), dim3(256), 0, raw,
+                   (const uint64_t *)ko, RANGE_KEY_SHIFT, rmin, (const uint32_t *)perm, gs, ge, gt, gd, go);
+            V.r_start = gs;
+            V.r_end = ge;
+            V.r_stream = gt;
+            V.r_depth = gd;
+            V.r_op = go;
+            V.perm = perm;
+            sort_ranges = false;
+            sorted = true;
         }
-        cudaStreamWaitEvent(c.stream, c.ev_join, 0);
-        if (K > 0 && nl == 0)
-            launch(c, "fill_unattributed", k_fill_unattributed, dim3(grid_for(K, 256, 65535)), dim3(256), 0, out_range,
-                   out_nop, K);
-        if (K > 0 && nl > 0) {
-            launch(c, "stream_windows", k_stream_windows, dim3(grid_for(NT * 32, 256, 65535)), dim3(256), 0,
-                   (const int64_t *)ls, (const uint32_t *)lvl_off, d_ndep, d_toff, d_koff, d_kcnt,
-                   (const uint32_t *)psk, kern->start_ns, NT, P, tinfo);
-            EncArgs A;
-            A.k_start = kern->start_ns;
-            A.psk = psk;
-            A.tinfo = tinfo;
-            A.toff = d_toff;
-            A.koff = d_koff;
-            A.kcnt = d_kcnt;
-            A.ndep = d_ndep;
-            A.ls = ls;
-            A.le = le;
-            A.li = li;
-            A.lvl_off = lvl_off;
-            A.P = P;
-            A.out_range = out_range;
-            A.out_nop = out_nop;
-            launch(c, "enclose", k_enclose, dim3((unsigned)NT), dim3(EN_THREADS), 0, A);
+        const ZeroRun zs{c.d_status, 2};              // err and flags
+        if ((st = zero_runs(c, 1, &zs))) return st;
+        const bool keys = V.k_key != nullptr;
+        if (!have_parts) {
+            launch(c, "enc_view", keys ? k_enc_parts<false, true> : k_enc_parts<false, false>, dim3((unsigned)B.parts),
+                   dim3(EP_THREADS), 0, V, EncCheck{}, B.parts, B.tp, B.tile_r, B.rows, B.row_len, B.lvlmask,
+                   c.d_status);
+            launch_carry(c, B);
         }
-        cudaStreamWaitEvent(c.stream, c.ev_join2, 0);
-        if (c.defer_status && k_sorted && !full_sort) {
-            // the status is read with the aggregation's, which the join checks
-            c.enclose_pending = true;
-            return OPATTR_OK;
-        }
+        have_parts = true;
+        if (!wide)
+            (keys ? launch_tiles<EncTileA, true> : launch_tiles<EncTileA, false>)(c, V, B, EN_LEVELS_A, 1, 0u, sorted,
+                                                                                  out_range, out_nop);
+        else if (nl <= EN_LEVELS_B)
+            (keys ? launch_tiles<EncTileB, true> : launch_tiles<EncTileB, false>)(c, V, B, nl, 1, 0u, sorted, out_range,
+                                                                                  out_nop);
+        else
+            (keys ? launch_tiles<EncTileB, true, true> : launch_tiles<EncTileB, false, true>)(
+                c, V, B, EN_LEVELS_B, 4, 0u, sorted, out_range, out_nop);
         if ((st = read_status(c))) return st;
-        if (!full_sort && (c.h_status->flags & F_LEVEL_FIXUP)) {
-            // equal starts out of (start, end) order within a level: the
-            // nesting checks above saw a level list out of order, so their
-            // verdict does not count; the pass on fully sorted ranges decides
-            c.h_status->flags &= ~F_LEVEL_FIXUP;
-            c.h_status->err = 0;
-            cudaMemsetAsync(c.d_status, 0, 2 * sizeof(unsigned), c.stream);   // err and flags
+        if (c.h_status->flags & F_LEVELS_MANY) {
+            nl = (int)c.h_status->nlevels;
+            wide = true;
             continue;
         }
-        if ((st = status_from_err(c.h_status->err))) return st;
-        // after the sort, equal starts out of (start, end) order in a level
-        // are two longer ranges with one start: overlapping, not laminar
-        if (c.h_status->flags & F_LEVEL_FIXUP) return OPATTR_E_NOT_NESTED;
-        return OPATTR_OK;
+        if ((c.h_status->flags & F_LEVEL_FIXUP) && !sorted) {
+            sort_ranges = true;
+            have_parts = false;
+            continue;
+        }
+        c.h_status->flags |= names_differ;
+        return enclose_verdict(*c.h_status, K);
     }
     return OPATTR_E_CUDA;
 }

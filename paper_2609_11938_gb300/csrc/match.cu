@@ -62,12 +62,6 @@ __global__ void k_match_identity(const uint32_t *__restrict__ kname, const uint3
     if (__any_sync(0xffffffffu, bad) && lane_id() == 0) set_flag(st, F_NAMES_DIFFER);
 }
 
-void launch_identity_match(Ctx &c, const uint32_t *kname, const uint32_t *nname, int64_t K, int32_t *out_idx,
-                           uint8_t *out_kind) {
-    launch(c, "match_identity", k_match_identity, dim3(grid_for(K, 256 * 16, REDUCE_GRID)), dim3(256), 0, kname,
-           nname, K, out_idx, out_kind, identity_vec(kname, nname, out_idx, out_kind), c.d_status);
-}
-
 // replayed kernels in time order (list rk) against rows 0..n-1
 __global__ void k_match_identity_list(const uint32_t *__restrict__ rk, const uint32_t *__restrict__ kname,
                                       const uint32_t *__restrict__ nname, int64_t n, int32_t *__restrict__ out_idx,
@@ -426,7 +420,7 @@ opattr_status do_match(Ctx &c, const opattr_kernels *kern, const opattr_ncu *ncu
     const int64_t NX = std::max(K, M);
     const bool per_stream = ncu->stream != nullptr;
     if (per_stream && M > 0 && !ncu->name_id) return OPATTR_E_INVALID_ARG;
-    // within a join the identity pairing ran beside the enclosure: with the
+    // within a join the identity pairing ran within the enclosure: with the
     // kernels in time order (the enclosure's verdict) and every name equal,
     // its outputs are the match
     // (with the enclosure's status still to be read, the names are taken to

@@ -66,13 +66,8 @@ extern "C" opattr_status opattr_match_noalloc(const opattr_kernels *kernels, con
     }
     char *base = static_cast<char *>(p);
     // status block first, the arena after it; host mirrors are plain host memory
-    DevStatus h_status, h_init;
-    memset(&h_init, 0, sizeof h_init);
-    h_init.mm[MM_KSTART_MIN] = LLONG_MAX;
-    h_init.mm[MM_KSTART_MAX] = LLONG_MIN;
-    h_init.mm[MM_RSTART_MIN] = LLONG_MAX;
-    h_init.mm[MM_REND_MAX] = LLONG_MIN;
-    h_status = h_init;
+    DevStatus h_status;
+    memset(&h_status, 0, sizeof h_status);
     Ctx c;
     c.device = dev;
     c.stream = (cudaStream_t)cuda_stream;
@@ -80,7 +75,6 @@ extern "C" opattr_status opattr_match_noalloc(const opattr_kernels *kernels, con
     c.cfg.dedup = 0;
     c.d_status = reinterpret_cast<DevStatus *>(base);
     c.h_status = &h_status;
-    c.h_init = &h_init;
     const size_t status_bytes = (sizeof(DevStatus) + 255) & ~(size_t)255;
     c.arena = base + status_bytes;
     c.arena_cap = NOALLOC_SCRATCH_BYTES - status_bytes;

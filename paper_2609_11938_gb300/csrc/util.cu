@@ -8,30 +8,19 @@ namespace opattr {
 
 constexpr int CHK_THREADS = 256;
 
-// Tiles of CHK_TILE consecutive kernels (the digit passes' tiles), a block
-// at a time, each thread taking two groups of eight consecutive kernels per
-// tile (16-byte loads when the arrays allow) and comparing each (start,
-// stream) with its successor; min / max and the order flag are reduced per
-// block and published with one atomic each.  With stream_hist the block also
-// counts the kernels of each stream (added to the 256 counters once per
-// block), and with tile_hist it writes each tile's counts as column `tile`
-// of a stream-major matrix (tile_hist[s * ntiles + tile]): the digit
-// histogram of a stable partition by stream, in array order.
+// Tiles of CHK_TILE consecutive kernels, a block at a time, each thread taking
+// two groups of eight consecutive kernels per tile (16-byte loads when the
+// arrays allow) and comparing each (start, stream) with its successor; min /
+// max and the order flag are reduced per block and published with one atomic
+// each.
 constexpr int CHK_G = 8;
 constexpr int CHK_TILE = 2 * CHK_THREADS * CHK_G;
-static_assert(CHK_TILE == RADIX_TILE, "the order check's tiles are the digit passes' tiles");
 __global__ void __launch_bounds__(CHK_THREADS) k_check_kernel_order(const uint8_t *__restrict__ stream,
                                                                     const int64_t *__restrict__ start, int64_t n,
-                                                                    int vec, DevStatus *st,
-                                                                    uint32_t *__restrict__ stream_hist,
-                                                                    uint32_t *__restrict__ tile_hist) {
+                                                                    int vec, DevStatus *st) {
     pdl_wait();
     __shared__ long long smin[CHK_THREADS / 32], smax[CHK_THREADS / 32];
     __shared__ int sbad[CHK_THREADS / 32];
-    __shared__ uint32_t sh[256], th[256];
-    const bool count = stream_hist || tile_hist;
-    for (int i = threadIdx.x; i < 256; i += CHK_THREADS) sh[i] = th[i] = 0;
-    __syncthreads();
     long long mn = LLONG_MAX, mx = LLONG_MIN;
     int unsorted = 0;
     const int64_t ntiles = (n + CHK_TILE - 1) / CHK_TILE;
@@ -70,23 +59,8 @@ __global__ void __launch_bounds__(CHK_THREADS) k_check_kernel_order(const uint8_
                 mn = t[u] < mn ? t[u] : mn;
                 mx = t[u] > mx ? t[u] : mx;
                 if (i0 + u + 1 < n) unsorted |= (t[u + 1] < t[u]) || (t[u + 1] == t[u] && s[u + 1] < s[u]);
-                if (count) atomicAdd(&th[s[u]], 1u);
             }
         }
-        if (count) {
-            __syncthreads();
-            for (int i = threadIdx.x; i < 256; i += CHK_THREADS) {
-                const uint32_t x = th[i];
-                if (tile_hist) tile_hist[(int64_t)i * ntiles + tile] = x;
-                sh[i] += x;
-                th[i] = 0;
-            }
-            __syncthreads();
-        }
-    }
-    if (stream_hist) {
-        for (int i = threadIdx.x; i < 256; i += CHK_THREADS)
-            if (sh[i]) atomicAdd(&stream_hist[i], sh[i]);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -114,12 +88,11 @@ __global__ void __launch_bounds__(CHK_THREADS) k_check_kernel_order(const uint8_
     }
 }
 
-void check_kernel_order(Ctx &c, const uint8_t *stream, const int64_t *start, int64_t n, uint32_t *stream_hist,
-                        uint32_t *tile_hist) {
+void check_kernel_order(Ctx &c, const uint8_t *stream, const int64_t *start, int64_t n) {
     if (n <= 0) return;
     const int vec = ((reinterpret_cast<uintptr_t>(start) & 15) == 0) && ((reinterpret_cast<uintptr_t>(stream) & 7) == 0);
     launch(c, "check_kernel_order", k_check_kernel_order, dim3(grid_for(n, CHK_TILE, REDUCE_GRID)),
-           dim3(CHK_THREADS), 0, stream, start, n, vec, c.d_status, stream_hist, tile_hist);
+           dim3(CHK_THREADS), 0, stream, start, n, vec, c.d_status);
 }
 
 // ------------------------------------------------------------------ time sort
@@ -130,7 +103,7 @@ void check_kernel_order(Ctx &c, const uint8_t *stream, const int64_t *start, int
 // every bin, a few records each, by key and index.  Two reads and two writes of
 // 8 bytes per record, where the radix sort makes a pass of 24 bytes per eight
 // key bits.  Times crowd when a trace has long gaps or many equal times: a
-// bucket above BK_CAP records or a bin above BK_BIN_MAX sets F_BUCKETS, and the
+// bucket above BK_CAP records or a bin above BK_BIN_MAX sets *crowded, and the
 // radix sort does the whole again.
 //
 // 6M kernel records in no order: 16 us to count, 77 to scatter (bound by the
@@ -188,7 +161,7 @@ __global__ void __launch_bounds__(BK_THREADS) k_bucket_scatter(Key key, int64_t 
 __global__ void __launch_bounds__(BK_THREADS) k_bucket_sort(const uint64_t *__restrict__ in,
                                                             const uint32_t *__restrict__ end, int shift,
                                                             uint64_t *__restrict__ keys, uint32_t *__restrict__ perm,
-                                                            DevStatus *st) {
+                                                            uint32_t *crowded) {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char bk_smem[];
     uint64_t *buf = reinterpret_cast<uint64_t *>(bk_smem);              // [BK_CAP]
@@ -198,7 +171,7 @@ __global__ void __launch_bounds__(BK_THREADS) k_bucket_sort(const uint64_t *__re
     const uint32_t s0 = b ? end[b - 1] : 0u, m = end[b] - s0;
     if (m == 0) return;
     if (m > (uint32_t)BK_CAP) {
-        if (threadIdx.x == 0) set_flag(st, F_BUCKETS);
+        if (threadIdx.x == 0) *crowded = 1u;
         return;
     }
     constexpr int PER = BK_BINS / BK_THREADS;
@@ -232,7 +205,7 @@ __global__ void __launch_bounds__(BK_THREADS) k_bucket_sort(const uint64_t *__re
         ex += c[q];
     }
     if (__syncthreads_or(full)) {
-        if (threadIdx.x == 0) set_flag(st, F_BUCKETS);
+        if (threadIdx.x == 0) *crowded = 1u;
         return;
     }
 #pragma unroll
@@ -284,24 +257,26 @@ static opattr_status time_sort(Ctx &c, Arena &a, Key key, int64_t n, uint64_t to
     while (shift > 0 && (int64_t)(top >> shift) + 1 < (n + BK_TARGET - 1) / BK_TARGET) --shift;
     const int64_t nb = (int64_t)(top >> shift) + 1;
     if (c.host_mapped && nb <= BK_MAX) {
-        int sms = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device);
+        const int sms = sm_count(c);
         const size_t smem = sizeof(uint32_t) * nb, sort_smem = sizeof(uint64_t) * BK_CAP + sizeof(uint32_t) * BK_BINS;
-        const dim3 g(grid_for(n, BK_THREADS * 8, (smem > 64 * 1024 ? 1 : 3) * std::max(1, sms)));
+        const dim3 g(grid_for(n, BK_THREADS * 8, (smem > 64 * 1024 ? 1 : 3) * sms));
         cudaFuncSetAttribute(k_bucket_count<Key>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(4 * BK_MAX));
         cudaFuncSetAttribute(k_bucket_scatter<Key>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(4 * BK_MAX));
         cudaFuncSetAttribute(k_bucket_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem);
-        cudaMemsetAsync(hist, 0, sizeof(uint32_t) * nb, c.stream);
+        uint32_t *crowded = hist + nb;                // after the counts: hist holds BK_MAX + 1 at least
+        const ZeroRun z{hist, nb + 1};
+        opattr_status st = zero_runs(c, 1, &z);
+        if (st) return st;
         launch(c, "bucket_count", k_bucket_count<Key>, g, dim3(BK_THREADS), smem, key, n, shift, (int)nb, hist);
         scan_exclusive_u32(c, hist, hist, nb, part, nullptr);
         launch(c, "bucket_scatter", k_bucket_scatter<Key>, g, dim3(BK_THREADS), smem, key, n, shift, (int)nb, hist, k0);
         launch(c, "bucket_sort", k_bucket_sort, dim3((unsigned)nb), dim3(BK_THREADS), sort_smem, (const uint64_t *)k0,
-               (const uint32_t *)hist, shift, k1, v1, c.d_status);
-        opattr_status st = read_status(c);
-        if (st) return st;
+               (const uint32_t *)hist, shift, k1, v1, crowded);
+        const SmallCopy verdict{c.h_small, crowded, sizeof(uint32_t)};
+        if ((st = read_status(c, 1, &verdict))) return st;
         *keys = k1;
         *perm = v1;
-        if (!(c.h_status->flags & F_BUCKETS)) return OPATTR_OK;
+        if (!c.h_small[0]) return OPATTR_OK;
     }
     launch(c, "time_keys", k_write_keys<Key>, dim3(grid_for(n, 256, 65535)), dim3(256), 0, key, n, k0);
     radix_sort_pairs<uint64_t>(c, k0, v0, k1, v1, n, bits_for(top), true, hist, part, keys, perm);
@@ -327,6 +302,27 @@ opattr_status kernel_time_order(Ctx &c, Arena &a, const uint8_t *stream, const i
                                        ((uint64_t)(tmax - tmin) << sbits) | ((1ull << sbits) - 1), &k, order);
     if (keys) *keys = k;
     return st;
+}
+
+// The order key of range i: its start, then its depth, so that parents come
+// before children that start with them, then 0 for a zero-length range and 1
+// for a longer one.  Within a level of laminar ranges two ranges share a start
+// only if all but the last of them have zero length, so a stable sort on this
+// key puts every level in (start, end, index) order -- the order of Algorithm
+// 2's one representative per depth; two longer ranges sharing a start in one
+// level are out of that order only when they overlap, which the laminar
+// checks report.
+struct RangeTimeKey {
+    const int64_t *start, *end;
+    const uint8_t *depth;
+    long long tmin;
+    __device__ __forceinline__ uint64_t operator()(int64_t i) const {
+        return (((uint64_t)(start[i] - tmin) << 5 | depth[i]) << 1) | (end[i] > start[i] ? 1u : 0u);
+    }
+};
+opattr_status range_time_order(Ctx &c, Arena &a, const int64_t *start, const int64_t *end, const uint8_t *depth,
+                               int64_t n, long long tmin, long long tmax, uint32_t **order, uint64_t **keys) {
+    return time_sort(c, a, RangeTimeKey{start, end, depth, tmin}, n, ((uint64_t)(tmax - tmin) << 6) | 63u, keys, order);
 }
 
 }  // namespace opattr

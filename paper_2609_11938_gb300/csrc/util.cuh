@@ -7,19 +7,15 @@
 namespace opattr {
 
 // Sets F_K_UNSORTED unless (start_ns, stream) is non-decreasing along the
-// array, and records min / max start in MM_KSTART_MIN / MM_KSTART_MAX.  With
-// stream_hist (256 zeroed counters), also counts the kernels of each stream;
-// with tile_hist (radix_hist_elems(n) counters), writes the stream counts of
-// every RADIX_TILE tile of the array as a stream-major matrix.
-void check_kernel_order(Ctx &c, const uint8_t *stream, const int64_t *start, int64_t n,
-                        uint32_t *stream_hist = nullptr, uint32_t *tile_hist = nullptr);
+// array, and records min / max start in MM_KSTART_MIN / MM_KSTART_MAX.
+void check_kernel_order(Ctx &c, const uint8_t *stream, const int64_t *start, int64_t n);
 
 // Scratch (bytes) of a time sort of n records (kernel_time_order).
 size_t time_sort_scratch(int64_t n);
 
 // Permutation of kernel indices into time order (start, stream, index): sorted
 // by (start - min_start) << sbits | stream.  Needs the min / max from
-// check_kernel_order in c.h_status.  With scmap (device, [256]: increasing
+// check_kernel_order (or the enclosure's checks) in c.h_status.  With scmap (device, [256]: increasing
 // compact ids of the streams that have kernels) the key holds the compact id
 // in stream_bits bits instead of the id in 8.  *order receives a device array
 // of n indices carved from `a`, *keys (if given) the sorted keys.  May wait on
@@ -27,5 +23,12 @@ size_t time_sort_scratch(int64_t n);
 opattr_status kernel_time_order(Ctx &c, struct Arena &a, const uint8_t *stream, const int64_t *start, int64_t n,
                                 uint32_t **order, const uint8_t *scmap = nullptr, int stream_bits = 8,
                                 uint64_t **keys = nullptr);
+
+// The same for ranges: sorted by (start - tmin) << 6 | depth << 1 | (longer than
+// zero), with tmin the smallest start and tmax no smaller than the largest.
+constexpr int RANGE_KEY_SHIFT = 6;
+opattr_status range_time_order(Ctx &c, struct Arena &a, const int64_t *start, const int64_t *end,
+                               const uint8_t *depth, int64_t n, long long tmin, long long tmax, uint32_t **order,
+                               uint64_t **keys);
 
 }  // namespace opattr

@@ -1,0 +1,53 @@
+"""The enclosure's tiles (GPU) where they can go wrong: parts and tiles of a few
+events and one more, more ranges in a tile than one step takes, more streams or
+levels than the common layout holds, and instants at which many ranges start
+and end together cut by a tile's edge.  Against the oracle."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import oracle
+import tracegen
+from gpu_util import assert_parity, gpu_run
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(t):
+    assert_parity(gpu_run(t), oracle.run(t, enclose_mode="indexed"))
+
+
+@pytest.mark.parametrize("n", [1, 395, 396, 397, 800, 16_000, 16_800, 70_001])
+def test_tile_edges(n):
+    """About 1.29 events per kernel; a tile holds 512 in small traces, and past
+    32 parts the carried ranges come from their own pass."""
+    _check(tracegen.generate("large", n_kernels=n, n_streams=3, seed=n))
+
+
+@pytest.mark.parametrize("streams,depth", [(64, 3), (65, 3), (70, 2), (16, 32), (17, 32), (20, 30), (64, 32), (66, 32)])
+@pytest.mark.parametrize("shuffle", [False, True])
+def test_layouts(streams, depth, shuffle):
+    """Streams and levels on both sides of the common layout (64 streams, 512
+    levels) and of the wide one (2,048 levels)."""
+    _check(tracegen.generate("adversarial", n_kernels=30_000, n_streams=streams, max_depth=depth, seed=streams + depth,
+                             shuffle=shuffle))
+
+
+@pytest.mark.parametrize("seed", range(6))
+def test_ties_across_tiles(seed):
+    """Thousands of events at few instants: ties of starts, ends and kernels
+    run over tile and step edges (ranges in array order and permuted)."""
+    t = tracegen.small_random(400 + seed, n_streams=1 + seed % 3, n_events=9000, t_max=40, max_depth=5,
+                              shuffle=bool(seed & 1), n_names=7)
+    _check(t)
+
+
+def test_ranges_without_kernels():
+    """Many more ranges than kernels: tiles of ranges alone, taken in steps."""
+    t = tracegen.generate("large", n_kernels=60_000, n_streams=2, seed=3)
+    keep = np.arange(t.K) < 40
+    n = int(keep.sum())
+    t = dataclasses.replace(t, k_stream=t.k_stream[:n].copy(), k_start=t.k_start[:n].copy(), k_dur=t.k_dur[:n].copy(),
+                            k_name=t.k_name[:n].copy(), ncu_name=t.ncu_name[:n].copy(), counters=t.counters[:n].copy())
+    _check(t)
