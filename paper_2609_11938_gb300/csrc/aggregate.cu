@@ -36,10 +36,12 @@ struct AggIn {
     const float *counters;
     int64_t M;                  // ncu rows: a row index at or past M is never read (the count pass reports it)
     int64_t n_ops;
-    unsigned *ctr;              // [0] next chunk of the ops pass, [1] ops listed in dirty; zeroed before it
+    uint32_t lane_max;          // longest op that one lane takes
+    unsigned *ctr;              // [0] next chunk of the ops pass, [1] ops listed in dirty, [2] in mids, [3] in longs;
+                                // zeroed before it
     uint32_t *dirty;            // ops whose fast sums saw a null or infinite value
-    uint32_t *longs;            // ops the ops pass leaves to the pieces pass (listed there)
-    unsigned *nlong;            //   and their number (zeroed before the ops pass)
+    uint32_t *mids;             // ops longer than a lane takes: a block each (k_agg_mid)
+    uint32_t *longs;            // ops longer than a block takes: the pieces pass
     const unsigned *nonident;   // nonzero unless ncu_idx[k] == k for every kernel (set by the count pass)
     opattr_op_aggregates out;
 };
@@ -433,28 +435,28 @@ __global__ void k_agg_place(const int32_t *__restrict__ rok, const uint32_t *__r
 }
 
 // ------------------------------------------------------------------ long segments
-// Segments of the ops longer than AG_HUGE (the pieces pass below) are sorted
-// by kernel index first, one block per segment: up to SL_SMEM entries by a
-// bitonic sort in shared memory; longer ones in SL_SMEM runs sorted that way,
-// then merged pairwise through `tmp` (merge path: each thread merges an equal
-// share of the output after a binary search on its diagonal).
+// Segments of the ops longer than AG_MID_MAX (the pieces pass below), when a
+// counting pass cannot place them in order, are sorted by kernel index first,
+// one block per segment: up to SL_SMEM entries by a bitonic sort in shared
+// memory; longer ones in SL_SMEM runs sorted that way, then merged pairwise
+// through `tmp` (merge path: each thread merges an equal share of the output
+// after a binary search on its diagonal).
 constexpr int SL_THREADS = 256;
 constexpr int SL_SMEM = 8192;
 
-constexpr uint32_t AG_SHORT_MAX = 64;           // segments up to this length: sorted in place by one lane
-constexpr uint32_t AG_HUGE = 256;               // longer segments: split into pieces over several warps
-constexpr uint32_t AG_PIECE = 1024;              // kernels of a huge op per warp of the pieces pass
-constexpr uint32_t AG_BLOCK_SORT_MAX = 4096;     // longer huge segments: placed by a counting pass, not sorted
+// Ops up to this length, or up to four times the average one, are left to one
+// lane of the ops pass; AG_LANE_TOP at most.
+constexpr uint32_t AG_LANE_MAX = 64, AG_LANE_TOP = 256;
+constexpr uint32_t AG_MID_MAX = 4096;           // up to this length: one block; longer: pieces over several warps
+constexpr uint32_t AG_PIECE = 1024;             // kernels of such an op per warp of the pieces pass
 
 __device__ void bitonic_smem(uint32_t *a, int n2) {     // n2 a power of two; the block sorts a[0..n2)
     for (int k = 2; k <= n2; k <<= 1)
         for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < n2; i += blockDim.x) {
-                const int p = i ^ j;
-                if (p > i) {
-                    const uint32_t x = a[i], y = a[p];
-                    if (((i & k) == 0) == (x > y)) { a[i] = y; a[p] = x; }
-                }
+            for (int q = threadIdx.x; q < n2 / 2; q += blockDim.x) {
+                const int i = 2 * q - (q & (j - 1)), p = i + j;
+                const uint32_t x = a[i], y = a[p];
+                if (((i & k) == 0) == (x > y)) { a[i] = y; a[p] = x; }
             }
             __syncthreads();
         }
@@ -528,10 +530,10 @@ __global__ void __launch_bounds__(SL_THREADS) k_agg_sort_long(const uint32_t *__
 // memory by coalesced loads, and each thread checks its segments there and,
 // in the rare case the count pass met an op in two runs, sorts them in place,
 // so segments are walked in ascending kernel index (a larger chunk reads the
-// list in place: segments up to AG_SHORT_MAX are checked and sorted there).
-// Ops longer than AG_HUGE, and longer than AG_SHORT_MAX in a chunk that does
-// not fit, are listed for the pieces pass instead (sorted there by a block
-// each).  While a kernel is added, the counter rows and durations
+// list in place).  Ops longer than lane_max are listed instead, for a block
+// each or for the pieces pass: a lane waits up to a microsecond for each of its
+// kernels, and one op of 250 held the pass (4M kernels with fusion operators:
+// 589 us) for four times as long as all the others.  While a kernel is added, the counter rows and durations
 // of the next two arrive in per-thread shared-memory slots by asynchronous
 // copy (cp.async), with their row indices loaded a step earlier still (or
 // taken to be the kernel indices when the count pass found every row to be
@@ -556,7 +558,20 @@ constexpr size_t AG_SMEM = sizeof(OpsWarp) * AG_WARPS;
 __device__ __noinline__ int op_careful(const uint32_t *seg, uint32_t len, AggIn A, int64_t o) {
     Acc acc;
     acc.init();
-    for (uint32_t t = 0; t < len; ++t) acc.add(A, seg[t]);
+    // kernel t + 1's duration and row index, and t + 2's index, in flight during t
+    uint32_t k = len > 1 ? seg[1] : 0u;
+    long long d = len > 0 ? A.dur[seg[0]] : 0;
+    int32_t j = len > 0 ? A.ncu_idx[seg[0]] : -1;
+    for (uint32_t t = 0; t < len; ++t) {
+        const long long d1 = t + 1 < len ? A.dur[k] : 0;
+        const int32_t j1 = t + 1 < len ? A.ncu_idx[k] : -1;
+        const uint32_t k2 = t + 2 < len ? seg[t + 2] : 0u;
+        const bool ok = j >= 0 && j < A.M;
+        acc.accumulate(d, ok, reinterpret_cast<const float4 *>(A.counters + (int64_t)(ok ? j : 0) * NC));
+        d = d1;
+        j = j1;
+        k = k2;
+    }
     acc.write(A, o);
     return acc.bad;
 }
@@ -651,8 +666,9 @@ __global__ void __launch_bounds__(AG_THREADS, 5) k_agg_ops(const uint32_t *__res
             if (i < nchunk) W.order[atomicAdd(&W.lcount[bkt[q]], 1u)] = (uint8_t)i;
             // each thread puts the segments of its own ops in ascending order
             const uint32_t len = i < nchunk ? ob[q] - oa[q] : 0u;
-            if (len > AG_HUGE || (!staged && len > AG_SHORT_MAX)) {
-                A.longs[atomicAdd(A.nlong, 1u)] = (uint32_t)(o0 + i);   // for the pieces pass
+            if (len > A.lane_max) {
+                const bool mid = len <= AG_MID_MAX;
+                (mid ? A.mids : A.longs)[atomicAdd(A.ctr + (mid ? 2 : 3), 1u)] = (uint32_t)(o0 + i);
             } else if (len > 1) {
                 if (staged) sort_segment(W.L + (oa[q] - cbase), len);
                 else sort_segment(list + oa[q], len);
@@ -683,7 +699,7 @@ __global__ void __launch_bounds__(AG_THREADS, 5) k_agg_ops(const uint32_t *__res
             if (i >= nchunk) continue;
             const int64_t o = o0 + il;
             const uint32_t s0 = sa, len = sb - sa;
-            if (len > AG_HUGE || (!staged && len > AG_SHORT_MAX)) continue;   // listed: k_agg_long_ops writes it
+            if (len > A.lane_max) continue;                       // listed
             const uint32_t *seg = staged ? W.L + (s0 - cbase) : list + s0;
             AccF acc;
             acc.init();
@@ -752,12 +768,12 @@ __global__ void k_agg_careful(const uint32_t *__restrict__ off, uint32_t *list, 
 
 // ------------------------------------------------------------------ host
 // ------------------------------------------------------------------ long ops
-// Ops the ops pass lists (longer than AG_HUGE, or longer than AG_SHORT_MAX
-// in a chunk it could not stage; sorted by k_agg_sort_long or placed in order
-// by a counting pass) are split into pieces of AG_PIECE kernels, so an
-// operator with a very long segment (an Inductor fusion-map operator gathers
-// every unattributed launch of its kernel name) is spread over many warps
-// instead of holding one thread for its whole length.  Each lane adds a
+// Ops longer than AG_MID_MAX that the ops pass lists (sorted by
+// k_agg_sort_long or placed in order by a counting pass) are split into pieces
+// of AG_PIECE kernels, so an operator with a very long segment (an Inductor
+// fusion-map operator gathers every unattributed launch of its kernel name) is
+// spread over many warps instead of holding one block for its whole length.
+// Each lane adds a
 // contiguous run of a piece in ascending kernel index with the careful
 // accumulator; partials are combined by fixed trees of pairwise float-float
 // additions (lane l takes lane l + 16, then l + 8, ...; a piece's partials in
@@ -971,6 +987,56 @@ __global__ void k_agg_pieces(const uint32_t *__restrict__ off, const uint32_t *_
     }
 }
 
+// Ops of more than lane_max and up to AG_MID_MAX kernels: a block each.  The
+// segment comes to shared memory and is put in ascending kernel index when it is
+// not; each thread adds a contiguous run of it, and the partials are merged by
+// fixed trees (each warp's, then the warps' in order).  Two launches share the
+// list: blocks of 128 threads take ops up to MID_SPLIT kernels, blocks of 512
+// the longer ones (an op of 4,000 kernels takes 128 threads 250 us, most of it
+// in the sort).
+constexpr uint32_t MID_SPLIT = 1024;
+template <int MID_THREADS>
+__global__ void __launch_bounds__(MID_THREADS) k_agg_mid(const uint32_t *__restrict__ off,
+                                                         const uint32_t *__restrict__ list, AggIn A, DevStatus *st) {
+    pdl_wait();
+    __shared__ uint32_t seg[AG_MID_MAX];
+    __shared__ Acc wpart[MID_THREADS / 32];
+    const unsigned lane = lane_id(), w = threadIdx.x >> 5, n = A.ctr[2];
+    int bad = 0;
+    for (unsigned q = blockIdx.x; q < n; q += gridDim.x) {
+        const uint32_t o = A.mids[q], s0 = off[o], len = off[o + 1] - s0;
+        if ((len > MID_SPLIT) != (MID_THREADS > 128)) continue;           // the other launch's
+        uint32_t n2 = MID_THREADS;
+        while (n2 < len) n2 <<= 1;
+        bool down = false;
+        for (uint32_t i = threadIdx.x; i < n2; i += MID_THREADS) {
+            const uint32_t x = i < len ? list[s0 + i] : 0xFFFFFFFFu;
+            down |= i + 1 < len && list[s0 + i + 1] < x;
+            seg[i] = x;
+        }
+        if (__syncthreads_or(down)) bitonic_smem(seg, (int)n2);
+        const uint32_t per = (len + MID_THREADS - 1) / MID_THREADS;
+        const uint32_t l0 = min(threadIdx.x * per, len), l1 = min(l0 + per, len);
+        Acc acc;
+        if (!piece_fast(A, seg, l0, l1, acc)) {           // a null or infinite value: redo with null handling
+            acc.init();
+            for (uint32_t t = l0; t < l1; ++t) acc.add(A, seg[t]);
+        }
+#pragma unroll 1
+        for (int d = 16; d > 0; d >>= 1) acc_merge_down(acc, d);
+        if (lane == 0) wpart[w] = acc;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            Acc total = wpart[0];
+            for (int v = 1; v < MID_THREADS / 32; ++v) acc_merge(total, wpart[v]);
+            total.write(A, o);
+            bad |= total.bad;
+        }
+        __syncthreads();
+    }
+    if (bad) set_err(st, ERR_INVALID);
+}
+
 // Finish: one block per huge op merges its pieces' partials -- thread t takes
 // pieces t, t + FIN_THREADS, ... in order, then each warp's fixed tree, then
 // thread 0 takes the warps' partials in warp order -- and writes the record.
@@ -1033,35 +1099,38 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
 
     Need nd;
     nd.add<uint32_t>(O + 1).add<uint32_t>(O + 1).add<uint32_t>(K).add<uint32_t>(K);
-    nd.add<uint32_t>(O + 1).add<unsigned>(3).add<unsigned>(1).add<uint32_t>(O + 1);
-    nd.add<uint32_t>(O + 1).add<Acc>(K / AG_PIECE + (K / (AG_SHORT_MAX + 1)) + 1);   // pieces per op, partials
+    const int64_t mids_n = std::min<int64_t>(O, K / (AG_LANE_MAX + 1)) + 1;        // ops longer than a lane takes
+    const int64_t part_n = K / AG_PIECE + K / (AG_MID_MAX + 1) + 1;                // pieces of the longest
+    nd.add<uint32_t>(mids_n).add<uint32_t>(mids_n).add<unsigned>(4).add<unsigned>(1).add<uint32_t>(O + 1);
+    nd.add<uint32_t>(mids_n).add<Acc>(part_n);
     nd.add<uint32_t>(scan_scratch_elems(std::max<int64_t>(O + 1, radix_hist_elems(K))));
     nd.add<uint32_t>(O + 1).add<uint32_t>(radix_hist_elems(K)).add<uint32_t>(8);   // huge-op index, histogram, info
-    nd.add<uint32_t>(O + 1);                                                         // huge ops
+    nd.add<uint32_t>(mids_n);                                                        // huge ops
     opattr_status st = ensure_arena(c, nd.bytes + 4096);
     if (st) return st;
     Arena a(c);
     uint32_t *cnt = a.take<uint32_t>(O + 1), *off = a.take<uint32_t>(O + 1);
     // tmp holds each kernel's slot among its op's kernels until the list is
     // placed, then serves the segment sorts
-    uint32_t *list = a.take<uint32_t>(K), *tmp = a.take<uint32_t>(K), *longs = a.take<uint32_t>(O + 1);
-    // ctr[0] next chunk, ctr[1] ops listed dirty, ctr[2] (nlong) ops listed long:
-    // the two counts come back together
-    unsigned *ctr = a.take<unsigned>(3);
-    unsigned *nlong = ctr ? ctr + 2 : nullptr;
+    uint32_t *list = a.take<uint32_t>(K), *tmp = a.take<uint32_t>(K);
+    uint32_t *mids = a.take<uint32_t>(mids_n), *longs = a.take<uint32_t>(mids_n);
+    // ctr[0] next chunk; the numbers of ops listed dirty, mid and long (nlong)
+    // come back together
+    unsigned *ctr = a.take<unsigned>(4);
+    unsigned *nlong = ctr ? ctr + 3 : nullptr;
     unsigned *nonident = a.take<unsigned>(1);
     uint32_t *dirty = a.take<uint32_t>(O + 1);
-    uint32_t *npc = a.take<uint32_t>(O + 1);
-    Acc *partials = a.take<Acc>(K / AG_PIECE + (K / (AG_SHORT_MAX + 1)) + 1);
+    uint32_t *npc = a.take<uint32_t>(mids_n);
+    Acc *partials = a.take<Acc>(part_n);
     if (!npc || !partials) return OPATTR_E_OOM;
     uint32_t *part = a.take<uint32_t>(scan_scratch_elems(std::max<int64_t>(O + 1, radix_hist_elems(K))));
     uint32_t *hidx = a.take<uint32_t>(O + 1), *hhist = a.take<uint32_t>(radix_hist_elems(K));
-    uint32_t *info = a.take<uint32_t>(8), *hop = a.take<uint32_t>(O + 1);
+    uint32_t *info = a.take<uint32_t>(8), *hop = a.take<uint32_t>(mids_n);
     if (!hidx || !hhist || !info || !hop) return OPATTR_E_OOM;
-    if (!cnt || !off || !list || !tmp || !longs || !nlong || !part || !nonident || !dirty) return OPATTR_E_OOM;
+    if (!cnt || !off || !list || !tmp || !mids || !longs || !nlong || !part || !nonident || !dirty) return OPATTR_E_OOM;
     // with the enclosure's verdict pending (a join) the status block keeps it:
     // the enclosure's reset left the aggregation's slots at zero
-    const ZeroRun zr[3] = {{cnt, O + 1}, {ctr, 3}, {nonident, 1}};
+    const ZeroRun zr[3] = {{cnt, O + 1}, {ctr, 4}, {nonident, 1}};
     if ((st = c.enclose_pending ? zero_runs(c, 3, zr) : reset_status(c, 3, zr))) return st;
     const int sms = sm_count(c);
     // runs long enough to keep most segments in one warp, short enough that
@@ -1078,10 +1147,11 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
     in.counters = ncu->counters;
     in.M = M;
     in.n_ops = O;
+    in.lane_max = (uint32_t)std::min<int64_t>(AG_LANE_TOP, std::max<int64_t>(AG_LANE_MAX, O > 0 ? 4 * K / O : 0));
     in.ctr = ctr;
     in.dirty = dirty;
+    in.mids = mids;
     in.longs = longs;
-    in.nlong = nlong;
     in.nonident = nonident;
     in.out = *out;
     bool status_fresh = false;        // no launch since the last status read
@@ -1100,27 +1170,33 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
         launch(c, "agg_ops", k_agg_ops, dim3(ops_grid(c, O)), dim3(AG_THREADS), AG_SMEM,
                (const uint32_t *)off, list, in, (int)c.enclose_pending, (const DevStatus *)c.d_status);
         // the ops the pass left: listed with a null or infinite value (redone
-        // by k_agg_careful), long ones (the pieces pass); both
-        // counts come back with the status
-        const SmallCopy counts{c.h_small, ctr + 1, 2 * sizeof(uint32_t)};
+        // by k_agg_careful, a thread each), longer than a lane takes (a block
+        // each) and longer still (the pieces pass); the counts come back with
+        // the status
+        const SmallCopy counts{c.h_small, ctr + 1, 3 * sizeof(uint32_t)};
         if ((st = read_status(c, 1, &counts))) return st;
-        const uint32_t n_dirty = c.h_small[0], n_long = c.h_small[1];
-        status_fresh = n_dirty == 0 && n_long == 0;
+        const uint32_t n_dirty = c.h_small[0], n_mid = c.h_small[1], n_long = c.h_small[2];
+        status_fresh = n_dirty == 0 && n_mid == 0 && n_long == 0;
         if (n_dirty > 0)
-            launch(c, "agg_careful", k_agg_careful, dim3(std::max(1, sms)), dim3(128), 0, (const uint32_t *)off, list,
-                   in, c.d_status);
-        uint32_t pieces = 0, longest = 0, n_huge = 0;
+            launch(c, "agg_careful", k_agg_careful, dim3(grid_for(n_dirty, 128)), dim3(128), 0, (const uint32_t *)off,
+                   list, in, c.d_status);
+        if (n_mid > 0) {
+            launch(c, "agg_mid", k_agg_mid<128>, dim3(std::min<uint32_t>(n_mid, 4u * sms)), dim3(128), 0,
+                   (const uint32_t *)off, (const uint32_t *)list, in, c.d_status);
+            launch(c, "agg_mid", k_agg_mid<512>, dim3(std::min<uint32_t>(n_mid, (unsigned)sms)), dim3(512), 0,
+                   (const uint32_t *)off, (const uint32_t *)list, in, c.d_status);
+        }
+        uint32_t pieces = 0, n_huge = 0;
         if (n_long > 0) {
             launch(c, "agg_piece_offsets", k_agg_piece_offsets, dim3(1), dim3(1024), 0, (const uint32_t *)off,
                    (const uint32_t *)longs, (const unsigned *)nlong, 0u, npc, info, hop);
             const SmallCopy pinfo{c.h_small, info, 5 * sizeof(uint32_t)};
             if ((st = read_status(c, 1, &pinfo))) return st;
             pieces = c.h_small[1];
-            longest = c.h_small[2];
             n_huge = c.h_small[4];
         }
         if (pieces > 0) {
-            if (n_huge <= (uint32_t)RADIX_BINS && longest > AG_BLOCK_SORT_MAX && K > 0) {
+            if (n_huge <= (uint32_t)RADIX_BINS && K > 0) {
                 // very long segments: placed in kernel order by one counting pass
                 cudaMemsetAsync(hidx, 0xFF, sizeof(uint32_t) * (O + 1), c.stream);
                 launch(c, "huge_index", k_huge_index, dim3(grid_for(n_huge, 256, 4096)), dim3(256), 0,
@@ -1279,10 +1355,11 @@ opattr_status do_rollup(Ctx &c, const opattr_kernels *kern, const opattr_ranges 
         in.counters = ncu->counters;
         in.M = M;
         in.n_ops = C;
+        in.lane_max = 0;
         in.ctr = nullptr;
         in.dirty = nullptr;
+        in.mids = nullptr;
         in.longs = nullptr;
-        in.nlong = nullptr;
         in.nonident = nullptr;
         in.out = *out;
         int sms = 0;
