@@ -1128,10 +1128,10 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
     uint32_t *info = a.take<uint32_t>(8), *hop = a.take<uint32_t>(mids_n);
     if (!hidx || !hhist || !info || !hop) return OPATTR_E_OOM;
     if (!cnt || !off || !list || !tmp || !mids || !longs || !nlong || !part || !nonident || !dirty) return OPATTR_E_OOM;
-    // with the enclosure's verdict pending (a join) the status block keeps it:
-    // the enclosure's reset left the aggregation's slots at zero
+    // with the enclosure's or the matching's verdict pending (a join) the status
+    // block keeps it: the enclosure's reset left the aggregation's slots at zero
     const ZeroRun zr[3] = {{cnt, O + 1}, {ctr, 4}, {nonident, 1}};
-    if ((st = c.enclose_pending ? zero_runs(c, 3, zr) : reset_status(c, 3, zr))) return st;
+    if ((st = c.enclose_pending || c.keep_status ? zero_runs(c, 3, zr) : reset_status(c, 3, zr))) return st;
     const int sms = sm_count(c);
     // runs long enough to keep most segments in one warp, short enough that
     // the grid is one wave of resident warps (five blocks of eight per SM)

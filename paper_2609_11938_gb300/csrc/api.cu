@@ -25,6 +25,7 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
                          uint8_t *out_nop);
 opattr_status do_match(Ctx &c, const opattr_kernels *kern, const opattr_ncu *ncu, const opattr_dedup *dd,
                        int32_t *out_idx, uint8_t *out_kind, opattr_match_summary *sum);
+bool match_layers_ahead(const opattr_dedup *dd);
 opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_ranges *rng, const int32_t *rok,
                            const opattr_ncu *ncu, const int32_t *nidx, uint32_t n_ops,
                            const opattr_op_aggregates *out, opattr_totals *tot_out);
@@ -416,7 +417,7 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
         Ctx &c;
         explicit JoinScope(Ctx &ctx) : c(ctx) { c.in_join = true; }
         ~JoinScope() {
-            if (c.enclose_pending) cudaStreamSynchronize(c.stream);     // an early return: nothing left running
+            if (c.enclose_pending || c.match_pending) cudaStreamSynchronize(c.stream);     // an early return: nothing left running
             c.in_join = false;
             c.order_from_enclose = false;
             c.join_korder = nullptr;
@@ -424,19 +425,28 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
             c.spec_k = 0;
             c.spec_ran = false;
             c.defer_status = false;
-            c.enclose_pending = false;
+            c.enclose_pending = c.match_pending = c.keep_status = c.no_spec = false;
+            c.max_ncu = nullptr;
+            c.max_known = false;
         }
     } scope(c);
-    // the matching's identity pairing may run within the enclosure: rows one
-    // for one with the kernels, no layer deduplication, no per-stream rows;
-    // then the enclosure's last status read can wait for the aggregation's
-    const bool spec = !dedup && !ncu->stream && kernels->n > 0 && kernels->n == ncu->n && kernels->name_id &&
-                      ncu->name_id && ncu_idx_of_kernel;
+    // The matching can go ahead on the taking that the records are in order, so
+    // that the enclosure's verdict is read with the aggregation's: the identity
+    // pairing (rows one for one with the kernels; it runs within the enclosure),
+    // the stream-partitioned pairing, or layer deduplication.  Else the matching
+    // may have to sort names, whose largest the enclosure's checks find.
+    const bool dd = c.cfg.dedup && dedup && kernels->layer_id;
+    const bool full = kernels->n > 0 && kernels->name_id && ncu->name_id && ncu_idx_of_kernel;
+    const bool same = full && !dd && kernels->n == ncu->n;
+    const bool spec = same && !ncu->stream;
+    const bool ahead = same || (full && dd && !ncu->stream && match_layers_ahead(dedup));
     for (int pass = 0; pass < 2; ++pass) {
         c.enclose_k_sorted = -1;
         c.spec_k = 0;
         c.spec_ran = false;
-        c.enclose_pending = false;
+        c.enclose_pending = c.match_pending = c.keep_status = c.no_spec = false;
+        c.max_ncu = full && !same && !dd && kernels->n + ncu->n < (1ll << 32) ? ncu : nullptr;
+        c.max_known = false;
         if (spec) {
             c.spec_kname = kernels->name_id;
             c.spec_nname = ncu->name_id;
@@ -444,7 +454,7 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
             c.spec_kind = match_kind;
             c.spec_k = kernels->n;
         }
-        c.defer_status = spec && pass == 0;
+        c.defer_status = ahead && pass == 0;
         opattr_status st = finish(c, do_enclose(c, kernels, ranges, range_of_kernel, n_op_enclosing));
         c.defer_status = false;
         if (st < 0) return st;
@@ -454,18 +464,24 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
         c.order_from_enclose = false;
         c.join_korder = nullptr;             // the aggregation needs no time order
         c.arena_keep = 0;
-        if (sm < 0) return sm;
+        if (sm < 0) {
+            // the enclosure's error comes before the matching's
+            if (!c.enclose_pending) return sm;
+            if ((st = read_status(c)) < 0) return st;
+            if (c.h_status->flags & (F_LEVEL_FIXUP | F_K_UNSORTED | F_R_UNSORTED | F_LEVELS_MANY)) continue;
+            st = enclose_verdict(*c.h_status, kernels->n);
+            return st < 0 ? st : sm;
+        }
         st = finish(c, do_aggregate(c, kernels, ranges, range_of_kernel, ncu, ncu_idx_of_kernel, n_ops, dev_out,
                                     host_totals));
+        if (st < 0 && (c.enclose_pending || c.match_pending)) {
+            // read once more if the aggregation stopped before reading it
+            const opattr_status s2 = read_status(c);
+            if (s2 < 0) return s2;
+        }
         if (c.enclose_pending) {
-            // the enclosure's verdict and the identity pairing's, read with the
-            // aggregation's status (read once more if the aggregation stopped
-            // before reading it)
+            // the enclosure's verdict and the pairing's, read with the aggregation's status
             c.enclose_pending = false;
-            if (st < 0) {
-                const opattr_status s2 = read_status(c);
-                if (s2 < 0) return s2;
-            }
             // redone without deferring
             if (c.h_status->flags & (F_LEVEL_FIXUP | F_K_UNSORTED | F_R_UNSORTED | F_LEVELS_MANY)) continue;
             // the enclosure's error before the aggregation's (nesting is only
@@ -477,13 +493,22 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
             if (st >= 0 && (c.h_status->flags & F_NAMES_DIFFER)) {
                 // the names disagree: the matching and the aggregation proper
                 c.order_from_enclose = true;
-                c.spec_ran = false;
+                c.spec_ran = c.match_pending = c.keep_status = false;
+                c.no_spec = true;
                 sm = finish(c, do_match(c, kernels, ncu, dedup, ncu_idx_of_kernel, match_kind, host_summary));
                 c.order_from_enclose = false;
                 if (sm < 0) return sm;
                 st = finish(c, do_aggregate(c, kernels, ranges, range_of_kernel, ncu, ncu_idx_of_kernel, n_ops,
                                             dev_out, host_totals));
+                if (st < 0 && c.match_pending) {
+                    const opattr_status s2 = read_status(c);
+                    if (s2 < 0) return s2;
+                }
             }
+        }
+        if (c.match_pending) {
+            sm = match_verdict(c, host_summary);
+            if (sm < 0) return sm;
         }
         if (st < 0) return st;
         return sm;

@@ -52,6 +52,7 @@ enum CountSlot {
     C_TIER_INDUCTOR,
     C_FUSED,
     C_CORR_USED,
+    C_MAX_KEY,               // largest matching key of kernels and rows
     C_NSLOTS = 24
 };
 enum MinMaxSlot { MM_KSTART_MIN = 0, MM_KSTART_MAX, MM_RSTART_MIN, MM_REND_MAX, MM_NSLOTS = 8 };
@@ -74,7 +75,7 @@ struct TimingSlot {
 };
 
 constexpr int N_LEVELS = 256 * 32;   // (stream, depth) levels of the enclosure
-constexpr size_t STAGE_BYTES = 1024;   // pinned staging of host-built tables
+constexpr size_t STAGE_BYTES = 32768;  // pinned staging of host-built tables
 constexpr int SMALL_WORDS = 512;
 
 struct Ctx {
@@ -114,6 +115,16 @@ struct Ctx {
     uint8_t *spec_kind = nullptr;
     int64_t spec_k = 0;
     bool spec_ran = false;
+    // within a join whose matching must sort its names: the largest key, found
+    // by the enclosure's checking pass (max_ncu), then max_known
+    const opattr_ncu *max_ncu = nullptr;
+    bool max_known = false;
+    // within a join: the matching's results are complete but its counts and
+    // verdict are read with the aggregation's status (match_pending); then the
+    // aggregation keeps the status block (keep_status).  no_spec: the fast
+    // pairing is known to fail
+    bool match_pending = false, keep_status = false, no_spec = false;
+    opattr_match_summary match_sum{};
     // within a join whose matching can be skipped: the enclosure's last status
     // read is left to the aggregation's (defer_status), and the enclosure's
     // verdict is pending until then (enclose_pending; the aggregation keeps
@@ -159,6 +170,9 @@ int sm_count(Ctx &c);
 // The status of an enclosure that read `H` (a NOT_NESTED found beside
 // F_LEVEL_FIXUP does not count: the run on sorted ranges decides).
 opattr_status enclose_verdict(const DevStatus &H, int64_t K);
+// The matching's counts and status from the status block (c.match_sum holds
+// what was known before it ran).
+opattr_status match_verdict(Ctx &c, opattr_match_summary *sum);
 // A small transfer between the context's pinned host buffers and device
 // memory, on c.stream.  When those buffers are mapped into the device's
 // address space (opattr_create checks), a small kernel moves the bytes through

@@ -98,6 +98,9 @@ struct EncCheck {
     uint8_t *kind;                       // may be NULL
     int vec;                             // kernel arrays aligned for 16-byte accesses
     int pair_vec;                        // the pairing's arrays too
+    const uint32_t *mk, *mn;             // names of kernels and rows whose largest key is wanted, or NULL
+    const uint8_t *ms;                   // streams of the rows: keys are name << 8 | stream
+    int64_t M;
 };
 
 constexpr int EP_THREADS = 256;
@@ -233,6 +236,20 @@ __global__ void __launch_bounds__(EP_THREADS) k_enc_parts(EncView V, EncCheck C,
                 rmx = ev[u] > rmx ? ev[u] : rmx;
                 if (dv[u] < OPATTR_MAX_DEPTH && !((dmask[tv[u]] >> dv[u]) & 1u)) atomicOr(&dmask[tv[u]], 1u << dv[u]);
             }
+        }
+        if (C.mk) {
+            uint32_t top_key = 0;
+            for (int64_t i = kb + tid; i < ke; i += EP_THREADS) {
+                const uint32_t x = C.ms ? C.mk[i] << 8 | V.k_stream[i] : C.mk[i];
+                top_key = x > top_key ? x : top_key;
+            }
+            const int64_t mshare = (C.M + parts - 1) / parts, me = (b + 1) * mshare < C.M ? (b + 1) * mshare : C.M;
+            for (int64_t i = b * mshare + tid; i < me; i += EP_THREADS) {
+                const uint32_t x = C.ms ? C.mn[i] << 8 | C.ms[i] : C.mn[i];
+                top_key = x > top_key ? x : top_key;
+            }
+            top_key = __reduce_max_sync(0xffffffffu, top_key);
+            if (lane == 0 && top_key) atomicMax(&st->cnt[C_MAX_KEY], (unsigned long long)top_key);
         }
         f = (int)__reduce_or_sync(0xffffffffu, (unsigned)f);
         if (lane == 0 && f) atomicOr(&flags_s, f);
@@ -988,6 +1005,13 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
         C.idx = c.spec_idx;
         C.kind = c.spec_kind;
         C.pair_vec = al(C.kname, 16) && al(C.nname, 16) && al(C.idx, 16) && al(C.kind, 8);
+    }
+    c.max_known = c.max_ncu != nullptr;
+    if (c.max_ncu) {
+        C.mk = kern->name_id;
+        C.mn = c.max_ncu->name_id;
+        C.ms = c.max_ncu->stream;
+        C.M = c.max_ncu->n;
     }
     launch(c, "enc_parts", k_enc_parts<true, false>, dim3((unsigned)B.parts), dim3(EP_THREADS), 0, V, C, B.parts,
            B.tp, B.tile_r, B.rows, B.row_len, B.lvlmask, c.d_status);

@@ -9,11 +9,11 @@
 // streams one after another) the same test runs on the replayed kernels and
 // the rows each partitioned stably by stream.
 //
-// General path.  Ordinals come from stable radix sorts: replayed kernels in
-// time order sorted by name give o(k) = position - start of the name's run;
-// ncu rows in array order sorted by name give the rows of each name in
-// launch order.  The join is row = rows_of_name[o(k)], subject to the
-// mismatch mode.  Dedup positions come the same way from a stable sort of
+// General path.  Ordinals come from one stable radix sort by name of the
+// replayed kernels in time order followed by the ncu rows in array order: a
+// name's run of kernels, in launch order, is followed by its run of rows, in
+// launch order, and the join is row = rows_of_name[position in the run], subject
+// to the mismatch mode.  Dedup positions come from a stable partition of the
 // layer-tagged kernels by layer id.
 #include <algorithm>
 
@@ -117,14 +117,6 @@ __global__ void k_check_names24(const uint32_t *__restrict__ name, int64_t n, De
     if (__any_sync(0xffffffffu, acc >> 24 != 0) && lane_id() == 0) set_err(st, ERR_INVALID);
 }
 
-__global__ void k_fill_match(int32_t *out_idx, uint8_t *out_kind, int64_t n) {
-    pdl_wait();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        out_idx[i] = -1;
-        if (out_kind) out_kind[i] = 0;
-    }
-}
-
 // ------------------------------------------------------------------ general path helpers
 // Flags in time order: flag[i] = predicate(korder[i]).
 //   what = 0: replayed (layer < 0 or the layer is its class representative)
@@ -146,35 +138,28 @@ __global__ void k_compact(const uint32_t *__restrict__ korder, const uint32_t *_
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         if (flag[i]) list[pos[i]] = korder ? korder[i] : (uint32_t)i;
 }
-__global__ void k_gather_u32(const uint32_t *__restrict__ src, const uint32_t *__restrict__ idx, int64_t n,
-                             uint32_t *__restrict__ dst) {
-    pdl_wait();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        dst[i] = idx ? src[idx[i]] : src[i];
-}
 __global__ void k_gather_i32_as_u32(const int32_t *__restrict__ src, const uint32_t *__restrict__ idx, int64_t n,
                                     uint32_t *__restrict__ dst) {
     pdl_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         dst[i] = (uint32_t)src[idx[i]];
 }
-__global__ void k_max_u32(const uint32_t *__restrict__ a, int64_t n, unsigned long long *out) {
+// The largest matching key (name, or name << 8 | stream with streams) of
+// kernels and rows.
+__global__ void k_max_key(const uint32_t *__restrict__ kname, const uint8_t *__restrict__ kstream, int64_t K,
+                          const uint32_t *__restrict__ nname, const uint8_t *__restrict__ nstream, int64_t M,
+                          DevStatus *st) {
     pdl_wait();
     uint32_t m = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        m = a[i] > m ? a[i] : m;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        uint32_t x = __shfl_xor_sync(0xffffffffu, m, o);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < K + M; i += (int64_t)gridDim.x * blockDim.x) {
+        const bool row = i >= K;
+        const int64_t j = row ? i - K : i;
+        uint32_t x = row ? nname[j] : kname[j];
+        if (nstream) x = x << 8 | (row ? nstream[j] : kstream[j]);
         m = x > m ? x : m;
     }
-    __shared__ uint32_t sm[32];
-    if (lane_id() == 0) sm[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (unsigned w = 1; w < blockDim.x / 32; ++w) m = sm[w] > m ? sm[w] : m;
-        if (m) atomicMax(out, (unsigned long long)m);
-    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane_id() == 0 && m) atomicMax(&st->cnt[C_MAX_KEY], (unsigned long long)m);
 }
 __global__ void k_check_layers(const int32_t *__restrict__ layer, int64_t n, int32_t n_layers,
                                const int32_t *__restrict__ rep_layer, DevStatus *st) {
@@ -208,111 +193,173 @@ __device__ __forceinline__ int64_t upper_bound_u32(const uint32_t *a, int64_t n,
     return lo;
 }
 
-// Runs of equal keys in a sorted array.  flag[i] = 1 at each run's first
-// element; after an exclusive scan pos[i] counts the runs that start before
-// i, so element i lies in run pos[i] + head(i) - 1 and start[pos[i]] = i at
-// each head.
-__device__ __forceinline__ bool run_head(const uint32_t *a, int64_t i) { return i == 0 || a[i - 1] != a[i]; }
-
-__global__ void k_run_heads(const uint32_t *__restrict__ a, int64_t n, uint32_t *__restrict__ flag) {
+// The sort's input: matching keys of the nrep replayed kernels in time order
+// (list rk, or the kernel array itself when rk is null), then of the M rows.
+// With streams the key is name << 8 | stream; a name id of 2^24 or more cannot
+// be packed and is an invalid argument.
+__global__ void k_pair_keys(const uint32_t *__restrict__ rk, const uint32_t *__restrict__ kname,
+                            const uint8_t *__restrict__ kstream, int64_t nrep, const uint32_t *__restrict__ nname,
+                            const uint8_t *__restrict__ nstream, int64_t n, uint32_t *__restrict__ key,
+                            DevStatus *st) {
     pdl_wait();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        flag[i] = run_head(a, i);
-}
-__global__ void k_run_starts(const uint32_t *__restrict__ a, const uint32_t *__restrict__ pos, int64_t n,
-                             uint32_t *__restrict__ start) {
-    pdl_wait();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        if (run_head(a, i)) start[pos[i]] = (uint32_t)i;
-}
-
-// First run r in [0, nr) whose key a[start[r]] is >= x.
-__device__ __forceinline__ int64_t lower_bound_runs(const uint32_t *a, const uint32_t *start, int64_t nr, uint32_t x) {
-    int64_t lo = 0, hi = nr;
-    while (lo < hi) {
-        int64_t m = (lo + hi) >> 1;
-        if (a[start[m]] < x) lo = m + 1; else hi = m;
+    int bad = 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const bool row = i >= nrep;
+        const int64_t j = row ? i - nrep : (rk ? (int64_t)rk[i] : i);
+        uint32_t x = row ? nname[j] : kname[j];
+        if (nstream) {
+            bad |= x >> 24 != 0;
+            x = x << 8 | (row ? nstream[j] : kstream[j]);
+        }
+        key[i] = x;
     }
-    return lo;
+    if (bad) set_err(st, ERR_INVALID);
 }
 
-// Per kernel name run u (replayed kernels sorted by (name, time)): the ncu
-// rows of the same name, as the first position b[u] in the sorted rows and
-// their count cq[u].  Runs whose kernel and row counts differ are counted
-// (and are an error in the error mode).
-__global__ void k_run_pair(const uint32_t *__restrict__ skn, const uint32_t *__restrict__ ustart,
-                           const uint32_t *__restrict__ n_urun, int64_t nrep, const uint32_t *__restrict__ snn,
-                           const uint32_t *__restrict__ vstart, const uint32_t *__restrict__ n_vrun, int64_t M,
-                           int mode, uint32_t *__restrict__ b_of, uint32_t *__restrict__ cq_of, DevStatus *st) {
+// Runs of the sorted keys sk (sv[i] < nrep: a kernel, else a row): a name's
+// kernels are one run, its rows the next.  run[i] is element i's run, start[u]
+// the first element of run u; *n_run their number, start[*n_run] = n.
+__device__ __forceinline__ bool run_head(const uint32_t *sk, const uint32_t *sv, int64_t nrep, int64_t i) {
+    return i == 0 || sk[i - 1] != sk[i] || ((int64_t)sv[i - 1] < nrep) != ((int64_t)sv[i] < nrep);
+}
+__global__ void __launch_bounds__(SCAN_THREADS) k_runs(const uint32_t *__restrict__ sk,
+                                                       const uint32_t *__restrict__ sv, int64_t nrep, int64_t n,
+                                                       Chain C, uint32_t *__restrict__ run,
+                                                       uint32_t *__restrict__ start, uint32_t *__restrict__ n_run) {
     pdl_wait();
-    const int64_t U = *n_urun, V = *n_vrun;
-    unsigned long long names_bad = 0;
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < U; u += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t lo = ustart[u], hi = u + 1 < U ? ustart[u + 1] : nrep;
-        const uint32_t name = skn[lo];
-        const int64_t v = lower_bound_runs(snn, vstart, V, name);
-        const bool found = v < V && snn[vstart[v]] == name;
-        const int64_t b = found ? vstart[v] : 0;
-        const int64_t cq = found ? (v + 1 < V ? vstart[v + 1] : M) - b : 0;
-        b_of[u] = (uint32_t)b;
-        cq_of[u] = (uint32_t)cq;
-        names_bad += hi - lo != cq;
-    }
-    __shared__ unsigned long long red[33];
-    if (__any_sync(0xffffffffu, names_bad != 0) && lane_id() == 0 && mode == OPATTR_MISMATCH_ERROR)
-        set_err(st, ERR_COUNT);
-    block_add_u64(names_bad, &st->cnt[C_NAMES_MISMATCH], red);
+    chained_scan(
+        C, n, [&](int64_t i) -> uint32_t { return run_head(sk, sv, nrep, i); },
+        [&](int64_t i, uint32_t head, uint32_t ex) {
+            const uint32_t u = ex + head - 1;
+            run[i] = u;
+            if (head) start[u] = (uint32_t)i;
+        },
+        [&](uint32_t total) {
+            *n_run = total;
+            start[total] = (uint32_t)n;
+        });
 }
 
-// Names that have ncu rows but no replayed kernel at all (one thread per
-// ncu name run).
-__global__ void k_ncu_only_names(const uint32_t *__restrict__ snn, const uint32_t *__restrict__ vstart,
-                                 const uint32_t *__restrict__ n_vrun, const uint32_t *__restrict__ skn,
-                                 const uint32_t *__restrict__ ustart, const uint32_t *__restrict__ n_urun, int mode,
-                                 DevStatus *st) {
+// The ordinal join over the sorted elements.  A kernel is the o-th of its name,
+// o = i - start of its run; its row is the o-th element of the next run when
+// that holds the name's rows, subject to the mismatch mode.  The first element
+// of a kernel run compares its name's counts, the first of a row run reports a
+// name without kernels.
+__global__ void k_ordinal_join(const uint32_t *__restrict__ sk, const uint32_t *__restrict__ sv, int64_t nrep,
+                               int64_t n, const uint32_t *__restrict__ run, const uint32_t *__restrict__ start,
+                               const uint32_t *__restrict__ n_run, const uint32_t *__restrict__ rk, int mode,
+                               int32_t *__restrict__ out_idx, uint8_t *__restrict__ out_kind, DevStatus *st) {
     pdl_wait();
-    const int64_t U = *n_urun, V = *n_vrun;
-    unsigned long long bad = 0;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t name = snn[vstart[v]];
-        const int64_t u = lower_bound_runs(skn, ustart, U, name);
-        bad += u == U || skn[ustart[u]] != name;
-    }
-    __shared__ unsigned long long red[33];
-    if (__any_sync(0xffffffffu, bad != 0) && lane_id() == 0 && mode == OPATTR_MISMATCH_ERROR) set_err(st, ERR_COUNT);
-    block_add_u64(bad, &st->cnt[C_NAMES_MISMATCH], red);
-}
-
-// The ordinal join.  i runs over replayed kernels sorted by (name, time):
-//   skn / skj: sorted names, and the time rank j of each (rk[j] = kernel)
-//   kpos / ustart / b_of / cq_of: the run tables of skn
-//   snj: the row index of each ncu row in name-sorted order
-// Kernel i is the o-th of its name with o = i - ustart[run]; its row is the
-// o-th row of the name, subject to the mismatch mode.
-__global__ void k_ordinal_join(const uint32_t *__restrict__ skn, const uint32_t *__restrict__ skj,
-                               const uint32_t *__restrict__ kpos, const uint32_t *__restrict__ ustart,
-                               const uint32_t *__restrict__ n_urun, const uint32_t *__restrict__ b_of,
-                               const uint32_t *__restrict__ cq_of, const uint32_t *__restrict__ rk, int64_t nrep,
-                               const uint32_t *__restrict__ snj, int mode, int32_t *__restrict__ out_idx,
-                               uint8_t *__restrict__ out_kind, DevStatus *st) {
-    pdl_wait();
-    const int64_t U = *n_urun;
-    unsigned long long direct = 0, unmatched = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nrep; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t u = (int64_t)kpos[i] + run_head(skn, i) - 1;
-        const int64_t lo = ustart[u], hi = u + 1 < U ? ustart[u + 1] : nrep;
-        const int64_t cq = cq_of[u], o = i - lo;
-        const bool ok = mode == OPATTR_MISMATCH_SKIP_NAME ? (hi - lo == cq) : (o < cq);
-        const int32_t idx = ok && o < cq ? (int32_t)snj[b_of[u] + o] : -1;
-        const uint32_t k = rk[skj[i]];
+    const uint32_t U = *n_run;
+    unsigned long long direct = 0, unmatched = 0, names = 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t j = sv[i], u = run[i], lo = start[u];
+        if ((int64_t)j >= nrep) {
+            names += lo == i && (i == 0 || sk[i - 1] != sk[i]);
+            continue;
+        }
+        const uint32_t hi = start[u + 1];
+        const bool rows = u + 1 < U && sk[hi] == sk[i];
+        const uint32_t cq = rows ? start[u + 2] - hi : 0u, o = (uint32_t)i - lo;
+        names += lo == i && hi - lo != cq;
+        const bool ok = o < cq && (mode != OPATTR_MISMATCH_SKIP_NAME || hi - lo == cq);
+        const int32_t idx = ok ? (int32_t)((int64_t)sv[hi + o] - nrep) : -1;
+        const uint32_t k = rk ? rk[j] : j;
         out_idx[k] = idx;
         if (out_kind) out_kind[k] = idx >= 0 ? 1 : 0;
         direct += idx >= 0;
         unmatched += idx < 0;
     }
     __shared__ unsigned long long red[33];
+    if (__any_sync(0xffffffffu, names != 0) && lane_id() == 0 && mode == OPATTR_MISMATCH_ERROR) set_err(st, ERR_COUNT);
     block_add_u64(direct, &st->cnt[C_DIRECT], red);
     block_add_u64(unmatched, &st->cnt[C_COUNT_UNMATCHED], red);
+    block_add_u64(names, &st->cnt[C_NAMES_MISMATCH], red);
+}
+
+// ------------------------------------------------------------------ layers
+// Layer deduplication with the kernels in time order, in one pass: each
+// replayed kernel's rank among them is its row when the names agree and the
+// rows are as many.  Layer ids are checked along the way.
+__global__ void __launch_bounds__(SCAN_THREADS) k_layer_pairs(const int32_t *__restrict__ layer,
+                                                              const int32_t *__restrict__ rep_layer, int32_t n_layers,
+                                                              const uint32_t *__restrict__ kname,
+                                                              const uint32_t *__restrict__ nname, int64_t K, int64_t M,
+                                                              Chain C, int32_t *__restrict__ out_idx,
+                                                              uint8_t *__restrict__ out_kind, DevStatus *st) {
+    pdl_wait();
+    int bad = 0, differ = 0;
+    chained_scan(
+        C, K,
+        [&](int64_t i) -> uint32_t {
+            const int32_t l = layer[i];
+            const bool ok = l >= -1 && l < n_layers;
+            bad |= !ok;
+            return l < 0 || (ok && rep_layer[l] == l);
+        },
+        [&](int64_t i, uint32_t replayed, uint32_t rank) {
+            if (!replayed) return;
+            const bool row = (int64_t)rank < M;
+            differ |= !row || kname[i] != nname[rank];
+            out_idx[i] = row ? (int32_t)rank : -1;
+            if (out_kind) out_kind[i] = 1;
+        },
+        [&](uint32_t total) {
+            st->cnt[C_REPLAYED] = total;
+            if ((int64_t)total != M) set_flag(st, F_NAMES_DIFFER);
+        });
+    if (bad) set_err(st, ERR_INVALID);
+    if (differ) set_flag(st, F_NAMES_DIFFER);
+}
+
+// Positions within layers, few layers: one stable counting pass over the
+// kernels in time order by layer id.
+constexpr int LAYERS_DIGIT = RADIX_BINS - 1;        // with a last, empty digit for the end of the layer before
+struct LayerDigit {
+    const int32_t *layer;
+    const uint32_t *korder;
+    __device__ __forceinline__ unsigned operator()(int64_t i) const {
+        const int32_t l = layer[korder ? korder[i] : (uint32_t)i];
+        return l >= 0 && l < LAYERS_DIGIT ? (unsigned)l : (unsigned)RADIX_BINS;
+    }
+};
+struct PlaceByLayer {
+    const uint32_t *korder;
+    uint32_t *list, *place;      // kernels layer by layer; each kernel's place there
+    __device__ __forceinline__ unsigned operator()(int64_t i, uint32_t dest, unsigned) const {
+        const uint32_t k = korder ? korder[i] : (uint32_t)i;
+        list[dest] = k;
+        place[k] = dest;
+        return 0u;
+    }
+    __device__ __forceinline__ void done(unsigned) const {}
+};
+// offs[l * ntiles] is the first place of layer l.
+__global__ void k_layer_broadcast(const int32_t *__restrict__ layer, const int32_t *__restrict__ rep_layer,
+                                  int32_t n_layers, const uint32_t *__restrict__ offs, int64_t ntiles,
+                                  const uint32_t *__restrict__ list, const uint32_t *__restrict__ place,
+                                  const uint32_t *__restrict__ kname, int64_t K, int32_t *__restrict__ out_idx,
+                                  uint8_t *__restrict__ out_kind, DevStatus *st) {
+    pdl_wait();
+    unsigned long long bc = 0, miss = 0;
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < K; k += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t l = layer[k];
+        if (l < 0 || l >= n_layers || rep_layer[l] == l) continue;
+        const int32_t r = rep_layer[l];
+        const uint32_t p = place[k] - offs[(int64_t)l * ntiles], r0 = offs[(int64_t)r * ntiles];
+        int32_t idx = -1;
+        if (p < offs[(int64_t)(r + 1) * ntiles] - r0) {
+            const uint32_t src = list[r0 + p];
+            if (kname[src] == kname[k]) idx = out_idx[src];
+        }
+        out_idx[k] = idx;
+        if (out_kind) out_kind[k] = idx >= 0 ? 2 : 0;
+        bc += idx >= 0;
+        miss += idx < 0;
+    }
+    __shared__ unsigned long long red[33];
+    block_add_u64(bc, &st->cnt[C_BROADCAST], red);
+    block_add_u64(miss, &st->cnt[C_DEDUP_MISMATCH], red);
 }
 
 // Broadcast.  i runs over layer-tagged kernels sorted by (layer, time).
@@ -348,26 +395,6 @@ __global__ void k_dedup_broadcast(const uint32_t *__restrict__ sll, const uint32
 }
 
 // ------------------------------------------------------------------ host
-// (name, stream) as one key, name << 8 | stream, for per-stream ordinals; a
-// name id of 2^24 or more cannot be packed and is an invalid argument.
-__global__ void k_stream_keys(const uint32_t *__restrict__ name, const uint8_t *__restrict__ stream, int64_t n,
-                              uint32_t *__restrict__ key, DevStatus *st) {
-    pdl_wait();
-    int bad = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t x = name[i];
-        bad |= x >> 24 != 0;
-        key[i] = (x << 8) | stream[i];
-    }
-    if (bad) set_err(st, ERR_INVALID);
-}
-
-__global__ void k_iota(uint32_t *dst, int64_t n) {
-    pdl_wait();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        dst[i] = (uint32_t)i;
-}
-
 static opattr_status read_u64(Ctx &c, const unsigned long long *d, unsigned long long *h) {
     if (cudaMemcpyAsync(h, d, sizeof(*h), cudaMemcpyDeviceToHost, c.stream) != cudaSuccess ||
         cudaStreamSynchronize(c.stream) != cudaSuccess)
@@ -391,6 +418,69 @@ static void stream_pairs(Ctx &c, const opattr_kernels *kern, const opattr_ncu *n
     const StreamPairs ep{rk, pn, kern->name_id, ncu->name_id, kern->stream, ncu->stream, out_idx, out_kind,
                          c.d_status};
     digit_rank(c, "match_stream_pairs", dg, n, offs, ep);
+}
+
+bool match_layers_ahead(const opattr_dedup *dd) { return dd->n_layers > 0 && dd->n_layers <= LAYERS_DIGIT; }
+
+// Every duplicate-layer kernel takes its representative's row.  Few layers:
+// place / list from one counting pass; else layer-tagged kernels compacted in
+// time order and sorted by layer.  korder: time order, or NULL.
+static opattr_status broadcast_layers(Ctx &c, const opattr_kernels *kern, const opattr_dedup *dd, const int32_t *d_rep,
+                                      const uint32_t *korder, uint32_t *flag, uint32_t *pos, uint32_t *lk,
+                                      uint32_t *const *sort, uint32_t *hist, uint32_t *part, unsigned long long *dsm,
+                                      int32_t *out_idx, uint8_t *out_kind) {
+    const int64_t K = kern->n;
+    const unsigned gK = grid_for(K, 256, REDUCE_GRID);
+    if (dd->n_layers <= LAYERS_DIGIT) {
+        const LayerDigit dg{kern->layer_id, korder};
+        const uint32_t *offs = digit_offsets(c, dg, K, hist, part, dd->n_layers + 1);
+        digit_rank(c, "layer_place", dg, K, offs, PlaceByLayer{korder, lk, pos});
+        launch(c, "layer_broadcast", k_layer_broadcast, dim3(gK), dim3(256), 0, kern->layer_id, d_rep, dd->n_layers,
+               offs, (K + RADIX_TILE - 1) / RADIX_TILE, (const uint32_t *)lk, (const uint32_t *)pos, kern->name_id, K,
+               out_idx, out_kind, c.d_status);      // plain names: a class may span streams
+        return OPATTR_OK;
+    }
+    launch(c, "flags", k_flags, dim3(gK), dim3(256), 0, korder, kern->layer_id, d_rep, K, 1, flag);
+    uint32_t *ntag = reinterpret_cast<uint32_t *>(dsm + 1);
+    scan_exclusive_u32(c, flag, pos, K, part, ntag);
+    launch(c, "compact", k_compact, dim3(gK), dim3(256), 0, korder, (const uint32_t *)flag, (const uint32_t *)pos, K,
+           lk);
+    unsigned long long ntag_h = 0;
+    const opattr_status st = read_u64(c, dsm + 1, &ntag_h);
+    if (st) return st;
+    const int64_t nlk = (int64_t)(ntag_h & 0xFFFFFFFFull);
+    if (nlk == 0) return OPATTR_OK;
+    launch(c, "gather_layers", k_gather_i32_as_u32, dim3(grid_for(nlk, 256, REDUCE_GRID)), dim3(256), 0,
+           kern->layer_id, (const uint32_t *)lk, nlk, sort[0]);
+    uint32_t *sll, *slj;
+    radix_sort_pairs<uint32_t>(c, sort[0], sort[1], sort[2], sort[3], nlk,
+                               bits_for((uint64_t)(dd->n_layers > 0 ? dd->n_layers - 1 : 0)), true, hist, part, &sll,
+                               &slj);
+    launch(c, "dedup_broadcast", k_dedup_broadcast, dim3(grid_for(nlk, 256, REDUCE_GRID)), dim3(256), 0,
+           (const uint32_t *)sll, (const uint32_t *)slj, (const uint32_t *)lk, nlk, d_rep, kern->name_id, out_idx,
+           out_kind, c.d_status);
+    return OPATTR_OK;
+}
+
+opattr_status match_verdict(Ctx &c, opattr_match_summary *sum) {
+    const DevStatus &H = *c.h_status;
+    opattr_match_summary &S = c.match_sum;
+    c.match_pending = false;
+    if (H.err & ERR_INVALID) return OPATTR_E_INVALID_ARG;
+    if (H.err & ERR_COUNT) return OPATTR_E_COUNT_MISMATCH;
+    if (S.replayed < 0) S.replayed = (int64_t)H.cnt[C_REPLAYED];     // layer pairs: counted on the way
+    S.direct = S.fast_path ? S.replayed : (int64_t)H.cnt[C_DIRECT];
+    S.broadcast = (int64_t)H.cnt[C_BROADCAST];
+    S.names_mismatched = (int64_t)H.cnt[C_NAMES_MISMATCH];
+    S.count_unmatched = S.fast_path ? 0 : (int64_t)H.cnt[C_COUNT_UNMATCHED];
+    S.dedup_mismatch = (int64_t)H.cnt[C_DEDUP_MISMATCH];
+    S.unmatched = S.kernels - S.direct - S.broadcast;
+    if (sum) *sum = S;
+    const int mode = (int)c.cfg.mismatch;
+    if (mode == OPATTR_MISMATCH_SKIP_NAME && S.names_mismatched > 0) return OPATTR_W_COUNT_MISMATCH;
+    if (mode == OPATTR_MISMATCH_PREFIX && S.count_unmatched > 0) return OPATTR_W_COUNT_MISMATCH;
+    if (S.dedup_mismatch > 0) return OPATTR_W_DEDUP_MISMATCH;
+    return OPATTR_OK;
 }
 
 opattr_status do_match(Ctx &c, const opattr_kernels *kern, const opattr_ncu *ncu, const opattr_dedup *dd,
@@ -417,9 +507,11 @@ opattr_status do_match(Ctx &c, const opattr_kernels *kern, const opattr_ncu *ncu
         for (int32_t l = 0; l < dd->n_layers; ++l) rep_layer[l] = dd->rep_of_class[dd->class_of_layer[l]];
     }
     const int64_t NL = dedup_on ? (dd->n_layers > 0 ? dd->n_layers : 1) : 1;
-    const int64_t NX = std::max(K, M);
     const bool per_stream = ncu->stream != nullptr;
-    if (per_stream && M > 0 && !ncu->name_id) return OPATTR_E_INVALID_ARG;
+    opattr_match_summary &S = c.match_sum;
+    S = opattr_match_summary{};
+    S.kernels = K;
+    S.replayed = K;
     // within a join the identity pairing ran within the enclosure: with the
     // kernels in time order (the enclosure's verdict) and every name equal,
     // its outputs are the match
@@ -429,227 +521,191 @@ opattr_status do_match(Ctx &c, const opattr_kernels *kern, const opattr_ncu *ncu
         c.spec_nname == ncu->name_id && c.spec_idx == out_idx &&
         c.spec_kind == out_kind && c.spec_k == K && K == M && !dedup_on && !per_stream &&
         (c.enclose_pending || !(c.h_status->flags & F_NAMES_DIFFER))) {
-        opattr_match_summary S{};
-        S.kernels = K;
-        S.replayed = K;
         S.direct = K;
         S.fast_path = 1;
         if (sum) *sum = S;
         c.rows_identity = true;
         return OPATTR_OK;
     }
+    // scratch: the sort of kernels and rows (keys and values twice; the free
+    // pair then holds the runs), the time order, and with layers the replayed
+    // kernels and the layer lists
+    const int64_t N = K + M, NX = std::max(K, M);
+    const int64_t LX = dedup_on ? K : 1, hist_n = std::max(radix_hist_elems(N), radix_hist_elems(NX));
+    const int64_t part_n = scan_scratch_elems(std::max(std::max(hist_n, N), K));
     Need nd;
-    if (per_stream) nd.add<uint32_t>(K).add<uint32_t>(M);        // (name, stream) keys
-    nd.add<int32_t>(NL);
-    for (int i = 0; i < 5; ++i) nd.add<uint32_t>(K);                 // flag, pos, rk, lk, keys
-    for (int i = 0; i < 3; ++i) nd.add<uint32_t>(NX);                // sort buffers
-    for (int i = 0; i < 4; ++i) nd.add<uint32_t>(M);                 // ncu sort
-    nd.add<uint32_t>(radix_hist_elems(NX)).add<uint32_t>(scan_scratch_elems(std::max(radix_hist_elems(NX), NX)));
-    nd.add<unsigned long long>(4);
+    nd.add<int32_t>(NL).add<unsigned long long>(4);
+    for (int i = 0; i < 4; ++i) nd.add<uint32_t>(N + 2).add<uint32_t>(LX);
+    nd.add<uint8_t>(NX).add<uint32_t>(hist_n).add<uint32_t>(part_n);
     size_t need = nd.bytes + time_sort_scratch(K) + 4096;
     opattr_status st = ensure_arena(c, need);
     if (st) return st;
     Arena a(c);
-    if ((st = reset_status(c))) return st;
     int32_t *d_rep = a.take<int32_t>(NL);
-    uint32_t *flag = a.take<uint32_t>(K), *pos = a.take<uint32_t>(K), *rk = a.take<uint32_t>(K);
-    uint32_t *lk = a.take<uint32_t>(K), *k0 = a.take<uint32_t>(K);
-    uint32_t *s0 = a.take<uint32_t>(NX), *s1 = a.take<uint32_t>(NX), *s2 = a.take<uint32_t>(NX);
-    uint32_t *n0 = a.take<uint32_t>(M), *n1 = a.take<uint32_t>(M), *n2 = a.take<uint32_t>(M), *n3 = a.take<uint32_t>(M);
-    uint32_t *hist = a.take<uint32_t>(radix_hist_elems(NX));
-    uint32_t *part = a.take<uint32_t>(scan_scratch_elems(std::max(radix_hist_elems(NX), NX)));
     unsigned long long *dsm = a.take<unsigned long long>(4);
-    if (!d_rep || !flag || !pos || !rk || !lk || !k0 || !s0 || !s1 || !s2 || !n0 || !n1 || !n2 || !n3 || !hist ||
-        !part || !dsm)
+    uint32_t *b0 = a.take<uint32_t>(N + 2), *b1 = a.take<uint32_t>(N + 2), *b2 = a.take<uint32_t>(N + 2),
+             *b3 = a.take<uint32_t>(N + 2);
+    uint32_t *flag = a.take<uint32_t>(LX), *pos = a.take<uint32_t>(LX), *rkb = a.take<uint32_t>(LX),
+             *lk = a.take<uint32_t>(LX);
+    uint8_t *nb = a.take<uint8_t>(NX);
+    uint32_t *hist = a.take<uint32_t>(hist_n), *part = a.take<uint32_t>(part_n);
+    if (!d_rep || !dsm || !b0 || !b1 || !b2 || !b3 || !flag || !pos || !rkb || !lk || !nb || !hist || !part)
         return OPATTR_E_OOM;
-    if (dedup_on && dd->n_layers > 0)
-        cudaMemcpyAsync(d_rep, rep_layer.data(), sizeof(int32_t) * dd->n_layers, cudaMemcpyHostToDevice, c.stream);
-    // the matching key: the name id, or (name, stream) when the rows carry
-    // streams (built only if the general path runs)
-    const uint32_t *kname = kern->name_id, *nname = ncu->name_id;
-    uint32_t *kkey = nullptr, *nkey = nullptr;
-    if (per_stream) {
-        kkey = a.take<uint32_t>(K);
-        nkey = a.take<uint32_t>(M);
-        if ((K > 0 && !kkey) || (M > 0 && !nkey)) return OPATTR_E_OOM;
+    // (nothing else uses the staging now: the enclosure before it in a join is
+    // through with it once its status was read, or never used it)
+    if (dedup_on && dd->n_layers > 0) {
+        const size_t bytes = sizeof(int32_t) * dd->n_layers;
+        if (bytes <= STAGE_BYTES && c.host_mapped) {
+            memcpy(c.h_stage, rep_layer.data(), bytes);
+            if ((st = copy_small(c, d_rep, c.h_stage, bytes, cudaMemcpyHostToDevice))) return st;
+        } else {
+            cudaMemcpyAsync(d_rep, rep_layer.data(), bytes, cudaMemcpyHostToDevice, c.stream);
+        }
     }
-
     const unsigned gK = grid_for(K, 256, REDUCE_GRID);
-    // within a join the enclosure has just verified these records' order, and
-    // kept their time order when they were out of it
+    uint32_t *const sort[4] = {b0, b1, b2, b3};
+    const bool few_layers = dedup_on && match_layers_ahead(dd);
+
+    // within a join the enclosure has just verified these records' order (or its
+    // verdict is pending and they are taken to be in order), and kept their time
+    // order when they were out of it
     const bool known_sorted = c.order_from_enclose && c.enclose_k_sorted == 1;
     const bool known_unsorted = c.order_from_enclose && c.enclose_k_sorted == 0 && c.join_korder;
-    if (!known_sorted && !known_unsorted) check_kernel_order(c, kern->stream, kern->start_ns, K);
-    if (dedup_on && K > 0)
-        launch(c, "check_layers", k_check_layers, dim3(gK), dim3(256), 0, kern->layer_id, K, dd->n_layers,
-               (const int32_t *)d_rep, c.d_status);
-    if (per_stream && dedup_on && K > 0)
-        launch(c, "check_names24", k_check_names24, dim3(grid_for(K, 256 * 8, REDUCE_GRID)), dim3(256), 0,
-               kern->name_id, K, c.d_status);
-    // Speculative fast paths, taking the kernel array to be in time order
-    // (confirmed or refuted by the order check in the same batch).
-    const bool try_identity = !dedup_on && !per_stream && K == M && K > 0 && !known_unsorted;
-    const bool try_streams = !dedup_on && per_stream && K == M && K > 0 && !known_unsorted;
-    if (try_identity)
-        launch(c, "match_identity", k_match_identity, dim3(grid_for(K, 256 * 16, REDUCE_GRID)), dim3(256), 0,
-               kname, nname, K, out_idx, out_kind, identity_vec(kname, nname, out_idx, out_kind), c.d_status);
-    if (try_streams)
-        stream_pairs(c, kern, ncu, nullptr, K, reinterpret_cast<uint8_t *>(n2), n0, n1, hist, part, out_idx,
-                     out_kind);
-    if ((st = read_status(c))) return st;
-    if (c.h_status->err & ERR_INVALID) return OPATTR_E_INVALID_ARG;
-    const bool k_sorted = known_sorted || (!known_unsorted && !(c.h_status->flags & F_K_UNSORTED));
-    opattr_match_summary S{};
-    S.kernels = K;
-    S.replayed = dedup_on ? (int64_t)c.h_status->cnt[C_REPLAYED] : K;
-    if ((try_identity || try_streams) && k_sorted && !(c.h_status->flags & F_NAMES_DIFFER)) {
-        S.direct = K;
-        S.fast_path = 1;
-        if (sum) *sum = S;
-        return OPATTR_OK;
+    // Fast paths, taking the kernel array to be in time order (confirmed or
+    // refuted by the order check in the same batch, or by the join).
+    const bool ahead = K > 0 && !known_unsorted && !c.no_spec;
+    const bool try_identity = ahead && !dedup_on && !per_stream && K == M;
+    const bool try_streams = ahead && !dedup_on && per_stream && K == M;
+    const bool try_layers = ahead && few_layers && !per_stream;
+    // with the enclosure's verdict pending the status block is its, and so is
+    // the one that found the largest key; what the fast path finds is read with
+    // the aggregation's status
+    const bool defer = known_sorted && c.enclose_pending && (try_streams || try_layers);
+    const bool sort_at_once = known_sorted && !dedup_on && c.max_known && !c.enclose_pending && !try_identity &&
+                              !try_streams;
+    const ZeroRun zc{part, chain_words(K)};
+    uint64_t max_key = 0;
+    if (defer) {
+        if (try_layers && (st = zero_runs(c, 1, &zc))) return st;
+    } else if (sort_at_once) {
+        max_key = c.h_status->cnt[C_MAX_KEY];
+    } else if ((st = reset_status(c, try_layers ? 1 : 0, &zc))) {
+        return st;
     }
-    // the speculative verdicts are spent: later checks start from clear flags
-    cudaMemsetAsync(&c.d_status->flags, 0, sizeof(unsigned), c.stream);
+    const bool want_max = !defer && !sort_at_once && N > 0;
+    if (!sort_at_once) {
+        if (!known_sorted && !known_unsorted) check_kernel_order(c, kern->stream, kern->start_ns, K);
+        if (try_layers)
+            launch(c, "layer_pairs", k_layer_pairs, dim3(grid_for(K, SCAN_TILE)), dim3(SCAN_THREADS), 0,
+                   kern->layer_id, (const int32_t *)d_rep, dd->n_layers, kern->name_id, ncu->name_id, K, M,
+                   make_chain(c, part, K), out_idx, out_kind, c.d_status);
+        else if (dedup_on && K > 0)
+            launch(c, "check_layers", k_check_layers, dim3(gK), dim3(256), 0, kern->layer_id, K, dd->n_layers,
+                   (const int32_t *)d_rep, c.d_status);
+        if (per_stream && dedup_on && K > 0)
+            launch(c, "check_names24", k_check_names24, dim3(grid_for(K, 256 * 8, REDUCE_GRID)), dim3(256), 0,
+                   kern->name_id, K, c.d_status);
+        if (try_identity)
+            launch(c, "match_identity", k_match_identity, dim3(grid_for(K, 256 * 16, REDUCE_GRID)), dim3(256), 0,
+                   kern->name_id, ncu->name_id, K, out_idx, out_kind,
+                   identity_vec(kern->name_id, ncu->name_id, out_idx, out_kind), c.d_status);
+        if (try_streams) stream_pairs(c, kern, ncu, nullptr, K, nb, b0, b1, hist, part, out_idx, out_kind);
+        if (try_layers && (st = broadcast_layers(c, kern, dd, d_rep, nullptr, flag, pos, lk, sort, hist, part, dsm,
+                                                 out_idx, out_kind)))
+            return st;
+        // (a pairing by rows as many as the kernels rarely fails: the largest key is then found afterwards)
+        const bool now = want_max && !try_identity && !try_streams && !try_layers;
+        if (now)
+            launch(c, "max_key", k_max_key, dim3(grid_for(N, 256 * 8, 1024)), dim3(256), 0, kern->name_id, kern->stream,
+                   K, ncu->name_id, ncu->stream, M, c.d_status);
+        if (defer) {
+            S.fast_path = 1;
+            if (try_layers) S.replayed = -1;
+            c.match_pending = true;
+            return OPATTR_OK;
+        }
+        if ((st = read_status(c))) return st;
+        if (c.h_status->err & ERR_INVALID) return OPATTR_E_INVALID_ARG;
+        max_key = c.h_status->cnt[C_MAX_KEY];
+        const bool sorted = known_sorted || (!known_unsorted && !(c.h_status->flags & F_K_UNSORTED));
+        if (dedup_on) S.replayed = (int64_t)c.h_status->cnt[C_REPLAYED];
+        if ((try_identity || try_streams || try_layers) && sorted && !(c.h_status->flags & F_NAMES_DIFFER)) {
+            S.fast_path = 1;
+            return match_verdict(c, sum);
+        }
+        // the speculative verdicts are spent: later checks start from clear flags and counts
+        const ZeroRun zr[2] = {{&c.d_status->flags, 1}, {&c.d_status->cnt[0], 2 * C_MAX_KEY}};
+        if ((st = zero_runs(c, 2, zr))) return st;
+    }
+    const bool k_sorted = known_sorted || (!known_unsorted && !(c.h_status->flags & F_K_UNSORTED));
 
     // ---- general path
-    if (K > 0) launch(c, "fill_match", k_fill_match, dim3(gK), dim3(256), 0, out_idx, out_kind, K);
     uint32_t *korder = nullptr;
     if (!k_sorted && K > 0) {
         if (known_unsorted) korder = c.join_korder;
         else if ((st = kernel_time_order(c, a, kern->stream, kern->start_ns, K, &korder))) return st;
     }
-    // rk[j] = kernel index of the j-th replayed kernel in time order
+    // rk[j] = kernel index of the j-th replayed kernel in time order (NULL: j itself)
     int64_t nrep = K;
+    const uint32_t *rk = korder;
     if (dedup_on && K > 0) {
         launch(c, "flags", k_flags, dim3(gK), dim3(256), 0, (const uint32_t *)korder, kern->layer_id,
                (const int32_t *)d_rep, K, 0, flag);
         scan_exclusive_u32(c, flag, pos, K, part, nullptr);
         launch(c, "compact", k_compact, dim3(gK), dim3(256), 0, (const uint32_t *)korder, (const uint32_t *)flag,
-               (const uint32_t *)pos, K, rk);
+               (const uint32_t *)pos, K, rkb);
         nrep = S.replayed;
-    } else if (K > 0) {
-        if (korder) cudaMemcpyAsync(rk, korder, sizeof(uint32_t) * K, cudaMemcpyDeviceToDevice, c.stream);
-        else launch(c, "iota", k_iota, dim3(gK), dim3(256), 0, rk, K);
+        rk = rkb;
+        // (duplicate-layer kernels are written by the broadcast, the others by the join)
     }
     bool direct_done = false;
     // rows equal to the replayed kernels in time order, tried before the name
-    // sorts: with layer deduplication, or when the kernels were out of time order
-    const bool retry_streams = per_stream && (dedup_on || korder) && nrep == M && nrep > 0;
-    if (((dedup_on || korder) && !per_stream && nrep == M && nrep > 0) || retry_streams) {
-        if (retry_streams)
-            stream_pairs(c, kern, ncu, rk, nrep, reinterpret_cast<uint8_t *>(n2), n0, n1, hist, part, out_idx,
-                         out_kind);
+    // sort: with layer deduplication, or when the kernels were out of time order
+    const bool retry_streams = per_stream && !c.no_spec && (dedup_on || korder) && nrep == M && nrep > 0;
+    const bool retry_list = !per_stream && !c.no_spec && (korder || (dedup_on && !try_layers)) && nrep == M &&
+                            nrep > 0;
+    if (retry_streams || retry_list) {
+        if (retry_streams) stream_pairs(c, kern, ncu, rk, nrep, nb, b0, b1, hist, part, out_idx, out_kind);
         else
             launch(c, "match_identity_list", k_match_identity_list, dim3(grid_for(nrep, 256, REDUCE_GRID)),
-                   dim3(256), 0, (const uint32_t *)rk, kname, nname, nrep, out_idx, out_kind, c.d_status);
+                   dim3(256), 0, rk, kern->name_id, ncu->name_id, nrep, out_idx, out_kind, c.d_status);
         if ((st = read_status(c))) return st;
         if (c.h_status->err & ERR_INVALID) return OPATTR_E_INVALID_ARG;
         direct_done = !(c.h_status->flags & F_NAMES_DIFFER);
-        if (direct_done) S.fast_path = 1;
-        else launch(c, "fill_match", k_fill_match, dim3(gK), dim3(256), 0, out_idx, out_kind, K);
     }
     if (!direct_done && (nrep > 0 || M > 0)) {
-        if (per_stream) {
-            if (K > 0)
-                launch(c, "stream_keys", k_stream_keys, dim3(grid_for(K, 256, REDUCE_GRID)), dim3(256), 0,
-                       kern->name_id, kern->stream, K, kkey, c.d_status);
-            if (M > 0)
-                launch(c, "stream_keys", k_stream_keys, dim3(grid_for(M, 256, REDUCE_GRID)), dim3(256), 0,
-                       ncu->name_id, ncu->stream, M, nkey, c.d_status);
-            kname = kkey;
-            nname = nkey;
+        const int64_t n = nrep + M;
+        if (max_key == 0) {
+            launch(c, "max_key", k_max_key, dim3(grid_for(N, 256 * 8, 1024)), dim3(256), 0, kern->name_id, kern->stream,
+                   K, ncu->name_id, ncu->stream, M, c.d_status);
+            if ((st = read_status(c))) return st;
+            max_key = c.h_status->cnt[C_MAX_KEY];
         }
-        cudaMemsetAsync(dsm, 0, sizeof(unsigned long long), c.stream);
-        if (nrep > 0) {
-            launch(c, "gather_names", k_gather_u32, dim3(grid_for(nrep, 256, REDUCE_GRID)), dim3(256), 0, kname,
-                   (const uint32_t *)rk, nrep, k0);
-            launch(c, "max_name", k_max_u32, dim3(grid_for(nrep, 256, 4096)), dim3(256), 0, (const uint32_t *)k0, nrep,
-                   dsm);
-        }
-        if (M > 0) {
-            cudaMemcpyAsync(n0, nname, sizeof(uint32_t) * M, cudaMemcpyDeviceToDevice, c.stream);
-            launch(c, "max_name", k_max_u32, dim3(grid_for(M, 256, 4096)), dim3(256), 0, (const uint32_t *)n0, M, dsm);
-        }
-        unsigned long long hmax = 0;
-        if ((st = read_u64(c, dsm, &hmax))) return st;
-        const int bits = bits_for(hmax);
-        uint32_t *skn = nullptr, *skj = nullptr, *snn = n0, *snj = n1;
-        if (nrep > 0) radix_sort_pairs<uint32_t>(c, k0, s0, s1, s2, nrep, bits, true, hist, part, &skn, &skj);
-        if (M > 0) radix_sort_pairs<uint32_t>(c, n0, n1, n2, n3, M, bits, true, hist, part, &snn, &snj);
-        // run tables of both sorted name arrays (pos / start pairs in the
-        // buffers the sorts left free)
-        uint32_t *kfree0 = skn == k0 ? s1 : k0, *kfree1 = skn == k0 ? s2 : s0;
-        uint32_t *nfree0 = snn == n0 ? n2 : n0, *nfree1 = snn == n0 ? n3 : n1;
-        uint32_t *kpos = flag, *ustart = pos, *b_of = kfree0, *cq_of = kfree1, *vpos = nfree0, *vstart = nfree1;
-        uint32_t *n_urun = reinterpret_cast<uint32_t *>(dsm + 2), *n_vrun = reinterpret_cast<uint32_t *>(dsm + 3);
-        if (nrep > 0) {
-            launch(c, "run_heads", k_run_heads, dim3(grid_for(nrep, 256, REDUCE_GRID)), dim3(256), 0,
-                   (const uint32_t *)skn, nrep, kpos);
-        }
-        scan_exclusive_u32(c, kpos, kpos, nrep, part, n_urun);
-        if (nrep > 0)
-            launch(c, "run_starts", k_run_starts, dim3(grid_for(nrep, 256, REDUCE_GRID)), dim3(256), 0,
-                   (const uint32_t *)skn, (const uint32_t *)kpos, nrep, ustart);
-        if (M > 0)
-            launch(c, "run_heads", k_run_heads, dim3(grid_for(M, 256, REDUCE_GRID)), dim3(256), 0,
-                   (const uint32_t *)snn, M, vpos);
-        scan_exclusive_u32(c, vpos, vpos, M, part, n_vrun);
-        if (M > 0)
-            launch(c, "run_starts", k_run_starts, dim3(grid_for(M, 256, REDUCE_GRID)), dim3(256), 0,
-                   (const uint32_t *)snn, (const uint32_t *)vpos, M, vstart);
-        if (nrep > 0) {
-            launch(c, "run_pair", k_run_pair, dim3(grid_for(nrep, 256, REDUCE_GRID)), dim3(256), 0,
-                   (const uint32_t *)skn, (const uint32_t *)ustart, (const uint32_t *)n_urun, nrep,
-                   (const uint32_t *)snn, (const uint32_t *)vstart, (const uint32_t *)n_vrun, M, mode, b_of, cq_of,
-                   c.d_status);
-            launch(c, "ordinal_join", k_ordinal_join, dim3(grid_for(nrep, 256, REDUCE_GRID)), dim3(256), 0,
-                   (const uint32_t *)skn, (const uint32_t *)skj, (const uint32_t *)kpos, (const uint32_t *)ustart,
-                   (const uint32_t *)n_urun, (const uint32_t *)b_of, (const uint32_t *)cq_of, (const uint32_t *)rk,
-                   nrep, (const uint32_t *)snj, mode, out_idx, out_kind, c.d_status);
-        }
-        if (M > 0)
-            launch(c, "ncu_only_names", k_ncu_only_names, dim3(grid_for(M, 256, REDUCE_GRID)), dim3(256), 0,
-                   (const uint32_t *)snn, (const uint32_t *)vstart, (const uint32_t *)n_vrun, (const uint32_t *)skn,
-                   (const uint32_t *)ustart, (const uint32_t *)n_urun, mode, c.d_status);
+        launch(c, "pair_keys", k_pair_keys, dim3(grid_for(n, 256 * 4, REDUCE_GRID)), dim3(256), 0, rk, kern->name_id,
+               kern->stream, nrep, ncu->name_id, ncu->stream, n, b0, c.d_status);
+        uint32_t *sk = nullptr, *sv = nullptr;
+        radix_sort_pairs<uint32_t>(c, b0, b1, b2, b3, n, bits_for(max_key), true, hist, part, &sk, &sv);
+        uint32_t *run = sk == b0 ? b2 : b0, *start = sv == b1 ? b3 : b1;
+        uint32_t *n_run = reinterpret_cast<uint32_t *>(dsm + 2);
+        const ZeroRun zn{part, chain_words(n)};
+        if ((st = zero_runs(c, 1, &zn))) return st;
+        launch(c, "runs", k_runs, dim3(grid_for(n, SCAN_TILE)), dim3(SCAN_THREADS), 0, (const uint32_t *)sk,
+               (const uint32_t *)sv, nrep, n, make_chain(c, part, n), run, start, n_run);
+        launch(c, "ordinal_join", k_ordinal_join, dim3(grid_for(n, 256 * 2, REDUCE_GRID)), dim3(256), 0,
+               (const uint32_t *)sk, (const uint32_t *)sv, nrep, n, (const uint32_t *)run, (const uint32_t *)start,
+               (const uint32_t *)n_run, rk, mode, out_idx, out_kind, c.d_status);
     }
-    if (dedup_on && K > 0) {
-        // positions within layers: layer-tagged kernels in time order, sorted by layer
-        launch(c, "flags", k_flags, dim3(gK), dim3(256), 0, (const uint32_t *)korder, kern->layer_id,
-               (const int32_t *)d_rep, K, 1, flag);
-        uint32_t *ntag = reinterpret_cast<uint32_t *>(dsm + 1);
-        scan_exclusive_u32(c, flag, pos, K, part, ntag);
-        launch(c, "compact", k_compact, dim3(gK), dim3(256), 0, (const uint32_t *)korder, (const uint32_t *)flag,
-               (const uint32_t *)pos, K, lk);
-        unsigned long long ntag_h = 0;
-        if ((st = read_u64(c, dsm + 1, &ntag_h))) return st;
-        const int64_t nlk = (int64_t)(ntag_h & 0xFFFFFFFFull);
-        if (nlk > 0) {
-            launch(c, "gather_layers", k_gather_i32_as_u32, dim3(grid_for(nlk, 256, REDUCE_GRID)), dim3(256), 0,
-                   kern->layer_id, (const uint32_t *)lk, nlk, k0);
-            uint32_t *sll, *slj;
-            radix_sort_pairs<uint32_t>(c, k0, s0, s1, s2, nlk,
-                                       bits_for((uint64_t)(dd->n_layers > 0 ? dd->n_layers - 1 : 0)), true, hist, part,
-                                       &sll, &slj);
-            launch(c, "dedup_broadcast", k_dedup_broadcast, dim3(grid_for(nlk, 256, REDUCE_GRID)), dim3(256), 0,
-                   (const uint32_t *)sll, (const uint32_t *)slj, (const uint32_t *)lk, nlk, (const int32_t *)d_rep,
-                   kern->name_id, out_idx, out_kind, c.d_status);   // plain names: a class may span streams
-        }
+    S.fast_path = direct_done ? 1 : 0;
+    if (dedup_on && K > 0 && (st = broadcast_layers(c, kern, dd, d_rep, korder, flag, pos, lk, sort, hist, part, dsm,
+                                                    out_idx, out_kind)))
+        return st;
+    if (c.in_join) {
+        // complete but for its counts, read with the aggregation's status
+        c.match_pending = c.keep_status = true;
+        return OPATTR_OK;
     }
     if ((st = read_status(c))) return st;
-    const DevStatus &H = *c.h_status;
-    if (H.err & ERR_INVALID) return OPATTR_E_INVALID_ARG;
-    if (H.err & ERR_COUNT) return OPATTR_E_COUNT_MISMATCH;
-    S.direct = direct_done ? nrep : (int64_t)H.cnt[C_DIRECT];
-    S.broadcast = (int64_t)H.cnt[C_BROADCAST];
-    S.names_mismatched = (int64_t)H.cnt[C_NAMES_MISMATCH];
-    S.count_unmatched = direct_done ? 0 : (int64_t)H.cnt[C_COUNT_UNMATCHED];
-    S.dedup_mismatch = (int64_t)H.cnt[C_DEDUP_MISMATCH];
-    S.unmatched = K - S.direct - S.broadcast;
-    if (sum) *sum = S;
-    if (mode == OPATTR_MISMATCH_SKIP_NAME && S.names_mismatched > 0) return OPATTR_W_COUNT_MISMATCH;
-    if (mode == OPATTR_MISMATCH_PREFIX && S.count_unmatched > 0) return OPATTR_W_COUNT_MISMATCH;
-    if (S.dedup_mismatch > 0) return OPATTR_W_DEDUP_MISMATCH;
-    return OPATTR_OK;
+    return match_verdict(c, sum);
 }
 
 }  // namespace opattr

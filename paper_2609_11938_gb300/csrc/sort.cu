@@ -89,47 +89,25 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(const uint32_t *in, 
 // before it.  Out of place only: a tile whose wait gives up sums the input of
 // the tiles before it that are still silent.
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_onepass(const uint32_t *__restrict__ in,
-                                                               uint32_t *__restrict__ out, int64_t n,
-                                                               unsigned long long *status, unsigned *tile_ctr,
-                                                               int64_t nt, uint32_t *total_dev, int64_t spin_limit,
-                                                               int fault, DevStatus *st) {
+                                                               uint32_t *__restrict__ out, int64_t n, Chain C,
+                                                               uint32_t *total_dev) {
     pdl_wait();
-    __shared__ uint32_t wbuf[33];
-    __shared__ unsigned tile_s;
-    __shared__ uint32_t off_s;
-    if (threadIdx.x == 0) tile_s = atomicAdd(tile_ctr, 1u);
-    __syncthreads();
-    const int64_t tile = tile_s;
-    const unsigned w = threadIdx.x >> 5;
-    const int64_t base = tile * SCAN_TILE + w * (SCAN_TILE / 8);
-    uint32_t v[SCAN_ITEMS];
-    uint32_t carry = 0;
-#pragma unroll
-    for (int it = 0; it < SCAN_ITEMS; ++it) {
-        const int64_t i = base + it * 32 + lane_id();
-        const uint32_t x = i < n ? in[i] : 0u;
-        const uint32_t inc = warp_inclusive_scan(x);
-        v[it] = carry + inc - x;
-        carry += __shfl_sync(0xffffffffu, inc, 31);
-    }
-    // carry = this warp's total; block-exclusive prefix over warps
-    uint32_t btot;
-    uint32_t wpre = block_exclusive_scan<uint32_t>(lane_id() == 0 ? carry : 0u, wbuf, &btot);
-    wpre = __shfl_sync(0xffffffffu, wpre, 0);
-    if (threadIdx.x < 32) {
-        const uint32_t ex = warp_lookback_exclusive(status, tile, btot, in, n, SCAN_TILE, spin_limit, fault != 0, st);
-        if (threadIdx.x == 0) {
-            off_s = ex;
-            if (tile == nt - 1 && total_dev) *total_dev = ex + btot;
-        }
-    }
-    __syncthreads();
-    const uint32_t off = off_s + wpre;
-#pragma unroll
-    for (int it = 0; it < SCAN_ITEMS; ++it) {
-        const int64_t i = base + it * 32 + lane_id();
-        if (i < n) out[i] = off + v[it];
-    }
+    chained_scan(
+        C, n, [&](int64_t i) { return in[i]; }, [&](int64_t i, uint32_t, uint32_t ex) { out[i] = ex; },
+        [&](uint32_t total) {
+            if (total_dev) *total_dev = total;
+        });
+}
+
+Chain make_chain(Ctx &c, uint32_t *words, int64_t n) {
+    const char *fault = getenv("OPATTR_FAULT");
+    Chain C;
+    C.status = reinterpret_cast<unsigned long long *>(words);
+    C.tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
+    C.spin_limit = c.cfg.spin_limit > 0 ? c.cfg.spin_limit : LB_SPIN_DEFAULT;
+    C.fault = fault && strcmp(fault, "lookback") == 0;
+    C.st = c.d_status;
+    return C;
 }
 
 // Small scans in one block (one launch instead of three): each of the 32
@@ -185,13 +163,10 @@ void scan_exclusive_u32(Ctx &c, const uint32_t *in, uint32_t *out, int64_t n, ui
                (const uint32_t *)partials);
         return;
     }
-    unsigned long long *status = reinterpret_cast<unsigned long long *>(partials);
-    cudaMemsetAsync(status, 0, sizeof(unsigned long long) * (nt + 1), c.stream);
-    const char *fault = getenv("OPATTR_FAULT");
-    const int lb_fault = fault && strcmp(fault, "lookback") == 0;
-    const int64_t spin = c.cfg.spin_limit > 0 ? c.cfg.spin_limit : LB_SPIN_DEFAULT;
-    launch(c, "scan", k_scan_onepass, dim3((unsigned)nt), dim3(SCAN_THREADS), 0, in, out, n, status,
-           reinterpret_cast<unsigned *>(status + nt), nt, total_dev, spin, lb_fault, c.d_status);
+    const ZeroRun z{partials, chain_words(n)};
+    zero_runs(c, 1, &z);
+    launch(c, "scan", k_scan_onepass, dim3((unsigned)nt), dim3(SCAN_THREADS), 0, in, out, n, make_chain(c, partials, n),
+           total_dev);
 }
 
 // ------------------------------------------------------------------ radix sort

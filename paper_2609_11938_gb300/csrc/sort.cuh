@@ -61,9 +61,10 @@ constexpr int64_t LB_SPIN_DEFAULT = 1 << 20;
 
 // Called by all 32 lanes of one warp with the same arguments; returns the
 // sum of `total` over the tiles before t (in every lane).  Tile q covers
-// in[q * tile_elems, min((q + 1) * tile_elems, n)).
+// elements [q * tile_elems, min((q + 1) * tile_elems, n)), at(i) is element i.
+template <typename At>
 __device__ __forceinline__ uint32_t warp_lookback_exclusive(unsigned long long *status, int64_t t, uint32_t total,
-                                                            const uint32_t *in, int64_t n, int64_t tile_elems,
+                                                            At at, int64_t n, int64_t tile_elems,
                                                             int64_t spin_limit, bool fault, DevStatus *st) {
     const unsigned lane = lane_id();
     volatile unsigned long long *word = status;
@@ -90,7 +91,7 @@ __device__ __forceinline__ uint32_t warp_lookback_exclusive(unsigned long long *
             if ((none >> lane) & 1u) {       // its total, from its input
                 const int64_t e = (q + 1) * tile_elems < n ? (q + 1) * tile_elems : n;
                 uint32_t s = 0;
-                for (int64_t i = q * tile_elems; i < e; ++i) s += in[i];
+                for (int64_t i = q * tile_elems; i < e; ++i) s += at(i);
                 v = LB_AGG | s;
             }
             inc = __ballot_sync(0xffffffffu, (v & LB_INC) != 0);
@@ -106,6 +107,65 @@ __device__ __forceinline__ uint32_t warp_lookback_exclusive(unsigned long long *
         word[t] = LB_INC | (uint32_t)(excl + total);
     }
     return excl;
+}
+
+// What a kernel that chains its tiles needs: status words and the tile counter
+// (zero before the launch), the bound of its wait.
+struct Chain {
+    unsigned long long *status;          // [tiles], the counter after them
+    int64_t tiles, spin_limit;
+    int fault;
+    DevStatus *st;
+};
+// Words of such a chain over n elements (scan_scratch_elems(n) of them hold it).
+inline int64_t chain_words(int64_t n) { return 2 * ((n + SCAN_TILE - 1) / SCAN_TILE) + 2; }
+Chain make_chain(Ctx &c, uint32_t *words, int64_t n);
+
+// Tiles of SCAN_TILE elements in the order blocks start, by blocks of
+// SCAN_THREADS: element i's value is at(i) (0 or more), put(i, value, exclusive
+// prefix) is called for every element, done(total) by one thread of the last tile.
+template <typename At, typename Put, typename Done>
+__device__ __forceinline__ void chained_scan(const Chain &C, int64_t n, At at, Put put, Done done) {
+    __shared__ uint32_t wbuf[33];
+    __shared__ unsigned tile_s;
+    __shared__ uint32_t off_s;
+    if (threadIdx.x == 0) tile_s = atomicAdd(reinterpret_cast<unsigned *>(C.status + C.tiles), 1u);
+    __syncthreads();
+    const int64_t tile = tile_s;
+    const unsigned w = threadIdx.x >> 5;
+    const int64_t base = tile * SCAN_TILE + w * (SCAN_TILE / 8);
+    uint32_t v[SCAN_ITEMS], x[SCAN_ITEMS];
+    uint32_t carry = 0;
+#pragma unroll
+    for (int it = 0; it < SCAN_ITEMS; ++it) {
+        const int64_t i = base + it * 32 + lane_id();
+        x[it] = i < n ? at(i) : 0u;
+    }
+#pragma unroll
+    for (int it = 0; it < SCAN_ITEMS; ++it) {
+        const uint32_t inc = warp_inclusive_scan(x[it]);
+        v[it] = carry + inc - x[it];
+        carry += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    // carry = this warp's total; block-exclusive prefix over warps
+    uint32_t btot;
+    uint32_t wpre = block_exclusive_scan<uint32_t>(lane_id() == 0 ? carry : 0u, wbuf, &btot);
+    wpre = __shfl_sync(0xffffffffu, wpre, 0);
+    if (threadIdx.x < 32) {
+        const uint32_t ex =
+            warp_lookback_exclusive(C.status, tile, btot, at, n, SCAN_TILE, C.spin_limit, C.fault != 0, C.st);
+        if (threadIdx.x == 0) {
+            off_s = ex;
+            if (tile == C.tiles - 1) done(ex + btot);
+        }
+    }
+    __syncthreads();
+    const uint32_t off = off_s + wpre;
+#pragma unroll
+    for (int it = 0; it < SCAN_ITEMS; ++it) {
+        const int64_t i = base + it * 32 + lane_id();
+        if (i < n) put(i, x[it], off + v[it]);
+    }
 }
 
 // ------------------------------------------------------------------ digit passes
