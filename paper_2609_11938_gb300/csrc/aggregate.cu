@@ -603,6 +603,22 @@ __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// The counter rows of a warp's 32 kernels to shared memory, dst[l] for lane l
+// (row index j, -1 for none).  The lanes together copy 16-byte parts in the
+// order they lie, so one copy instruction touches the seven rows its 512 bytes
+// fall in, where each lane copying its own row touched 32 lines with every
+// instruction and the L1's tag lookups bound the pass.  Every lane must call it;
+// after the wait for its own copies a __syncwarp() makes the others' visible.
+__device__ __forceinline__ void cp_async_rows(float4 (*dst)[NC / 4], const float4 *rows, int32_t j) {
+    float4 *flat = &dst[0][0];
+#pragma unroll
+    for (int q = 0; q < NC / 4; ++q) {
+        const unsigned e = q * 32 + lane_id(), r = e / (NC / 4), c = e - r * (NC / 4);
+        const int32_t jr = __shfl_sync(0xffffffffu, j, (int)r);
+        if (jr >= 0) cp_async16(flat + e, rows + (int64_t)jr * (NC / 4) + c);
+    }
+}
+
 __global__ void __launch_bounds__(AG_THREADS, 5) k_agg_ops(const uint32_t *__restrict__ off, uint32_t *list,
                                                           AggIn A, int pending, const DevStatus *st) {
     pdl_wait();
@@ -919,21 +935,9 @@ __global__ void k_huge_index(const uint32_t *__restrict__ hop, int64_t n_huge, u
         hidx[hop[c]] = (uint32_t)c;
 }
 
-// A lane's run of a piece with the fast accumulator: returns false when a
-// null or infinite value took part (the caller redoes the run carefully),
-// else the run's partial in careful form (every counter non-null).
-__device__ __forceinline__ bool piece_fast(const AggIn &A, const uint32_t *seg, uint32_t l0, uint32_t l1, Acc &out) {
-    AccF f;
-    f.init();
-#pragma unroll 4
-    for (uint32_t t = l0; t < l1; ++t) {
-        const uint32_t k = seg[t];
-        const int32_t j = A.ncu_idx[k];
-        const bool ok = j >= 0 && j < A.M;
-        f.accumulate(A.dur[k], ok, reinterpret_cast<const float4 *>(A.counters + (int64_t)(ok ? j : 0) * NC));
-    }
-    if (!f.clean()) return false;
-    out.kc = (int)(l1 - l0);
+// A fast partial in careful form (every counter of every matched kernel non-null).
+__device__ __forceinline__ void acc_from_fast(Acc &out, const AccF &f, int kc) {
+    out.kc = kc;
     out.mc = f.mc;
     out.dsum = f.dsum;
     out.dall = f.dall;
@@ -949,21 +953,115 @@ __device__ __forceinline__ bool piece_fast(const AggIn &A, const uint32_t *seg, 
     out.seen = f.mc > 0 ? ALL_COUNTERS : 0u;
     out.bad = 0;
     out.terms = 0;
+}
+// A lane's run of a piece with the fast accumulator: returns false when a
+// null or infinite value took part (the caller redoes the run carefully),
+// else the run's partial in careful form (every counter non-null).
+__device__ __forceinline__ bool piece_fast(const AggIn &A, const uint32_t *seg, uint32_t l0, uint32_t l1, Acc &out) {
+    AccF f;
+    f.init();
+#pragma unroll 4
+    for (uint32_t t = l0; t < l1; ++t) {
+        const uint32_t k = seg[t];
+        const int32_t j = A.ncu_idx[k];
+        const bool ok = j >= 0 && j < A.M;
+        f.accumulate(A.dur[k], ok, reinterpret_cast<const float4 *>(A.counters + (int64_t)(ok ? j : 0) * NC));
+    }
+    if (!f.clean()) return false;
+    acc_from_fast(out, f, (int)(l1 - l0));
     return true;
 }
 
-// Pieces: one warp per AG_PIECE kernels of a huge op (lane l adds AG_PIECE /
-// 32 consecutive kernels), the warp's 32 partials merged by the fixed tree,
-// the piece's partial stored at its index.
-__global__ void k_agg_pieces(const uint32_t *__restrict__ off, const uint32_t *__restrict__ list,
+// The same partial with the rows ahead: kernel t + PC_AHEAD's row and duration
+// arrive in the lane's shared-memory slots by asynchronous copy while kernel t
+// is added, its indices loaded two steps earlier still.  Every lane of the warp
+// calls it.
+constexpr int PC_SLOTS = 4, PC_AHEAD = PC_SLOTS - 1, PC_THREADS = 256;
+struct PieceSlots {
+    float4 row[PC_SLOTS][32][NC / 4];
+    long long dur[PC_SLOTS][32];
+};
+constexpr size_t PC_SMEM = sizeof(PieceSlots) * (PC_THREADS / 32);
+template <typename At>                       // at(t): the lane's t-th kernel, t < n
+__device__ __forceinline__ bool piece_ahead(const AggIn &A, At at, uint32_t n, PieceSlots &S, Acc &out) {
+    const unsigned lane = lane_id();
+    const float4 *rows = reinterpret_cast<const float4 *>(A.counters);
+    auto row_of = [&](uint32_t k) -> int32_t {
+        const int32_t j = A.ncu_idx[k];
+        return j < A.M ? j : -1;
+    };
+    auto issue = [&](uint32_t t, uint32_t k, int32_t j) {
+        if (t < n) cp_async8(&S.dur[t % PC_SLOTS][lane], A.dur + k);
+        cp_async_rows(S.row[t % PC_SLOTS], rows, j);
+        cp_async_commit();
+    };
+    const uint32_t most = __reduce_max_sync(0xffffffffu, n);       // the lanes copy together
+    AccF f;
+    f.init();
+    unsigned have = 0;                       // bit t % PC_SLOTS: the kernel in that slot has a row
+    uint32_t k = 0;
+    int32_t j = -1;
+#pragma unroll
+    for (uint32_t t = 0; t < (uint32_t)PC_AHEAD; ++t) {
+        const uint32_t kt = t < n ? at(t) : 0u;
+        const int32_t jt = t < n ? row_of(kt) : -1;
+        issue(t, kt, jt);
+        have |= (jt >= 0 ? 1u : 0u) << t;
+    }
+    if (PC_AHEAD < n) {
+        k = at(PC_AHEAD);
+        j = row_of(k);
+    }
+    uint32_t k2 = PC_AHEAD + 1 < n ? at(PC_AHEAD + 1) : 0u;
+    for (uint32_t t = 0; t < most; ++t) {
+        const int32_t j2 = t + PC_AHEAD + 1 < n ? row_of(k2) : -1;
+        const uint32_t k3 = t + PC_AHEAD + 2 < n ? at(t + PC_AHEAD + 2) : 0u;
+        cp_async_wait<PC_AHEAD - 1>();
+        __syncwarp();
+        if (t < n) f.accumulate(S.dur[t % PC_SLOTS][lane], (have >> (t % PC_SLOTS)) & 1u, S.row[t % PC_SLOTS][lane]);
+        __syncwarp();
+        issue(t + PC_AHEAD, k, j);
+        const unsigned bit = 1u << ((t + PC_AHEAD) % PC_SLOTS);
+        have = j >= 0 ? have | bit : have & ~bit;
+        k = k2;
+        j = j2;
+        k2 = k3;
+    }
+    cp_async_wait<0>();
+    if (!f.clean()) return false;
+    acc_from_fast(out, f, (int)n);
+    return true;
+}
+
+// A warp's kernels, n of them this lane's: the 32 partials merged by the fixed
+// tree into *part.
+template <typename At>
+__device__ __forceinline__ void piece_by_warp(const AggIn &A, At at, uint32_t n, PieceSlots &S, Acc *part) {
+    const uint32_t lane = lane_id();
+    Acc acc;
+    if (!piece_ahead(A, at, n, S, acc)) {                 // a null or infinite value: redo with null handling
+        acc.init();
+        for (uint32_t t = 0; t < n; ++t) acc.add(A, at(t));
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int d = 16; d > 0; d >>= 1) acc_merge_down(acc, d);
+    if (lane == 0) *part = acc;
+}
+
+// Pieces: one warp per AG_PIECE kernels of a huge op, the piece's partial stored
+// at its index.  Bound by the gathers of the rows (80 bytes in three or four
+// sectors each).
+__global__ void __launch_bounds__(PC_THREADS, 2) k_agg_pieces(const uint32_t *__restrict__ off, const uint32_t *__restrict__ list,
                              const uint32_t *__restrict__ longs, const unsigned *__restrict__ nlong,
                              const uint32_t *__restrict__ poff, AggIn A, Acc *__restrict__ part) {
     pdl_wait();
+    extern __shared__ __align__(16) unsigned char ag_smem[];
+    PieceSlots &S = reinterpret_cast<PieceSlots *>(ag_smem)[threadIdx.x / 32];
     const int64_t n = *nlong;
     const int64_t P = poff[n];
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const unsigned lane = lane_id();
     for (int64_t p = warp; p < P; p += nwarps) {
         int64_t lo = 0, hi = n;                   // the listed op: last j with poff[j] <= p
         while (hi - lo > 1) {
@@ -974,17 +1072,16 @@ __global__ void k_agg_pieces(const uint32_t *__restrict__ off, const uint32_t *_
         const uint32_t s0 = off[o], len = off[o + 1] - s0;
         const uint32_t b0 = (uint32_t)(p - poff[lo]) * AG_PIECE;
         const uint32_t b1 = b0 + AG_PIECE < len ? b0 + AG_PIECE : len;
-        const uint32_t per = AG_PIECE / 32;
-        const uint32_t l0 = min(b0 + lane * per, b1), l1 = min(l0 + per, b1);
-        Acc acc;
-        if (!piece_fast(A, list + s0, l0, l1, acc)) {     // a null or infinite value: redo with null handling
-            acc.init();
-            for (uint32_t t = l0; t < l1; ++t) acc.add(A, list[s0 + t]);
-        }
-#pragma unroll 1
-        for (int d = 16; d > 0; d >>= 1) acc_merge_down(acc, d);
-        if (lane == 0) part[p] = acc;
+        const uint32_t *seg = list + s0 + b0;
+        const uint32_t m = b1 - b0, per = (m + 31) / 32, l0 = min(lane_id() * per, m);   // consecutive shares
+        piece_by_warp(A, [&](uint32_t t) { return seg[l0 + t]; }, min(l0 + per, m) - l0, S, part + p);
     }
+}
+static void launch_pieces(Ctx &c, const uint32_t *off, const uint32_t *list, const uint32_t *longs,
+                          const unsigned *nlong, const uint32_t *poff, const AggIn &in, Acc *part) {
+    cudaFuncSetAttribute(k_agg_pieces, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PC_SMEM);
+    launch(c, "agg_pieces", k_agg_pieces, dim3(4 * sm_count(c)), dim3(PC_THREADS), PC_SMEM, off, list, longs, nlong,
+           poff, in, part);
 }
 
 // Ops of more than lane_max and up to AG_MID_MAX kernels: a block each.  The
@@ -1211,9 +1308,7 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
                        (const uint32_t *)off, (const uint32_t *)longs, (const unsigned *)nlong, 2u,
                        0xFFFFFFFFu, list, tmp);
             }
-            launch(c, "agg_pieces", k_agg_pieces, dim3(4 * std::max(1, sms)), dim3(256), 0, (const uint32_t *)off,
-                   (const uint32_t *)list, (const uint32_t *)longs, (const unsigned *)nlong, (const uint32_t *)npc,
-                   in, partials);
+            launch_pieces(c, off, list, longs, nlong, npc, in, partials);
             launch(c, "agg_long_ops", k_agg_long_ops, dim3(2 * std::max(1, sms)), dim3(FIN_THREADS), 0,
                    (const uint32_t *)longs, (const unsigned *)nlong, (const uint32_t *)npc,
                    (const Acc *)partials, 0, in, c.d_status);
@@ -1294,6 +1389,116 @@ __global__ void k_class_keys(const int32_t *__restrict__ rok, const uint32_t *__
             if (h[i]) atomicAdd(&cnt[i], h[i]);
     }
 }
+// Few classes: the kernels grouped by class in one counting pass (kernel order
+// kept).  The class is read off the kernel's operator by the count, which keeps
+// it for the placing launch (CLASS_DIGIT: none).
+constexpr int CLASS_DIGIT = RADIX_BINS - 1;         // and the empty digit that ends the last class
+struct ClassDigit {
+    const int32_t *rok;
+    const uint32_t *r_op, *class_of_op;
+    int64_t R, n_ops;
+    uint32_t n_classes;
+    uint8_t *keep;
+    __device__ __forceinline__ unsigned operator()(int64_t k) const {
+        unsigned d = CLASS_DIGIT;
+        const int32_t r = range_of(rok, r_op, k);
+        if (r >= 0 && r < R) {
+            const uint32_t op = r_op[r];
+            if ((int64_t)op < n_ops) {
+                const uint32_t x = class_of_op[op];
+                if (x < n_classes) d = x;
+            }
+        }
+        keep[k] = (uint8_t)d;
+        return d < CLASS_DIGIT ? d : (unsigned)RADIX_BINS;
+    }
+};
+struct KeptDigit {
+    const uint8_t *keep;
+    __device__ __forceinline__ unsigned operator()(int64_t k) const {
+        const unsigned d = keep[k];
+        return d < CLASS_DIGIT ? d : (unsigned)RADIX_BINS;
+    }
+};
+struct PlaceByClass {
+    uint32_t *list;
+    __device__ __forceinline__ unsigned operator()(int64_t k, uint32_t dest, unsigned) const {
+        list[dest] = (uint32_t)k;
+        return 0u;
+    }
+    __device__ __forceinline__ void done(unsigned) const {}
+};
+// The classes over the warps of the summing pass (one block): class c's kernels
+// are list positions [off[c], off[c + 1]); it gets warps [first[c], first[c + 1]),
+// in proportion to its kernels and one at least.
+__global__ void __launch_bounds__(RADIX_BINS) k_class_warps(const uint32_t *__restrict__ offs, int64_t ntiles,
+                                                            int n_classes, uint32_t warps, uint32_t *__restrict__ off,
+                                                            uint32_t *__restrict__ first) {
+    pdl_wait();
+    __shared__ uint32_t wbuf[33];
+    const int c = threadIdx.x;
+    const uint32_t a = c <= n_classes ? offs[(int64_t)c * ntiles] : 0u;
+    const uint32_t z = c < n_classes ? offs[(int64_t)(c + 1) * ntiles] : a;
+    const unsigned long long all = offs[(int64_t)n_classes * ntiles];
+    const uint32_t share =
+        all ? (uint32_t)((unsigned long long)(z - a) * (warps - (uint32_t)n_classes) / all) : 0u;
+    const uint32_t ex = block_exclusive_scan<uint32_t>(c < n_classes ? share + 1 : 0u, wbuf, (uint32_t *)nullptr);
+    if (c <= n_classes) {
+        off[c] = a;
+        first[c] = ex;
+    }
+}
+// The classes' sums.  Warp i of a class's m takes every m-th group of 32
+// consecutive kernels of its list, so that all warps go through the kernel array
+// at one pace and the rows in flight are one band of it: neighbouring rows of
+// different classes share their 64-byte pieces of memory, and taken class by
+// class each of them was fetched again (220 bytes from memory per kernel).  One
+// partial per warp.
+//
+// Bound by issue (some 300 instructions per 32 kernels) and the rows' latency at
+// 16 warps per multiprocessor.  8M kernels in 64 classes: class by class in
+// pieces of 1,024 318 us, by windows of 32,768 kernels (as many partials as
+// windows times classes) 255 us, so 141 us.
+__global__ void __launch_bounds__(PC_THREADS, 2) k_class_sums(const uint32_t *__restrict__ off,
+                                                              const uint32_t *__restrict__ first, int n_classes,
+                                                              const uint32_t *__restrict__ list, AggIn A,
+                                                              Acc *__restrict__ part) {
+    pdl_wait();
+    extern __shared__ __align__(16) unsigned char ag_smem[];
+    PieceSlots &S = reinterpret_cast<PieceSlots *>(ag_smem)[threadIdx.x / 32];
+    const uint32_t g = (blockIdx.x * PC_THREADS + threadIdx.x) >> 5;
+    if (g >= first[n_classes]) return;
+    int c = 0, hi = n_classes;                    // the warp's class: last one with first <= g
+    while (hi - c > 1) {
+        const int m = (c + hi) >> 1;
+        if (first[m] <= g) c = m; else hi = m;
+    }
+    const uint32_t m = first[c + 1] - first[c], n = off[c + 1] - off[c], e0 = (g - first[c]) * 32 + lane_id();
+    const uint32_t *seg = list + off[c] + e0;
+    piece_by_warp(A, [&](uint32_t t) { return seg[(size_t)t * m * 32]; }, e0 < n ? (n - e0 + m * 32 - 1) / (m * 32) : 0u,
+                  S, part + g);
+}
+// One block per class merges its warps' partials: thread t takes t, t +
+// FIN_THREADS, ... in order, then the trees of k_agg_long_ops.
+__global__ void __launch_bounds__(FIN_THREADS) k_class_records(const uint32_t *__restrict__ first,
+                                                               const Acc *__restrict__ part, AggIn A, DevStatus *st) {
+    pdl_wait();
+    __shared__ Acc wpart[FIN_THREADS / 32];
+    const int c = blockIdx.x;
+    Acc acc;
+    acc.init();
+    for (uint32_t p = first[c] + threadIdx.x; p < first[c + 1]; p += FIN_THREADS) acc_merge(acc, part[p]);
+#pragma unroll 1
+    for (int d = 16; d > 0; d >>= 1) acc_merge_down(acc, d);
+    if (lane_id() == 0) wpart[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        Acc total = wpart[0];
+        for (int v = 1; v < FIN_THREADS / 32; ++v) acc_merge(total, wpart[v]);
+        total.write(A, c);
+        if (total.bad) set_err(st, ERR_INVALID);
+    }
+}
 __global__ void k_iota_u32(uint32_t *dst, int64_t n, unsigned *count) {
     pdl_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -1317,7 +1522,13 @@ opattr_status do_rollup(Ctx &c, const opattr_kernels *kern, const opattr_ranges 
         return OPATTR_E_INVALID_ARG;
     if ((reinterpret_cast<uintptr_t>(ncu->counters) & 15) != 0) return OPATTR_E_INVALID_ARG;
 
-    const int64_t maxp = K / AG_PIECE + C + 1;
+    // few classes: one counting pass, every warp of one wave for a share of one
+    // class; else a sort by class and pieces
+    const bool few = K > 0 && C > 0 && C <= CLASS_DIGIT;
+    const int sms = sm_count(c);
+    const unsigned sum_blocks = (unsigned)std::min<int64_t>(2 * sms, (K + 32 * 64 - 1) / (32 * 64) + C / 8 + 1);
+    const uint32_t sum_warps = sum_blocks * (PC_THREADS / 32);
+    const int64_t maxp = std::max<int64_t>(K / AG_PIECE + C + 1, sum_warps);
     Need nd;
     for (int i = 0; i < 4; ++i) nd.add<uint32_t>(K);
     nd.add<uint32_t>(radix_hist_elems(K)).add<uint32_t>(scan_scratch_elems(std::max(radix_hist_elems(K), C + 2)));
@@ -1339,17 +1550,28 @@ opattr_status do_rollup(Ctx &c, const opattr_kernels *kern, const opattr_ranges 
     if (O > 0)
         launch(c, "class_check", k_class_check, dim3(grid_for(O, 256, REDUCE_GRID)), dim3(256), 0, class_of_op, O,
                n_classes, c.d_status);
-    cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * (C + 2), c.stream);
     uint32_t *list = nullptr;
-    if (K > 0) {
+    if (few) {
+        uint8_t *keep = reinterpret_cast<uint8_t *>(v0);
+        const ClassDigit dg{rok, rng->op_id, class_of_op, R, O, n_classes, keep};
+        list = k0;
+        const uint32_t *offs = digit_offsets(c, dg, K, hist, part, (int)C + 1);
+        digit_rank(c, "class_place", KeptDigit{keep}, K, offs, PlaceByClass{list});
+        launch(c, "class_warps", k_class_warps, dim3(1), dim3(RADIX_BINS), 0, offs, (K + RADIX_TILE - 1) / RADIX_TILE,
+               (int)C, sum_warps, off, poff);
+    } else {
+        const ZeroRun z{cnt, C + 2};
+        if ((st = zero_runs(c, 1, &z))) return st;
+    }
+    if (K > 0 && !few) {
         launch(c, "class_keys", k_class_keys, dim3(grid_for(K, 256, REDUCE_GRID)), dim3(256), 0, rok, rng->op_id, K, R,
                O, class_of_op, n_classes, k0, cnt);
         uint32_t *ko;
         radix_sort_pairs<uint32_t>(c, k0, v0, k1, v1, K, bits_for((uint64_t)C), true, hist, part, &ko, &list);
     }
-    scan_exclusive_u32(c, cnt, off, C + 1, part, nullptr);           // off[C] = kernels with a class
+    if (!few) scan_exclusive_u32(c, cnt, off, C + 1, part, nullptr);   // off[C] = kernels with a class
     if (C > 0) {
-        AggIn in;
+        AggIn in{};
         in.dur = kern->dur_ns;
         in.ncu_idx = nidx;
         in.counters = ncu->counters;
@@ -1362,18 +1584,20 @@ opattr_status do_rollup(Ctx &c, const opattr_kernels *kern, const opattr_ranges 
         in.longs = nullptr;
         in.nonident = nullptr;
         in.out = *out;
-        int sms = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device);
-        launch(c, "class_iota", k_iota_u32, dim3(grid_for(C, 256, 4096)), dim3(256), 0, cls, C, ncls);
-        launch(c, "agg_piece_offsets", k_agg_piece_offsets, dim3(1), dim3(1024), 0, (const uint32_t *)off,
-               (const uint32_t *)cls, (const unsigned *)ncls, 0u, poff, (uint32_t *)nullptr, (uint32_t *)nullptr);
-        if (K > 0)
-            launch(c, "agg_pieces", k_agg_pieces, dim3(4 * std::max(1, sms)), dim3(256), 0, (const uint32_t *)off,
-                   (const uint32_t *)list, (const uint32_t *)cls, (const unsigned *)ncls, (const uint32_t *)poff, in,
-                   partials);
-        launch(c, "class_records", k_agg_long_ops, dim3(2 * std::max(1, sms)), dim3(FIN_THREADS), 0,
-               (const uint32_t *)cls,
-               (const unsigned *)ncls, (const uint32_t *)poff, (const Acc *)partials, 1, in, c.d_status);
+        if (few) {
+            cudaFuncSetAttribute(k_class_sums, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PC_SMEM);
+            launch(c, "class_sums", k_class_sums, dim3(sum_blocks), dim3(PC_THREADS), PC_SMEM, (const uint32_t *)off,
+                   (const uint32_t *)poff, (int)C, (const uint32_t *)list, in, partials);
+            launch(c, "class_records", k_class_records, dim3((unsigned)C), dim3(FIN_THREADS), 0,
+                   (const uint32_t *)poff, (const Acc *)partials, in, c.d_status);
+        } else {
+            launch(c, "class_iota", k_iota_u32, dim3(grid_for(C, 256, 4096)), dim3(256), 0, cls, C, ncls);
+            launch(c, "agg_piece_offsets", k_agg_piece_offsets, dim3(1), dim3(1024), 0, (const uint32_t *)off,
+                   (const uint32_t *)cls, (const unsigned *)ncls, 0u, poff, (uint32_t *)nullptr, (uint32_t *)nullptr);
+            if (K > 0) launch_pieces(c, off, list, cls, ncls, poff, in, partials);
+            launch(c, "class_records", k_agg_long_ops, dim3(2 * sms), dim3(FIN_THREADS), 0, (const uint32_t *)cls,
+                   (const unsigned *)ncls, (const uint32_t *)poff, (const Acc *)partials, 1, in, c.d_status);
+        }
     }
     if ((st = read_status(c))) return st;
     if (c.h_status->err & ERR_INVALID) return OPATTR_E_INVALID_ARG;
