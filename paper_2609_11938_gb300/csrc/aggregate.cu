@@ -199,28 +199,30 @@ struct Acc {
 
 // The common case, without per-value tests: a null (NaN) or infinite value
 // anywhere poisons a sum, and the op is then done again with Acc, which
-// handles nulls and flags infinities.  MAX values also enter a plain sum for
-// that test.  Every counter of every matched kernel is non-null here, so a
-// counter is defined iff some kernel matched, and the DW weight is dall.
+// handles nulls and flags infinities.  Every counter of every matched kernel is
+// non-null here, so a counter is defined iff some kernel matched, and the DW
+// weight is dall.
+//
+// Counters go two to a register through the packed fp32 instructions (97M warp
+// instructions for 4M kernels against 152M), neighbours as they lie in the row: a pair of DW counters weighs the duration, SUM beside
+// DW weighs (1, duration) -- exact, 1 * x + 0 -- and the two MAX counters ride
+// along as probes (their sums are not used; should one overflow, the op is done
+// again like any with an infinite value).
 struct AccF {
+    static constexpr int PAIRS = NC / 2;
     int mc;
     long long dsum, dall;
-    ff s[N_SUM];
-    ff w[N_DW];
+    f32x2 hi[PAIRS], lo[PAIRS];     // counters 2p, 2p + 1: float-float sums
     float mx[N_MAX];
-    float probe;                // sum of the MAX values: non-finite iff one was
     int terms;
 
     __device__ __forceinline__ void init() {
         mc = 0;
         dsum = dall = 0;
 #pragma unroll
-        for (int i = 0; i < N_SUM; ++i) s[i] = ff{0.f, 0.f};
-#pragma unroll
-        for (int i = 0; i < N_DW; ++i) w[i] = ff{0.f, 0.f};
+        for (int p = 0; p < PAIRS; ++p) hi[p] = lo[p] = 0ull;
 #pragma unroll
         for (int i = 0; i < N_MAX; ++i) mx[i] = -INFINITY;
-        probe = 0.f;
         terms = 0;
     }
 
@@ -229,46 +231,44 @@ struct AccF {
         if (!matched) return;
         mc++;
         dall += d;
-        float v[NC];
+        f32x2 v[PAIRS];
 #pragma unroll
         for (int q = 0; q < NC / 4; ++q) {
-            const float4 x = row[q];
-            v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
+            const ulonglong2 x = reinterpret_cast<const ulonglong2 *>(row)[q];
+            v[2 * q] = x.x;
+            v[2 * q + 1] = x.y;
         }
         const ff dd = split_dur(d);
+        const f32x2 dw = f2_pack(dd.hi, dd.hi), dn = f2_pack(-dd.hi, -dd.hi), dl = f2_pack(dd.lo, dd.lo);
+        const f32x2 sw = f2_pack(1.f, dd.hi), sn = f2_pack(-1.f, -dd.hi), sl = f2_pack(0.f, dd.lo);
 #pragma unroll
-        for (int i = 0; i < N_SUM; ++i) {
-            const ff t = two_sum(s[i].hi, v[Acc::sum_col(i)]);
-            s[i].hi = t.hi;
-            s[i].lo = __fadd_rn(s[i].lo, t.lo);
+        for (int p = 0; p < PAIRS; ++p) {
+            if (p == 0 || p == 9) f2_accum(hi[p], lo[p], v[p]);                                     // SUM SUM, SUM MAX
+            else if (p == 1 || p == 5 || p == 7) f2_accum_mul(hi[p], lo[p], v[p], sw, sn, sl);      // SUM DW
+            else f2_accum_mul(hi[p], lo[p], v[p], dw, dn, dl);                                      // DW DW, DW MAX
         }
 #pragma unroll
-        for (int i = 0; i < N_DW; ++i) {
-            const ff p = mul_split(v[Acc::dw_col(i)], dd);
-            ff_accum(w[i], p.hi, p.lo);
-        }
-#pragma unroll
-        for (int i = 0; i < N_MAX; ++i) {
-            mx[i] = fmaxf(mx[i], v[Acc::max_col(i)]);
-            probe = __fadd_rn(probe, v[Acc::max_col(i)]);
-        }
+        for (int i = 0; i < N_MAX; ++i) mx[i] = fmaxf(mx[i], f2_unpack(v[Acc::max_col(i) / 2]).y);
         if (++terms >= RENORM) {
             terms = 0;
 #pragma unroll
-            for (int i = 0; i < N_SUM; ++i) ff_renorm(s[i]);
-#pragma unroll
-            for (int i = 0; i < N_DW; ++i) ff_renorm(w[i]);
+            for (int p = 0; p < PAIRS; ++p) f2_renorm(hi[p], lo[p]);
         }
+    }
+
+    // counter c's sum
+    __device__ __forceinline__ ff sum(int c) const {
+        const float2 h = f2_unpack(hi[c / 2]), l = f2_unpack(lo[c / 2]);
+        return c & 1 ? ff{h.y, l.y} : ff{h.x, l.x};
     }
 
     // True when no null or infinite value took part (then write() is exact to spec).
     __device__ __forceinline__ bool clean() const {
-        float z = __fmul_rn(probe, 0.f);
+        f32x2 z = 0ull;
 #pragma unroll
-        for (int i = 0; i < N_SUM; ++i) z = __fmaf_rn(__fadd_rn(s[i].hi, s[i].lo), 0.f, z);
-#pragma unroll
-        for (int i = 0; i < N_DW; ++i) z = __fmaf_rn(__fadd_rn(w[i].hi, w[i].lo), 0.f, z);
-        return z == 0.f;
+        for (int p = 0; p < PAIRS; ++p) z = f2_fma(f2_add(hi[p], lo[p]), 0ull, z);
+        const float2 r = f2_unpack(z);
+        return __fadd_rn(r.x, r.y) == 0.f;
     }
 
     __device__ __forceinline__ void write(const AggIn &A, int64_t op, int kc) const {
@@ -286,14 +286,15 @@ struct AccF {
         }
 #pragma unroll
         for (int i = 0; i < N_SUM; ++i) {
-            ff x = s[i];
+            ff x = sum(Acc::sum_col(i));
             ff_renorm(x);
             agg[(int64_t)Acc::sum_col(i) * n + op] = ff_to_f64_fast(x);
         }
         if (dall > 0) {
             const ff rcp = ff_recip_i64(dall);
 #pragma unroll
-            for (int i = 0; i < N_DW; ++i) agg[(int64_t)Acc::dw_col(i) * n + op] = ff_mul_to_f64(w[i], rcp);
+            for (int i = 0; i < N_DW; ++i)
+                agg[(int64_t)Acc::dw_col(i) * n + op] = ff_mul_to_f64(sum(Acc::dw_col(i)), rcp);
         } else {
 #pragma unroll
             for (int i = 0; i < N_DW; ++i) agg[(int64_t)Acc::dw_col(i) * n + op] = qnan;
@@ -542,11 +543,16 @@ constexpr int AG_THREADS = 128;
 constexpr int AG_WARPS = AG_THREADS / 32;
 constexpr int AG_CHUNK = 64;                    // op ids per warp and chunk
 constexpr int AG_LBUCKETS = 32;
+// Four blocks of four warps per multiprocessor: with the 96 registers of five
+// the accumulators spill (730 us on 20M kernels, 446 on 6M whose records were out
+// of order; four blocks 696 and 343; three 748 and 380).  Four slots gave 718 and
+// 434, chunks of 128 ops 888 and 466.
+constexpr int AG_SLOTS = 2, AG_BLOCKS = 4;
 constexpr int AG_STAGE = 1024;                  // list entries of a chunk staged in shared memory
 
 struct OpsWarp {
-    float4 row[2][32][NC / 4];      // two kernels in flight per thread: counter rows
-    long long dur[2][32];           // and durations, by asynchronous copy
+    float4 row[AG_SLOTS][32][NC / 4];      // kernels in flight per thread: counter rows
+    long long dur[AG_SLOTS][32];           // and durations, by asynchronous copy
     uint32_t L[AG_STAGE];           // the chunk's list run (when it fits)
     uint32_t lcount[AG_LBUCKETS];
     uint8_t order[AG_CHUNK];
@@ -619,7 +625,7 @@ __device__ __forceinline__ void cp_async_rows(float4 (*dst)[NC / 4], const float
     }
 }
 
-__global__ void __launch_bounds__(AG_THREADS, 5) k_agg_ops(const uint32_t *__restrict__ off, uint32_t *list,
+__global__ void __launch_bounds__(AG_THREADS, AG_BLOCKS) k_agg_ops(const uint32_t *__restrict__ off, uint32_t *list,
                                                           AggIn A, int pending, const DevStatus *st) {
     pdl_wait();
     if (pending && stopped(st)) return;
@@ -712,42 +718,42 @@ __global__ void __launch_bounds__(AG_THREADS, 5) k_agg_ops(const uint32_t *__res
                 const uint32_t xb = __shfl_sync(0xffffffffu, ob[q], il & 31);
                 if ((il >> 5) == q) { sa = xa; sb = xb; }
             }
-            if (i >= nchunk) continue;
             const int64_t o = o0 + il;
-            const uint32_t s0 = sa, len = sb - sa;
-            if (len > A.lane_max) continue;                       // listed
+            const bool mine = i < nchunk && sb - sa <= A.lane_max;             // (longer ones are listed)
+            const uint32_t s0 = sa, len = mine ? sb - sa : 0u;
+            const uint32_t most = __reduce_max_sync(0xffffffffu, len);         // the lanes copy rows together
             const uint32_t *seg = staged ? W.L + (s0 - cbase) : list + s0;
             AccF acc;
             acc.init();
-            if (len > 0) {
-                // kernel t's row and duration land in slot t & 1 while kernel
-                // t - 1 is added; row indices are loaded one step further ahead
+            if (most > 0) {
+                // kernel t's row and duration land in slot t % AG_SLOTS while the
+                // kernels before it are added; row indices are loaded one step
+                // further ahead
                 auto issue = [&](uint32_t t, uint32_t k, int32_t j) {
-                    if (t < len) {
-                        cp_async8(&W.dur[t & 1][lane], A.dur + k);
-                        if (j >= 0) {
-                            const float4 *src = rows + (int64_t)j * (NC / 4);
-#pragma unroll
-                            for (int c = 0; c < NC / 4; ++c) cp_async16(&W.row[t & 1][lane][c], src + c);
-                        }
-                    }
+                    if (t < len) cp_async8(&W.dur[t % AG_SLOTS][lane], A.dur + k);
+                    cp_async_rows(W.row[t % AG_SLOTS], rows, j);
                     cp_async_commit();
                 };
-                const uint32_t k0 = seg[0], k1 = len > 1 ? seg[1] : 0u;
-                const int32_t j0 = row_of(k0), j1 = len > 1 ? row_of(k1) : -1;
-                uint32_t k2 = len > 2 ? seg[2] : 0u;
-                int32_t j2 = len > 2 ? row_of(k2) : -1;
-                issue(0, k0, j0);
-                issue(1, k1, j1);
-                int32_t js0 = j0, js1 = j1;           // row index of the kernel in each slot
-                for (uint32_t t = 0; t < len; ++t) {
-                    const uint32_t k3 = t + 3 < len ? seg[t + 3] : 0u;
-                    const int32_t j3 = t + 3 < len ? row_of(k3) : -1;
-                    cp_async_wait<1>();
-                    const int32_t j = (t & 1) ? js1 : js0;
-                    acc.accumulate(W.dur[t & 1][lane], j >= 0, W.row[t & 1][lane]);
-                    issue(t + 2, k2, j2);
-                    if (t & 1) js1 = j2; else js0 = j2;
+                unsigned have = 0;                    // bit t % AG_SLOTS: the kernel in that slot has a row
+#pragma unroll
+                for (uint32_t t = 0; t < (uint32_t)AG_SLOTS; ++t) {
+                    const uint32_t kt = t < len ? seg[t] : 0u;
+                    const int32_t jt = t < len ? row_of(kt) : -1;
+                    issue(t, kt, jt);
+                    have |= (jt >= 0 ? 1u : 0u) << t;
+                }
+                uint32_t k2 = AG_SLOTS < len ? seg[AG_SLOTS] : 0u;
+                int32_t j2 = AG_SLOTS < len ? row_of(k2) : -1;
+                for (uint32_t t = 0; t < most; ++t) {
+                    const uint32_t k3 = t + AG_SLOTS + 1 < len ? seg[t + AG_SLOTS + 1] : 0u;
+                    const int32_t j3 = t + AG_SLOTS + 1 < len ? row_of(k3) : -1;
+                    cp_async_wait<AG_SLOTS - 1>();
+                    __syncwarp();
+                    const unsigned bit = 1u << (t % AG_SLOTS);
+                    if (t < len) acc.accumulate(W.dur[t % AG_SLOTS][lane], have & bit, W.row[t % AG_SLOTS][lane]);
+                    __syncwarp();
+                    issue(t + AG_SLOTS, k2, j2);
+                    have = j2 >= 0 ? have | bit : have & ~bit;
                     k2 = k3;
                     j2 = j3;
                 }
@@ -755,6 +761,7 @@ __global__ void __launch_bounds__(AG_THREADS, 5) k_agg_ops(const uint32_t *__res
             }
             // a null or infinite value poisons a sum: the op is listed for
             // k_agg_careful
+            if (!mine) continue;
             if (acc.clean()) acc.write(A, o, (int)len);
             else A.dirty[atomicAdd(A.ctr + 1, 1u)] = (uint32_t)o;
         }
@@ -942,10 +949,10 @@ __device__ __forceinline__ void acc_from_fast(Acc &out, const AccF &f, int kc) {
     out.dsum = f.dsum;
     out.dall = f.dall;
 #pragma unroll
-    for (int i = 0; i < N_SUM; ++i) out.s[i] = f.s[i];
+    for (int i = 0; i < N_SUM; ++i) out.s[i] = f.sum(Acc::sum_col(i));
 #pragma unroll
     for (int i = 0; i < N_DW; ++i) {
-        out.w[i] = f.w[i];
+        out.w[i] = f.sum(Acc::dw_col(i));
         out.nanw[i] = 0;
     }
 #pragma unroll

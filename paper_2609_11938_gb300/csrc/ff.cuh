@@ -30,6 +30,62 @@ __device__ __forceinline__ ff two_sum(float a, float b) {
     float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
     return ff{s, e};
 }
+// Two floats in one 64-bit register (x the low half), under the packed fp32
+// instructions: two roundings to nearest per issue slot.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 f2_pack(float x, float y) {
+    f32x2 v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+    return v;
+}
+__device__ __forceinline__ float2 f2_unpack(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 f2_sub(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// hi + lo += x, both halves: two_sum into hi, its error into lo
+__device__ __forceinline__ void f2_accum(f32x2 &hi, f32x2 &lo, f32x2 x) {
+    const f32x2 s = f2_add(hi, x), bb = f2_sub(s, hi);
+    const f32x2 e = f2_add(f2_sub(hi, f2_sub(s, bb)), f2_sub(x, bb));
+    hi = s;
+    lo = f2_add(lo, e);
+}
+// hi + lo += m * (w + wl) for nw = -w: mul_split and ff_accum on both halves,
+// with the product carried as its negative (every rounding is symmetric)
+__device__ __forceinline__ void f2_accum_mul(f32x2 &hi, f32x2 &lo, f32x2 m, f32x2 w, f32x2 nw, f32x2 wl) {
+    const f32x2 np = f2_mul(m, nw);
+    const f32x2 pl = f2_fma(m, wl, f2_fma(m, w, np));
+    const f32x2 s = f2_sub(hi, np), bb = f2_sub(s, hi);
+    const f32x2 e = f2_sub(f2_sub(hi, f2_sub(s, bb)), f2_add(np, bb));
+    hi = s;
+    lo = f2_add(lo, f2_add(e, pl));
+}
+__device__ __forceinline__ void f2_renorm(f32x2 &hi, f32x2 &lo) {
+    const f32x2 s = f2_add(hi, lo), bb = f2_sub(s, hi);
+    lo = f2_add(f2_sub(hi, f2_sub(s, bb)), f2_sub(lo, bb));
+    hi = s;
+}
+
 // s + e == a + b exactly when |a| >= |b| or a == 0 (Dekker fast two-sum)
 __device__ __forceinline__ ff fast_two_sum(float a, float b) {
     float s = __fadd_rn(a, b);
