@@ -71,7 +71,10 @@ class MatchSummary(ctypes.Structure):
                [("fast_path", ctypes.c_int32), ("reserved", ctypes.c_int32)]
 
     def as_dict(self) -> dict:
-        return {f: int(getattr(self, f)) for f, _ in self._fields_ if f != "reserved"}
+        return {"kernels": self.kernels, "replayed": self.replayed, "direct": self.direct, "broadcast": self.broadcast,
+                "unmatched": self.unmatched, "names_mismatched": self.names_mismatched,
+                "count_unmatched": self.count_unmatched, "dedup_mismatch": self.dedup_mismatch,
+                "fast_path": self.fast_path}
 
 
 class Corr(ctypes.Structure):
@@ -109,7 +112,10 @@ class Totals(ctypes.Structure):
                [("attributed_frac", ctypes.c_double), ("unattributed_frac", ctypes.c_double)]
 
     def as_dict(self) -> dict:
-        return {f: getattr(self, f) for f, _ in self._fields_}
+        return {"total_ns": self.total_ns, "attributed_ns": self.attributed_ns, "unattributed_ns": self.unattributed_ns,
+                "kernels": self.kernels, "attributed_kernels": self.attributed_kernels,
+                "matched_kernels": self.matched_kernels, "attributed_frac": self.attributed_frac,
+                "unattributed_frac": self.unattributed_frac}
 
 
 _lib_lock = threading.Lock()
@@ -189,48 +195,48 @@ def opattr_create(device: int = 0, stream: int | None = None, mismatch: str = "s
 
 
 def opattr_enclose(handle, kernels: Kernels, ranges: Ranges, range_of_kernel_ptr: int, n_op_ptr: int | None) -> int:
-    return library().opattr_enclose(handle, ctypes.byref(kernels), ctypes.byref(ranges), _vp(range_of_kernel_ptr),
-                                    _vp(n_op_ptr or 0))
+    return (_lib or library()).opattr_enclose(handle, ctypes.byref(kernels), ctypes.byref(ranges), range_of_kernel_ptr,
+                                              n_op_ptr)
 
 
 def opattr_match(handle, kernels: Kernels, ncu: Ncu, dedup: Dedup | None, idx_ptr: int, kind_ptr: int | None,
                  summary: MatchSummary) -> int:
-    return library().opattr_match(handle, ctypes.byref(kernels), ctypes.byref(ncu),
-                                  ctypes.byref(dedup) if dedup is not None else None, _vp(idx_ptr),
-                                  _vp(kind_ptr or 0), ctypes.byref(summary))
+    return (_lib or library()).opattr_match(handle, ctypes.byref(kernels), ctypes.byref(ncu),
+                                            ctypes.byref(dedup) if dedup is not None else None, idx_ptr,
+                                            kind_ptr, ctypes.byref(summary))
 
 
 def opattr_aggregate(handle, kernels: Kernels, ranges: Ranges, rok_ptr: int, ncu: Ncu, idx_ptr: int, n_ops: int,
                      out: OpAggregates, totals: Totals) -> int:
-    return library().opattr_aggregate(handle, ctypes.byref(kernels), ctypes.byref(ranges), _vp(rok_ptr),
-                                      ctypes.byref(ncu), _vp(idx_ptr), ctypes.c_uint32(n_ops), ctypes.byref(out),
-                                      ctypes.byref(totals))
+    return (_lib or library()).opattr_aggregate(handle, ctypes.byref(kernels), ctypes.byref(ranges), rok_ptr,
+                                                ctypes.byref(ncu), idx_ptr, ctypes.c_uint32(n_ops), ctypes.byref(out),
+                                                ctypes.byref(totals))
 
 
 def opattr_join(handle, kernels: Kernels, ranges: Ranges, ncu: Ncu, dedup: Dedup | None, n_ops: int, rok_ptr: int,
                 nop_ptr: int | None, idx_ptr: int, kind_ptr: int | None, out: OpAggregates, summary: MatchSummary,
                 totals: Totals) -> int:
-    return library().opattr_join(handle, ctypes.byref(kernels), ctypes.byref(ranges), ctypes.byref(ncu),
-                                 ctypes.byref(dedup) if dedup is not None else None, ctypes.c_uint32(n_ops),
-                                 _vp(rok_ptr), _vp(nop_ptr or 0), _vp(idx_ptr), _vp(kind_ptr or 0), ctypes.byref(out),
-                                 ctypes.byref(summary), ctypes.byref(totals))
+    return (_lib or library()).opattr_join(handle, ctypes.byref(kernels), ctypes.byref(ranges), ctypes.byref(ncu),
+                                           ctypes.byref(dedup) if dedup is not None else None, ctypes.c_uint32(n_ops),
+                                           rok_ptr, nop_ptr, idx_ptr, kind_ptr, ctypes.byref(out),
+                                           ctypes.byref(summary), ctypes.byref(totals))
 
 
 def opattr_attribute(handle, kernels: Kernels, ranges: Ranges, rok_ptr: int, nop_ptr: int | None,
                      corr: Corr | None, fusion: Fusion | None, n_ops: int, op_ptr: int, tier_ptr: int | None,
                      fused_with_ptr: int | None, is_fused_ptr: int | None, summary: AttrSummary) -> int:
-    return library().opattr_attribute(handle, ctypes.byref(kernels), ctypes.byref(ranges), _vp(rok_ptr),
-                                      _vp(nop_ptr or 0), ctypes.byref(corr) if corr is not None else None,
-                                      ctypes.byref(fusion) if fusion is not None else None, ctypes.c_uint32(n_ops),
-                                      _vp(op_ptr), _vp(tier_ptr or 0), _vp(fused_with_ptr or 0),
-                                      _vp(is_fused_ptr or 0), ctypes.byref(summary))
+    return (_lib or library()).opattr_attribute(handle, ctypes.byref(kernels), ctypes.byref(ranges), rok_ptr,
+                                                nop_ptr, ctypes.byref(corr) if corr is not None else None,
+                                                ctypes.byref(fusion) if fusion is not None else None,
+                                                ctypes.c_uint32(n_ops), op_ptr, tier_ptr, fused_with_ptr, is_fused_ptr,
+                                                ctypes.byref(summary))
 
 
 def opattr_rollup(handle, kernels: Kernels, ranges: Ranges, rok_ptr: int | None, ncu: Ncu, idx_ptr: int, n_ops: int,
                   class_ptr: int, n_classes: int, out: OpAggregates) -> int:
-    return library().opattr_rollup(handle, ctypes.byref(kernels), ctypes.byref(ranges), _vp(rok_ptr or 0),
-                                   ctypes.byref(ncu), _vp(idx_ptr), ctypes.c_uint32(n_ops), _vp(class_ptr),
-                                   ctypes.c_uint32(n_classes), ctypes.byref(out))
+    return (_lib or library()).opattr_rollup(handle, ctypes.byref(kernels), ctypes.byref(ranges), rok_ptr,
+                                             ctypes.byref(ncu), idx_ptr, ctypes.c_uint32(n_ops), class_ptr,
+                                             ctypes.c_uint32(n_classes), ctypes.byref(out))
 
 
 def write_profile(path: str, k_stream, k_dur, k_name, op_of_kernel, ncu_idx, counters, ops: dict, tier=None,
@@ -306,9 +312,15 @@ def _ptr(t, dtype, name, device):
     return t.data_ptr() if t.numel() else None
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 @dataclass
@@ -376,6 +388,7 @@ class Context:
                  spin_limit: int = 0):
         import torch
         self.device = device
+        self._dev = torch.device("cuda", device)
         if stream is None:
             stream = torch.cuda.current_stream(device)
         self.stream = stream
@@ -402,29 +415,29 @@ class Context:
 
     # -- structs
     def kernels(self, tr: DeviceTrace) -> Kernels:
-        import torch
+        torch = _torch()
         dv = self.device
         return Kernels(_ptr(tr.k_stream, torch.uint8, "k_stream", dv), _ptr(tr.k_start, torch.int64, "k_start", dv),
                        _ptr(tr.k_dur, torch.int64, "k_dur", dv), _ptr(tr.k_name, torch.uint32, "k_name", dv),
                        _ptr(tr.k_layer, torch.int32, "k_layer", dv), tr.K)
 
     def ranges(self, tr: DeviceTrace) -> Ranges:
-        import torch
+        torch = _torch()
         dv = self.device
         return Ranges(_ptr(tr.r_stream, torch.uint8, "r_stream", dv), _ptr(tr.r_start, torch.int64, "r_start", dv),
                       _ptr(tr.r_end, torch.int64, "r_end", dv), _ptr(tr.r_depth, torch.uint8, "r_depth", dv),
                       _ptr(tr.r_op, torch.uint32, "r_op", dv), tr.R)
 
     def ncu(self, tr: DeviceTrace) -> Ncu:
-        import torch
+        torch = _torch()
         dv = self.device
         return Ncu(_ptr(tr.ncu_name, torch.uint32, "ncu_name", dv), _ptr(tr.counters, torch.float32, "counters", dv),
                    tr.M, _ptr(tr.ncu_stream, torch.uint8, "ncu_stream", dv))
 
     # -- calls
     def enclose(self, tr: DeviceTrace, out_range=None, out_nop=None, need_nop: bool = True):
-        import torch
-        dev = f"cuda:{self.device}"
+        torch = _torch()
+        dev = self._dev
         if out_range is None:
             out_range = torch.empty(tr.K, dtype=torch.int32, device=dev)
         if out_nop is None and need_nop:
@@ -449,8 +462,8 @@ class Context:
                      len(roc)), (col, roc)
 
     def match(self, tr: DeviceTrace, dedup: bool | None = None, out_idx=None, out_kind=None):
-        import torch
-        dev = f"cuda:{self.device}"
+        torch = _torch()
+        dev = self._dev
         if out_idx is None:
             out_idx = torch.empty(tr.K, dtype=torch.int32, device=dev)
         if out_kind is None:
@@ -469,8 +482,8 @@ class Context:
         """enclose + match + aggregate in one call (opattr_join).  `out` may hold
         preallocated range_of_kernel / n_op_enclosing / ncu_idx / match_kind
         tensors; returns (status, out, ops, match summary, totals)."""
-        import torch
-        dev = f"cuda:{self.device}"
+        torch = _torch()
+        dev = self._dev
         dv = self.device
         out = dict(out or {})
         for k, dt in (("range_of_kernel", torch.int32), ("n_op_enclosing", torch.uint8), ("ncu_idx", torch.int32),
@@ -496,8 +509,8 @@ class Context:
         return st, out, ops, summ.as_dict(), tot.as_dict()
 
     def alloc_ops(self, n_ops: int):
-        import torch
-        dev = f"cuda:{self.device}"
+        torch = _torch()
+        dev = self._dev
         return dict(kernel_count=torch.empty(n_ops, dtype=torch.int64, device=dev),
                     total_duration_ns=torch.empty(n_ops, dtype=torch.int64, device=dev),
                     matched_count=torch.empty(n_ops, dtype=torch.int64, device=dev),
@@ -506,9 +519,9 @@ class Context:
     def attribute(self, tr: DeviceTrace, range_of_kernel, n_op_enclosing=None, use_corr: bool = True,
                   use_fusion: bool = True, out=None):
         """The attribution tiers of Fig. 2: returns (status, op_of_kernel, tier, fused_with, is_fused, summary)."""
-        import torch
+        torch = _torch()
         dv = self.device
-        dev = f"cuda:{dv}"
+        dev = self._dev
         if out is None:
             out = dict(op=torch.empty(tr.K, dtype=torch.int32, device=dev),
                        tier=torch.empty(tr.K, dtype=torch.uint8, device=dev),
@@ -536,7 +549,7 @@ class Context:
     def aggregate(self, tr: DeviceTrace, range_of_kernel, ncu_idx, ops=None, op_of_kernel=None):
         """Eq. (1) per operator.  With op_of_kernel (opattr_attribute's output)
         in place of range_of_kernel, each kernel's operator is taken from it."""
-        import torch
+        torch = _torch()
         if ops is None:
             ops = self.alloc_ops(tr.n_ops)
         dv = self.device
@@ -560,7 +573,7 @@ class Context:
     def rollup(self, tr: DeviceTrace, range_of_kernel, ncu_idx, class_of_op, n_classes: int, out=None,
                op_of_kernel=None):
         """Per-class records (opattr_rollup); class_of_op: int32/uint32 device tensor of n_ops entries."""
-        import torch
+        torch = _torch()
         if out is None:
             out = self.alloc_ops(n_classes)
         dv = self.device
