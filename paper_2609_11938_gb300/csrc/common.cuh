@@ -64,7 +64,7 @@ struct DevStatus {
     long long mm[MM_NSLOTS];
     unsigned int kstreams[8];    // streams with kernels, one bit each (the enclosure's checks)
     unsigned int nlevels;        // range levels present (the enclosure)
-    unsigned int pad;
+    unsigned int nstreams;       // and streams with ranges
 };
 
 // ------------------------------------------------------------------ context

@@ -358,27 +358,30 @@ __global__ void __launch_bounds__(1024) k_enc_carry(uint32_t *__restrict__ rows,
 // entries, E_NONE none.
 constexpr unsigned E_NONE = 0xFFFFu;
 constexpr unsigned D_DEPTH = 31u, D_MIXED = 32u;     // bits of `dep`
-template <int THREADS_, int BLOCKS_, int RW_, int RPT_>
+template <int THREADS_, int BLOCKS_>
 struct EncTile {
-    static constexpr int THREADS = THREADS_, BLOCKS = BLOCKS_, RW = RW_, RPT = RPT_;
-    static constexpr int SR = RW * 32 * RPT;         // ranges of a step at most
-    static constexpr int WORDS = SR / 32;
+    static constexpr int THREADS = THREADS_, BLOCKS = BLOCKS_;
+    static constexpr int WORDS = 16;                 // ranges of a step, 32 to a group
+    static constexpr int SR = 32 * WORDS;
+    static constexpr int RPT = WORDS / (THREADS / 32);   // groups of a warp
     uint32_t *ss, *se, *si;      // start, end (relative), position | kind << 30
     uint32_t *re;                // end of the outermost ancestor
     uint32_t *amask;             // [ns] depths with an open range, per compact stream
     uint32_t *smask;             // [ns][WORDS] the stream's ranges among the tile's, one bit each
+    uint32_t *sgroups;           // [ns] the groups that hold some
     uint16_t *par, *prev, *best; // parent; the entry before on the stream; where the climb begins (below)
     uint16_t *va;                // innermost operator of the entry's chain
-    uint16_t *last;              // [RW + 1][nl] last range of each level in a warp's run, index + 1; then in
-                                 // the runs before it, and at last in all
-    uint16_t *swords;            // [ns] which words of smask are not empty
-    uint16_t *dopen;             // [ns] deepest open range, E_NONE none
+    uint16_t *before;            // [ns][WORDS] the stream's last entry before each group (before the first one
+                                 // its deepest open range), E_NONE none
+    uint32_t *lgroups;           // [nl / 2] the groups that hold ranges of a level, 16 bits each
+    uint8_t *last;               // [WORDS][nl] last range of each level in such a group
     uint16_t *cbase;             // [256] first level of a stream
     uint16_t *scid;              // [256] compact id of a stream (streams with levels, in order), E_NONE none
     uint8_t *dep, *vn;           // depth | D_MIXED; operators in the chain
-    uint8_t *sid;                // compact stream
+    uint8_t *sid;                // compact stream of the tile's ranges
     uint8_t *ndep;               // [256] levels of a stream
     uint8_t *slist;              // [256] the stream of a compact id
+    uint8_t *tlist;              // [ns] the streams that have ranges in the tile
     __device__ __forceinline__ EncTile(unsigned char *p, int nl, int ns) {
         const int cap = SR + nl;
         auto take = [&](size_t n) { unsigned char *q = p; p += n; return q; };
@@ -388,27 +391,29 @@ struct EncTile {
         re = reinterpret_cast<uint32_t *>(take((size_t)cap * 4));
         amask = reinterpret_cast<uint32_t *>(take((size_t)ns * 4));
         smask = reinterpret_cast<uint32_t *>(take((size_t)ns * WORDS * 4));
+        sgroups = reinterpret_cast<uint32_t *>(take((size_t)ns * 4));
+        lgroups = reinterpret_cast<uint32_t *>(take((size_t)nl * 2));
         par = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
         prev = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
         best = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
         va = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
-        last = reinterpret_cast<uint16_t *>(take((size_t)(RW + 1) * nl * 2));
-        swords = reinterpret_cast<uint16_t *>(take((size_t)ns * 2));
-        dopen = reinterpret_cast<uint16_t *>(take((size_t)ns * 2));
+        before = reinterpret_cast<uint16_t *>(take((size_t)ns * WORDS * 2));
         cbase = reinterpret_cast<uint16_t *>(take(512));
         scid = reinterpret_cast<uint16_t *>(take(512));
         dep = take(cap);
         vn = take(cap);
-        sid = take(cap);
+        sid = take(SR);
         ndep = take(256);
         slist = take(256);
+        tlist = take(ns);
+        last = take((size_t)WORDS * nl);
     }
     static size_t smem(int nl, int ns) {
-        return (size_t)(SR + nl) * 27 + (size_t)(RW + 1) * nl * 2 + (size_t)ns * (4 + 4 * WORDS + 4) + 1024 + 512;
+        return (size_t)(SR + nl) * 26 + SR + (size_t)(WORDS + 2) * nl + (size_t)ns * (8 + 6 * WORDS + 1) + 1024 + 512;
     }
 };
-using EncTileA = EncTile<256, 4, 8, 2>;
-using EncTileB = EncTile<512, 2, 4, 4>;
+using EncTileA = EncTile<256, 4>;
+using EncTileB = EncTile<512, 2>;
 constexpr int EN_LEVELS_A = 512, EN_STREAMS_A = 64;      // levels and streams of the common layout
 constexpr int EN_LEVELS_B = 2048;                        // of the wide one: 64 streams of every depth
 constexpr int64_t EN_TILE = 2048, EN_TILE_MIN = 512;     // events of a tile; of a part's one tile in small traces
@@ -417,8 +422,9 @@ constexpr uint32_t EN_SPAN = 0xFFFFFFF0u;                // a step's times fit 3
 
 // One block per part, tile by tile; a tile with more ranges than SR, or whose
 // times span 2^32 ns, is taken in steps.  A step's ranges, and the ranges open
-// when it begins, lie in shared memory (times relative to its first event, 32
-// bits), and once per range this is worked out:
+// when it begins, lie in shared memory (times relative to the part's first
+// event, or to the step's after 2^32 ns, in 32 bits), and once per range this
+// is worked out:
 //   parent  the last range of the level above that starts no later
 //   chain   Algorithm 2's result for the range and its ancestors: walking
 //           outward to the first structural range, the innermost operator
@@ -444,9 +450,18 @@ constexpr uint32_t EN_SPAN = 0xFFFFFFF0u;                // a step's times fit 3
 // Ranges that are not laminar give wrong answers but no stray access: parents
 // lie one level up, so every climb and walk ends within 32 steps.
 //
+// Open ranges are kept from step to step, a warp to a stream and a lane to a
+// level, and only for the streams that the step touched: their chains are read
+// off the warp's ballots, so a range of the tile walks outward only to the
+// first open one, and a step's tables are cleared by the entries it made.
+//
 // Bound by issue (2.4 instructions a cycle) and by the shared-memory chains of
-// the links, not by HBM: 490 us for 20M kernels and 5.1M ranges on 16 streams,
-// 17 us for 2,000.  The level lists, stream partition, windows and per-stream
+// the links, not by HBM: 425 us for 20M kernels and 5.1M ranges on 16 streams
+// of 8 levels, 1,990 us for 50M and 14.5M on 64 streams of 32, 14 us for 2,000.
+// With every open range's chain walked, and every level's tables cleared,
+// counted up and made relative to the next event at each step, 490, 3,840 and
+// 17 us; steps of 1,024 ranges (one block of 1,024 threads) 2,780 us where 512
+// took 2,610.  The level lists, stream partition, windows and per-stream
 // tiles it replaces took 436 us in their largest kernel and another 300 us in
 // eight more launches (partly side by side) for the same trace, two host waits
 // and 60 us for the small one.  Also measured: one search per depth and kernel
@@ -463,15 +478,15 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
               const uint32_t *__restrict__ lvlmask, int nlcap, int nscap, int gshift, unsigned leave_on, int final,
               int32_t *__restrict__ out_range, uint8_t *__restrict__ out_nop, DevStatus *st) {
     pdl_wait();
-    constexpr int THREADS = TL::THREADS, WARPS = THREADS / 32, RW = TL::RW, RPT = TL::RPT, SR = TL::SR,
-                  WORDS = TL::WORDS;
+    constexpr int THREADS = TL::THREADS, WARPS = THREADS / 32, RPT = TL::RPT, SR = TL::SR, WORDS = TL::WORDS;
     static_assert(THREADS >= 256, "a thread per stream");
-    static_assert(WORDS <= 16, "words of a stream's mask");
+    static_assert(WORDS == 16 && RPT * WARPS == WORDS, "half a warp per stream, 16 bits per level");
     if ((st->err & (ERR_INVALID | ERR_DEPTH)) || (st->flags & leave_on)) return;
     extern __shared__ __align__(16) unsigned char en_smem[];
     const TL S(en_smem, nlcap, nscap);
     __shared__ uint32_t wbuf[33];
     __shared__ int taken[2];
+    __shared__ int ntouched;
     const int tid = threadIdx.x;
     const unsigned lane = lane_id(), warp = tid >> 5, lt = lanemask_lt();
     const int64_t b = blockIdx.x;
@@ -493,6 +508,7 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
         if (nl > nlcap || ns > nscap) {
             if (b == 0 && tid == 0) {
                 atomicMax(&st->nlevels, (unsigned)nl);
+                atomicMax(&st->nstreams, (unsigned)ns);
                 set_flag(st, F_LEVELS_MANY);
             }
             return;
@@ -501,12 +517,12 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
             S.cbase[tid] = (uint16_t)(ex & 0xFFFFu);
             S.ndep[tid] = (uint8_t)n;
             S.scid[tid] = n ? (uint16_t)(ex >> 16) : (uint16_t)E_NONE;
-            if (n) {
-                S.slist[ex >> 16] = (uint8_t)tid;
-                S.amask[ex >> 16] = 0;
-            }
+            if (n) S.slist[ex >> 16] = (uint8_t)tid;
         }
     }
+    for (int l = tid; l < (nl + 1) / 2; l += THREADS) S.lgroups[l] = 0;
+    for (int i = tid; i < ns * WORDS; i += THREADS) S.smask[i] = 0;
+    for (int q = tid; q < ns; q += THREADS) S.sgroups[q] = 0;
     const int64_t nt = parts * tp, events = V.K + V.R;
     int64_t r = tile_r[b * tp];
     int64_t k = tile_event(b * tp, nt, events) - r;
@@ -516,44 +532,95 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
         const long long t = kk < V.K ? V.time<KEYS>(kk) : LLONG_MAX, a = rr < V.R ? V.r_start[rr] : LLONG_MAX;
         return t < a ? t : a;
     };
-    long long base = first_time(k, r);
+    long long base = first_time(k, r), first = base;      // times are relative to base; the step's first event
     auto rel = [&](long long x) -> uint32_t {
         const unsigned long long v = (unsigned long long)x - (unsigned long long)base;
         return x < base ? 0u : (v >= 0xFFFFFFFEull ? 0xFFFFFFFFu : (uint32_t)v + 1u);
     };
-    for (int l = tid; l < LEVELS; l += THREADS) {
-        const int s = l >> 5, d = l & 31;
-        if (d >= S.ndep[s]) continue;
-        uint32_t v = 0;
-        if (carried) v = rows[b * LEVELS + l];
-        else
-            for (int64_t q = 0; q < b; ++q) {
-                const uint32_t x = (uint32_t)l < row_len[q] ? rows[q * LEVELS + l] : 0u;
-                v = x > v ? x : v;
-            }
-        if (v == 0) continue;
-        const long long z = V.r_end[v - 1];
-        if (z < base) continue;
-        const int e = SR + S.cbase[s] + d;
-        S.ss[e] = rel(V.r_start[v - 1]);
-        S.se[e] = rel(z);
-        S.si[e] = (v - 1) | kind_of(V.r_op[v - 1]) << 30;
-        S.dep[e] = (uint8_t)(d | D_MIXED);
-        atomicOr(&S.amask[S.scid[s]], 1u << d);
+    // What a warp writes of a stream's open ranges, lane by depth: the chain of
+    // each is the run of open levels above it, read off four ballots.
+    auto open_ranges = [&](int q, uint32_t e0, bool live, uint32_t a, uint32_t z, uint32_t i) {
+        const uint32_t kind = i >> 30;
+        const unsigned m = __ballot_sync(0xffffffffu, live), le = lt | 1u << lane;
+        const unsigned ops = __ballot_sync(0xffffffffu, live && kind == KIND_OP);
+        const unsigned walls = __ballot_sync(0xffffffffu, live && kind == KIND_STRUCT);
+        const unsigned longs = __ballot_sync(0xffffffffu, live && a < z);
+        const unsigned gap = ~m & le;
+        const unsigned lo = gap ? 32u - __clz(gap) : 0u;                         // the run's outermost level
+        const uint32_t out = __shfl_sync(0xffffffffu, z, (int)(lo & 31u));
+        if (lane == 0) S.amask[q] = m;
+        if (lane < WORDS) S.before[q * WORDS + lane] = m ? (uint16_t)(e0 + 31u - __clz(m)) : (uint16_t)E_NONE;
+        if (!live) return;
+        const uint32_t e = e0 + lane;
+        const unsigned run = le & ~((1u << lo) - 1u), wall = walls & run;
+        const unsigned seen = ops & (wall ? run & ~((2u << (31 - __clz(wall))) - 1u) : run);
+        S.ss[e] = a;
+        S.se[e] = z;
+        S.si[e] = i;
+        S.dep[e] = (uint8_t)(lane | D_MIXED);
+        S.par[e] = lane > 0 && ((m >> (lane - 1)) & 1u) ? (uint16_t)(e - 1) : (uint16_t)E_NONE;
+        S.prev[e] = m & lt ? (uint16_t)(e0 + 31u - __clz(m & lt)) : (uint16_t)E_NONE;
+        S.va[e] = seen ? (uint16_t)(e0 + 31u - __clz(seen)) : (uint16_t)E_NONE;
+        S.vn[e] = (uint8_t)__popc(seen);
+        S.re[e] = out;
+        S.best[e] = longs & le ? (uint16_t)(e0 + 31u - __clz(longs & le)) : (uint16_t)E_NONE;
+    };
+    for (int q = (int)warp; q < ns; q += WARPS) {                                // a warp per stream, a lane per depth
+        const unsigned s = S.slist[q], l = s * 32u + lane;
+        uint32_t v = 0, a = 0, z = 0, i = 0;
+        if (lane < S.ndep[s]) {
+            if (carried) v = rows[b * LEVELS + l];
+            else
+#pragma unroll 4
+                for (int64_t x = 0; x < b; ++x) {
+                    const uint32_t u = l < row_len[x] ? rows[x * LEVELS + l] : 0u;
+                    v = u > v ? u : v;
+                }
+        }
+        bool live = v != 0;
+        if (live) {
+            const long long end = V.r_end[v - 1];
+            live = end >= base;
+            a = rel(V.r_start[v - 1]);
+            z = rel(end);
+            i = (v - 1) | kind_of(V.r_op[v - 1]) << 30;
+        }
+        open_ranges(q, (uint32_t)SR + S.cbase[s], live, a, z, i);
     }
     bool err = false, fix = false;
+    int64_t r_end_n = tile_r[b * tp + 1];           // the next step's end
     __syncthreads();
-    for (int64_t t = b * tp; t < (b + 1) * tp; ++t) {
-        const int64_t r1 = tile_r[t + 1], k1 = tile_event(t + 1, nt, events) - r1;
+    for (int64_t t = b * tp + 1; t <= (b + 1) * tp; ++t) {
+        const int64_t r1 = r_end_n, k1 = tile_event(t, nt, events) - r1;
+        if (t < (b + 1) * tp) r_end_n = tile_r[t + 1];
         while (k < k1 || r < r1) {
             int nr = (int)(r1 - r < SR ? r1 - r : SR), nk = (int)(k1 - k);
+            long long nbase = first_time(k + nk, r + nr);
             // ---- the step: the whole tile, or up to the first event that
             // must wait (a kernel that starts no earlier than a range not
-            // loaded; 2^32 ns)
+            // loaded; 2^32 ns from base)
             auto near = [&](long long x) { return (unsigned long long)x - (unsigned long long)base < EN_SPAN; };
-            bool whole = r1 - r <= SR;
-            if (nk > 0) whole = whole && near(V.time<KEYS>(k + nk - 1));
-            if (nr > 0) whole = whole && near(V.r_start[r + nr - 1]);
+            const long long t_last = nk > 0 ? V.time<KEYS>(k + nk - 1) : first, a_last = nr > 0 ? V.r_start[r + nr - 1] : first;
+            if (!(near(t_last) && near(a_last)) && base != first) {
+                // the open ranges relative to this step's first event (once in some 4 s of the trace)
+                const unsigned long long shift = (unsigned long long)first - (unsigned long long)base;
+                base = first;
+                for (int q = (int)warp; q < ns; q += WARPS) {
+                    const unsigned s = S.slist[q];
+                    const uint32_t e0 = (uint32_t)SR + S.cbase[s], e = e0 + lane;
+                    uint32_t a2 = 0, z2 = 0, i = 0;
+                    if ((S.amask[q] >> lane) & 1u) {
+                        const uint32_t a = S.ss[e], z = S.se[e];
+                        i = S.si[e];
+                        a2 = (unsigned long long)a > shift ? a - (uint32_t)shift : 0u;
+                        z2 = z == 0xFFFFFFFFu ? rel(V.r_end[i & POS_MASK])
+                                              : ((unsigned long long)z > shift ? z - (uint32_t)shift : 0u);
+                    }
+                    open_ranges(q, e0, z2 > 0, a2, z2, i);
+                }
+                __syncthreads();
+            }
+            bool whole = r1 - r <= SR && near(t_last) && near(a_last);
             if (!whole) {
                 // by two warps, 32 probes a round
                 if (warp < 2) {
@@ -579,6 +646,7 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                 __syncthreads();
                 nk = taken[0];
                 nr = taken[1];
+                nbase = first_time(k + nk, r + nr);
                 if (nk == 0 && nr == 0) {                                // cannot happen on ordered records
                     if (tid == 0) set_err(st, ERR_INVALID);
                     return;
@@ -592,186 +660,174 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
             // times of this step as 32 bits: exact for its events
             auto rel_near = [&](long long x) { return (uint32_t)x - (uint32_t)base + 1u; };
             // ---- ranges, 32 at a time: the stream's and the level's earlier
-            // ranges in the warp's run by lane masks, before it by tables
+            // ranges in the group by lane masks, before it by tables (links)
             uint32_t lk[RPT], pk[RPT];               // the level's range before | level << 16; parent | prev on stream << 16
-            if (warp < RW) {
-                uint16_t *wl = S.last + warp * nlcap;
-                for (int l = (int)lane; l < nl; l += 32) wl[l] = 0;
-                for (int q = (int)lane; q < ns; q += 32)
+            if (tid == 0) ntouched = 0;
 #pragma unroll
-                    for (int i = 0; i < RPT; ++i) S.smask[q * WORDS + warp * RPT + i] = 0;
-                __syncwarp();
+            for (int i = 0; i < RPT; ++i) {
+                const unsigned g = i * WARPS + warp;
+                const int at = (int)g * 32, e = at + (int)lane;
+                lk[i] = 0xFFFFu << 16;
+                pk[i] = 0;
+                if (at >= nr) continue;
+                const bool in = e < nr;
+                const int64_t p = r + e;
+                const long long a = in ? V.r_start[p] : 0, z = in ? V.r_end[p] : 0;
+                const unsigned s = in ? V.r_stream[p] : 0u, d = in ? V.r_depth[p] : 0u;
+                const uint32_t op = in ? V.r_op[p] : 0u;
+                const bool lvl = in && d < S.ndep[s];
+                err |= in && !lvl && mine(s);
+                const unsigned q = lvl ? S.scid[s] : 256u;
+                const unsigned ps = __match_any_sync(0xffffffffu, q);
+                unsigned pl = ps, pp = ps;           // lanes of the level, of the level above
 #pragma unroll
-                for (int i = 0; i < RPT; ++i) {
-                    const int e = (int)warp * 32 * RPT + i * 32 + (int)lane;
-                    if (e - (int)lane >= nr) {
-                        lk[i] = 0xFFFFu << 16;
-                        continue;
+                for (int bit = 0; bit < 5; ++bit) {
+                    const unsigned x = __ballot_sync(0xffffffffu, (d >> bit) & 1u);
+                    pl &= (d >> bit) & 1u ? x : ~x;
+                    pp &= ((d - 1u) >> bit) & 1u ? x : ~x;
+                }
+                if (lvl) {
+                    const unsigned c = S.cbase[s] + d;
+                    const unsigned ml = pl & lt, mp = d ? pp & lt : 0u, ms = ps & lt;
+                    lk[i] = (ml ? at + 32u - __clz(ml) : 0u) | c << 16;                  // index + 1, 0 not here
+                    pk[i] = (mp ? at + 32u - __clz(mp) : 0u) | (ms ? at + 32u - __clz(ms) : 0u) << 16;
+                    S.ss[e] = rel_near(a);
+                    S.se[e] = rel(z);
+                    S.si[e] = (uint32_t)p | kind_of(op) << 30;
+                    S.dep[e] = (uint8_t)d;
+                    S.sid[e] = (uint8_t)q;
+                    if ((pl >> lane) == 1u) {                                            // the level's last of the 32
+                        S.last[g * nlcap + c] = (uint8_t)lane;
+                        atomicOr(&S.lgroups[c / 2], 1u << (g + 16 * (c & 1u)));
                     }
-                    const bool in = e < nr;
-                    const int64_t p = r + (in ? e : 0);
-                    const long long a = in ? V.r_start[p] : 0, z = in ? V.r_end[p] : 0;
-                    const unsigned s = in ? V.r_stream[p] : 0u, d = in ? V.r_depth[p] : 0u;
-                    const uint32_t op = in ? V.r_op[p] : 0u;
-                    const bool lvl = in && d < S.ndep[s];
-                    err |= in && !lvl && mine(s);
-                    const unsigned q = lvl ? S.scid[s] : 256u;
-                    const unsigned c = lvl ? S.cbase[s] + d : 0u;
-                    const unsigned ps = __match_any_sync(0xffffffffu, q);
-                    unsigned pl = ps, pp = ps;       // lanes of the level, of the level above
-#pragma unroll
-                    for (int bit = 0; bit < 5; ++bit) {
-                        const unsigned x = __ballot_sync(0xffffffffu, (d >> bit) & 1u);
-                        pl &= (d >> bit) & 1u ? x : ~x;
-                        pp &= ((d - 1u) >> bit) & 1u ? x : ~x;
+                    if (ms == 0) {
+                        S.smask[q * WORDS + g] = ps;
+                        atomicOr(&S.sgroups[q], 1u << g);
                     }
-                    lk[i] = pk[i] = 0;
-                    if (lvl) {
-                        const unsigned at = (unsigned)e - lane;
-                        const unsigned ml = pl & lt, mp = d ? pp & lt : 0u, ms = ps & lt;
-                        unsigned u;
-                        u = ml ? at + 31u - __clz(ml) + 1u : wl[c];                      // index + 1, 0 not here
-                        lk[i] = u | c << 16;
-                        u = mp ? at + 31u - __clz(mp) + 1u : (d ? wl[c - 1] : 0u);
-                        pk[i] = u | (ms ? at + 31u - __clz(ms) + 1u : 0u) << 16;
-                        S.ss[e] = rel_near(a);
-                        S.se[e] = rel(z);
-                        S.si[e] = (uint32_t)p | kind_of(op) << 30;
-                        S.dep[e] = (uint8_t)d;
-                        S.sid[e] = (uint8_t)q;
-                    } else if (in) {                 // another group's, or below a gap: on no stream's chain
-                        S.ss[e] = rel_near(a);
-                        S.se[e] = 0;
-                        S.si[e] = KIND_STRUCT << 30;
-                        S.dep[e] = (uint8_t)(D_DEPTH | D_MIXED);
-                        S.sid[e] = 255;
-                        S.par[e] = S.prev[e] = (uint16_t)E_NONE;
-                    }
-                    __syncwarp();
-                    if (lvl) {
-                        if ((pl >> lane) == 1u) wl[c] = (uint16_t)(e + 1);               // the level's last of the 32
-                        if ((ps & lt) == 0) S.smask[q * WORDS + warp * RPT + i] = ps;
-                    }
-                    if (!lvl) lk[i] = 0xFFFFu << 16;
-                    __syncwarp();
+                } else if (in) {                     // another group's, or below a gap: on no stream's chain
+                    S.ss[e] = rel_near(a);
+                    S.se[e] = 0;
+                    S.si[e] = KIND_STRUCT << 30;
+                    S.dep[e] = (uint8_t)(D_DEPTH | D_MIXED);
+                    S.sid[e] = 255;
+                    S.par[e] = S.prev[e] = (uint16_t)E_NONE;
                 }
             }
             __syncthreads();
             // ---- links, and the laminar checks.  Relative times are exact
             // below 2^32 - 1; two clamped ends are compared as they are.
-            for (int l = tid; l < nl; l += THREADS) {
-                uint32_t u = 0;
+            auto last_of = [&](uint32_t l, unsigned below) -> uint32_t {                 // the level's, in groups below; + 1
+                const unsigned h = (S.lgroups[l / 2] >> (16 * (l & 1u))) & ((1u << below) - 1u);
+                const unsigned g = 31 - __clz(h);
+                return h ? g * 32 + S.last[g * nlcap + l] + 1u : 0u;
+            };
 #pragma unroll
-                for (int w = 0; w < RW; ++w) {
-                    const uint32_t x = S.last[w * nlcap + l];
-                    S.last[w * nlcap + l] = (uint16_t)u;
-                    u = x ? x : u;
+            for (int i = 0; i < RPT; ++i) {
+                const unsigned g = i * WARPS + warp;
+                const uint32_t c = lk[i] >> 16;
+                if (c == 0xFFFFu) continue;
+                const uint32_t e = g * 32 + lane;
+                const unsigned q = S.sid[e], d = S.dep[e] & D_DEPTH, am = S.amask[q];
+                const uint32_t a = S.ss[e];
+                auto earlier = [&](uint32_t u, uint32_t l, unsigned depth) -> uint32_t {
+                    if (u == 0) u = last_of(l, g);
+                    return u ? u - 1 : ((am >> depth) & 1u ? (uint32_t)SR + l : (uint32_t)E_NONE);
+                };
+                const uint32_t y = earlier(lk[i] & 0xFFFFu, c, d);
+                uint32_t p = d ? earlier(pk[i] & 0xFFFFu, c - 1, d - 1) : (uint32_t)E_NONE;
+                uint32_t x = pk[i] >> 16;                                            // before it on the stream
+                if (x) --x;
+                else {
+                    const unsigned h = S.sgroups[q] & ((1u << g) - 1u), w = 31 - __clz(h);
+                    x = h ? w * 32 + 31 - __clz(S.smask[q * WORDS + w]) : (uint32_t)S.before[q * WORDS];
                 }
-                S.last[RW * nlcap + l] = (uint16_t)u;
+                bool mixed = x != E_NONE && S.ss[x] == a;
+                for (int f = (int)e + 1; f < nr && S.ss[f] == a; ++f) {              // equal starts further on
+                    if (S.sid[f] != q) continue;
+                    mixed = true;
+                    if (d && (S.dep[f] & D_DEPTH) == d - 1) p = f;
+                }
+                auto end_of = [&](uint32_t w) { return V.r_end[S.si[w] & POS_MASK]; };
+                auto ends_before = [&](uint32_t w, uint32_t v) {                     // entry w ends before entry v
+                    const uint32_t f = S.se[w], g = S.se[v];
+                    return f == 0xFFFFFFFFu && g == 0xFFFFFFFFu ? end_of(w) < end_of(v) : f < g;
+                };
+                if (y != E_NONE) {
+                    if (S.ss[y] == a && ends_before(e, y)) fix = true;               // starts with it, ends before it
+                    else if (S.se[y] > a) err = true;
+                    mixed |= S.se[y] == a;
+                }
+                if (d && (p == E_NONE || ends_before(p, e))) {
+                    if (more && !final && next == V.r_start[r + e]) fix = true;
+                    else err = true;
+                }
+                S.par[e] = (uint16_t)p;
+                S.prev[e] = (uint16_t)x;
+                if (mixed) S.dep[e] = (uint8_t)(d | D_MIXED);
             }
-            for (int q = THREADS - 1 - tid; q < ns; q += THREADS) {
-                unsigned m = 0;
+            // the last entry before each group, half a warp to a stream
+            for (int q2 = (int)warp * 2; q2 < ns; q2 += WARPS * 2) {
+                const int q = q2 + (int)(lane >> 4), w = (int)(lane & 15u);
+                const bool some = q < ns && S.sgroups[q] != 0;
+                if (!__any_sync(0xffffffffu, some)) continue;
+                const uint32_t m = some ? S.smask[q * WORDS + w] : 0u;
+                uint32_t u = m ? w * 32 + 32 - __clz(m) : 0u;
 #pragma unroll
-                for (int w = 0; w < WORDS; ++w) m |= (S.smask[q * WORDS + w] ? 1u : 0u) << w;
-                S.swords[q] = (uint16_t)m;
-                const uint32_t o = S.amask[q];
-                S.dopen[q] = o ? (uint16_t)(SR + S.cbase[S.slist[q]] + 31 - __clz(o)) : (uint16_t)E_NONE;
+                for (int h = 1; h < 16; h <<= 1) {
+                    const uint32_t v = __shfl_up_sync(0xffffffffu, u, h, 16);
+                    u = v > u ? v : u;
+                }
+                u = __shfl_up_sync(0xffffffffu, u, 1, 16);
+                if (some && w > 0) S.before[q * WORDS + w] = u ? (uint16_t)(u - 1) : S.before[q * WORDS];
+                if (some && w == 0) S.tlist[atomicAdd(&ntouched, 1)] = (uint8_t)q;
             }
             __syncthreads();
-            if (warp < RW) {
-#pragma unroll
-                for (int i = 0; i < RPT; ++i) {
-                    const uint32_t c = lk[i] >> 16;
-                    if (c == 0xFFFFu) continue;
-                    const uint32_t e = warp * 32 * RPT + i * 32 + lane;
-                    const unsigned q = S.sid[e], d = S.dep[e] & D_DEPTH, am = S.amask[q];
-                    const uint32_t a = S.ss[e];
-                    auto earlier = [&](uint32_t u, uint32_t l, unsigned depth) -> uint32_t {
-                        if (u == 0) u = S.last[warp * nlcap + l];
-                        return u ? u - 1 : ((am >> depth) & 1u ? (uint32_t)SR + l : (uint32_t)E_NONE);
-                    };
-                    const uint32_t y = earlier(lk[i] & 0xFFFFu, c, d);
-                    uint32_t p = d ? earlier(pk[i] & 0xFFFFu, c - 1, d - 1) : (uint32_t)E_NONE;
-                    uint32_t x = pk[i] >> 16;                                            // before it on the stream
-                    if (x) --x;
-                    else {
-                        const unsigned h = S.swords[q] & ((1u << (warp * RPT + i)) - 1u);
-                        const unsigned w = 31 - __clz(h);
-                        x = h ? w * 32 + 31 - __clz(S.smask[q * WORDS + w]) : (uint32_t)S.dopen[q];
-                    }
-                    bool mixed = x != E_NONE && S.ss[x] == a;
-                    for (int f = (int)e + 1; f < nr && S.ss[f] == a; ++f) {              // equal starts further on
-                        if (S.sid[f] != q) continue;
-                        mixed = true;
-                        if (d && (S.dep[f] & D_DEPTH) == d - 1) p = f;
-                    }
-                    auto end_of = [&](uint32_t w) { return V.r_end[S.si[w] & POS_MASK]; };
-                    auto ends_before = [&](uint32_t w, uint32_t v) {                     // entry w ends before entry v
-                        const uint32_t f = S.se[w], g = S.se[v];
-                        return f == 0xFFFFFFFFu && g == 0xFFFFFFFFu ? end_of(w) < end_of(v) : f < g;
-                    };
-                    if (y != E_NONE) {
-                        if (S.ss[y] == a && ends_before(e, y)) fix = true;               // starts with it, ends before it
-                        else if (S.se[y] > a) err = true;
-                        mixed |= S.se[y] == a;
-                    }
-                    if (d && (p == E_NONE || ends_before(p, e))) {
-                        if (more && !final && next == V.r_start[r + e]) fix = true;
-                        else err = true;
-                    }
-                    S.par[e] = (uint16_t)p;
-                    S.prev[e] = (uint16_t)x;
-                    if (mixed) S.dep[e] = (uint8_t)(d | D_MIXED);
-                }
+            // ---- the kernels: each warp an equal run, 32 at a time (the first of them on their way already)
+            const int per = (nk + 32 * WARPS - 1) / (32 * WARPS) * 32;
+            const int j0 = (int)warp * per, j1 = j0 + per < nk ? j0 + per : nk;
+            long long t_n = 0;
+            unsigned s_n = 0;
+            if (j0 + (int)lane < j1) {
+                t_n = V.time<KEYS>(k + j0 + lane);
+                s_n = V.stream<KEYS>(k + j0 + lane);
             }
-            for (int q = (int)warp; q < ns; q += WARPS) {                                // a warp per stream, a lane per depth
-                const uint32_t m = S.amask[q];
-                if (!((m >> lane) & 1u)) continue;
-                const uint32_t e = (uint32_t)SR + S.cbase[S.slist[q]] + lane;
-                S.par[e] = lane > 0 && ((m >> (lane - 1)) & 1u) ? (uint16_t)(e - 1) : (uint16_t)E_NONE;
-                S.prev[e] = m & lt ? (uint16_t)(e - lane + 31u - __clz(m & lt)) : (uint16_t)E_NONE;
-            }
-            __syncthreads();
-            // ---- chains and `best`
+            // ---- chains and `best`, up to the first open range, which has its own
             auto best_of = [&](uint32_t e) -> uint32_t {
-                while (e != E_NONE && S.ss[e] >= S.se[e]) e = S.prev[e];                 // zero length
-                if (e == E_NONE) return e;
+                while (e < SR && S.ss[e] >= S.se[e]) e = S.prev[e];                      // zero length
+                if (e >= SR) return e == E_NONE ? e : (uint32_t)S.best[e];
                 uint32_t w = e;
                 const uint32_t a = S.ss[e];
                 for (uint32_t x = S.prev[e]; x != E_NONE && S.ss[x] == a; x = S.prev[x])
                     if (S.se[x] > a && (S.dep[x] & D_DEPTH) > (S.dep[w] & D_DEPTH)) w = x;
                 return w;
             };
-            auto chain = [&](uint32_t e) {
-                uint32_t ans = E_NONE, n = 0, top = e;
+            for (int e = tid; e < nr; e += THREADS) {
+                uint32_t ans = E_NONE, n = 0, x = e, top;
                 bool on = true;
-                for (uint32_t x = e; x != E_NONE; x = S.par[x]) {
+                do {
                     const uint32_t kind = S.si[x] >> 30;
                     on = on && kind != KIND_STRUCT;
                     if (on && kind == KIND_OP && n++ == 0) ans = x;
                     top = x;
+                    x = S.par[x];
+                } while (x < SR);
+                uint32_t end = S.se[top];
+                if (x != E_NONE) {
+                    if (on) {
+                        if (n == 0) ans = S.va[x];
+                        n += S.vn[x];
+                    }
+                    end = S.re[x];
                 }
                 S.va[e] = (uint16_t)ans;
                 S.vn[e] = (uint8_t)n;
-                S.re[e] = S.se[top];
+                S.re[e] = end;
                 S.best[e] = (uint16_t)best_of(e);
-            };
-            for (int e = tid; e < nr; e += THREADS) chain(e);
-            for (int q = (int)warp; q < ns; q += WARPS)
-                if ((S.amask[q] >> lane) & 1u) chain((uint32_t)SR + S.cbase[S.slist[q]] + lane);
+            }
             __syncthreads();
-            // ---- the kernels: each warp an equal run, 32 at a time
             {
-                const int per = (nk + 32 * WARPS - 1) / (32 * WARPS) * 32;
-                const int j0 = (int)warp * per, j1 = j0 + per < nk ? j0 + per : nk;
                 int q0 = 0;                                                              // ranges before the run
-                long long t_n = 0;
-                unsigned s_n = 0;
                 if (j0 < j1) {
-                    if (j0 + (int)lane < j1) {
-                        t_n = V.time<KEYS>(k + j0 + lane);
-                        s_n = V.stream<KEYS>(k + j0 + lane);
-                    }
                     const uint32_t T0 = __shfl_sync(0xffffffffu, rel_near(t_n), 0);
                     int hi = nr;
                     while (q0 < hi) {
@@ -796,24 +852,26 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                     for (;;) {
                         const uint32_t v = q0 + (int)lane < nr ? S.ss[q0 + lane] : 0xFFFFFFFFu;
                         const int c = __popc(__ballot_sync(0xffffffffu, v <= Tm));
-                        for (int i = 0; i < c; ++i) qn += __shfl_sync(0xffffffffu, v, i) <= T ? 1 : 0;
+                        int h = 0;
+#pragma unroll
+                        for (int i = 16; i > 0; i >>= 1) h += __shfl_sync(0xffffffffu, v, h + i - 1) <= T ? i : 0;
                         q0 += c;
-                        if (c < 32) break;
+                        if (c < 32) {
+                            qn += h;
+                            break;
+                        }
+                        const uint32_t v31 = __shfl_sync(0xffffffffu, v, 31);
+                        qn += h + (v31 <= T ? 1 : 0);
                     }
                     if (!in || !mine(s)) continue;
                     uint32_t ans = E_NONE;
                     unsigned n = 0;
                     const unsigned q = S.scid[s];
                     if (q != E_NONE) {
-                        uint32_t x, m = 0;                                               // the stream's last one
-                        unsigned w = (unsigned)qn >> 5;
-                        if (w < WORDS) m = S.smask[q * WORDS + w] & ((1u << (qn & 31)) - 1u);
-                        if (m == 0) {
-                            const unsigned h = S.swords[q] & ((1u << w) - 1u);
-                            w = 31 - __clz(h);
-                            if (h) m = S.smask[q * WORDS + w];
-                        }
-                        x = m ? w * 32 + 31 - __clz(m) : (uint32_t)S.dopen[q];
+                        // the stream's last one
+                        const unsigned l = qn ? (unsigned)qn - 1u : 0u, w = q * WORDS + (l >> 5);
+                        const uint32_t m = qn ? S.smask[w] & ((2u << (l & 31)) - 1u) : 0u;
+                        uint32_t x = m ? (l | 31u) - __clz(m) : (uint32_t)S.before[w];
                         if (x != E_NONE) {
                             const bool at_start = S.ss[x] == T;
                             if (!at_start || !(S.dep[x] & D_MIXED)) {
@@ -861,37 +919,29 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
             // ---- the range each level carries on: its last one, unless it is over
             k += nk;
             r += nr;
-            const long long nbase = first_time(k, r);
-            const unsigned long long shift = (unsigned long long)nbase - (unsigned long long)base;
-            for (int q = (int)warp; q < ns; q += WARPS) {
+            const unsigned long long now = (unsigned long long)nbase - (unsigned long long)base;
+            const int nq = ntouched;             // the others stay (ranges that have ended are climbed past)
+            for (int j = (int)warp; j < nq; j += WARPS) {
+                const int q = S.tlist[j];
                 const unsigned s = S.slist[q];
+                const uint32_t l = S.cbase[s] + lane;
+                uint32_t a = 0, z = 0, i = 0;
                 bool live = false;
-                if ((int)lane < S.ndep[s]) {
-                    const uint32_t l = S.cbase[s] + lane;
-                    const uint32_t u = S.last[RW * nlcap + l];
-                    const uint32_t e = SR + l, f = u ? u - 1 : e;
+                if (lane < S.ndep[s]) {
+                    const uint32_t u = last_of(l, WORDS), f = u ? u - 1 : (uint32_t)SR + l;
                     if (u || ((S.amask[q] >> lane) & 1u)) {
-                        const uint32_t a = S.ss[f], z = S.se[f], i = S.si[f];
-                        // times relative to the next step
-                        uint32_t z2;
-                        if (z == 0xFFFFFFFFu) {
-                            const long long end = V.r_end[i & POS_MASK];
-                            const unsigned long long v = (unsigned long long)end - (unsigned long long)nbase;
-                            z2 = end < nbase ? 0u : (v >= 0xFFFFFFFEull ? 0xFFFFFFFFu : (uint32_t)v + 1u);
-                        } else {
-                            z2 = (unsigned long long)z > shift ? z - (uint32_t)shift : 0u;
-                        }
-                        live = z2 > 0;
-                        S.ss[e] = (unsigned long long)a > shift ? a - (uint32_t)shift : 0u;
-                        S.se[e] = z2;
-                        S.si[e] = i;
-                        S.dep[e] = (uint8_t)(lane | D_MIXED);
+                        a = S.ss[f];
+                        z = S.se[f];
+                        i = S.si[f];
+                        live = z == 0xFFFFFFFFu ? V.r_end[i & POS_MASK] >= nbase : (unsigned long long)z > now;
                     }
+                    if (u) reinterpret_cast<uint16_t *>(S.lgroups)[l] = 0;
                 }
-                const unsigned m = __ballot_sync(0xffffffffu, live);
-                if (lane == 0) S.amask[q] = m;
+                if (lane < WORDS) S.smask[q * WORDS + lane] = 0;
+                if (lane == WORDS) S.sgroups[q] = 0;
+                open_ranges(q, (uint32_t)SR + l - lane, live, a, z, i);
             }
-            base = nbase;
+            first = nbase;
             __syncthreads();
         }
     }
@@ -939,9 +989,10 @@ struct EncBufs {
 };
 constexpr int64_t EN_DIRECT_PARTS = 32;          // up to this many: a block scans the rows before its own itself
 template <typename TL, bool KEYS, bool GROUPS = false>
-static void launch_tiles(Ctx &c, const EncView &V, const EncBufs &B, int nl, int groups, unsigned leave_on,
+static void launch_tiles(Ctx &c, const EncView &V, const EncBufs &B, int nl, int ns, int groups, unsigned leave_on,
                          bool final, int32_t *out_range, uint8_t *out_nop) {
-    const int ns = std::is_same<TL, EncTileA>::value ? EN_STREAMS_A : 256;
+    nl = (nl + 7) & ~7;                          // (whole words in every table)
+    ns = (ns + 7) & ~7;
     const size_t smem = TL::smem(nl, ns);
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(k_enclose<TL, KEYS, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1021,7 +1072,7 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     const SmallCopy masks{c.h_small, B.lvlmask, 256 * sizeof(uint32_t)};
     if (early && (st = post_status(c, 1, &masks))) return st;
     launch_carry(c, B);
-    launch_tiles<EncTileA, false>(c, V, B, EN_LEVELS_A, 1, F_K_UNSORTED | F_R_UNSORTED, false, out_range, out_nop);
+    launch_tiles<EncTileA, false>(c, V, B, EN_LEVELS_A, EN_STREAMS_A, 1, F_K_UNSORTED | F_R_UNSORTED, false, out_range, out_nop);
     if (c.defer_status) {
         bool usual = true;
         if (early) {
@@ -1114,7 +1165,7 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     // ranges sorted so that parents come first: their verdict is final
     bool sort_ranges = !r_sorted || fixup, sorted = false;
     bool have_parts = k_sorted && !sort_ranges;       // (too many levels only: the checking pass's parts stand)
-    int nl = many ? (int)levels : EN_LEVELS_A;
+    int nl = many ? (int)levels : EN_LEVELS_A, ns = many ? (int)c.h_status->nstreams : EN_STREAMS_A;
     bool wide = many;
     for (int attempt = 0; attempt < 4; ++attempt) {
         if (sort_ranges && R > 0) {
@@ -1144,17 +1195,18 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
         }
         have_parts = true;
         if (!wide)
-            (keys ? launch_tiles<EncTileA, true> : launch_tiles<EncTileA, false>)(c, V, B, EN_LEVELS_A, 1, 0u, sorted,
+            (keys ? launch_tiles<EncTileA, true> : launch_tiles<EncTileA, false>)(c, V, B, EN_LEVELS_A, EN_STREAMS_A, 1, 0u, sorted,
                                                                                   out_range, out_nop);
         else if (nl <= EN_LEVELS_B)
-            (keys ? launch_tiles<EncTileB, true> : launch_tiles<EncTileB, false>)(c, V, B, nl, 1, 0u, sorted, out_range,
+            (keys ? launch_tiles<EncTileB, true> : launch_tiles<EncTileB, false>)(c, V, B, nl, ns, 1, 0u, sorted, out_range,
                                                                                   out_nop);
         else
             (keys ? launch_tiles<EncTileB, true, true> : launch_tiles<EncTileB, false, true>)(
-                c, V, B, EN_LEVELS_B, 4, 0u, sorted, out_range, out_nop);
+                c, V, B, EN_LEVELS_B, 64, 4, 0u, sorted, out_range, out_nop);
         if ((st = read_status(c))) return st;
         if (c.h_status->flags & F_LEVELS_MANY) {
             nl = (int)c.h_status->nlevels;
+            ns = (int)c.h_status->nstreams;
             wide = true;
             continue;
         }

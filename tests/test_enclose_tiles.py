@@ -1,7 +1,8 @@
 """The enclosure's tiles (GPU) where they can go wrong: parts and tiles of a few
 events and one more, more ranges in a tile than one step takes, more streams or
-levels than the common layout holds, and instants at which many ranges start
-and end together cut by a tile's edge.  Against the oracle."""
+levels than the common layout holds, instants at which many ranges start and
+end together cut by a tile's edge, and times that outgrow 32 bits.  Against the
+oracle."""
 import dataclasses
 
 import numpy as np
@@ -51,3 +52,15 @@ def test_ranges_without_kernels():
     t = dataclasses.replace(t, k_stream=t.k_stream[:n].copy(), k_start=t.k_start[:n].copy(), k_dur=t.k_dur[:n].copy(),
                             k_name=t.k_name[:n].copy(), ncu_name=t.ncu_name[:n].copy(), counters=t.counters[:n].copy())
     _check(t)
+
+
+@pytest.mark.parametrize("streams,depth", [(3, 6), (66, 12)])
+@pytest.mark.parametrize("bits", [12, 17, 24])
+def test_long_traces(streams, depth, bits):
+    """Times stretched until a part, then a step, then the gap between two
+    events is longer than the 32 bits that times in a step have: open ranges
+    are made relative to a later event, with ends past 32 bits among them."""
+    t = tracegen.generate("adversarial", n_kernels=20_000, n_streams=streams, max_depth=depth, seed=bits)
+    t0 = min(int(t.k_start.min()), int(t.r_start.min()))
+    _check(dataclasses.replace(t, k_start=(t.k_start - t0) << bits, r_start=(t.r_start - t0) << bits,
+                               r_end=(t.r_end - t0) << bits))
