@@ -334,68 +334,74 @@ __device__ __forceinline__ bool stopped(const DevStatus *st) {
 // op's kernels: one atomic per distinct op id of a warp on cnt[op], whose old
 // value plus the kernel's rank among its warp peers is the slot (rank[k]);
 // cnt ends as the per-op counts.  Each warp takes a run of `run` consecutive
-// kernels (a multiple of 32, up to AF_RUN) 32 at a time in index order, so an
-// op whose kernels all lie in one run gets ascending slots; the ops pass
-// sorts the few segments that do not.
+// kernels (a multiple of 32, up to AF_RUN) in index order, so an op whose
+// kernels all lie in one run gets ascending slots; the ops pass sorts the few
+// segments that do not.
+//
+// Bound by the latency of the gathers and atomics of a step, so AC_GROUPS
+// groups of 32 kernels go together: 116 us for 20M kernels, 264 for 50M (143
+// and 409 one group at a time with its loads a step ahead; two groups 142 and
+// 415, four with the registers of AC_BLOCKS blocks spilling 114 and 254, four
+// with a block fewer 124 and 260).
 constexpr int AF_RUN = 4096;
+constexpr int AC_GROUPS = 3, AC_BLOCKS = 5;
 
 template <bool DIRECT>
-__global__ void __launch_bounds__(256, 5) k_agg_count(const int64_t *__restrict__ dur, const int32_t *__restrict__ rok,
-                            const int32_t *__restrict__ nidx, const uint32_t *__restrict__ r_op, int64_t K, int64_t R,
-                            int64_t M, int64_t n_ops, uint32_t *__restrict__ cnt, uint32_t *__restrict__ rank,
-                            int64_t run, int ident_rows, unsigned *__restrict__ nonident, int pending,
-                            DevStatus *st) {
+__global__ void __launch_bounds__(256, AC_BLOCKS)
+    k_agg_count(const int64_t *__restrict__ dur, const int32_t *__restrict__ rok, const int32_t *__restrict__ nidx,
+                const uint32_t *__restrict__ r_op, int64_t K, int64_t R, int64_t M, int64_t n_ops,
+                uint32_t *__restrict__ cnt, uint32_t *__restrict__ rank, int64_t run, int ident_rows,
+                unsigned *__restrict__ nonident, int pending, DevStatus *st) {
     pdl_wait();
     if (pending && stopped(st)) return;
     const unsigned lane = lane_id(), lt = lanemask_lt();
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
     const int64_t nwarps = (int64_t)gridDim.x * blockDim.x / 32;
-    unsigned long long tot = 0, att = 0, natt = 0, nmatch = 0;
+    unsigned long long tot = 0, att = 0;
+    unsigned natt = 0, nmatch = 0;
     int bad = 0, nid = 0;
-    auto op_of = [&](int32_t r) -> uint32_t { return (r >= 0 && r < R) ? r_op[r] : 0xFFFFFFFFu; };
     for (int64_t k0 = warp * run; k0 < K; k0 += nwarps * run) {
         const int64_t k1 = k0 + run < K ? k0 + run : K;
-        // ranges two groups ahead; op ids, durations and row indices one group
-        // ahead, so each step waits only on its own atomic
-        int64_t k = k0 + lane;
-        int32_t r_c = k < k1 ? range_of_t<DIRECT>(rok, r_op, k) : -1;
-        uint32_t op_c = op_of(r_c);
-        long long d_c = k < k1 ? dur[k] : 0;
-        int32_t j_c = k < k1 ? (ident_rows ? (int32_t)k : nidx[k]) : -1;
-        int32_t r_n = k + 32 < k1 ? range_of_t<DIRECT>(rok, r_op, k + 32) : -1;
-        for (int64_t kb = k0; kb < k1; kb += 32) {
-            k = kb + lane;
-            const bool in = k < k1;
-            const int32_t r = r_c, j = j_c;
-            const uint32_t op = op_c;
-            const long long d = d_c;
-            r_c = r_n;
-            op_c = op_of(r_n);
-            d_c = k + 32 < k1 ? dur[k + 32] : 0;
-            j_c = k + 32 < k1 ? (ident_rows ? (int32_t)(k + 32) : nidx[k + 32]) : -1;
-            r_n = k + 64 < k1 ? range_of_t<DIRECT>(rok, r_op, k + 64) : -1;
-            nid |= in && (int64_t)j != k;
-            bool valid = in;
-            if (in && (d < 0 || r < -1 || r >= R || j < -1 || j >= M || (r >= 0 && (int64_t)op >= n_ops))) {
-                bad = 1;
-                valid = false;
+        for (int64_t kb = k0; kb < k1; kb += 32 * AC_GROUPS) {
+            int32_t r[AC_GROUPS], j[AC_GROUPS];
+            long long d[AC_GROUPS];
+            uint32_t op[AC_GROUPS];
+            unsigned peers[AC_GROUPS], base[AC_GROUPS];
+            // the sums of a call with a bad record are not given out, so no
+            // record waits for its checks
+#pragma unroll
+            for (int u = 0; u < AC_GROUPS; ++u) {
+                const int64_t k = kb + u * 32 + lane;
+                const bool in = k < k1;
+                r[u] = in ? range_of_t<DIRECT>(rok, r_op, k) : -1;
+                d[u] = in ? dur[k] : 0;
+                j[u] = in ? (ident_rows ? (int32_t)k : nidx[k]) : -1;
             }
-            if (valid) {
-                tot += (unsigned long long)d;
-                if (r >= 0) {
-                    att += (unsigned long long)d;
+#pragma unroll
+            for (int u = 0; u < AC_GROUPS; ++u) op[u] = (r[u] >= 0 && r[u] < R) ? r_op[r[u]] : 0xFFFFFFFFu;
+#pragma unroll
+            for (int u = 0; u < AC_GROUPS; ++u) {
+                const int64_t k = kb + u * 32 + lane;
+                nid |= k < k1 && (int64_t)j[u] != k;
+                bad |= d[u] < 0 || r[u] < -1 || r[u] >= R || j[u] < -1 || j[u] >= M;
+                tot += (unsigned long long)d[u];
+                if (r[u] >= 0) {
+                    att += (unsigned long long)d[u];
                     natt++;
-                    nmatch += j >= 0;
+                    nmatch += j[u] >= 0;
+                    bad |= (int64_t)op[u] >= n_ops;
                 }
+                // slotted exactly as k_agg_place places it: by range and op id alone
+                if ((int64_t)op[u] >= n_ops) op[u] = 0xFFFFFFFFu;
+                peers[u] = __match_any_sync(0xffffffffu, op[u]);
+                base[u] = 0;
+                if (op[u] != 0xFFFFFFFFu && (peers[u] & lt) == 0) base[u] = atomicAdd(&cnt[op[u]], (unsigned)__popc(peers[u]));
             }
-            // slotted exactly as k_agg_place places it: by range and op id alone
-            const unsigned key = (in && r >= 0 && r < R && (int64_t)op < n_ops) ? op : 0xFFFFFFFFu;
-            const unsigned peers = __match_any_sync(0xffffffffu, key);
-            const int leader = __ffs(peers) - 1;
-            unsigned base = 0;
-            if (key != 0xFFFFFFFFu && (int)lane == leader) base = atomicAdd(&cnt[key], (unsigned)__popc(peers));
-            base = __shfl_sync(0xffffffffu, base, leader);
-            if (key != 0xFFFFFFFFu) rank[k] = base + __popc(peers & lt);
+#pragma unroll
+            for (int u = 0; u < AC_GROUPS; ++u) {
+                base[u] = __shfl_sync(0xffffffffu, base[u], __ffs(peers[u]) - 1);
+                if (op[u] != 0xFFFFFFFFu) rank[kb + u * 32 + lane] = base[u] + __popc(peers[u] & lt);
+            }
         }
     }
     __shared__ unsigned long long red[33];
@@ -403,8 +409,8 @@ __global__ void __launch_bounds__(256, 5) k_agg_count(const int64_t *__restrict_
     if (__any_sync(0xffffffffu, nid) && lane_id() == 0) atomicOr(nonident, 1u);
     block_add_u64(tot, &st->cnt[C_TOTAL_NS], red);
     block_add_u64(att, &st->cnt[C_ATTR_NS], red);
-    block_add_u64(natt, &st->cnt[C_ATTR_K], red);
-    block_add_u64(nmatch, &st->cnt[C_MATCHED_K], red);
+    block_add_u64((unsigned long long)natt, &st->cnt[C_ATTR_K], red);
+    block_add_u64((unsigned long long)nmatch, &st->cnt[C_MATCHED_K], red);
 }
 
 // ------------------------------------------------------------------ place
@@ -1237,10 +1243,10 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
     const ZeroRun zr[3] = {{cnt, O + 1}, {ctr, 4}, {nonident, 1}};
     if ((st = c.enclose_pending || c.keep_status ? zero_runs(c, 3, zr) : reset_status(c, 3, zr))) return st;
     const int sms = sm_count(c);
-    // runs long enough to keep most segments in one warp, short enough that
-    // the grid is one wave of resident warps (five blocks of eight per SM)
-    const int64_t warps = (int64_t)std::max(1, sms) * 40;
-    const int64_t run = std::min<int64_t>(AF_RUN, std::max<int64_t>(32, ((K + warps - 1) / warps + 31) / 32 * 32));
+    // runs long enough to keep most segments in one warp, in as few full waves
+    // of resident warps as runs of up to AF_RUN allow
+    const int64_t warps = (int64_t)std::max(1, sms) * AC_BLOCKS * 8, waves = (K + warps * AF_RUN - 1) / (warps * AF_RUN);
+    const int64_t run = std::max<int64_t>(32, waves > 0 ? ((K + warps * waves - 1) / (warps * waves) + 31) / 32 * 32 : 0);
     if (K > 0)
         launch(c, "agg_count", rok ? k_agg_count<false> : k_agg_count<true>,
                dim3(grid_for(K, 256 / 32 * run, 65535)), dim3(256), 0, kern->dur_ns, rok, nidx, rng->op_id, K, R, M,
