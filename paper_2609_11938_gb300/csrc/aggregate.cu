@@ -37,8 +37,9 @@ struct AggIn {
     int64_t M;                  // ncu rows: a row index at or past M is never read (the count pass reports it)
     int64_t n_ops;
     uint32_t lane_max;          // longest op that one lane takes
-    unsigned *ctr;              // [0] next chunk of the ops pass, [1] ops listed in dirty, [2] in mids, [3] in longs;
-                                // zeroed before it
+    int chunk;                  // op ids of a chunk of the ops pass
+    unsigned *ctr;              // [0] chunks drawn in the ops pass, [1] ops listed in dirty, [2] in mids, [3] in longs,
+                                // [4] blocks done (here), [5] nonident, [6] blocks done (count); zeroed before it
     uint32_t *dirty;            // ops whose fast sums saw a null or infinite value
     uint32_t *mids;             // ops longer than a lane takes: a block each (k_agg_mid)
     uint32_t *longs;            // ops longer than a block takes: the pieces pass
@@ -345,13 +346,15 @@ __device__ __forceinline__ bool stopped(const DevStatus *st) {
 // with a block fewer 124 and 260).
 constexpr int AF_RUN = 4096;
 constexpr int AC_GROUPS = 3, AC_BLOCKS = 5;
+constexpr int AC_PER = 16;                      // counts that a thread of the last block scans
+constexpr int64_t AC_SCAN = 256 * AC_PER;
 
 template <bool DIRECT>
 __global__ void __launch_bounds__(256, AC_BLOCKS)
     k_agg_count(const int64_t *__restrict__ dur, const int32_t *__restrict__ rok, const int32_t *__restrict__ nidx,
                 const uint32_t *__restrict__ r_op, int64_t K, int64_t R, int64_t M, int64_t n_ops,
-                uint32_t *__restrict__ cnt, uint32_t *__restrict__ rank, int64_t run, int ident_rows,
-                unsigned *__restrict__ nonident, int pending, DevStatus *st) {
+                uint32_t *cnt, uint32_t *__restrict__ rank, int64_t run, int ident_rows,
+                unsigned *__restrict__ nonident, int pending, uint32_t *off, unsigned *done, DevStatus *st) {
     pdl_wait();
     if (pending && stopped(st)) return;
     const unsigned lane = lane_id(), lt = lanemask_lt();
@@ -411,6 +414,29 @@ __global__ void __launch_bounds__(256, AC_BLOCKS)
     block_add_u64(att, &st->cnt[C_ATTR_NS], red);
     block_add_u64((unsigned long long)natt, &st->cnt[C_ATTR_K], red);
     block_add_u64((unsigned long long)nmatch, &st->cnt[C_MATCHED_K], red);
+    if (!off) return;
+    // few ops: the last block turns the counts into offsets
+    __shared__ bool last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(done, 1u) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    const int64_t i0 = threadIdx.x * AC_PER;
+    uint32_t v[AC_PER], sum = 0;
+#pragma unroll
+    for (int i = 0; i < AC_PER; ++i) v[i] = i0 + i <= n_ops ? __ldcg(cnt + i0 + i) : 0u;
+#pragma unroll
+    for (int i = 0; i < AC_PER; ++i) sum += v[i];
+    uint32_t ex = block_exclusive_scan<uint32_t>(sum, reinterpret_cast<uint32_t *>(red), nullptr);
+#pragma unroll
+    for (int i = 0; i < AC_PER; ++i) {
+        if (i0 + i <= n_ops) off[i0 + i] = ex;
+        ex += v[i];
+    }
 }
 
 // ------------------------------------------------------------------ place
@@ -631,10 +657,18 @@ __device__ __forceinline__ void cp_async_rows(float4 (*dst)[NC / 4], const float
     }
 }
 
+// Where the last block of the ops pass stores the status block and the numbers
+// of listed ops for the host (mapped pinned memory), or NULL: a launch fewer
+// before the host's wait.
+struct OpsReport {
+    uint32_t *status, *counts;
+};
+
 __global__ void __launch_bounds__(AG_THREADS, AG_BLOCKS) k_agg_ops(const uint32_t *__restrict__ off, uint32_t *list,
-                                                          AggIn A, int pending, const DevStatus *st) {
+                                                          AggIn A, int pending, const DevStatus *st,
+                                                          OpsReport report) {
     pdl_wait();
-    if (pending && stopped(st)) return;
+    const bool idle = pending && stopped(st);
     extern __shared__ __align__(16) unsigned char ag_smem[];
     OpsWarp &W = reinterpret_cast<OpsWarp *>(ag_smem)[threadIdx.x / 32];
     const unsigned lane = lane_id();
@@ -647,13 +681,14 @@ __global__ void __launch_bounds__(AG_THREADS, AG_BLOCKS) k_agg_ops(const uint32_
     };
     auto draw = [&]() -> unsigned {
         unsigned v = 0;
-        if (lane == 0) v = atomicAdd(A.ctr, 1u);
+        if (lane == 0) v = gridDim.x * AG_WARPS + atomicAdd(A.ctr, 1u);
         return v;
     };
     constexpr int PER = AG_CHUNK / 32;
-    // the first chunk's offsets; afterwards the next chunk is drawn and its
-    // offsets loaded while the current one runs
-    int64_t o0 = (int64_t)__shfl_sync(0xffffffffu, draw(), 0) * AG_CHUNK;
+    const int CHUNK = A.chunk;
+    // the first chunk's offsets (each warp has one); afterwards the next chunk
+    // is drawn and its offsets loaded while the current one runs
+    int64_t o0 = idle ? A.n_ops : (int64_t)(blockIdx.x * AG_WARPS + threadIdx.x / 32) * CHUNK;
     uint32_t oa[PER], ob[PER];
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
@@ -663,7 +698,7 @@ __global__ void __launch_bounds__(AG_THREADS, AG_BLOCKS) k_agg_ops(const uint32_
     }
     while (o0 < A.n_ops) {
         const unsigned next_raw = draw();           // in flight during this chunk
-        const int nchunk = A.n_ops - o0 < AG_CHUNK ? (int)(A.n_ops - o0) : AG_CHUNK;
+        const int nchunk = A.n_ops - o0 < CHUNK ? (int)(A.n_ops - o0) : CHUNK;
         const uint32_t cbase = __shfl_sync(0xffffffffu, oa[0], 0);          // the chunk's list run
         const uint32_t cend = __shfl_sync(0xffffffffu, ob[(nchunk - 1) >> 5], (nchunk - 1) & 31);
         const uint32_t ctot = cend - cbase;
@@ -704,7 +739,7 @@ __global__ void __launch_bounds__(AG_THREADS, AG_BLOCKS) k_agg_ops(const uint32_
         }
         __syncwarp();
         // the next chunk's offsets, in flight during the rounds
-        const int64_t o1 = (int64_t)__shfl_sync(0xffffffffu, next_raw, 0) * AG_CHUNK;
+        const int64_t o1 = (int64_t)__shfl_sync(0xffffffffu, next_raw, 0) * CHUNK;
         uint32_t na[PER], nb[PER];
 #pragma unroll
         for (int q = 0; q < PER; ++q) {
@@ -776,6 +811,19 @@ __global__ void __launch_bounds__(AG_THREADS, AG_BLOCKS) k_agg_ops(const uint32_
 #pragma unroll
         for (int q = 0; q < PER; ++q) { oa[q] = na[q]; ob[q] = nb[q]; }
     }
+    if (!report.status) return;
+    __shared__ bool last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(A.ctr + 4, 1u) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    for (unsigned i = threadIdx.x; i < sizeof(DevStatus) / 4; i += AG_THREADS)
+        report.status[i] = __ldcg(reinterpret_cast<const uint32_t *>(st) + i);
+    if (threadIdx.x < 3) report.counts[threadIdx.x] = __ldcg(A.ctr + 1 + threadIdx.x);
 }
 
 // The ops k_agg_ops listed as dirty: one thread each puts the segment in
@@ -1182,15 +1230,24 @@ __global__ void __launch_bounds__(FIN_THREADS) k_agg_long_ops(const uint32_t *__
     if (bad) set_err(st, ERR_INVALID);
 }
 
-// Blocks of the ops pass: what stays resident, fewer for few ops.
-static unsigned ops_grid(Ctx &c, int64_t O) {
+// Blocks of the ops pass: what stays resident, fewer for few ops.  A chunk is
+// half as long where every warp still has one at most: a lane then walks one op
+// instead of two (14,300 ops 20 us -> 11; 114,400 ops, past that line, 23 us
+// with chunks of 64).
+static unsigned ops_grid(Ctx &c, int64_t O, int *chunk) {
     const int sms = sm_count(c);
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_agg_ops, AG_THREADS, AG_SMEM);
     cudaGetLastError();
     const int64_t resident = (int64_t)std::max(1, sms) * std::max(1, per_sm);
-    const int64_t need = (O + (int64_t)AG_WARPS * AG_CHUNK - 1) / ((int64_t)AG_WARPS * AG_CHUNK);
+    *chunk = O <= resident * AG_WARPS * (AG_CHUNK / 2) ? AG_CHUNK / 2 : AG_CHUNK;
+    const int64_t need = (O + (int64_t)AG_WARPS * *chunk - 1) / ((int64_t)AG_WARPS * *chunk);
     return (unsigned)std::max<int64_t>(1, std::min(resident, need));
+}
+
+int64_t agg_counter_words(uint32_t n_ops) {
+    const int64_t n = (int64_t)n_ops + 1;
+    return AGG_OWN_WORDS + (scan_clean_words(n) + 7) / 8 * 8 + n;
 }
 
 opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_ranges *rng, const int32_t *rok,
@@ -1208,27 +1265,36 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
     if ((reinterpret_cast<uintptr_t>(ncu->counters) & 15) != 0) return OPATTR_E_INVALID_ARG;
 
     Need nd;
-    nd.add<uint32_t>(O + 1).add<uint32_t>(O + 1).add<uint32_t>(K).add<uint32_t>(K);
+    nd.add<uint32_t>(O + 1).add<uint32_t>(K).add<uint32_t>(K);
     const int64_t mids_n = std::min<int64_t>(O, K / (AG_LANE_MAX + 1)) + 1;        // ops longer than a lane takes
     const int64_t part_n = K / AG_PIECE + K / (AG_MID_MAX + 1) + 1;                // pieces of the longest
-    nd.add<uint32_t>(mids_n).add<uint32_t>(mids_n).add<unsigned>(4).add<unsigned>(1).add<uint32_t>(O + 1);
+    nd.add<uint32_t>(mids_n).add<uint32_t>(mids_n).add<uint32_t>(O + 1);
     nd.add<uint32_t>(mids_n).add<Acc>(part_n);
     nd.add<uint32_t>(scan_scratch_elems(std::max<int64_t>(O + 1, radix_hist_elems(K))));
     nd.add<uint32_t>(O + 1).add<uint32_t>(radix_hist_elems(K)).add<uint32_t>(8);   // huge-op index, histogram, info
     nd.add<uint32_t>(mids_n);                                                        // huge ops
+    // the counters lie ready at the start of the arena, or are taken and zeroed here
+    const int64_t words = agg_counter_words(n_ops);          // ctr, the scan's, cnt
+    const bool keeps = c.enclose_pending || c.keep_status;
+    if (!(keeps && c.agg_words == words)) c.agg_ready = false;
+    if (!c.agg_ready) c.arena_keep = 0;
     opattr_status st = ensure_arena(c, nd.bytes + 4096);
+    if (!st && !c.agg_ready) st = ensure_arena(c, nd.add<uint32_t>(words).bytes + 4096);
     if (st) return st;
     Arena a(c);
-    uint32_t *cnt = a.take<uint32_t>(O + 1), *off = a.take<uint32_t>(O + 1);
+    const bool ready = c.agg_ready;
+    uint32_t *counters = ready ? reinterpret_cast<uint32_t *>(c.arena) : a.take<uint32_t>(words);
+    c.agg_ready = false;
+    c.arena_keep = 0;
+    uint32_t *off = a.take<uint32_t>(O + 1);
     // tmp holds each kernel's slot among its op's kernels until the list is
     // placed, then serves the segment sorts
     uint32_t *list = a.take<uint32_t>(K), *tmp = a.take<uint32_t>(K);
     uint32_t *mids = a.take<uint32_t>(mids_n), *longs = a.take<uint32_t>(mids_n);
-    // ctr[0] next chunk; the numbers of ops listed dirty, mid and long (nlong)
-    // come back together
-    unsigned *ctr = a.take<unsigned>(4);
-    unsigned *nlong = ctr ? ctr + 3 : nullptr;
-    unsigned *nonident = a.take<unsigned>(1);
+    // the numbers of ops listed dirty, mid and long (nlong) come back together
+    if (!counters) return OPATTR_E_OOM;
+    unsigned *ctr = counters, *nlong = ctr + 3, *nonident = ctr + 5;
+    uint32_t *chain = counters + AGG_OWN_WORDS, *cnt = counters + (words - (O + 1));
     uint32_t *dirty = a.take<uint32_t>(O + 1);
     uint32_t *npc = a.take<uint32_t>(mids_n);
     Acc *partials = a.take<Acc>(part_n);
@@ -1237,12 +1303,16 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
     uint32_t *hidx = a.take<uint32_t>(O + 1), *hhist = a.take<uint32_t>(radix_hist_elems(K));
     uint32_t *info = a.take<uint32_t>(8), *hop = a.take<uint32_t>(mids_n);
     if (!hidx || !hhist || !info || !hop) return OPATTR_E_OOM;
-    if (!cnt || !off || !list || !tmp || !mids || !longs || !nlong || !part || !nonident || !dirty) return OPATTR_E_OOM;
+    if (!off || !list || !tmp || !mids || !longs || !part || !dirty) return OPATTR_E_OOM;
     // with the enclosure's or the matching's verdict pending (a join) the status
     // block keeps it: the enclosure's reset left the aggregation's slots at zero
-    const ZeroRun zr[3] = {{cnt, O + 1}, {ctr, 4}, {nonident, 1}};
-    if ((st = c.enclose_pending || c.keep_status ? zero_runs(c, 3, zr) : reset_status(c, 3, zr))) return st;
+    const ZeroRun zr{counters, words};
+    if (!ready && (st = keeps ? zero_runs(c, 1, &zr) : reset_status(c, 1, &zr))) return st;
     const int sms = sm_count(c);
+    // Fewer than AC_SCAN ops: the count's last block scans the counts (340 ops:
+    // 2 us more in the count, where the launch of a scan took 5); with 7,150 it
+    // takes 8 us more, with 14,300 14 us, and one block of 1,024 threads 5 to 6.
+    const bool scan = K > 0 && O > 0 && O < AC_SCAN;
     // runs long enough to keep most segments in one warp, in as few full waves
     // of resident warps as runs of up to AF_RUN allow
     const int64_t warps = (int64_t)std::max(1, sms) * AC_BLOCKS * 8, waves = (K + warps * AF_RUN - 1) / (warps * AF_RUN);
@@ -1250,7 +1320,8 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
     if (K > 0)
         launch(c, "agg_count", rok ? k_agg_count<false> : k_agg_count<true>,
                dim3(grid_for(K, 256 / 32 * run, 65535)), dim3(256), 0, kern->dur_ns, rok, nidx, rng->op_id, K, R, M,
-               O, cnt, tmp, run, (int)(c.in_join && c.rows_identity), nonident, (int)c.enclose_pending, c.d_status);
+               O, cnt, tmp, run, (int)(c.in_join && c.rows_identity), nonident, (int)c.enclose_pending, scan ? off : nullptr,
+               ctr + 6, c.d_status);
     AggIn in;
     in.dur = kern->dur_ns;
     in.ncu_idx = nidx;
@@ -1266,7 +1337,7 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
     in.out = *out;
     bool status_fresh = false;        // no launch since the last status read
     if (O > 0) {
-        scan_exclusive_u32(c, cnt, off, O + 1, part, nullptr);
+        if (!scan) scan_exclusive_u32(c, cnt, off, O + 1, chain, nullptr, true);
         if (K > 0)
             launch(c, "agg_place", rok ? k_agg_place<false> : k_agg_place<true>,
                    dim3(grid_for(K, 256 * 4, REDUCE_GRID)), dim3(256), 0, rok, rng->op_id, K, R, O,
@@ -1277,14 +1348,17 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
             cudaFuncSetAttribute(k_agg_ops, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AG_SMEM);
             attr_done |= 1u << c.device;
         }
-        launch(c, "agg_ops", k_agg_ops, dim3(ops_grid(c, O)), dim3(AG_THREADS), AG_SMEM,
-               (const uint32_t *)off, list, in, (int)c.enclose_pending, (const DevStatus *)c.d_status);
+        const unsigned grid = ops_grid(c, O, &in.chunk);
+        OpsReport report{};
+        if (c.host_mapped) report = {reinterpret_cast<uint32_t *>(c.h_status), c.h_small};
+        launch(c, "agg_ops", k_agg_ops, dim3(grid), dim3(AG_THREADS), AG_SMEM, (const uint32_t *)off, list, in,
+               (int)c.enclose_pending, (const DevStatus *)c.d_status, report);
         // the ops the pass left: listed with a null or infinite value (redone
         // by k_agg_careful, a thread each), longer than a lane takes (a block
         // each) and longer still (the pieces pass); the counts come back with
         // the status
         const SmallCopy counts{c.h_small, ctr + 1, 3 * sizeof(uint32_t)};
-        if ((st = read_status(c, 1, &counts))) return st;
+        if ((st = c.host_mapped ? sync_status(c) : read_status(c, 1, &counts))) return st;
         const uint32_t n_dirty = c.h_small[0], n_mid = c.h_small[1], n_long = c.h_small[2];
         status_fresh = n_dirty == 0 && n_mid == 0 && n_long == 0;
         if (n_dirty > 0)

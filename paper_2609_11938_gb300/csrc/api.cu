@@ -52,8 +52,14 @@ opattr_status cuda_status(Ctx &c, cudaError_t e) {
 // environment makes growth fail, to exercise the out-of-memory path without
 // a GPU fault.
 opattr_status ensure_arena(Ctx &c, size_t bytes) {
+    if (bytes + c.arena_keep <= c.arena_cap) return OPATTR_OK;
+    if (c.agg_ready && !c.join_korder) {
+        // nothing but zeroed counters: no reason to hold two arenas
+        c.agg_ready = false;
+        c.arena_keep = 0;
+        if (bytes <= c.arena_cap) return OPATTR_OK;
+    }
     bytes += c.arena_keep;
-    if (bytes <= c.arena_cap) return OPATTR_OK;
     if (c.arena_fixed) return OPATTR_E_OOM;
     const char *fault = getenv("OPATTR_FAULT");
     if (fault && strcmp(fault, "alloc") == 0) return OPATTR_E_OOM;
@@ -233,7 +239,11 @@ opattr_status read_status(Ctx &c, int n_extra, const SmallCopy *extra) {
     cp[n++] = SmallCopy{c.h_status, c.d_status, sizeof(DevStatus)};
     for (int q = 0; q < n_extra; ++q) cp[n++] = extra[q];
     opattr_status st = copy_small_n(c, n, cp, cudaMemcpyDeviceToHost);
-    if (st) return st;
+    return st ? st : sync_status(c);
+}
+
+opattr_status sync_status(Ctx &c) {
+    if (c.last_error != cudaSuccess) return cuda_status(c, c.last_error);
     cudaError_t e = cudaStreamSynchronize(c.stream);
     if (e != cudaSuccess) return cuda_status(c, e);
     if (c.timing) timing_collect(c);
@@ -428,6 +438,8 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
             c.enclose_pending = c.match_pending = c.keep_status = c.no_spec = false;
             c.max_ncu = nullptr;
             c.max_known = false;
+            c.agg_words = 0;
+            c.agg_ready = false;
         }
     } scope(c);
     // The matching can go ahead on the taking that the records are in order, so
@@ -444,6 +456,10 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
         c.enclose_k_sorted = -1;
         c.spec_k = 0;
         c.spec_ran = false;
+        c.arena_keep = 0;
+        c.agg_ready = false;
+        // (an n_ops beyond the records is left to the aggregation's own request)
+        c.agg_words = (int64_t)n_ops <= kernels->n + ranges->n ? agg_counter_words(n_ops) : 0;
         c.enclose_pending = c.match_pending = c.keep_status = c.no_spec = false;
         c.max_ncu = full && !same && !dd && kernels->n + ncu->n < (1ll << 32) ? ncu : nullptr;
         c.max_known = false;
@@ -458,12 +474,15 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
         opattr_status st = finish(c, do_enclose(c, kernels, ranges, range_of_kernel, n_op_enclosing));
         c.defer_status = false;
         if (st < 0) return st;
+        const size_t agg_bytes = (sizeof(uint32_t) * (size_t)c.agg_words + 255) & ~(size_t)255;
+        c.agg_ready = c.agg_words > 0;
+        c.arena_keep = std::max(c.arena_keep, agg_bytes);
         c.order_from_enclose = true;
         opattr_status sm =
             finish(c, do_match(c, kernels, ncu, dedup, ncu_idx_of_kernel, match_kind, host_summary));
         c.order_from_enclose = false;
         c.join_korder = nullptr;             // the aggregation needs no time order
-        c.arena_keep = 0;
+        c.arena_keep = c.agg_ready ? agg_bytes : 0;
         if (sm < 0) {
             // the enclosure's error comes before the matching's
             if (!c.enclose_pending) return sm;

@@ -133,6 +133,11 @@ struct Ctx {
     // within a join: the matching was the identity pairing (row k for kernel
     // k), so the aggregation need not read the row indices
     bool rows_identity = false;
+    // within a join: the aggregation's counters, agg_words of them at the start
+    // of the arena, are zeroed by the enclosure's reset (agg_ready) unless the
+    // arena has to grow on the way
+    int64_t agg_words = 0;
+    bool agg_ready = false;
     int64_t launches = 0;
     bool timing = false;
     std::string timing_only;         // with timing on: bracket only this kernel (empty = all)
@@ -170,6 +175,10 @@ int sm_count(Ctx &c);
 // The status of an enclosure that read `H` (a NOT_NESTED found beside
 // F_LEVEL_FIXUP does not count: the run on sorted ranges decides).
 opattr_status enclose_verdict(const DevStatus &H, int64_t K);
+// Words of the aggregation's counters for n_ops operators: a few of its own,
+// the status words of the scan, and one per operator and one more.
+constexpr int AGG_OWN_WORDS = 8;
+int64_t agg_counter_words(uint32_t n_ops);
 // The matching's counts and status from the status block (c.match_sum holds
 // what was known before it ran).
 opattr_status match_verdict(Ctx &c, opattr_match_summary *sum);
@@ -203,6 +212,8 @@ opattr_status await_status(Ctx &c);
 // The status block back to the host (with up to three more device->host
 // transfers in the same launch), then a stream synchronize.
 opattr_status read_status(Ctx &c, int n_extra = 0, const SmallCopy *extra = nullptr);
+// The same where a kernel on the stream has stored the block to h_status itself.
+opattr_status sync_status(Ctx &c);
 opattr_status cuda_status(Ctx &c, cudaError_t e);
 int timing_slot(Ctx &c, const char *name);
 void timing_begin(Ctx &c, int slot, cudaEvent_t *e0, cudaEvent_t *e1);
@@ -324,6 +335,11 @@ __device__ __forceinline__ T block_sum(T v, T *warp_buf) {
     T total;
     block_exclusive_scan(v, warp_buf, &total);
     return total;
+}
+
+// p[0 .. n) = 0 by the whole grid: scratch of the launch after this one.
+__device__ __forceinline__ void zero_words(uint32_t *p, int64_t n) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = 0;
 }
 
 // Sum v over the block and add the total to *dst with one atomic.  Every

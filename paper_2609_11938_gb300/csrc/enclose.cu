@@ -1022,19 +1022,22 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     const int64_t tiles = B.parts * B.tp;
     Need nd;
     nd.add<uint32_t>(tiles + 1).add<uint32_t>(B.parts).add<uint32_t>(B.parts * LEVELS).add<uint32_t>(256);
+    if (c.agg_words > 0) nd.add<uint32_t>(c.agg_words);
     const bool keep_order = c.in_join && K > 0;       // a join keeps the time order for its matching
     if (keep_order) nd.add<uint32_t>(K);
     opattr_status st = ensure_arena(c, nd.bytes + 4096);
     if (st) return st;
     Arena a(c);
-    uint32_t *kept_order = keep_order ? a.take<uint32_t>(K) : nullptr;     // first: the start of the arena
+    // first, at the start of the arena, what outlives the enclosure
+    uint32_t *agg = c.agg_words > 0 ? a.take<uint32_t>(c.agg_words) : nullptr;
+    uint32_t *kept_order = keep_order ? a.take<uint32_t>(K) : nullptr;
     B.lvlmask = a.take<uint32_t>(256);
     B.tile_r = a.take<uint32_t>(tiles + 1);
     B.row_len = a.take<uint32_t>(B.parts);
     B.rows = a.take<uint32_t>(B.parts * LEVELS);
     if (!B.lvlmask || !B.tile_r || !B.row_len || !B.rows) return OPATTR_E_OOM;
-    const ZeroRun z{B.lvlmask, 256};
-    if ((st = reset_status(c, 1, &z))) return st;
+    const ZeroRun z[2] = {{B.lvlmask, 256}, {agg, agg ? c.agg_words : 0}};
+    if ((st = reset_status(c, 2, z))) return st;
 
     EncView V{};
     V.k_start = kern->start_ns;
@@ -1154,7 +1157,7 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
         if (kept_order) {
             cudaMemcpyAsync(kept_order, korder, sizeof(uint32_t) * K, cudaMemcpyDeviceToDevice, c.stream);
             c.join_korder = kept_order;
-            c.arena_keep = (sizeof(uint32_t) * (size_t)K + 255) & ~(size_t)255;
+            c.arena_keep = (size_t)(reinterpret_cast<char *>(kept_order + K) - c.arena + 255) & ~(size_t)255;
         }
     }
     const EncView raw = V;

@@ -200,8 +200,9 @@ __device__ __forceinline__ int64_t upper_bound_u32(const uint32_t *a, int64_t n,
 __global__ void k_pair_keys(const uint32_t *__restrict__ rk, const uint32_t *__restrict__ kname,
                             const uint8_t *__restrict__ kstream, int64_t nrep, const uint32_t *__restrict__ nname,
                             const uint8_t *__restrict__ nstream, int64_t n, uint32_t *__restrict__ key,
-                            DevStatus *st) {
+                            uint32_t *chain, int64_t nchain, DevStatus *st) {
     pdl_wait();
+    zero_words(chain, nchain);               // of the runs' scan
     int bad = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const bool row = i >= nrep;
@@ -675,6 +676,7 @@ opattr_status do_match(Ctx &c, const opattr_kernels *kern, const opattr_ncu *ncu
     }
     if (!direct_done && (nrep > 0 || M > 0)) {
         const int64_t n = nrep + M;
+        uint32_t *chain = reinterpret_cast<uint32_t *>(nb);          // free by now; two words per 4,096 elements fit
         if (max_key == 0) {
             launch(c, "max_key", k_max_key, dim3(grid_for(N, 256 * 8, 1024)), dim3(256), 0, kern->name_id, kern->stream,
                    K, ncu->name_id, ncu->stream, M, c.d_status);
@@ -682,15 +684,13 @@ opattr_status do_match(Ctx &c, const opattr_kernels *kern, const opattr_ncu *ncu
             max_key = c.h_status->cnt[C_MAX_KEY];
         }
         launch(c, "pair_keys", k_pair_keys, dim3(grid_for(n, 256 * 4, REDUCE_GRID)), dim3(256), 0, rk, kern->name_id,
-               kern->stream, nrep, ncu->name_id, ncu->stream, n, b0, c.d_status);
+               kern->stream, nrep, ncu->name_id, ncu->stream, n, b0, chain, chain_words(n), c.d_status);
         uint32_t *sk = nullptr, *sv = nullptr;
         radix_sort_pairs<uint32_t>(c, b0, b1, b2, b3, n, bits_for(max_key), true, hist, part, &sk, &sv);
         uint32_t *run = sk == b0 ? b2 : b0, *start = sv == b1 ? b3 : b1;
         uint32_t *n_run = reinterpret_cast<uint32_t *>(dsm + 2);
-        const ZeroRun zn{part, chain_words(n)};
-        if ((st = zero_runs(c, 1, &zn))) return st;
         launch(c, "runs", k_runs, dim3(grid_for(n, SCAN_TILE)), dim3(SCAN_THREADS), 0, (const uint32_t *)sk,
-               (const uint32_t *)sv, nrep, n, make_chain(c, part, n), run, start, n_run);
+               (const uint32_t *)sv, nrep, n, make_chain(c, chain, n), run, start, n_run);
         launch(c, "ordinal_join", k_ordinal_join, dim3(grid_for(n, 256 * 2, REDUCE_GRID)), dim3(256), 0,
                (const uint32_t *)sk, (const uint32_t *)sv, nrep, n, (const uint32_t *)run, (const uint32_t *)start,
                (const uint32_t *)n_run, rk, mode, out_idx, out_kind, c.d_status);

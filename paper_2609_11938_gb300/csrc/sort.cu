@@ -145,8 +145,10 @@ __global__ void __launch_bounds__(1024) k_scan_small(const uint32_t *in, uint32_
     if (threadIdx.x == 0 && total_dev) *total_dev = tot;
 }
 
+int64_t scan_clean_words(int64_t n) { return n <= SCAN_ONE_BLOCK ? 0 : chain_words(n); }
+
 void scan_exclusive_u32(Ctx &c, const uint32_t *in, uint32_t *out, int64_t n, uint32_t *partials,
-                        uint32_t *total_dev) {
+                        uint32_t *total_dev, bool clean) {
     int64_t nt = (n + SCAN_TILE - 1) / SCAN_TILE;
     if (n <= 0) {
         if (total_dev) cudaMemsetAsync(total_dev, 0, sizeof(uint32_t), c.stream);
@@ -164,7 +166,7 @@ void scan_exclusive_u32(Ctx &c, const uint32_t *in, uint32_t *out, int64_t n, ui
         return;
     }
     const ZeroRun z{partials, chain_words(n)};
-    zero_runs(c, 1, &z);
+    if (!clean) zero_runs(c, 1, &z);
     launch(c, "scan", k_scan_onepass, dim3((unsigned)nt), dim3(SCAN_THREADS), 0, in, out, n, make_chain(c, partials, n),
            total_dev);
 }
@@ -178,8 +180,10 @@ __device__ __forceinline__ unsigned digit_of(K key, int shift) {
 // Per tile, the count of each digit; hist is digit-major: hist[d * ntiles + tile].
 template <typename K>
 __global__ void __launch_bounds__(RADIX_THREADS) k_radix_upsweep(const K *__restrict__ keys, int64_t n, int shift,
-                                                                 uint32_t *__restrict__ hist, int64_t ntiles) {
+                                                                 uint32_t *__restrict__ hist, int64_t ntiles,
+                                                                 uint32_t *clean, int64_t nclean) {
     pdl_wait();
+    zero_words(clean, nclean);
     __shared__ uint32_t h[RADIX_THREADS / 32][RADIX_BINS];
     const unsigned w = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < (RADIX_THREADS / 32) * RADIX_BINS; i += RADIX_THREADS) (&h[0][0])[i] = 0;
@@ -316,8 +320,8 @@ void radix_sort_pairs(Ctx &c, K *k0, uint32_t *v0, K *k1, uint32_t *v1, int64_t 
     for (int shift = 0; shift < bits && n > 0; shift += RADIX_BITS) {
         const bool first = shift == 0;
         launch(c, "radix_upsweep", k_radix_upsweep<K>, dim3((unsigned)ntiles), dim3(RADIX_THREADS), 0,
-               (const K *)ka, n, shift, hcount, ntiles);
-        scan_exclusive_u32(c, hcount, hoff, ntiles * RADIX_BINS, partials, nullptr);
+               (const K *)ka, n, shift, hcount, ntiles, partials, scan_clean_words(ntiles * RADIX_BINS));
+        scan_exclusive_u32(c, hcount, hoff, ntiles * RADIX_BINS, partials, nullptr, true);
         launch(c, "radix_downsweep", k_radix_downsweep<K>, dim3((unsigned)ntiles), dim3(RADIX_THREADS),
                downsweep_smem<K>(), (const K *)ka, (const uint32_t *)((first && iota) ? nullptr : va), kb, vb, n,
                shift, (const uint32_t *)hoff, ntiles);

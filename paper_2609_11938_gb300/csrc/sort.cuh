@@ -19,9 +19,12 @@ constexpr int RADIX_BINS = 1 << RADIX_BITS;
 inline int64_t scan_scratch_elems(int64_t n) { return 2 * ((n + SCAN_TILE - 1) / SCAN_TILE) + 4; }
 
 // out[i] = in[0] + ... + in[i-1]; *total_dev (device, may be NULL) = sum of all.
-// in and out may alias.  `partials` holds scan_scratch_elems(n) u32.
+// in and out may alias.  `partials` holds scan_scratch_elems(n) u32; with
+// `clean` its first scan_clean_words(n) are zero already (the launch before
+// cleared them: 3 us less than a launch of their own).
 void scan_exclusive_u32(Ctx &c, const uint32_t *in, uint32_t *out, int64_t n, uint32_t *partials,
-                        uint32_t *total_dev);
+                        uint32_t *total_dev, bool clean = false);
+int64_t scan_clean_words(int64_t n);
 
 // Scratch for a radix sort or a digit pass over n keys: the tiles' digit
 // counts (a tiles x RADIX_BINS matrix) and, after them, room for their scan
@@ -181,8 +184,9 @@ __device__ __forceinline__ void chained_scan(const Chain &C, int64_t n, At at, P
 // peer groups from one ballot per digit bit.
 template <typename DigitFn>
 __global__ void __launch_bounds__(RADIX_THREADS) k_digit_hist(DigitFn digit, int64_t n, uint32_t *__restrict__ hist,
-                                                              int64_t ntiles) {
+                                                              int64_t ntiles, uint32_t *clean, int64_t nclean) {
     pdl_wait();
+    zero_words(clean, nclean);
     __shared__ uint32_t h[RADIX_THREADS / 32][RADIX_BINS];
     const unsigned w = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < (RADIX_THREADS / 32) * RADIX_BINS; i += RADIX_THREADS) (&h[0][0])[i] = 0;
@@ -267,11 +271,11 @@ uint32_t *digit_offsets(Ctx &c, DigitFn digit, int64_t n, uint32_t *hist, uint32
                         int nbins = RADIX_BINS) {
     if (n <= 0) return hist;
     const int64_t ntiles = (n + RADIX_TILE - 1) / RADIX_TILE;
-    launch(c, "digit_hist", k_digit_hist<DigitFn>, dim3((unsigned)ntiles), dim3(RADIX_THREADS), 0, digit, n, hist,
-           ntiles);
     const int64_t m = ntiles * (int64_t)(nbins < 1 ? 1 : nbins);
+    launch(c, "digit_hist", k_digit_hist<DigitFn>, dim3((unsigned)ntiles), dim3(RADIX_THREADS), 0, digit, n, hist,
+           ntiles, partials, scan_clean_words(m));
     uint32_t *offs = hist + ntiles * RADIX_BINS;
-    scan_exclusive_u32(c, hist, offs, m, partials, nullptr);
+    scan_exclusive_u32(c, hist, offs, m, partials, nullptr, true);
     return offs;
 }
 

@@ -1,10 +1,14 @@
 """Where the aggregation hands an operator over (GPU): one lane, a block of 128
 threads, a block of 512, the pieces pass, with the lane's share following the
 average length; with and without null counters, against the oracle."""
+import dataclasses
+
 import numpy as np
 import pytest
 
 import oracle
+import tracegen
+from gpu_util import assert_parity, gpu_run
 from test_gpu_parity import _agg_inputs, _check_aggregate, _gpu_aggregate, opa  # noqa: F401
 
 pytestmark = pytest.mark.gpu
@@ -19,6 +23,31 @@ def test_operator_lengths(opa, n_small, k, nan_frac):  # noqa: F811
     t, rk, idx = _agg_inputs(31 + n_small, sum(lens) + k, lens, n_small, nan_frac)
     o = oracle.aggregate(t.k_dur, rk, t.r_op, t.counters, idx, t.n_ops)
     _check_aggregate(_gpu_aggregate(opa, t, rk, idx), o)
+
+
+@pytest.mark.parametrize("n_ops", [1, 4094, 4095, 4096, 32_766, 32_767, 32_768, 77_823, 77_824, 77_825])
+@pytest.mark.parametrize("call", ["aggregate", "join", "join_many"])
+def test_operator_counts(opa, n_ops, call):  # noqa: F811
+    """Where the offsets come from (the count's last block, one block, a chained
+    scan) and how many operators a warp takes; with the counters zeroed for the
+    call, in a join with those the enclosure's reset left (twice: the arena
+    grows in the first), and in one with more operators than records."""
+    if call == "aggregate":
+        t, rk, idx = _agg_inputs(n_ops, n_ops + 5000, [], n_ops)
+        _check_aggregate(_gpu_aggregate(opa, t, rk, idx),
+                         oracle.aggregate(t.k_dur, rk, t.r_op, t.counters, idx, t.n_ops))
+        return
+    t = tracegen.generate("large", n_kernels=int(n_ops * 4.2) if call == "join" else 500, n_streams=2, seed=9)
+    t = dataclasses.replace(t, n_ops=max(n_ops, t.n_ops))
+    want = gpu_run(t)
+    assert_parity(want, oracle.run(t, enclose_mode="indexed"))
+    tr = opa.to_device(t)
+    with opa.Context(0) as ctx:
+        for _ in range(2):
+            st, out, ops, summary, totals = ctx.join(tr)
+            assert st == want["match_status"] and summary == want["summary"] and totals == want["totals"]
+            for k, v in ops.items():
+                np.testing.assert_array_equal(v.cpu().numpy(), want["ops"][k])
 
 
 def test_infinite_counter_in_a_long_operator(opa):  # noqa: F811
