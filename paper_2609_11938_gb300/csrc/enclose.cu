@@ -358,19 +358,21 @@ __global__ void __launch_bounds__(1024) k_enc_carry(uint32_t *__restrict__ rows,
 // entries, E_NONE none.
 constexpr unsigned E_NONE = 0xFFFFu;
 constexpr unsigned D_DEPTH = 31u, D_MIXED = 32u;     // bits of `dep`
-template <int THREADS_, int BLOCKS_>
+template <int THREADS_, int BLOCKS_, bool JUMP_>
 struct EncTile {
     static constexpr int THREADS = THREADS_, BLOCKS = BLOCKS_;
+    static constexpr bool JUMP = JUMP_;
     static constexpr int WORDS = 16;                 // ranges of a step, 32 to a group
     static constexpr int SR = 32 * WORDS;
     static constexpr int RPT = WORDS / (THREADS / 32);   // groups of a warp
     uint32_t *ss, *se, *si;      // start, end (relative), position | kind << 30
-    uint32_t *re;                // end of the outermost ancestor
     uint32_t *amask;             // [ns] depths with an open range, per compact stream
     uint32_t *smask;             // [ns][WORDS] the stream's ranges among the tile's, one bit each
     uint32_t *sgroups;           // [ns] the groups that hold some
     uint16_t *par, *prev, *best; // parent; the entry before on the stream; where the climb begins (below)
     uint16_t *va;                // innermost operator of the entry's chain
+    uint16_t *top;               // outermost ancestor
+    uint16_t *jump;              // ancestor four levels up, E_NONE none (where chains are long)
     uint16_t *before;            // [ns][WORDS] the stream's last entry before each group (before the first one
                                  // its deepest open range), E_NONE none
     uint32_t *lgroups;           // [nl / 2] the groups that hold ranges of a level, 16 bits each
@@ -388,7 +390,6 @@ struct EncTile {
         ss = reinterpret_cast<uint32_t *>(take((size_t)cap * 4));
         se = reinterpret_cast<uint32_t *>(take((size_t)cap * 4));
         si = reinterpret_cast<uint32_t *>(take((size_t)cap * 4));
-        re = reinterpret_cast<uint32_t *>(take((size_t)cap * 4));
         amask = reinterpret_cast<uint32_t *>(take((size_t)ns * 4));
         smask = reinterpret_cast<uint32_t *>(take((size_t)ns * WORDS * 4));
         sgroups = reinterpret_cast<uint32_t *>(take((size_t)ns * 4));
@@ -397,6 +398,8 @@ struct EncTile {
         prev = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
         best = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
         va = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
+        top = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
+        jump = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
         before = reinterpret_cast<uint16_t *>(take((size_t)ns * WORDS * 2));
         cbase = reinterpret_cast<uint16_t *>(take(512));
         scid = reinterpret_cast<uint16_t *>(take(512));
@@ -412,8 +415,8 @@ struct EncTile {
         return (size_t)(SR + nl) * 26 + SR + (size_t)(WORDS + 2) * nl + (size_t)ns * (8 + 6 * WORDS + 1) + 1024 + 512;
     }
 };
-using EncTileA = EncTile<256, 4>;
-using EncTileB = EncTile<512, 2>;
+using EncTileA = EncTile<256, 4, false>;
+using EncTileB = EncTile<512, 2, true>;
 constexpr int EN_LEVELS_A = 512, EN_STREAMS_A = 64;      // levels and streams of the common layout
 constexpr int EN_LEVELS_B = 2048;                        // of the wide one: 64 streams of every depth
 constexpr int64_t EN_TILE = 2048, EN_TILE_MIN = 512;     // events of a tile; of a part's one tile in small traces
@@ -547,7 +550,6 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
         const unsigned longs = __ballot_sync(0xffffffffu, live && a < z);
         const unsigned gap = ~m & le;
         const unsigned lo = gap ? 32u - __clz(gap) : 0u;                         // the run's outermost level
-        const uint32_t out = __shfl_sync(0xffffffffu, z, (int)(lo & 31u));
         if (lane == 0) S.amask[q] = m;
         if (lane < WORDS) S.before[q * WORDS + lane] = m ? (uint16_t)(e0 + 31u - __clz(m)) : (uint16_t)E_NONE;
         if (!live) return;
@@ -562,7 +564,8 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
         S.prev[e] = m & lt ? (uint16_t)(e0 + 31u - __clz(m & lt)) : (uint16_t)E_NONE;
         S.va[e] = seen ? (uint16_t)(e0 + 31u - __clz(seen)) : (uint16_t)E_NONE;
         S.vn[e] = (uint8_t)__popc(seen);
-        S.re[e] = out;
+        S.top[e] = (uint16_t)(e0 + lo);
+        if (TL::JUMP) S.jump[e] = lane >= lo + 4 ? (uint16_t)(e - 4) : (uint16_t)E_NONE;
         S.best[e] = longs & le ? (uint16_t)(e0 + 31u - __clz(longs & le)) : (uint16_t)E_NONE;
     };
     for (int q = (int)warp; q < ns; q += WARPS) {                                // a warp per stream, a lane per depth
@@ -802,7 +805,8 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                 return w;
             };
             for (int e = tid; e < nr; e += THREADS) {
-                uint32_t ans = E_NONE, n = 0, x = e, top;
+                uint32_t ans = E_NONE, n = 0, x = e, top, far = E_NONE;
+                int up = 0;
                 bool on = true;
                 do {
                     const uint32_t kind = S.si[x] >> 30;
@@ -810,18 +814,23 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                     if (on && kind == KIND_OP && n++ == 0) ans = x;
                     top = x;
                     x = S.par[x];
+                    if (TL::JUMP && ++up == 4) far = x;
                 } while (x < SR);
-                uint32_t end = S.se[top];
                 if (x != E_NONE) {
                     if (on) {
                         if (n == 0) ans = S.va[x];
                         n += S.vn[x];
                     }
-                    end = S.re[x];
+                    top = S.top[x];
+                    if (TL::JUMP && up < 4) {                // on along the open ones, one slot to a level
+                        far = x - (4 - up);
+                        if (far < top) far = E_NONE;
+                    }
                 }
+                if (TL::JUMP) S.jump[e] = (uint16_t)far;
                 S.va[e] = (uint16_t)ans;
                 S.vn[e] = (uint8_t)n;
-                S.re[e] = end;
+                S.top[e] = (uint16_t)top;
                 S.best[e] = (uint16_t)best_of(e);
             }
             __syncthreads();
@@ -876,7 +885,9 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                             const bool at_start = S.ss[x] == T;
                             if (!at_start || !(S.dep[x] & D_MIXED)) {
                                 if (!at_start) x = S.best[x];
-                                if (x != E_NONE && S.re[x] >= T) {
+                                if (x != E_NONE && S.se[S.top[x]] >= T) {
+                                    if (TL::JUMP)
+                                        for (uint32_t u = x; u != E_NONE && S.se[u] < T; u = S.jump[u]) x = u;
                                     while (S.se[x] < T) x = S.par[x];
                                     ans = S.va[x];
                                     n = S.vn[x];
