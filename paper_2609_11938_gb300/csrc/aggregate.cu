@@ -61,14 +61,14 @@ constexpr int RENORM = 128;
 __device__ __noinline__ double finish_sum(float hi, float lo) {
     ff v{hi, lo};
     ff_renorm(v);
-    return ff_to_f64(v);
+    return ff_to_f64_fast(v);
 }
 __device__ __noinline__ double finish_dw(float hi, float lo, long long den) {
     ff v{hi, lo};
     ff_renorm(v);
-    return ff_div_i64_to_f64(v, den);
+    return ff_div_to_f64(v, split_i64(den));
 }
-__device__ __noinline__ double finish_max(float x) { return f32_to_f64_bits(x); }
+__device__ __noinline__ double finish_max(float x) { return f32_to_f64_fast(x); }
 constexpr unsigned ALL_COUNTERS = (1u << NC) - 1;
 
 // A duration as a normalised pair (as split_i64), the common case (< 2^48 ns)
@@ -239,6 +239,13 @@ struct AccF {
             v[2 * q] = x.x;
             v[2 * q + 1] = x.y;
         }
+        add(d, v);
+#pragma unroll
+        for (int i = 0; i < N_MAX; ++i) mx[i] = fmaxf(mx[i], f2_unpack(v[Acc::max_col(i) / 2]).y);
+    }
+
+    // One row's values into the sums.
+    __device__ __forceinline__ void add(long long d, const f32x2 (&v)[PAIRS]) {
         const ff dd = split_dur(d);
         const f32x2 dw = f2_pack(dd.hi, dd.hi), dn = f2_pack(-dd.hi, -dd.hi), dl = f2_pack(dd.lo, dd.lo);
         const f32x2 sw = f2_pack(1.f, dd.hi), sn = f2_pack(-1.f, -dd.hi), sl = f2_pack(0.f, dd.lo);
@@ -248,8 +255,6 @@ struct AccF {
             else if (p == 1 || p == 5 || p == 7) f2_accum_mul(hi[p], lo[p], v[p], sw, sn, sl);      // SUM DW
             else f2_accum_mul(hi[p], lo[p], v[p], dw, dn, dl);                                      // DW DW, DW MAX
         }
-#pragma unroll
-        for (int i = 0; i < N_MAX; ++i) mx[i] = fmaxf(mx[i], f2_unpack(v[Acc::max_col(i) / 2]).y);
         if (++terms >= RENORM) {
             terms = 0;
 #pragma unroll
@@ -302,6 +307,99 @@ struct AccF {
         }
 #pragma unroll
         for (int i = 0; i < N_MAX; ++i) agg[(int64_t)Acc::max_col(i) * n + op] = f32_to_f64_fast(mx[i]);
+    }
+};
+
+// AccF with nulls left out and infinite values reported, as Acc has it: a value
+// that takes no part adds zero, and its kernel's duration leaves that DW
+// counter's weight.
+struct AccN {
+    AccF f;
+    long long nanw[N_DW];
+    unsigned seen;
+    int bad;
+
+    __device__ __forceinline__ void init() {
+        f.init();
+#pragma unroll
+        for (int i = 0; i < N_DW; ++i) nanw[i] = 0;
+        seen = 0;
+        bad = 0;
+    }
+
+    __device__ __forceinline__ void accumulate(long long d, bool matched, const float4 *row) {
+        f.dsum += d;
+        if (!matched) return;
+        f.mc++;
+        f.dall += d;
+        f32x2 v[AccF::PAIRS], z = 0ull;
+#pragma unroll
+        for (int q = 0; q < NC / 4; ++q) {
+            const ulonglong2 x = reinterpret_cast<const ulonglong2 *>(row)[q];
+            v[2 * q] = x.x;
+            v[2 * q + 1] = x.y;
+        }
+        // (fmaxf passes a null over; an infinite one fails the call)
+#pragma unroll
+        for (int i = 0; i < N_MAX; ++i) f.mx[i] = fmaxf(f.mx[i], f2_unpack(v[Acc::max_col(i) / 2]).y);
+#pragma unroll
+        for (int p = 0; p < AccF::PAIRS; ++p) z = f2_fma(v[p], 0ull, z);
+        const float2 zz = f2_unpack(z);
+        unsigned valid = ALL_COUNTERS;
+        if (__fadd_rn(zz.x, zz.y) != 0.f) {          // NaN iff some value is NaN or infinite
+            unsigned inf = 0;
+#pragma unroll
+            for (int p = 0; p < AccF::PAIRS; ++p) {
+                float2 x = f2_unpack(v[p]);
+                const unsigned a = __float_as_uint(x.x) & 0x7FFFFFFFu, b = __float_as_uint(x.y) & 0x7FFFFFFFu;
+                if (a >= 0x7F800000u) {
+                    valid &= ~(1u << (2 * p));
+                    inf |= a == 0x7F800000u;
+                    x.x = 0.f;
+                }
+                if (b >= 0x7F800000u) {
+                    valid &= ~(2u << (2 * p));
+                    inf |= b == 0x7F800000u;
+                    x.y = 0.f;
+                }
+                v[p] = f2_pack(x.x, x.y);
+            }
+            bad |= (int)inf;
+#pragma unroll
+            for (int i = 0; i < N_DW; ++i)
+                if (!((valid >> Acc::dw_col(i)) & 1u)) nanw[i] += d;
+        }
+        seen |= valid;
+        f.add(d, v);
+    }
+
+    __device__ __forceinline__ void write(const AggIn &A, int64_t op, int kc) const {
+        A.out.kernel_count[op] = kc;
+        A.out.total_duration_ns[op] = f.dsum;
+        A.out.matched_count[op] = f.mc;
+        double *agg = A.out.agg;
+        const int64_t n = A.n_ops;
+        const double qnan = __longlong_as_double(0x7FF8000000000000ll);
+#pragma unroll
+        for (int i = 0; i < N_SUM; ++i) {
+            const int c = Acc::sum_col(i);
+            ff x = f.sum(c);
+            ff_renorm(x);
+            agg[(int64_t)c * n + op] = ((seen >> c) & 1u) ? ff_to_f64_fast(x) : qnan;
+        }
+#pragma unroll
+        for (int i = 0; i < N_DW; ++i) {
+            const int c = Acc::dw_col(i);
+            const long long den = f.dall - nanw[i];
+            ff x = f.sum(c);
+            ff_renorm(x);
+            agg[(int64_t)c * n + op] = (((seen >> c) & 1u) && den > 0) ? ff_div_to_f64(x, split_dur(den)) : qnan;
+        }
+#pragma unroll
+        for (int i = 0; i < N_MAX; ++i) {
+            const int c = Acc::max_col(i);
+            agg[(int64_t)c * n + op] = ((seen >> c) & 1u) ? f32_to_f64_fast(f.mx[i]) : qnan;
+        }
     }
 };
 
@@ -591,29 +689,6 @@ struct OpsWarp {
 };
 constexpr size_t AG_SMEM = sizeof(OpsWarp) * AG_WARPS;
 
-// An op whose fast sums saw a null or infinite value: the segment again, in
-// the same order, with Acc.  Returns 1 if a value was infinite.
-__device__ __noinline__ int op_careful(const uint32_t *seg, uint32_t len, AggIn A, int64_t o) {
-    Acc acc;
-    acc.init();
-    // kernel t + 1's duration and row index, and t + 2's index, in flight during t
-    uint32_t k = len > 1 ? seg[1] : 0u;
-    long long d = len > 0 ? A.dur[seg[0]] : 0;
-    int32_t j = len > 0 ? A.ncu_idx[seg[0]] : -1;
-    for (uint32_t t = 0; t < len; ++t) {
-        const long long d1 = t + 1 < len ? A.dur[k] : 0;
-        const int32_t j1 = t + 1 < len ? A.ncu_idx[k] : -1;
-        const uint32_t k2 = t + 2 < len ? seg[t + 2] : 0u;
-        const bool ok = j >= 0 && j < A.M;
-        acc.accumulate(d, ok, reinterpret_cast<const float4 *>(A.counters + (int64_t)(ok ? j : 0) * NC));
-        d = d1;
-        j = j1;
-        k = k2;
-    }
-    acc.write(A, o);
-    return acc.bad;
-}
-
 // Ascending order of a segment, sorted in place when it is not (insertion
 // sort: the segment is two ascending runs at worst).
 __device__ __forceinline__ void sort_segment(uint32_t *seg, uint32_t len) {
@@ -826,19 +901,74 @@ __global__ void __launch_bounds__(AG_THREADS, AG_BLOCKS) k_agg_ops(const uint32_
     if (threadIdx.x < 3) report.counts[threadIdx.x] = __ldcg(A.ctr + 1 + threadIdx.x);
 }
 
-// The ops k_agg_ops listed as dirty: one thread each puts the segment in
-// ascending kernel index (in place) and redoes it with Acc, which leaves
-// nulls out and reports infinite values.  A separate pass keeps that rare,
-// register-hungry path out of the ops pass.
-__global__ void k_agg_careful(const uint32_t *__restrict__ off, uint32_t *list, AggIn A, DevStatus *st) {
+// The ops k_agg_ops listed as dirty: one lane each puts the segment in
+// ascending kernel index (in place) and redoes it with AccN, which leaves
+// nulls out and reports infinite values.  A separate pass keeps that
+// register-hungry path out of the ops pass (within it, for the lanes concerned,
+// the pass spilled: 853 us on 20M kernels without any null against 696).  Rows
+// reach the lanes as they do there, the warp copying together and AG_SLOTS
+// kernels ahead, counters two to a register.  Bound by issue at 12 warps a
+// multiprocessor (1.6 instructions a cycle): 176,000 ops, 1M kernels with 2 % of
+// nulls, 75 us; 86 with Acc and each lane reading its own rows.
+__global__ void __launch_bounds__(AG_THREADS, AG_BLOCKS) k_agg_careful(const uint32_t *__restrict__ off,
+                                                                       uint32_t *list, AggIn A, DevStatus *st) {
     pdl_wait();
+    __shared__ float4 row_s[AG_WARPS][AG_SLOTS][32][NC / 4];
+    __shared__ long long dur_s[AG_WARPS][AG_SLOTS][32];
+    const unsigned lane = lane_id(), w = threadIdx.x / 32;
+    auto &row = row_s[w];
+    auto &dur = dur_s[w];
+    const float4 *rows = reinterpret_cast<const float4 *>(A.counters);
+    auto row_of = [&](uint32_t k) -> int32_t {
+        const int32_t j = A.ncu_idx[k];
+        return j < A.M ? j : -1;
+    };
     int bad = 0;
     const unsigned n = A.ctr[1];
-    for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-        const uint32_t o = A.dirty[e];
-        const uint32_t s0 = off[o], len = off[o + 1] - s0;
-        sort_segment(list + s0, len);
-        bad |= op_careful(list + s0, len, A, o);
+    for (unsigned e0 = (blockIdx.x * AG_WARPS + w) * 32; e0 < n; e0 += gridDim.x * AG_WARPS * 32) {
+        const bool mine = e0 + lane < n;
+        const uint32_t o = mine ? A.dirty[e0 + lane] : 0u;
+        const uint32_t s0 = mine ? off[o] : 0u, len = mine ? off[o + 1] - s0 : 0u;
+        const uint32_t most = __reduce_max_sync(0xffffffffu, len);
+        uint32_t *seg = list + s0;
+        sort_segment(seg, len);
+        __syncwarp();
+        auto issue = [&](uint32_t t, uint32_t k, int32_t j) {
+            if (t < len) cp_async8(&dur[t % AG_SLOTS][lane], A.dur + k);
+            cp_async_rows(row[t % AG_SLOTS], rows, j);
+            cp_async_commit();
+        };
+        AccN acc;
+        acc.init();
+        unsigned have = 0;
+#pragma unroll
+        for (uint32_t t = 0; t < (uint32_t)AG_SLOTS; ++t) {
+            const uint32_t kt = t < len ? seg[t] : 0u;
+            const int32_t jt = t < len ? row_of(kt) : -1;
+            issue(t, kt, jt);
+            have |= (jt >= 0 ? 1u : 0u) << t;
+        }
+        uint32_t k2 = AG_SLOTS < len ? seg[AG_SLOTS] : 0u;
+        int32_t j2 = AG_SLOTS < len ? row_of(k2) : -1;
+        for (uint32_t t = 0; t < most; ++t) {
+            const uint32_t k3 = t + AG_SLOTS + 1 < len ? seg[t + AG_SLOTS + 1] : 0u;
+            const int32_t j3 = t + AG_SLOTS + 1 < len ? row_of(k3) : -1;
+            cp_async_wait<AG_SLOTS - 1>();
+            __syncwarp();
+            const unsigned bit = 1u << (t % AG_SLOTS);
+            if (t < len) acc.accumulate(dur[t % AG_SLOTS][lane], have & bit, row[t % AG_SLOTS][lane]);
+            __syncwarp();
+            issue(t + AG_SLOTS, k2, j2);
+            have = j2 >= 0 ? have | bit : have & ~bit;
+            k2 = k3;
+            j2 = j3;
+        }
+        cp_async_wait<0>();
+        __syncwarp();
+        if (mine) {
+            acc.write(A, o, (int)len);
+            bad |= acc.bad;
+        }
     }
     if (bad) set_err(st, ERR_INVALID);
 }
@@ -1354,7 +1484,7 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
         launch(c, "agg_ops", k_agg_ops, dim3(grid), dim3(AG_THREADS), AG_SMEM, (const uint32_t *)off, list, in,
                (int)c.enclose_pending, (const DevStatus *)c.d_status, report);
         // the ops the pass left: listed with a null or infinite value (redone
-        // by k_agg_careful, a thread each), longer than a lane takes (a block
+        // by k_agg_careful, a lane each), longer than a lane takes (a block
         // each) and longer still (the pieces pass); the counts come back with
         // the status
         const SmallCopy counts{c.h_small, ctr + 1, 3 * sizeof(uint32_t)};
@@ -1362,8 +1492,8 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
         const uint32_t n_dirty = c.h_small[0], n_mid = c.h_small[1], n_long = c.h_small[2];
         status_fresh = n_dirty == 0 && n_mid == 0 && n_long == 0;
         if (n_dirty > 0)
-            launch(c, "agg_careful", k_agg_careful, dim3(grid_for(n_dirty, 128)), dim3(128), 0, (const uint32_t *)off,
-                   list, in, c.d_status);
+            launch(c, "agg_careful", k_agg_careful, dim3(grid_for(n_dirty, AG_THREADS)), dim3(AG_THREADS), 0,
+                   (const uint32_t *)off, list, in, c.d_status);
         if (n_mid > 0) {
             launch(c, "agg_mid", k_agg_mid<128>, dim3(std::min<uint32_t>(n_mid, 4u * sms)), dim3(128), 0,
                    (const uint32_t *)off, (const uint32_t *)list, in, c.d_status);

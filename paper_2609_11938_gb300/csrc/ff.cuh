@@ -255,18 +255,17 @@ __device__ __forceinline__ double ff_mul_to_f64(ff a, ff b) {
     return ff_to_f64_fast(fast_two_sum(p, e));
 }
 
-// (n.hi + n.lo) / D for an int64 D > 0, as a double within a few units of
-// 2^-46 relative: q1 from an approximate reciprocal, then one correction from
-// the exact residual.
-__device__ __forceinline__ double ff_div_i64_to_f64(ff n, long long D) {
-    const ff d = split_i64(D);
+// (n.hi + n.lo) / (d.hi + d.lo), d a normalised pair above 0, as a double within
+// a few units of 2^-46 relative: q1 from an approximate reciprocal, then one
+// correction from the exact residual.
+__device__ __forceinline__ double ff_div_to_f64(ff n, ff d) {
     float inv;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(d.hi));
     const float q1 = __fmul_rn(n.hi, inv);
     const float r0 = __fmaf_rn(-q1, d.hi, n.hi);            // exact residual of the leading quotient
     const float r = __fadd_rn(__fmaf_rn(-q1, d.lo, r0), n.lo);
     const float q2 = __fmul_rn(r, inv);
-    return ff_to_f64(fast_two_sum(q1, q2));
+    return ff_to_f64_fast(fast_two_sum(q1, q2));
 }
 
 }  // namespace opattr
