@@ -205,9 +205,9 @@ struct Acc {
 // weight is dall.
 //
 // Counters go two to a register through the packed fp32 instructions (97M warp
-// instructions for 4M kernels against 152M), neighbours as they lie in the row: a pair of DW counters weighs the duration, SUM beside
-// DW weighs (1, duration) -- exact, 1 * x + 0 -- and the two MAX counters ride
-// along as probes (their sums are not used; should one overflow, the op is done
+// instructions for 4M kernels against 152M), neighbours as they lie in the row:
+// a pair of DW counters weighs the duration, SUM beside DW weighs (1, duration)
+// -- exact, 1 * x + 0 -- and the two MAX counters ride along as probes (their sums are not used; should one overflow, the op is done
 // again like any with an infinite value).
 struct AccF {
     static constexpr int PAIRS = NC / 2;
@@ -658,25 +658,29 @@ __global__ void __launch_bounds__(SL_THREADS) k_agg_sort_long(const uint32_t *__
 // band of op ids whatever each warp's pace, and with op ids in range order
 // the kernels and outputs of that band stay in L2.  The chunk's segments are
 // one contiguous run of the list; when it fits it is first copied to shared
-// memory by coalesced loads, and each thread checks its segments there and,
+// memory, and each thread checks its segments there and,
 // in the rare case the count pass met an op in two runs, sorts them in place,
 // so segments are walked in ascending kernel index (a larger chunk reads the
 // list in place).  Ops longer than lane_max are listed instead, for a block
 // each or for the pieces pass: a lane waits up to a microsecond for each of its
 // kernels, and one op of 250 held the pass (4M kernels with fusion operators:
-// 589 us) for four times as long as all the others.  While a kernel is added, the counter rows and durations
-// of the next two arrive in per-thread shared-memory slots by asynchronous
-// copy (cp.async), with their row indices loaded a step earlier still (or
-// taken to be the kernel indices when the count pass found every row to be
-// its kernel's own index).
+// 589 us) for four times as long as all the others.  While a kernel is added,
+// the counter rows and durations of the next two arrive in per-thread
+// shared-memory slots by asynchronous copy (cp.async), with their row indices
+// loaded a step earlier still (or taken to be the kernel indices when the count
+// pass found every row to be its kernel's own index).
 constexpr int AG_THREADS = 128;
 constexpr int AG_WARPS = AG_THREADS / 32;
-constexpr int AG_CHUNK = 64;                    // op ids per warp and chunk
+constexpr int AG_CHUNK = 64;                   // op ids per warp and chunk, at most
 constexpr int AG_LBUCKETS = 32;
-// Four blocks of four warps per multiprocessor: with the 96 registers of five
-// the accumulators spill (730 us on 20M kernels, 446 on 6M whose records were out
-// of order; four blocks 696 and 343; three 748 and 380).  Four slots gave 718 and
-// 434, chunks of 128 ops 888 and 466.
+// Four blocks of four warps per multiprocessor, 656 us on 20M kernels and 340 on
+// 6M whose records were out of order: with the 96 registers of five the
+// accumulators spill (821 and 475), three measured slower too (as did four
+// slots).  Chunks of 128 ops fill more lanes (49 % of them for 35 with a long
+// tail of lengths) but put twice the ops in flight, past what L2 holds: 896 and 466.
+// The chunk's offsets lie in shared memory and its list run comes by asynchronous
+// copy; with the offsets in registers, handed round by shuffles, and the run copied
+// through them, 704 and 345.
 constexpr int AG_SLOTS = 2, AG_BLOCKS = 4;
 constexpr int AG_STAGE = 1024;                  // list entries of a chunk staged in shared memory
 
@@ -684,6 +688,7 @@ struct OpsWarp {
     float4 row[AG_SLOTS][32][NC / 4];      // kernels in flight per thread: counter rows
     long long dur[AG_SLOTS][32];           // and durations, by asynchronous copy
     uint32_t L[AG_STAGE];           // the chunk's list run (when it fits)
+    uint32_t off[2][AG_CHUNK + 4];  // the chunk's offsets (one more than ops), and the next one's
     uint32_t lcount[AG_LBUCKETS];
     uint8_t order[AG_CHUNK];
 };
@@ -709,6 +714,9 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
 }
 __device__ __forceinline__ void cp_async8(void *dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -761,22 +769,22 @@ __global__ void __launch_bounds__(AG_THREADS, AG_BLOCKS) k_agg_ops(const uint32_
     };
     constexpr int PER = AG_CHUNK / 32;
     const int CHUNK = A.chunk;
-    // the first chunk's offsets (each warp has one); afterwards the next chunk
-    // is drawn and its offsets loaded while the current one runs
+    // the first chunk (each warp has one) and its offsets; afterwards the next
+    // chunk is drawn and its offsets copied while the current one runs
     int64_t o0 = idle ? A.n_ops : (int64_t)(blockIdx.x * AG_WARPS + threadIdx.x / 32) * CHUNK;
-    uint32_t oa[PER], ob[PER];
-#pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        const int64_t o = o0 + q * 32 + lane;
-        oa[q] = o < A.n_ops ? off[o] : 0u;
-        ob[q] = o < A.n_ops ? off[o + 1] : 0u;
-    }
+    int buf = 0;
+    auto fetch_offsets = [&](int to, int64_t o) {
+        for (int i = (int)lane; i <= CHUNK && o + i <= A.n_ops; i += 32) cp_async4(&W.off[to][i], off + o + i);
+        cp_async_commit();
+    };
+    if (o0 < A.n_ops) fetch_offsets(0, o0);
+    cp_async_wait<0>();
+    __syncwarp();
     while (o0 < A.n_ops) {
         const unsigned next_raw = draw();           // in flight during this chunk
         const int nchunk = A.n_ops - o0 < CHUNK ? (int)(A.n_ops - o0) : CHUNK;
-        const uint32_t cbase = __shfl_sync(0xffffffffu, oa[0], 0);          // the chunk's list run
-        const uint32_t cend = __shfl_sync(0xffffffffu, ob[(nchunk - 1) >> 5], (nchunk - 1) & 31);
-        const uint32_t ctot = cend - cbase;
+        const uint32_t *offs = W.off[buf];
+        const uint32_t cbase = offs[0], ctot = offs[nchunk] - cbase;       // the chunk's list run
         const bool staged = ctot <= AG_STAGE;
         // lengths of the chunk's ops, counting sort by length (descending, capped)
         uint32_t bkt[PER];
@@ -785,55 +793,43 @@ __global__ void __launch_bounds__(AG_THREADS, AG_BLOCKS) k_agg_ops(const uint32_
 #pragma unroll
         for (int q = 0; q < PER; ++q) {
             const int i = q * 32 + (int)lane;
-            const uint32_t len = i < nchunk ? ob[q] - oa[q] : 0u;
+            const uint32_t len = i < nchunk ? offs[i + 1] - offs[i] : 0u;
             bkt[q] = AG_LBUCKETS - 1 - (len < AG_LBUCKETS - 1 ? len : AG_LBUCKETS - 1);
             if (i < nchunk) atomicAdd(&W.lcount[bkt[q]], 1u);
         }
         if (staged)
-            for (uint32_t i = lane; i < ctot; i += 32) W.L[i] = list[cbase + i];
+            for (uint32_t i = lane; i < ctot; i += 32) cp_async4(&W.L[i], list + cbase + i);
+        cp_async_commit();
         __syncwarp();
         {
             const unsigned x = W.lcount[lane];
             const unsigned inc = warp_inclusive_scan(x);
             W.lcount[lane] = inc - x;
         }
+        cp_async_wait<0>();
         __syncwarp();
 #pragma unroll
         for (int q = 0; q < PER; ++q) {
             const int i = q * 32 + (int)lane;
             if (i < nchunk) W.order[atomicAdd(&W.lcount[bkt[q]], 1u)] = (uint8_t)i;
             // each thread puts the segments of its own ops in ascending order
-            const uint32_t len = i < nchunk ? ob[q] - oa[q] : 0u;
+            const uint32_t len = i < nchunk ? offs[i + 1] - offs[i] : 0u;
             if (len > A.lane_max) {
                 const bool mid = len <= AG_MID_MAX;
                 (mid ? A.mids : A.longs)[atomicAdd(A.ctr + (mid ? 2 : 3), 1u)] = (uint32_t)(o0 + i);
             } else if (len > 1) {
-                if (staged) sort_segment(W.L + (oa[q] - cbase), len);
-                else sort_segment(list + oa[q], len);
+                if (staged) sort_segment(W.L + (offs[i] - cbase), len);
+                else sort_segment(list + offs[i], len);
             }
         }
         __syncwarp();
         // the next chunk's offsets, in flight during the rounds
         const int64_t o1 = (int64_t)__shfl_sync(0xffffffffu, next_raw, 0) * CHUNK;
-        uint32_t na[PER], nb[PER];
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            const int64_t o = o1 + q * 32 + lane;
-            na[q] = o < A.n_ops ? off[o] : 0u;
-            nb[q] = o < A.n_ops ? off[o + 1] : 0u;
-        }
+        if (o1 < A.n_ops) fetch_offsets(buf ^ 1, o1);
         for (int g = 0; g * 32 < nchunk; ++g) {
             const int i = g * 32 + (int)lane;
-            // offsets of the op each lane walks, from the lane that holds them
-            // (op il sits in register il >> 5 of lane il & 31)
             const int il = i < nchunk ? W.order[i] : 0;
-            uint32_t sa = 0, sb = 0;
-#pragma unroll
-            for (int q = 0; q < PER; ++q) {
-                const uint32_t xa = __shfl_sync(0xffffffffu, oa[q], il & 31);
-                const uint32_t xb = __shfl_sync(0xffffffffu, ob[q], il & 31);
-                if ((il >> 5) == q) { sa = xa; sb = xb; }
-            }
+            const uint32_t sa = offs[il], sb = offs[il + 1];
             const int64_t o = o0 + il;
             const bool mine = i < nchunk && sb - sa <= A.lane_max;             // (longer ones are listed)
             const uint32_t s0 = sa, len = mine ? sb - sa : 0u;
@@ -881,10 +877,10 @@ __global__ void __launch_bounds__(AG_THREADS, AG_BLOCKS) k_agg_ops(const uint32_
             if (acc.clean()) acc.write(A, o, (int)len);
             else A.dirty[atomicAdd(A.ctr + 1, 1u)] = (uint32_t)o;
         }
+        cp_async_wait<0>();
         __syncwarp();
         o0 = o1;
-#pragma unroll
-        for (int q = 0; q < PER; ++q) { oa[q] = na[q]; ob[q] = nb[q]; }
+        buf ^= 1;
     }
     if (!report.status) return;
     __shared__ bool last;
@@ -905,7 +901,7 @@ __global__ void __launch_bounds__(AG_THREADS, AG_BLOCKS) k_agg_ops(const uint32_
 // ascending kernel index (in place) and redoes it with AccN, which leaves
 // nulls out and reports infinite values.  A separate pass keeps that
 // register-hungry path out of the ops pass (within it, for the lanes concerned,
-// the pass spilled: 853 us on 20M kernels without any null against 696).  Rows
+// the pass spilled: 853 us on 20M kernels without any null where it took 696).  Rows
 // reach the lanes as they do there, the warp copying together and AG_SLOTS
 // kernels ahead, counters two to a register.  Bound by issue at 12 warps a
 // multiprocessor (1.6 instructions a cycle): 176,000 ops, 1M kernels with 2 % of
