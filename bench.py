@@ -36,18 +36,13 @@ KERNEL_BYTES = {
     # list 4 + duration 8 + row index 4 + counter row 80 per kernel (the row
     # index is not read when every kernel's row is its own index: 92)
     "agg_ops": lambda K, R, M, O: 96 * K + 188 * O,
-    "enclose": lambda K, R, M, O: 14 * K + 20 * R,
+    "enc_parts": lambda K, R, M, O: 9 * K + 18 * R,
+    "enclose": lambda K, R, M, O: 14 * K + 22 * R,
     "agg_place": lambda K, R, M, O: 16 * K,
     "agg_count": lambda K, R, M, O: 24 * K + 4 * O,
     "match_identity": lambda K, R, M, O: 13 * K,
     "check_kernel_order": lambda K, R, M, O: 9 * K,
-    "check_ranges": lambda K, R, M, O: 18 * R,
-    "level_gather": lambda K, R, M, O: 44 * R,
-    "level_place": lambda K, R, M, O: 42 * R,
     "match_stream_pairs": lambda K, R, M, O: 18 * K,
-    "validate_levels": lambda K, R, M, O: 22 * R,
-    "stream_place": lambda K, R, M, O: 5 * K,
-    "stream_windows": lambda K, R, M, O: 0,
 }
 
 WORKLOADS = {
@@ -444,6 +439,7 @@ def main():
         if (tq is tr and tiers_out is None and not use_dedup and not args.per_stream_ncu and M == K
                 and not args.shuffle):
             KERNEL_BYTES["agg_count"] = lambda K, R, M, O: 20 * K + 4 * O
+            KERNEL_BYTES["enc_parts"] = lambda K, R, M, O: 22 * K + 18 * R
     # per-kernel breakdown: a few steps with every launch bracketed by events
     n_brk = max(1, min(args.steps, 10))
     ctx.set_timing(True)

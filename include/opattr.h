@@ -21,12 +21,10 @@
  *    tables, the summaries and totals) live in HOST memory.
  *  - Work is ordered on the context's CUDA stream.  A call returns once its
  *    small host-side results have been copied back; the device outputs are
- *    then complete on that stream.  Inside a call, independent steps may run
- *    on a second stream the context owns, forked from and joined back into
- *    the caller's stream before the call returns.
- *  - Those small transfers (status block, level offsets, host-built tables)
- *    go through the device mapping of the context's pinned host buffers,
- *    moved by a small kernel of the library, not through the copy engines:
+ *    then complete on that stream.
+ *  - Those small transfers (status block, counts, host-built tables) go
+ *    through the device mapping of the context's pinned host buffers, moved
+ *    by kernels of the library, not through the copy engines:
  *    a call does not wait behind bulk copies the caller has in flight on
  *    other streams (where the device cannot map them, cudaMemcpyAsync).
  *  - The library's kernels are programmatic dependent launches: each is
@@ -344,7 +342,7 @@ opattr_status opattr_aggregate(opattr_ctx *ctx, const opattr_kernels *kernels, c
  * matching).  The kernel records' time order is verified once for both the
  * enclosure and the matching.  With as many ncu rows as kernels (no
  * deduplication, no per-stream rows), the identity pairing of the matching
- * runs beside the enclosure and, when the kernels are in time order, the
+ * is written by the enclosure's checks and, when the kernels are in time order, the
  * enclosure's verdict is read with the aggregation's status: the outputs are
  * those of the three calls all the same (a disagreeing name redoes the
  * matching and the aggregation; ranges that need the enclosure's fully
