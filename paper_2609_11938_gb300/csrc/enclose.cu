@@ -501,7 +501,8 @@ constexpr uint32_t EN_SPAN = 0xFFFFFFF0u;                // a step's times fit 3
 //
 // Bound by issue (2.4 instructions a cycle) and by the shared-memory chains of
 // the links, not by HBM: 425 us for 20M kernels and 5.1M ranges on 16 streams
-// of 8 levels, 1,990 us for 50M and 14.5M on 64 streams of 32, 14 us for 2,000.
+// of 8 levels, 1,950 us for 50M and 14.5M on 64 streams of 32 (1,990 with climbs
+// of one level at a time), 14 us for 2,000.
 // With every open range's chain walked, and every level's tables cleared,
 // counted up and made relative to the next event at each step, 490, 3,840 and
 // 17 us; steps of 1,024 ranges (one block of 1,024 threads) 2,780 us where 512
