@@ -316,12 +316,15 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_layer_pairs(const int32_t *__r
 // Positions within layers, few layers: one stable counting pass over the
 // kernels in time order by layer id.
 constexpr int LAYERS_DIGIT = RADIX_BINS - 1;        // with a last, empty digit for the end of the layer before
+// (ids past the table are left out: this runs before the host has seen the check
+// of the ids, and only the table's digits, and the empty one after them, have offsets)
 struct LayerDigit {
     const int32_t *layer;
     const uint32_t *korder;
+    int32_t n_layers;            // LAYERS_DIGIT at most
     __device__ __forceinline__ unsigned operator()(int64_t i) const {
         const int32_t l = layer[korder ? korder[i] : (uint32_t)i];
-        return l >= 0 && l < LAYERS_DIGIT ? (unsigned)l : (unsigned)RADIX_BINS;
+        return l >= 0 && l < n_layers ? (unsigned)l : (unsigned)RADIX_BINS;
     }
 };
 struct PlaceByLayer {
@@ -433,7 +436,7 @@ static opattr_status broadcast_layers(Ctx &c, const opattr_kernels *kern, const 
     const int64_t K = kern->n;
     const unsigned gK = grid_for(K, 256, REDUCE_GRID);
     if (dd->n_layers <= LAYERS_DIGIT) {
-        const LayerDigit dg{kern->layer_id, korder};
+        const LayerDigit dg{kern->layer_id, korder, dd->n_layers};
         const uint32_t *offs = digit_offsets(c, dg, K, hist, part, dd->n_layers + 1);
         digit_rank(c, "layer_place", dg, K, offs, PlaceByLayer{korder, lk, pos});
         launch(c, "layer_broadcast", k_layer_broadcast, dim3(gK), dim3(256), 0, kern->layer_id, d_rep, dd->n_layers,

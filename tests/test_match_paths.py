@@ -108,3 +108,31 @@ def test_join_errors_in_order():
         st, out, *_ = ctx.join(opa.to_device(t))
         assert st == opa.OK
         np.testing.assert_array_equal(out["ncu_idx"].cpu().numpy(), oracle.run(t)["ncu_idx"])
+
+
+@pytest.mark.parametrize("call", ["match", "join"])
+@pytest.mark.parametrize("shuffle", [False, True])
+@pytest.mark.parametrize("slots,streams,bad", [(3, 2, 6), (3, 2, 7), (3, 2, 254), (3, 2, 255), (3, 2, 1 << 30), (3, 2, -2),
+                                               (254, 1, 254), (255, 1, 255), (255, 1, 256), (300, 1, 301)])
+def test_bad_layer_ids(slots, streams, bad, shuffle, call):
+    """Layer ids past the table, next to it and far off, on both sides of the
+    counting pass: refused, and the context is as good as new."""
+    import paper_2609_11938_gb300 as opa
+    t = _layered(slots, streams, shuffle)
+    ids = t.k_layer.copy()
+    ids[[7, t.K // 2, t.K - 1]] = bad
+    with opa.Context(0) as ctx:
+        for trace in (dataclasses.replace(t, k_layer=ids), t):
+            tr = opa.to_device(trace)
+            run = (lambda: ctx.match(tr)[:3]) if call == "match" else \
+                (lambda: (lambda st, out, *_: (st, out["ncu_idx"], out["match_kind"]))(*ctx.join(tr)))
+            if trace is not t:
+                with pytest.raises(opa.OpattrError) as ei:
+                    run()
+                assert ei.value.status == opa.E_INVALID_ARG
+                continue
+            st, idx, kind = run()
+            o = oracle.run(t)
+            assert st == o["match_status"]
+            np.testing.assert_array_equal(idx.cpu().numpy(), o["ncu_idx"])
+            np.testing.assert_array_equal(kind.cpu().numpy(), o["match_kind"])
