@@ -1007,7 +1007,8 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
 }
 
 // ------------------------------------------------------------------ sorted views
-// Range records in the order of the sorted keys (which hold the starts).
+// Range records in the order of the sorted keys (which hold the starts), or of
+// perm alone where the keys are too wide to be kept (NULL).
 __global__ void k_range_gather(EncView V, const uint64_t *__restrict__ key, int shift, long long tmin,
                                const uint32_t *__restrict__ perm, int64_t *__restrict__ start,
                                int64_t *__restrict__ end, uint8_t *__restrict__ stream, uint8_t *__restrict__ depth,
@@ -1015,7 +1016,7 @@ __global__ void k_range_gather(EncView V, const uint64_t *__restrict__ key, int 
     pdl_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < V.R; i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t r = perm[i];
-        start[i] = tmin + (long long)(key[i] >> shift);
+        start[i] = key ? tmin + (long long)(key[i] >> shift) : V.r_start[r];
         end[i] = V.r_end[r];
         stream[i] = V.r_stream[r];
         depth[i] = V.r_depth[r];

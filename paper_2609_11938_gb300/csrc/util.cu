@@ -236,6 +236,20 @@ __global__ void k_write_keys(Key key, int64_t n, uint64_t *__restrict__ keys) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         keys[i] = key(i);
 }
+// The two halves of a key that does not fit 64 bits: what follows the time, and
+// then the times in the order that this gave.
+template <typename Key>
+__global__ void k_write_low(Key key, int64_t n, uint64_t *__restrict__ keys) {
+    pdl_wait();
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        keys[i] = key.low(i);
+}
+template <typename Key>
+__global__ void k_gather_times(Key key, const uint32_t *__restrict__ perm, int64_t n, uint64_t *__restrict__ keys) {
+    pdl_wait();
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        keys[i] = key.time(perm[i]);
+}
 
 size_t time_sort_scratch(int64_t n) {
     Need nd;
@@ -245,13 +259,30 @@ size_t time_sort_scratch(int64_t n) {
     return nd.bytes;
 }
 
+// Records 0 .. n - 1 by key(i) = time(i) << bits | low(i), with time(i) at most
+// `span`; *keys receives the sorted keys.  Where span << bits does not fit 64
+// bits the sort goes by low(i) first and by time(i) then, and *keys is NULL.
 template <typename Key>
-static opattr_status time_sort(Ctx &c, Arena &a, Key key, int64_t n, uint64_t top, uint64_t **keys, uint32_t **perm) {
+static opattr_status time_sort(Ctx &c, Arena &a, Key key, int64_t n, uint64_t span, uint64_t **keys, uint32_t **perm) {
     const int64_t hist_n = std::max<int64_t>(radix_hist_elems(n), BK_MAX + 1);
     uint64_t *k0 = a.take<uint64_t>(n), *k1 = a.take<uint64_t>(n);
     uint32_t *v0 = a.take<uint32_t>(n), *v1 = a.take<uint32_t>(n);
     uint32_t *hist = a.take<uint32_t>(hist_n), *part = a.take<uint32_t>(scan_scratch_elems(hist_n));
     if (!k0 || !k1 || !v0 || !v1 || !hist || !part) return OPATTR_E_OOM;
+    if (bits_for(span) + key.bits > 64) {
+        const dim3 g(grid_for(n, 256, 65535));
+        uint64_t *k = nullptr;
+        uint32_t *v = nullptr;
+        launch(c, "time_keys", k_write_low<Key>, g, dim3(256), 0, key, n, k0);
+        radix_sort_pairs<uint64_t>(c, k0, v0, k1, v1, n, key.bits, true, hist, part, &k, &v);
+        launch(c, "time_keys", k_gather_times<Key>, g, dim3(256), 0, key, (const uint32_t *)v, n, k);
+        radix_sort_pairs<uint64_t>(c, k, v, k == k0 ? k1 : k0, v == v0 ? v1 : v0, n, bits_for(span), false, hist, part,
+                                   &k, perm);
+        *keys = nullptr;
+        return OPATTR_OK;
+    }
+    // no key is above it: the bucket counts in shared memory are indexed by the key's high bits
+    const uint64_t top = span << key.bits | ((1ull << key.bits) - 1);
     // widest buckets of BK_TARGET records on average whose span fits the entries' 32 bits
     int shift = 32;
     while (shift > 0 && (int64_t)(top >> shift) + 1 < (n + BK_TARGET - 1) / BK_TARGET) --shift;
@@ -287,21 +318,24 @@ struct KernelTimeKey {
     const int64_t *start;
     const uint8_t *stream, *scmap;      // scmap may be NULL
     long long tmin;
-    int sbits;
-    __device__ __forceinline__ uint64_t operator()(int64_t i) const {
+    int bits;
+    __device__ __forceinline__ uint64_t time(int64_t i) const { return (uint64_t)start[i] - (uint64_t)tmin; }
+    __device__ __forceinline__ unsigned low(int64_t i) const {
         const unsigned s = stream[i];
-        return ((uint64_t)(start[i] - tmin) << sbits) | (scmap ? scmap[s] : s);
+        return scmap ? scmap[s] : s;
     }
+    __device__ __forceinline__ uint64_t operator()(int64_t i) const { return time(i) << bits | low(i); }
 };
 opattr_status kernel_time_order(Ctx &c, Arena &a, const uint8_t *stream, const int64_t *start, int64_t n,
                                 uint32_t **order, const uint8_t *scmap, int stream_bits, uint64_t **keys) {
     const long long tmin = c.h_status->mm[MM_KSTART_MIN], tmax = c.h_status->mm[MM_KSTART_MAX];
-    const int sbits = scmap ? stream_bits : 8;
     uint64_t *k = nullptr;
-    const opattr_status st = time_sort(c, a, KernelTimeKey{start, stream, scmap, tmin, sbits}, n,
-                                       ((uint64_t)(tmax - tmin) << sbits) | ((1ull << sbits) - 1), &k, order);
+    const opattr_status st = time_sort(c, a, KernelTimeKey{start, stream, scmap, tmin, scmap ? stream_bits : 8}, n,
+                                       (uint64_t)tmax - (uint64_t)tmin, &k, order);
+    if (st) return st;
+    if (keys && !k) return OPATTR_E_INVALID_ARG;
     if (keys) *keys = k;
-    return st;
+    return OPATTR_OK;
 }
 
 // The order key of range i: its start, then its depth, so that parents come
@@ -313,16 +347,17 @@ opattr_status kernel_time_order(Ctx &c, Arena &a, const uint8_t *stream, const i
 // level are out of that order only when they overlap, which the laminar
 // checks report.
 struct RangeTimeKey {
+    static constexpr int bits = RANGE_KEY_SHIFT;
     const int64_t *start, *end;
     const uint8_t *depth;
     long long tmin;
-    __device__ __forceinline__ uint64_t operator()(int64_t i) const {
-        return (((uint64_t)(start[i] - tmin) << 5 | depth[i]) << 1) | (end[i] > start[i] ? 1u : 0u);
-    }
+    __device__ __forceinline__ uint64_t time(int64_t i) const { return (uint64_t)start[i] - (uint64_t)tmin; }
+    __device__ __forceinline__ unsigned low(int64_t i) const { return depth[i] << 1 | (end[i] > start[i] ? 1u : 0u); }
+    __device__ __forceinline__ uint64_t operator()(int64_t i) const { return time(i) << bits | low(i); }
 };
 opattr_status range_time_order(Ctx &c, Arena &a, const int64_t *start, const int64_t *end, const uint8_t *depth,
                                int64_t n, long long tmin, long long tmax, uint32_t **order, uint64_t **keys) {
-    return time_sort(c, a, RangeTimeKey{start, end, depth, tmin}, n, ((uint64_t)(tmax - tmin) << 6) | 63u, keys, order);
+    return time_sort(c, a, RangeTimeKey{start, end, depth, tmin}, n, (uint64_t)tmax - (uint64_t)tmin, keys, order);
 }
 
 }  // namespace opattr
