@@ -587,17 +587,20 @@ opattr_status do_match(Ctx &c, const opattr_kernels *kern, const opattr_ncu *ncu
     const bool defer = known_sorted && c.enclose_pending && (try_streams || try_layers);
     const bool sort_at_once = known_sorted && !dedup_on && c.max_known && !c.enclose_pending && !try_identity &&
                               !try_streams;
+    // kernels that the enclosure found out of order, as many rows: the pairing
+    // through the time order comes first, on the clear status it left
+    const bool list_at_once = known_unsorted && !dedup_on && K == M && !c.no_spec;
+    const bool at_once = sort_at_once || list_at_once;
     const ZeroRun zc{part, chain_words(K)};
     uint64_t max_key = 0;
     if (defer) {
         if (try_layers && (st = zero_runs(c, 1, &zc))) return st;
-    } else if (sort_at_once) {
-        max_key = c.h_status->cnt[C_MAX_KEY];
+    } else if (at_once) {
+        if (sort_at_once) max_key = c.h_status->cnt[C_MAX_KEY];
     } else if ((st = reset_status(c, try_layers ? 1 : 0, &zc))) {
         return st;
     }
-    const bool want_max = !defer && !sort_at_once && N > 0;
-    if (!sort_at_once) {
+    if (!at_once) {
         if (!known_sorted && !known_unsorted) check_kernel_order(c, kern->stream, kern->start_ns, K);
         if (try_layers)
             launch(c, "layer_pairs", k_layer_pairs, dim3(grid_for(K, SCAN_TILE)), dim3(SCAN_THREADS), 0,
@@ -617,9 +620,9 @@ opattr_status do_match(Ctx &c, const opattr_kernels *kern, const opattr_ncu *ncu
         if (try_layers && (st = broadcast_layers(c, kern, dd, d_rep, nullptr, flag, pos, lk, sort, hist, part, dsm,
                                                  out_idx, out_kind)))
             return st;
-        // (a pairing by rows as many as the kernels rarely fails: the largest key is then found afterwards)
-        const bool now = want_max && !try_identity && !try_streams && !try_layers;
-        if (now)
+        // (a pairing that is tried before the sort, here or below, rarely fails:
+        // the largest key is then found afterwards)
+        if (!defer && N > 0 && !try_identity && !try_streams && !try_layers && (!dedup_on || c.no_spec))
             launch(c, "max_key", k_max_key, dim3(grid_for(N, 256 * 8, 1024)), dim3(256), 0, kern->name_id, kern->stream,
                    K, ncu->name_id, ncu->stream, M, c.d_status);
         if (defer) {

@@ -136,3 +136,22 @@ def test_bad_layer_ids(slots, streams, bad, shuffle, call):
             assert st == o["match_status"]
             np.testing.assert_array_equal(idx.cpu().numpy(), o["ncu_idx"])
             np.testing.assert_array_equal(kind.cpu().numpy(), o["match_kind"])
+
+
+@pytest.mark.parametrize("case", ["plain", "streams", "layers"])
+def test_join_out_of_order_finds_no_key(case):
+    """Records out of order whose rows follow the launches: paired through the
+    time order, without the largest name that only the sort by names needs."""
+    import paper_2609_11938_gb300 as opa
+    t = tracegen.generate("dedup" if case == "layers" else "gpt2", n_iters=5, shuffle=True)
+    if case == "streams":
+        t = tracegen.per_stream_runs(t)
+    o = oracle.run(t, dedup=case == "layers")
+    tr = opa.to_device(t)
+    with opa.Context(0) as ctx:
+        ctx.set_timing(True)
+        st, out, _, summ, _ = ctx.join(tr, dedup=case == "layers")
+        ran = {k for k, (_, n) in ctx.timing_report().items() if n}
+    assert st == opa.OK and summ["fast_path"] == 1
+    np.testing.assert_array_equal(out["ncu_idx"].cpu().numpy(), o["ncu_idx"])
+    assert "bucket_sort" in ran and not ran & {"max_key", "pair_keys"}
