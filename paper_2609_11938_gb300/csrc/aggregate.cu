@@ -576,8 +576,11 @@ constexpr int SL_THREADS = 256;
 constexpr int SL_SMEM = 8192;
 
 // Ops up to this length, or up to four times the average one, are left to one
-// lane of the ops pass; AG_LANE_TOP at most.
-constexpr uint32_t AG_LANE_MAX = 64, AG_LANE_TOP = 256;
+// lane of the ops pass; AG_LANE_TOP at most.  4M kernels, ops of 200 in order /
+// in any order / of skewed lengths: 743 / 869 / 1,157 us with 128 at most, where
+// 256 took 2,387 / 3,294 / 2,032 (few lanes at work, each sorting by itself); ops
+// of 100 in order 648, where 64 for all took 1,113.
+constexpr uint32_t AG_LANE_MAX = 64, AG_LANE_TOP = 128;
 constexpr uint32_t AG_MID_MAX = 4096;           // up to this length: one block; longer: pieces over several warps
 constexpr uint32_t AG_PIECE = 1024;             // kernels of such an op per warp of the pieces pass
 
@@ -694,8 +697,10 @@ struct OpsWarp {
 };
 constexpr size_t AG_SMEM = sizeof(OpsWarp) * AG_WARPS;
 
-// Ascending order of a segment, sorted in place when it is not (insertion
-// sort: the segment is two ascending runs at worst).
+// Ascending order of a segment of at most AG_LANE_TOP, sorted in place when it is
+// not.  An op whose kernels lie in one run of the count pass is in order; in two
+// neighbouring ones, two ascending runs, which insertion takes in one pass; one
+// whose kernels lie anywhere, up to len^2 / 4 moves.
 __device__ __forceinline__ void sort_segment(uint32_t *seg, uint32_t len) {
     bool up = true;
     for (uint32_t t = 1; t < len; ++t) up &= seg[t - 1] < seg[t];

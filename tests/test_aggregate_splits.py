@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("nan_frac", [0.0, 0.03])
 @pytest.mark.parametrize("n_small,k", [(20_000, 80_000),      # short operators: lanes take up to 64 kernels
-                                       (200, 30_000),         # long ones: up to 256
+                                       (200, 30_000),         # long ones: up to 128
                                        (1, 6_000)])           # one more, longer than any other
 def test_operator_lengths(opa, n_small, k, nan_frac):  # noqa: F811
     lens = [1, 2, 63, 64, 65, 127, 128, 129, 255, 256, 257, 1023, 1024, 1025, 4095, 4096, 4097]
