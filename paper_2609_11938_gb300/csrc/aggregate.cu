@@ -1381,6 +1381,21 @@ int64_t agg_counter_words(uint32_t n_ops) {
     return AGG_OWN_WORDS + (scan_clean_words(n) + 7) / 8 * 8 + n;
 }
 
+// Ops longer than a lane takes, at most; pieces of the longest.
+static int64_t agg_mids(int64_t K, int64_t O) { return std::min<int64_t>(O, K / (AG_LANE_MAX + 1)) + 1; }
+static int64_t agg_partials(int64_t K) { return K / AG_PIECE + K / (AG_MID_MAX + 1) + 1; }
+size_t aggregate_scratch(int64_t K, uint32_t n_ops) {
+    const int64_t O = n_ops, mids_n = agg_mids(K, O);
+    Need nd;
+    nd.add<uint32_t>(O + 1).add<uint32_t>(K).add<uint32_t>(K);
+    nd.add<uint32_t>(mids_n).add<uint32_t>(mids_n).add<uint32_t>(O + 1);
+    nd.add<uint32_t>(mids_n).add<Acc>(agg_partials(K));
+    nd.add<uint32_t>(scan_scratch_elems(std::max<int64_t>(O + 1, radix_hist_elems(K))));
+    nd.add<uint32_t>(O + 1).add<uint32_t>(radix_hist_elems(K)).add<uint32_t>(8);   // huge-op index, histogram, info
+    nd.add<uint32_t>(mids_n);                                                        // huge ops
+    return nd.bytes + 4096;
+}
+
 opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_ranges *rng, const int32_t *rok,
                            const opattr_ncu *ncu, const int32_t *nidx, uint32_t n_ops,
                            const opattr_op_aggregates *out, opattr_totals *tot_out) {
@@ -1395,22 +1410,15 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
         return OPATTR_E_INVALID_ARG;
     if ((reinterpret_cast<uintptr_t>(ncu->counters) & 15) != 0) return OPATTR_E_INVALID_ARG;
 
-    Need nd;
-    nd.add<uint32_t>(O + 1).add<uint32_t>(K).add<uint32_t>(K);
-    const int64_t mids_n = std::min<int64_t>(O, K / (AG_LANE_MAX + 1)) + 1;        // ops longer than a lane takes
-    const int64_t part_n = K / AG_PIECE + K / (AG_MID_MAX + 1) + 1;                // pieces of the longest
-    nd.add<uint32_t>(mids_n).add<uint32_t>(mids_n).add<uint32_t>(O + 1);
-    nd.add<uint32_t>(mids_n).add<Acc>(part_n);
-    nd.add<uint32_t>(scan_scratch_elems(std::max<int64_t>(O + 1, radix_hist_elems(K))));
-    nd.add<uint32_t>(O + 1).add<uint32_t>(radix_hist_elems(K)).add<uint32_t>(8);   // huge-op index, histogram, info
-    nd.add<uint32_t>(mids_n);                                                        // huge ops
+    const int64_t mids_n = agg_mids(K, O), part_n = agg_partials(K);
+    const size_t need = aggregate_scratch(K, n_ops);
     // the counters lie ready at the start of the arena, or are taken and zeroed here
     const int64_t words = agg_counter_words(n_ops);          // ctr, the scan's, cnt
     const bool keeps = c.enclose_pending || c.keep_status;
     if (!(keeps && c.agg_words == words)) c.agg_ready = false;
     if (!c.agg_ready) c.arena_keep = 0;
-    opattr_status st = ensure_arena(c, nd.bytes + 4096);
-    if (!st && !c.agg_ready) st = ensure_arena(c, nd.add<uint32_t>(words).bytes + 4096);
+    opattr_status st = ensure_arena(c, need);
+    if (!st && !c.agg_ready) st = ensure_arena(c, need + Need().add<uint32_t>(words).bytes);
     if (st) return st;
     Arena a(c);
     const bool ready = c.agg_ready;

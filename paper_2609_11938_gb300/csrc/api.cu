@@ -95,6 +95,14 @@ opattr_status ensure_arena(Ctx &c, size_t bytes) {
     return OPATTR_OK;
 }
 
+static opattr_status drop_arena(Ctx &c) {
+    if (cudaStreamSynchronize(c.stream) != cudaSuccess) return cuda_status(c, cudaGetLastError());
+    if (c.arena) cudaFree(c.arena);
+    c.arena = nullptr;
+    c.arena_cap = 0;
+    return OPATTR_OK;
+}
+
 int sm_count(Ctx &c) {
     if (c.sms == 0) {
         cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, c.device);
@@ -440,6 +448,7 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
             c.max_known = false;
             c.agg_words = 0;
             c.agg_ready = false;
+            c.join_scratch = 0;
         }
     } scope(c);
     // The matching can go ahead on the taking that the records are in order, so
@@ -452,6 +461,7 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
     const bool same = full && !dd && kernels->n == ncu->n;
     const bool spec = same && !ncu->stream;
     const bool ahead = same || (full && dd && !ncu->stream && match_layers_ahead(dedup));
+    bool lean = false;                   // each step asks for its own scratch
     for (int pass = 0; pass < 2; ++pass) {
         c.enclose_k_sorted = -1;
         c.spec_k = 0;
@@ -463,6 +473,13 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
         c.enclose_pending = c.match_pending = c.keep_status = c.no_spec = false;
         c.max_ncu = full && !same && !dd && kernels->n + ncu->n < (1ll << 32) ? ncu : nullptr;
         c.max_known = false;
+        c.join_scratch = 0;
+        if (!lean && c.agg_words > 0 && full && ncu->n >= 0 && kernels->n < (1ll << 31) && ncu->n < (1ll << 31)) {
+            const size_t keep = Need().add<uint32_t>(c.agg_words).bytes;
+            const int64_t layers = dd ? std::min<int64_t>(dedup->n_layers, kernels->n) : 0;
+            c.join_scratch = keep + aggregate_scratch(kernels->n, n_ops);
+            if (!spec) c.join_scratch = std::max(c.join_scratch, keep + match_scratch(kernels->n, ncu->n, dd, layers));
+        }
         if (spec) {
             c.spec_kname = kernels->name_id;
             c.spec_nname = ncu->name_id;
@@ -473,6 +490,11 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
         c.defer_status = ahead && pass == 0;
         opattr_status st = finish(c, do_enclose(c, kernels, ranges, range_of_kernel, n_op_enclosing));
         c.defer_status = false;
+        if (st == OPATTR_E_OOM && c.join_scratch > 0 && drop_arena(c) == OPATTR_OK) {
+            lean = true;                 // the steps one by one need less at a time
+            --pass;
+            continue;
+        }
         if (st < 0) return st;
         const size_t agg_bytes = (sizeof(uint32_t) * (size_t)c.agg_words + 255) & ~(size_t)255;
         c.agg_ready = c.agg_words > 0;

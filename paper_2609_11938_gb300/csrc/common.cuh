@@ -138,6 +138,10 @@ struct Ctx {
     // arena has to grow on the way
     int64_t agg_words = 0;
     bool agg_ready = false;
+    // within a join: scratch that its matching and aggregation will ask for on
+    // records in order (beyond what is kept), so that the enclosure's request is
+    // the join's only one
+    size_t join_scratch = 0;
     int64_t launches = 0;
     bool timing = false;
     std::string timing_only;         // with timing on: bracket only this kernel (empty = all)
@@ -179,6 +183,9 @@ opattr_status enclose_verdict(const DevStatus &H, int64_t K);
 // the status words of the scan, and one per operator and one more.
 constexpr int AGG_OWN_WORDS = 8;
 int64_t agg_counter_words(uint32_t n_ops);
+// Scratch (bytes) of the aggregation beside those counters, and of the matching.
+size_t aggregate_scratch(int64_t K, uint32_t n_ops);
+size_t match_scratch(int64_t K, int64_t M, bool dedup_on, int64_t n_layers);
 // The matching's counts and status from the status block (c.match_sum holds
 // what was known before it ran).
 opattr_status match_verdict(Ctx &c, opattr_match_summary *sum);

@@ -1079,7 +1079,7 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     if (c.agg_words > 0) nd.add<uint32_t>(c.agg_words);
     const bool keep_order = c.in_join && K > 0;       // a join keeps the time order for its matching
     if (keep_order) nd.add<uint32_t>(K);
-    opattr_status st = ensure_arena(c, nd.bytes + 4096);
+    opattr_status st = ensure_arena(c, std::max(nd.bytes + 4096, c.join_scratch));
     if (st) return st;
     Arena a(c);
     // first, at the start of the arena, what outlives the enclosure

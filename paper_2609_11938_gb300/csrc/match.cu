@@ -487,6 +487,30 @@ opattr_status match_verdict(Ctx &c, opattr_match_summary *sum) {
     return OPATTR_OK;
 }
 
+// Scratch: the sort of kernels and rows (keys and values twice; the free pair then
+// holds the runs), the time order, and with layers the replayed kernels and the
+// layer lists.
+struct MatchSizes {
+    int64_t NL, N, NX, LX, hist_n, part_n;
+    size_t bytes;
+    MatchSizes(int64_t K, int64_t M, bool dedup_on, int64_t n_layers) {
+        NL = dedup_on && n_layers > 0 ? n_layers : 1;
+        N = K + M;
+        NX = std::max(K, M);
+        LX = dedup_on ? K : 1;
+        hist_n = std::max(radix_hist_elems(N), radix_hist_elems(NX));
+        part_n = scan_scratch_elems(std::max(std::max(hist_n, N), K));
+        Need nd;
+        nd.add<int32_t>(NL).add<unsigned long long>(4);
+        for (int i = 0; i < 4; ++i) nd.add<uint32_t>(N + 2).add<uint32_t>(LX);
+        nd.add<uint8_t>(NX).add<uint32_t>(hist_n).add<uint32_t>(part_n);
+        bytes = nd.bytes + time_sort_scratch(K) + 4096;
+    }
+};
+size_t match_scratch(int64_t K, int64_t M, bool dedup_on, int64_t n_layers) {
+    return MatchSizes(K, M, dedup_on, n_layers).bytes;
+}
+
 opattr_status do_match(Ctx &c, const opattr_kernels *kern, const opattr_ncu *ncu, const opattr_dedup *dd,
                        int32_t *out_idx, uint8_t *out_kind, opattr_match_summary *sum) {
     const int64_t K = kern->n, M = ncu->n;
@@ -510,7 +534,6 @@ opattr_status do_match(Ctx &c, const opattr_kernels *kern, const opattr_ncu *ncu
         rep_layer.resize(dd->n_layers > 0 ? dd->n_layers : 1);
         for (int32_t l = 0; l < dd->n_layers; ++l) rep_layer[l] = dd->rep_of_class[dd->class_of_layer[l]];
     }
-    const int64_t NL = dedup_on ? (dd->n_layers > 0 ? dd->n_layers : 1) : 1;
     const bool per_stream = ncu->stream != nullptr;
     opattr_match_summary &S = c.match_sum;
     S = opattr_match_summary{};
@@ -531,18 +554,9 @@ opattr_status do_match(Ctx &c, const opattr_kernels *kern, const opattr_ncu *ncu
         c.rows_identity = true;
         return OPATTR_OK;
     }
-    // scratch: the sort of kernels and rows (keys and values twice; the free
-    // pair then holds the runs), the time order, and with layers the replayed
-    // kernels and the layer lists
-    const int64_t N = K + M, NX = std::max(K, M);
-    const int64_t LX = dedup_on ? K : 1, hist_n = std::max(radix_hist_elems(N), radix_hist_elems(NX));
-    const int64_t part_n = scan_scratch_elems(std::max(std::max(hist_n, N), K));
-    Need nd;
-    nd.add<int32_t>(NL).add<unsigned long long>(4);
-    for (int i = 0; i < 4; ++i) nd.add<uint32_t>(N + 2).add<uint32_t>(LX);
-    nd.add<uint8_t>(NX).add<uint32_t>(hist_n).add<uint32_t>(part_n);
-    size_t need = nd.bytes + time_sort_scratch(K) + 4096;
-    opattr_status st = ensure_arena(c, need);
+    const MatchSizes Z(K, M, dedup_on, dedup_on ? dd->n_layers : 0);
+    const int64_t NL = Z.NL, N = Z.N, NX = Z.NX, LX = Z.LX, hist_n = Z.hist_n, part_n = Z.part_n;
+    opattr_status st = ensure_arena(c, Z.bytes);
     if (st) return st;
     Arena a(c);
     int32_t *d_rep = a.take<int32_t>(NL);

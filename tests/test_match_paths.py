@@ -155,3 +155,26 @@ def test_join_out_of_order_finds_no_key(case):
     assert st == opa.OK and summ["fast_path"] == 1
     np.testing.assert_array_equal(out["ncu_idx"].cpu().numpy(), o["ncu_idx"])
     assert "bucket_sort" in ran and not ran & {"max_key", "pair_keys"}
+
+
+@pytest.mark.parametrize("case", ["plain", "names", "streams", "layers"])
+def test_first_join_asks_for_scratch_once(case):
+    """A context's first join launches what the next ones do: no scratch grows
+    between its steps, which would leave the aggregation to zero its counters."""
+    import paper_2609_11938_gb300 as opa
+    if case == "layers":
+        t = tracegen.generate("dedup", n_iters=400)
+    else:
+        t = tracegen.generate("large", n_kernels=3_000_000 if case == "plain" else 600_000, n_streams=4, seed=4)
+        if case == "names":
+            t = _drop_row(t)
+        elif case == "streams":
+            t = tracegen.per_stream_runs(t)
+    tr = opa.to_device(t)
+    with opa.Context(0) as ctx:
+        n = []
+        for _ in range(3):
+            at = ctx.launch_count()
+            ctx.join(tr, dedup=case == "layers")
+            n.append(ctx.launch_count() - at)
+    assert n[0] == n[1] == n[2], n
