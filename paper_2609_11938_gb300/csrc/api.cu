@@ -199,7 +199,7 @@ __global__ void k_reset(DevStatus *st, ZeroRuns z) {
                               : threadIdx.x == MM_KSTART_MAX || threadIdx.x == MM_REND_MAX ? LLONG_MIN
                                                                                            : 0;
     if (threadIdx.x < 8) st->kstreams[threadIdx.x] = 0;
-    if (threadIdx.x == 0) st->err = st->flags = st->nlevels = st->nstreams = 0;
+    if (threadIdx.x == 0) st->err = st->flags = 0;
 }
 
 static opattr_status launch_reset(Ctx &c, DevStatus *st, int n, const ZeroRun *z) {

@@ -63,8 +63,6 @@ struct DevStatus {
     unsigned long long cnt[C_NSLOTS];
     long long mm[MM_NSLOTS];
     unsigned int kstreams[8];    // streams with kernels, one bit each (the enclosure's checks)
-    unsigned int nlevels;        // range levels present (the enclosure)
-    unsigned int nstreams;       // and streams with ranges
 };
 
 // ------------------------------------------------------------------ context

@@ -69,6 +69,44 @@ __device__ __forceinline__ int64_t tile_event(int64_t i, int64_t n, int64_t even
     return (int64_t)((unsigned long long)events * (unsigned long long)i / (unsigned long long)n);   // below 2^52
 }
 
+// Traces with more streams or levels than one block's tables hold are taken group
+// by group of 16 consecutive stream ids (512 levels at most): kernels and ranges
+// partitioned stably by group, every group a sequence of its own with a share of
+// the parts in proportion to its events.  20M kernels, enclosure and partition:
+// 255 streams of 12 levels 510 + 390 us, where four walks of the whole trace with the
+// streams of one group each took 2,388; of 32 levels 690 + 395 and 2,805.
+constexpr int GROUP_SHIFT = 4, N_GROUPS = 256 >> GROUP_SHIFT;
+struct EncGroup {
+    int64_t k0, K, r0, R, tile0;         // its kernels, ranges and tile bounds begin at
+    int part0, parts, tp;
+};
+// View and parts narrowed to the group of part b; false for a block past the last part.
+__device__ __forceinline__ bool enter_group(const EncGroup *__restrict__ G, EncView &V, int64_t &b, int64_t &parts, int &tp,
+                                            int64_t &tile0, int64_t &part0, unsigned &grp) {
+    unsigned g = 0;
+    while (g < N_GROUPS && b >= G[g].part0 + G[g].parts) ++g;
+    if (g == N_GROUPS) return false;
+    const EncGroup E = G[g];
+    V.k_start += E.k0;
+    V.k_stream += E.k0;
+    V.korder += E.k0;
+    V.K = E.K;
+    V.r_start += E.r0;
+    V.r_end += E.r0;
+    V.r_stream += E.r0;
+    V.r_depth += E.r0;
+    V.r_op += E.r0;
+    V.perm += E.r0;
+    V.R = E.R;
+    b -= E.part0;
+    parts = E.parts;
+    tp = E.tp;
+    tile0 = E.tile0;
+    part0 = E.part0;
+    grp = g;
+    return true;
+}
+
 // Ranges among the first d[i] merged events for each i, by one warp: 32 probes
 // a round, the N searches' side by side (a round is two gathers' latency).  A
 // range precedes the kernels that start no earlier.  Ends in [0, R] whatever the
@@ -136,11 +174,12 @@ constexpr int EP_SEARCH = 4;             // tile bounds a warp looks for at once
 // Bound by HBM: 9 bytes per kernel and 18 per range (13 more per kernel with
 // the pairing), each read or written once: 121 us for 20M kernels and 5.1M
 // ranges in order, 4.4 TB/s (130 with a tile bound and a range at a time).
-template <bool CHECK, bool KEYS>
+template <bool CHECK, bool KEYS, bool GROUPS = false>
 __global__ void __launch_bounds__(EP_THREADS) k_enc_parts(EncView V, EncCheck C, int64_t parts, int tp,
                                                           uint32_t *__restrict__ tile_r, uint32_t *__restrict__ rows,
                                                           uint32_t *__restrict__ row_len,
-                                                          uint32_t *__restrict__ lvlmask, DevStatus *st) {
+                                                          uint32_t *__restrict__ lvlmask, const EncGroup *__restrict__ G,
+                                                          DevStatus *st) {
     pdl_wait();
     __shared__ uint32_t last[LEVELS];
     __shared__ uint32_t dmask[256];
@@ -150,7 +189,15 @@ __global__ void __launch_bounds__(EP_THREADS) k_enc_parts(EncView V, EncCheck C,
     __shared__ int64_t bound[2];
     __shared__ uint32_t top_s;
     const int tid = threadIdx.x;
-    const int64_t b = blockIdx.x;
+    int64_t b = blockIdx.x;
+    if (GROUPS) {
+        int64_t tile0, part0;
+        unsigned grp;
+        if (!enter_group(G, V, b, parts, tp, tile0, part0, grp)) return;
+        tile_r += tile0;
+        rows += part0 * LEVELS;
+        row_len += part0;
+    }
     const unsigned lane = lane_id(), warp = tid >> 5;
     for (int i = tid; i < LEVELS; i += EP_THREADS) last[i] = 0;
     if (CHECK) {
@@ -366,9 +413,16 @@ __global__ void __launch_bounds__(EP_THREADS) k_enc_parts(EncView V, EncCheck C,
 // a running maximum down every column.  One block per stream: lane d of a
 // warp takes depth d, each of the 32 warps an equal run of the parts.
 __global__ void __launch_bounds__(1024) k_enc_carry(uint32_t *__restrict__ rows, const uint32_t *__restrict__ row_len,
-                                                    int64_t parts, const uint32_t *__restrict__ lvlmask) {
+                                                    int64_t parts, const uint32_t *__restrict__ lvlmask,
+                                                    const EncGroup *__restrict__ G) {
     pdl_wait();
     if (lvlmask[blockIdx.x] == 0) return;
+    if (G) {                                     // the parts of the stream's group
+        G += blockIdx.x >> GROUP_SHIFT;
+        rows += (int64_t)G->part0 * LEVELS;
+        row_len += G->part0;
+        parts = G->parts;
+    }
     __shared__ uint32_t seg[32][33];
     const unsigned lane = lane_id(), w = threadIdx.x >> 5;
     const uint32_t l = blockIdx.x * 32u + lane;
@@ -459,7 +513,15 @@ struct EncTile {
 using EncTileA = EncTile<256, 4, false>;
 using EncTileB = EncTile<512, 2, true>;
 constexpr int EN_LEVELS_A = 512, EN_STREAMS_A = 64;      // levels and streams of the common layout
-constexpr int EN_LEVELS_B = 2048;                        // of the wide one: 64 streams of every depth
+constexpr int EN_LEVELS_B = 2048;                        // levels of the wide one
+// Groups of streams: past the wide layout's levels, and where a step of the whole
+// trace touches so many streams that carrying their open ranges on costs more than
+// the partition.  300k / 4M / 20M kernels on 200 streams of 4 levels: 265 / 546 /
+// 1,860 us per join by groups, 243 / 543 / 2,022 in the wide layout; on 255 streams
+// 274 / 551 / 1,882 and 257 / 568 / 2,117; on 100 streams 258 / 527 / 1,817 and
+// 221 / 486 / 1,795.
+constexpr int EN_STREAMS_B = 160;
+constexpr int64_t EN_GROUP_EVENTS = 4 << 20;
 constexpr int64_t EN_TILE = 2048, EN_TILE_MIN = 512;     // events of a tile; of a part's one tile in small traces
 constexpr int64_t EN_EARLY = 1 << 20;                    // events from which a join looks at the checks before the end
 constexpr uint32_t EN_SPAN = 0xFFFFFFF0u;                // a step's times fit 32 bits relative to its first
@@ -513,15 +575,14 @@ constexpr uint32_t EN_SPAN = 0xFFFFFFF0u;                // a step's times fit 3
 // in level lists of the tile (1,170 us), entries grouped by stream with a
 // search per kernel (696 us).
 //
-// blockIdx.y is a group of 2^gshift consecutive stream ids: the block leaves
-// the other groups' kernels and ranges alone (traces with more levels than the
-// wide layout holds; else one group of all 256).
+// GROUPS: the parts are those of groups of streams (EncGroup).
 template <typename TL, bool KEYS, bool GROUPS>
 __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
     k_enclose(EncView V, int64_t parts, int tp, const uint32_t *__restrict__ tile_r,
               const uint32_t *__restrict__ rows, const uint32_t *__restrict__ row_len, int carried,
-              const uint32_t *__restrict__ lvlmask, int nlcap, int nscap, int gshift, unsigned leave_on, int final,
-              int32_t *__restrict__ out_range, uint8_t *__restrict__ out_nop, DevStatus *st) {
+              const uint32_t *__restrict__ lvlmask, int nlcap, int nscap, const EncGroup *__restrict__ G,
+              unsigned leave_on, int final, int32_t *__restrict__ out_range,
+              uint8_t *__restrict__ out_nop, DevStatus *st) {
     pdl_wait();
     constexpr int THREADS = TL::THREADS, WARPS = THREADS / 32, RPT = TL::RPT, SR = TL::SR, WORDS = TL::WORDS;
     static_assert(THREADS >= 256, "a thread per stream");
@@ -534,15 +595,21 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
     __shared__ int ntouched;
     const int tid = threadIdx.x;
     const unsigned lane = lane_id(), warp = tid >> 5, lt = lanemask_lt();
-    const int64_t b = blockIdx.x;
-    const unsigned grp = blockIdx.y;
-    auto mine = [&](unsigned s) { return !GROUPS || (s >> gshift) == grp; };
+    int64_t b = blockIdx.x;
+    unsigned grp = 0;
+    if (GROUPS) {
+        int64_t tile0, part0;
+        if (!enter_group(G, V, b, parts, tp, tile0, part0, grp)) return;
+        tile_r += tile0;
+        rows += part0 * LEVELS;
+        row_len += part0;
+    }
     // levels present: depths 0 .. ndep - 1 of each stream (a depth below a gap
     // has no parent level: its ranges are not nested)
     int nl, ns;
     {
         uint32_t n = 0;
-        if (tid < 256 && mine(tid)) {
+        if (tid < 256 && (!GROUPS || tid >> GROUP_SHIFT == (int)grp)) {
             const uint32_t m = lvlmask[tid];
             n = m == 0xFFFFFFFFu ? 32u : (uint32_t)__ffs(~m) - 1u;
         }
@@ -551,11 +618,7 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
         nl = (int)(tot & 0xFFFFu);
         ns = (int)(tot >> 16);
         if (nl > nlcap || ns > nscap) {
-            if (b == 0 && tid == 0) {
-                atomicMax(&st->nlevels, (unsigned)nl);
-                atomicMax(&st->nstreams, (unsigned)ns);
-                set_flag(st, F_LEVELS_MANY);
-            }
+            if (b == 0 && tid == 0) set_flag(st, F_LEVELS_MANY);
             return;
         }
         if (tid < 256) {
@@ -721,7 +784,7 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                 const unsigned s = in ? V.r_stream[p] : 0u, d = in ? V.r_depth[p] : 0u;
                 const uint32_t op = in ? V.r_op[p] : 0u;
                 const bool lvl = in && d < S.ndep[s];
-                err |= in && !lvl && mine(s);
+                err |= in && !lvl;
                 const unsigned q = lvl ? S.scid[s] : 256u;
                 const unsigned ps = __match_any_sync(0xffffffffu, q);
                 unsigned pl = ps, pp = ps;           // lanes of the level, of the level above
@@ -749,7 +812,7 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                         S.smask[q * WORDS + g] = ps;
                         atomicOr(&S.sgroups[q], 1u << g);
                     }
-                } else if (in) {                     // another group's, or below a gap: on no stream's chain
+                } else if (in) {                     // below a gap: on no stream's chain
                     S.ss[e] = rel_near(a);
                     S.se[e] = 0;
                     S.si[e] = KIND_STRUCT << 30;
@@ -914,7 +977,7 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                         const uint32_t v31 = __shfl_sync(0xffffffffu, v, 31);
                         qn += h + (v31 <= T ? 1 : 0);
                     }
-                    if (!in || !mine(s)) continue;
+                    if (!in) continue;
                     uint32_t ans = E_NONE;
                     unsigned n = 0;
                     const unsigned q = S.scid[s];
@@ -1024,6 +1087,73 @@ __global__ void k_range_gather(EncView V, const uint64_t *__restrict__ key, int 
     }
 }
 
+// ------------------------------------------------------------------ groups of streams
+// Kernels and ranges of the view, each partitioned by one stable counting pass.
+template <bool KEYS>
+struct GroupDigitK {
+    EncView V;
+    __device__ __forceinline__ unsigned operator()(int64_t i) const { return V.stream<KEYS>(i) >> GROUP_SHIFT; }
+};
+template <bool KEYS>
+struct GroupPlaceK {
+    EncView V;
+    int64_t *start;
+    uint8_t *stream;
+    uint32_t *order;
+    __device__ __forceinline__ void operator()(int64_t i, uint32_t dest, unsigned) const {
+        start[dest] = V.time<KEYS>(i);
+        stream[dest] = (uint8_t)V.stream<KEYS>(i);
+        order[dest] = V.korder ? V.korder[i] : (uint32_t)i;
+    }
+};
+struct GroupDigitR {
+    const uint8_t *stream;
+    __device__ __forceinline__ unsigned operator()(int64_t i) const { return stream[i] >> GROUP_SHIFT; }
+};
+struct GroupPlaceR {
+    EncView V;
+    int64_t *start, *end;
+    uint8_t *stream, *depth;
+    uint32_t *op, *perm;
+    __device__ __forceinline__ void operator()(int64_t i, uint32_t dest, unsigned) const {
+        start[dest] = V.r_start[i];
+        end[dest] = V.r_end[i];
+        stream[dest] = V.r_stream[i];
+        depth[dest] = V.r_depth[i];
+        op[dest] = V.r_op[i];
+        perm[dest] = V.perm ? V.perm[i] : (uint32_t)i;
+    }
+};
+// koffs / roffs: digit-major offsets of the counting passes (kt / rt tiles each).
+__global__ void k_enc_groups(const uint32_t *__restrict__ koffs, int64_t kt, int64_t K, const uint32_t *__restrict__ roffs,
+                             int64_t rt, int64_t R, int64_t parts, EncGroup *__restrict__ G) {
+    pdl_wait();
+    __shared__ EncGroup E[N_GROUPS];
+    const int g = threadIdx.x;
+    auto first = [](const uint32_t *offs, int64_t tiles, int64_t n, int d) -> int64_t {
+        return n == 0 ? 0 : d == N_GROUPS ? n : (int64_t)offs[d * tiles];
+    };
+    EncGroup &e = E[g];
+    e.k0 = first(koffs, kt, K, g);
+    e.r0 = first(roffs, rt, R, g);
+    e.K = first(koffs, kt, K, g + 1) - e.k0;
+    e.R = first(roffs, rt, R, g + 1) - e.r0;
+    const int64_t n = e.K + e.R, p = n * parts / (K + R);
+    e.parts = n == 0 ? 0 : (int)(p > 0 ? p : 1);
+    const int64_t tp = n == 0 ? 0 : (n + e.parts * EN_TILE - 1) / (e.parts * EN_TILE);
+    e.tp = (int)(tp > 0 ? tp : 1);
+    __syncwarp((1u << N_GROUPS) - 1u);
+    int64_t part0 = 0, tile0 = 0;
+    for (int q = 0; q < g; ++q) {
+        part0 += E[q].parts;
+        tile0 += (int64_t)E[q].parts * E[q].tp + 1;
+    }
+    EncGroup out = e;
+    out.part0 = (int)part0;
+    out.tile0 = tile0;
+    G[g] = out;
+}
+
 // ------------------------------------------------------------------ host
 opattr_status enclose_verdict(const DevStatus &H, int64_t K) {
     if (H.err & ERR_INVALID) return OPATTR_E_INVALID_ARG;
@@ -1040,25 +1170,91 @@ struct EncBufs {
     int64_t parts;
     int tp;                      // tiles of a part
     uint32_t *tile_r, *rows, *row_len, *lvlmask;
+    EncGroup *groups;            // NULL: one sequence
 };
 constexpr int64_t EN_DIRECT_PARTS = 32;          // up to this many: a block scans the rows before its own itself
 template <typename TL, bool KEYS, bool GROUPS = false>
-static void launch_tiles(Ctx &c, const EncView &V, const EncBufs &B, int nl, int ns, int groups, unsigned leave_on,
-                         bool final, int32_t *out_range, uint8_t *out_nop) {
+static void launch_tiles(Ctx &c, const EncView &V, const EncBufs &B, int nl, int ns, unsigned leave_on, bool final,
+                         int32_t *out_range, uint8_t *out_nop) {
     nl = (nl + 7) & ~7;                          // (whole words in every table)
     ns = (ns + 7) & ~7;
     const size_t smem = TL::smem(nl, ns);
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(k_enclose<TL, KEYS, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch(c, "enclose", k_enclose<TL, KEYS, GROUPS>, dim3((unsigned)B.parts, (unsigned)groups), dim3(TL::THREADS), smem, V,
+    launch(c, "enclose", k_enclose<TL, KEYS, GROUPS>, dim3((unsigned)B.parts), dim3(TL::THREADS), smem, V,
            B.parts, B.tp, (const uint32_t *)B.tile_r, (const uint32_t *)B.rows, (const uint32_t *)B.row_len,
-           (int)(B.parts > EN_DIRECT_PARTS), (const uint32_t *)B.lvlmask, nl, ns, groups > 1 ? 6 : 8, leave_on, (int)final,
-           out_range, out_nop, c.d_status);
+           (int)(GROUPS || B.parts > EN_DIRECT_PARTS), (const uint32_t *)B.lvlmask, nl, ns, (const EncGroup *)B.groups,
+           leave_on, (int)final, out_range, out_nop, c.d_status);
 }
 static void launch_carry(Ctx &c, const EncBufs &B) {
-    if (B.parts > EN_DIRECT_PARTS)
+    if (B.groups || B.parts > EN_DIRECT_PARTS)
         launch(c, "enc_carry", k_enc_carry, dim3(256), dim3(1024), 0, B.rows, (const uint32_t *)B.row_len, B.parts,
-               (const uint32_t *)B.lvlmask);
+               (const uint32_t *)B.lvlmask, (const EncGroup *)B.groups);
+}
+
+// Levels and streams with ranges, from the depths present on every stream.
+struct LevelCount {
+    int levels = 0, streams = 0;
+    explicit LevelCount(const uint32_t *masks) {
+        for (int s = 0; s < 256; ++s) {
+            levels += masks[s] == 0xFFFFFFFFu ? 32 : __builtin_ctz(~masks[s]);
+            streams += (masks[s] & 1u) != 0;
+        }
+    }
+};
+
+// Room for the partition by groups, and the partition: the view on it, its parts
+// in B.
+struct GroupArrays {
+    int64_t *k_start, *r_start, *r_end;
+    uint8_t *k_stream, *r_stream, *r_depth;
+    uint32_t *korder, *r_op, *perm, *k_hist, *r_hist, *part, *tile_r, *row_len, *rows;
+    EncGroup *groups;
+    bool take(Arena &a, int64_t K, int64_t R, int64_t n_part, int64_t tiles, int64_t parts) {
+        bool ok = (k_start = a.take<int64_t>(K)) && (k_stream = a.take<uint8_t>(K)) && (korder = a.take<uint32_t>(K));
+        ok = ok && (k_hist = a.take<uint32_t>(radix_hist_elems(K))) && (part = a.take<uint32_t>(n_part));
+        ok = ok && (r_start = a.take<int64_t>(R)) && (r_end = a.take<int64_t>(R)) && (r_stream = a.take<uint8_t>(R));
+        ok = ok && (r_depth = a.take<uint8_t>(R)) && (r_op = a.take<uint32_t>(R)) && (perm = a.take<uint32_t>(R));
+        ok = ok && (r_hist = a.take<uint32_t>(radix_hist_elems(R))) && (groups = a.take<EncGroup>(N_GROUPS));
+        ok = ok && (tile_r = a.take<uint32_t>(tiles)) && (row_len = a.take<uint32_t>(parts));
+        return ok && (rows = a.take<uint32_t>(parts * LEVELS));
+    }
+};
+static EncView launch_groups(Ctx &c, const EncView &V, const GroupArrays &ga, EncBufs &B) {
+    const uint32_t *koffs = nullptr;
+    if (V.k_key) {
+        koffs = digit_offsets(c, GroupDigitK<true>{V}, V.K, ga.k_hist, ga.part, N_GROUPS);
+        digit_move(c, "group_kernels", GroupDigitK<true>{V}, V.K, koffs,
+                   GroupPlaceK<true>{V, ga.k_start, ga.k_stream, ga.korder});
+    } else {
+        koffs = digit_offsets(c, GroupDigitK<false>{V}, V.K, ga.k_hist, ga.part, N_GROUPS);
+        digit_move(c, "group_kernels", GroupDigitK<false>{V}, V.K, koffs,
+                   GroupPlaceK<false>{V, ga.k_start, ga.k_stream, ga.korder});
+    }
+    const uint32_t *roffs = digit_offsets(c, GroupDigitR{V.r_stream}, V.R, ga.r_hist, ga.part, N_GROUPS);
+    digit_move(c, "group_ranges", GroupDigitR{V.r_stream}, V.R, roffs,
+               GroupPlaceR{V, ga.r_start, ga.r_end, ga.r_stream, ga.r_depth, ga.r_op, ga.perm});
+    auto tiles = [](int64_t n) { return (n + RADIX_TILE - 1) / RADIX_TILE; };
+    launch(c, "enc_groups", k_enc_groups, dim3(1), dim3(N_GROUPS), 0, koffs, tiles(V.K), V.K, roffs, tiles(V.R), V.R,
+           B.parts, ga.groups);
+    EncView G{};
+    G.k_start = ga.k_start;
+    G.k_stream = ga.k_stream;
+    G.korder = ga.korder;
+    G.K = V.K;
+    G.r_start = ga.r_start;
+    G.r_end = ga.r_end;
+    G.r_stream = ga.r_stream;
+    G.r_depth = ga.r_depth;
+    G.r_op = ga.r_op;
+    G.perm = ga.perm;
+    G.R = V.R;
+    B.parts += N_GROUPS;             // rounded up to one part at least for every group
+    B.tile_r = ga.tile_r;
+    B.row_len = ga.row_len;
+    B.rows = ga.rows;
+    B.groups = ga.groups;
+    return G;
 }
 
 opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges *rng, int32_t *out_range,
@@ -1122,25 +1318,21 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
         C.M = c.max_ncu->n;
     }
     launch(c, "enc_parts", k_enc_parts<true, false>, dim3((unsigned)B.parts), dim3(EP_THREADS), 0, V, C, B.parts,
-           B.tp, B.tile_r, B.rows, B.row_len, B.lvlmask, c.d_status);
+           B.tp, B.tile_r, B.rows, B.row_len, B.lvlmask, (const EncGroup *)nullptr, c.d_status);
     // a large join looks at the checks' verdict while the rest runs on the
     // taking that the records are in order; a small one reads it once, at its end
     const bool early = c.defer_status && K + R >= EN_EARLY;
     const SmallCopy masks{c.h_small, B.lvlmask, 256 * sizeof(uint32_t)};
     if (early && (st = post_status(c, 1, &masks))) return st;
     launch_carry(c, B);
-    launch_tiles<EncTileA, false>(c, V, B, EN_LEVELS_A, EN_STREAMS_A, 1, F_K_UNSORTED | F_R_UNSORTED, false, out_range, out_nop);
+    launch_tiles<EncTileA, false>(c, V, B, EN_LEVELS_A, EN_STREAMS_A, F_K_UNSORTED | F_R_UNSORTED, false, out_range, out_nop);
     if (c.defer_status) {
         bool usual = true;
         if (early) {
             if ((st = await_status(c))) return st;
-            int levels = 0, streams = 0;
-            for (int s = 0; s < 256; ++s) {
-                levels += __builtin_popcount(c.h_small[s]);
-                streams += c.h_small[s] != 0;
-            }
-            usual = !(c.h_status->flags & (F_K_UNSORTED | F_R_UNSORTED)) && levels <= EN_LEVELS_A &&
-                    streams <= EN_STREAMS_A;
+            const LevelCount n(c.h_small);
+            usual = !(c.h_status->flags & (F_K_UNSORTED | F_R_UNSORTED)) && n.levels <= EN_LEVELS_A &&
+                    n.streams <= EN_STREAMS_A;
         }
         if (usual) {
             // the rest of the verdict comes with the aggregation's status, which the join checks
@@ -1149,21 +1341,22 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
             return OPATTR_OK;
         }
     }
-    if ((st = read_status(c))) return st;
+    if ((st = read_status(c, 1, &masks))) return st;
     bool k_sorted = !(c.h_status->flags & F_K_UNSORTED), r_sorted = !(c.h_status->flags & F_R_UNSORTED);
     c.enclose_k_sorted = k_sorted ? 1 : 0;
-    const bool many = (c.h_status->flags & F_LEVELS_MANY) != 0;
+    const LevelCount present(c.h_small);
+    const bool many = present.levels > EN_LEVELS_A || present.streams > EN_STREAMS_A;
+    const bool grouped = present.levels > EN_LEVELS_B || (present.streams > EN_STREAMS_B && K + R > EN_GROUP_EVENTS);
     const bool fixup = (c.h_status->flags & F_LEVEL_FIXUP) != 0;
     if ((st = enclose_verdict(*c.h_status, K)) && !(fixup && st == OPATTR_E_NOT_NESTED)) return st;
     if (k_sorted && r_sorted && !many && !fixup) return OPATTR_OK;
 
     // ---- records out of order, ranges of one level that share a start and are
     // out of (start, end) order, or more levels than the common layout holds:
-    // the tiles again, on the sorted view, with room for every level
+    // the tiles again, on the sorted view, with room for every level or by groups
     const unsigned names_differ = c.h_status->flags & F_NAMES_DIFFER;   // the pairing's verdict stays
     const long long rmin = c.h_status->mm[MM_RSTART_MIN], rmax = c.h_status->mm[MM_REND_MAX];
     const long long kmin = c.h_status->mm[MM_KSTART_MIN];
-    const unsigned levels = c.h_status->nlevels;
     int nks = 0;                                  // streams with kernels
     uint8_t *scmap = c.h_stage, *unmap = c.h_stage + 256;
     memset(c.h_stage, 0, 512);
@@ -1178,6 +1371,15 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
         Need n2;
         n2.add<int64_t>(R).add<int64_t>(R).add<uint8_t>(R).add<uint8_t>(R).add<uint32_t>(R);
         more += n2.bytes + time_sort_scratch(R) + 4096;
+    }
+    const int64_t g_parts = B.parts + N_GROUPS, g_tiles = (K + R) / EN_TILE + B.parts + 3 * N_GROUPS;
+    const int64_t g_part = scan_scratch_elems(std::max(radix_hist_elems(K), radix_hist_elems(R)));
+    if (grouped) {
+        Need n3;
+        n3.add<int64_t>(K).add<uint8_t>(K).add<uint32_t>(K).add<uint32_t>(radix_hist_elems(K)).add<uint32_t>(g_part);
+        n3.add<int64_t>(R).add<int64_t>(R).add<uint8_t>(R).add<uint8_t>(R).add<uint32_t>(R).add<uint32_t>(R);
+        n3.add<uint32_t>(radix_hist_elems(R)).add<EncGroup>(N_GROUPS).add<uint32_t>(g_tiles).add<uint32_t>(g_parts);
+        more += n3.add<uint32_t>(g_parts * LEVELS).bytes + 4096;
     }
     // growing the arena keeps the prefix taken so far
     c.arena_keep = (c.arena_used + 255) & ~(size_t)255;
@@ -1221,10 +1423,10 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     if (!gs || !ge || !gt || !gd || !go) return OPATTR_E_OOM;
     // ranges sorted so that parents come first: their verdict is final
     bool sort_ranges = !r_sorted || fixup, sorted = false;
-    bool have_parts = k_sorted && !sort_ranges;       // (too many levels only: the checking pass's parts stand)
-    int nl = many ? (int)levels : EN_LEVELS_A, ns = many ? (int)c.h_status->nstreams : EN_STREAMS_A;
-    bool wide = many;
-    for (int attempt = 0; attempt < 4; ++attempt) {
+    bool have_parts = k_sorted && !sort_ranges && !grouped;       // (too many levels only: the checking pass's parts stand)
+    GroupArrays ga{};
+    if (grouped && !ga.take(a, K, R, g_part, g_tiles, g_parts)) return OPATTR_E_OOM;
+    for (int attempt = 0; attempt < 2; ++attempt) {
         if (sort_ranges && R > 0) {
             uint64_t *ko = nullptr;
             uint32_t *perm = nullptr;
@@ -1244,29 +1446,28 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
         const ZeroRun zs{c.d_status, 2};              // err and flags
         if ((st = zero_runs(c, 1, &zs))) return st;
         const bool keys = V.k_key != nullptr;
-        if (!have_parts) {
+        if (grouped) {
+            EncBufs BG = B;
+            const EncView VG = launch_groups(c, V, ga, BG);
+            launch(c, "enc_view", k_enc_parts<false, false, true>, dim3((unsigned)BG.parts), dim3(EP_THREADS), 0, VG,
+                   EncCheck{}, BG.parts, BG.tp, BG.tile_r, BG.rows, BG.row_len, BG.lvlmask, (const EncGroup *)BG.groups,
+                   c.d_status);
+            launch_carry(c, BG);
+            launch_tiles<EncTileA, false, true>(c, VG, BG, EN_LEVELS_A, EN_STREAMS_A, 0u, sorted, out_range, out_nop);
+        } else if (!have_parts) {
             launch(c, "enc_view", keys ? k_enc_parts<false, true> : k_enc_parts<false, false>, dim3((unsigned)B.parts),
                    dim3(EP_THREADS), 0, V, EncCheck{}, B.parts, B.tp, B.tile_r, B.rows, B.row_len, B.lvlmask,
-                   c.d_status);
+                   (const EncGroup *)nullptr, c.d_status);
             launch_carry(c, B);
+            have_parts = true;
         }
-        have_parts = true;
-        if (!wide)
-            (keys ? launch_tiles<EncTileA, true> : launch_tiles<EncTileA, false>)(c, V, B, EN_LEVELS_A, EN_STREAMS_A, 1, 0u, sorted,
+        if (!grouped && !many)
+            (keys ? launch_tiles<EncTileA, true> : launch_tiles<EncTileA, false>)(c, V, B, EN_LEVELS_A, EN_STREAMS_A, 0u, sorted,
                                                                                   out_range, out_nop);
-        else if (nl <= EN_LEVELS_B)
-            (keys ? launch_tiles<EncTileB, true> : launch_tiles<EncTileB, false>)(c, V, B, nl, ns, 1, 0u, sorted, out_range,
-                                                                                  out_nop);
-        else
-            (keys ? launch_tiles<EncTileB, true, true> : launch_tiles<EncTileB, false, true>)(
-                c, V, B, EN_LEVELS_B, 64, 4, 0u, sorted, out_range, out_nop);
+        else if (!grouped)
+            (keys ? launch_tiles<EncTileB, true> : launch_tiles<EncTileB, false>)(c, V, B, present.levels, present.streams, 0u,
+                                                                                  sorted, out_range, out_nop);
         if ((st = read_status(c))) return st;
-        if (c.h_status->flags & F_LEVELS_MANY) {
-            nl = (int)c.h_status->nlevels;
-            ns = (int)c.h_status->nstreams;
-            wide = true;
-            continue;
-        }
         if ((c.h_status->flags & F_LEVEL_FIXUP) && !sorted) {
             sort_ranges = true;
             have_parts = false;

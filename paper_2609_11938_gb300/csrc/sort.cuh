@@ -262,6 +262,66 @@ __global__ void __launch_bounds__(RADIX_THREADS) k_digit_rank(DigitFn digit, int
     epi.done(bits);
 }
 
+// The same for an epi that moves wide elements: it is called in order of the
+// destinations, so that a tile's elements of one digit are written side by side
+// (and read from the 4,096 of the tile).
+template <typename DigitFn, typename Epi>
+__global__ void __launch_bounds__(RADIX_THREADS) k_digit_move(DigitFn digit, int64_t n,
+                                                              const uint32_t *__restrict__ offs, int64_t ntiles,
+                                                              Epi epi) {
+    pdl_wait();
+    constexpr int WARPS = RADIX_THREADS / 32;
+    __shared__ uint32_t wcnt[WARPS * RADIX_BINS];
+    __shared__ uint32_t gbase[RADIX_BINS], dstart[RADIX_BINS], wbuf[33];
+    __shared__ uint16_t src[RADIX_TILE];
+    __shared__ uint8_t sdig[RADIX_TILE];
+    const unsigned w = threadIdx.x >> 5, lane = lane_id(), lt = lanemask_lt();
+    for (int i = threadIdx.x; i < WARPS * RADIX_BINS; i += RADIX_THREADS) wcnt[i] = 0;
+    __syncthreads();
+    const int64_t tile0 = (int64_t)blockIdx.x * RADIX_TILE;
+    const int at = (int)w * (RADIX_TILE / WARPS) + (int)lane;
+    unsigned dig[RADIX_ITEMS], peers[RADIX_ITEMS];
+    uint32_t rank[RADIX_ITEMS];
+#pragma unroll
+    for (int it = 0; it < RADIX_ITEMS; ++it) {
+        const int64_t i = tile0 + at + it * 32;
+        dig[it] = i < n ? digit(i) : (unsigned)RADIX_BINS;
+        peers[it] = warp_peers8(dig[it], dig[it] < RADIX_BINS);
+    }
+#pragma unroll
+    for (int it = 0; it < RADIX_ITEMS; ++it) {
+        const unsigned d = dig[it], before = d < RADIX_BINS ? wcnt[w * RADIX_BINS + d] : 0u;
+        __syncwarp();
+        if (d < RADIX_BINS && (peers[it] & lt) == 0) wcnt[w * RADIX_BINS + d] = before + __popc(peers[it]);
+        __syncwarp();
+        rank[it] = before + __popc(peers[it] & lt);
+    }
+    __syncthreads();
+    uint32_t sum = 0, total;
+#pragma unroll
+    for (int q = 0; q < WARPS; ++q) {                 // thread d: digit d over the warps
+        const uint32_t x = wcnt[q * RADIX_BINS + threadIdx.x];
+        wcnt[q * RADIX_BINS + threadIdx.x] = sum;
+        sum += x;
+    }
+    dstart[threadIdx.x] = block_exclusive_scan<uint32_t>(sum, wbuf, &total);
+    gbase[threadIdx.x] = sum ? offs[(int64_t)threadIdx.x * ntiles + blockIdx.x] : 0u;
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < RADIX_ITEMS; ++it) {
+        if (dig[it] >= RADIX_BINS) continue;
+        const uint32_t p = dstart[dig[it]] + wcnt[w * RADIX_BINS + dig[it]] + rank[it];
+        src[p] = (uint16_t)(at + it * 32);
+        sdig[p] = (uint8_t)dig[it];
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (uint32_t j = threadIdx.x; j < total; j += RADIX_THREADS) {
+        const unsigned d = sdig[j];
+        epi(tile0 + src[j], gbase[d] + (j - dstart[d]), d);
+    }
+}
+
 // nbins: digits used (every digit below it); only those rows of the matrix
 // are counted on and scanned.  The scan goes out of place, into the second
 // half of `hist` (radix_hist_elems(n) entries: one pass); the offsets'
@@ -284,6 +344,14 @@ void digit_rank(Ctx &c, const char *name, DigitFn digit, int64_t n, const uint32
     if (n <= 0) return;
     const int64_t ntiles = (n + RADIX_TILE - 1) / RADIX_TILE;
     launch(c, name, k_digit_rank<DigitFn, Epi>, dim3((unsigned)ntiles), dim3(RADIX_THREADS), 0, digit, n, hist,
+           ntiles, epi);
+}
+
+template <typename DigitFn, typename Epi>
+void digit_move(Ctx &c, const char *name, DigitFn digit, int64_t n, const uint32_t *hist, Epi epi) {
+    if (n <= 0) return;
+    const int64_t ntiles = (n + RADIX_TILE - 1) / RADIX_TILE;
+    launch(c, name, k_digit_move<DigitFn, Epi>, dim3((unsigned)ntiles), dim3(RADIX_THREADS), 0, digit, n, hist,
            ntiles, epi);
 }
 

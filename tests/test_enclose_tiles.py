@@ -35,6 +35,38 @@ def test_layouts(streams, depth, shuffle):
                              shuffle=shuffle))
 
 
+@pytest.mark.parametrize("shuffle", [False, True])
+@pytest.mark.parametrize("streams,depth,n", [(130, 5, 30_000), (255, 4, 30_000), (130, 32, 300), (200, 32, 80_000),
+                                             (256, 32, 60_000)])
+def test_groups_of_streams(streams, depth, n, shuffle):
+    """Past 64 streams, and taken by groups of 16 past 2,048 levels: groups
+    without kernels, without ranges and with neither, few events and many."""
+    t = tracegen.generate("adversarial", n_kernels=n, n_streams=streams, max_depth=depth, seed=n + depth, shuffle=shuffle)
+    _check(t)
+    k, r = t.k_stream // 16, t.r_stream // 16
+    keep_k, keep_r = ~np.isin(k, (1, 4, 7)), ~np.isin(r, (2, 4))
+    t = dataclasses.replace(t, **{f: getattr(t, f)[keep_k].copy() for f in ("k_stream", "k_start", "k_dur", "k_name")},
+                            **{f: getattr(t, f)[keep_r].copy() for f in ("r_stream", "r_start", "r_end", "r_depth", "r_op")})
+    _check(t)
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_ties_in_groups_of_streams(seed):
+    """Equal starts out of (start, end) order on many streams: sorted, then grouped."""
+    t = tracegen.small_random(500 + seed, n_streams=90, n_events=300, t_max=40, max_depth=5, shuffle=bool(seed & 1),
+                              n_names=7)
+    # with a chain of 32 levels on every stream, long before
+    s, d = np.divmod(np.arange(90 * 32), 32)
+    add = lambda a, v: np.concatenate([a, v.astype(a.dtype)])
+    _check(dataclasses.replace(t, r_stream=add(t.r_stream, s), r_depth=add(t.r_depth, d), r_start=add(t.r_start, d - 500),
+                               r_end=add(t.r_end, -400 - d), r_op=add(t.r_op, 0 * s)))
+
+
+def test_groups_of_many_short_streams():
+    """More than 160 streams and 4M events: by groups, though the levels are few."""
+    _check(tracegen.generate("adversarial", n_kernels=4_400_000, n_streams=200, max_depth=3, seed=8))
+
+
 @pytest.mark.parametrize("seed", range(6))
 def test_ties_across_tiles(seed):
     """Thousands of events at few instants: ties of starts, ends and kernels
