@@ -415,10 +415,10 @@ __device__ __forceinline__ int32_t range_of_t(const int32_t *rok, const uint32_t
 }
 
 // Within a join whose enclosure's verdict is still to be read (pending): the
-// enclosure found records out of order, more levels than its layout holds or
-// an error, and wrote nothing to aggregate.
+// enclosure found records out of order, more levels than its layout holds, events
+// too far apart or an error, and did not write all there is to aggregate.
 __device__ __forceinline__ bool stopped(const DevStatus *st) {
-    return (st->err & (ERR_INVALID | ERR_DEPTH)) || (st->flags & (F_K_UNSORTED | F_R_UNSORTED | F_LEVELS_MANY));
+    return (st->err & (ERR_INVALID | ERR_DEPTH)) || (st->flags & (F_REDO & ~F_LEVEL_FIXUP));
 }
 
 // ------------------------------------------------------------------ count

@@ -449,6 +449,7 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
             c.agg_words = 0;
             c.agg_ready = false;
             c.join_scratch = 0;
+            c.redo = 0;
         }
     } scope(c);
     // The matching can go ahead on the taking that the records are in order, so
@@ -509,7 +510,7 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
             // the enclosure's error comes before the matching's
             if (!c.enclose_pending) return sm;
             if ((st = read_status(c)) < 0) return st;
-            if (c.h_status->flags & (F_LEVEL_FIXUP | F_K_UNSORTED | F_R_UNSORTED | F_LEVELS_MANY)) continue;
+            if ((c.redo = c.h_status->flags & F_REDO)) continue;
             st = enclose_verdict(*c.h_status, kernels->n);
             return st < 0 ? st : sm;
         }
@@ -524,7 +525,7 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
             // the enclosure's verdict and the pairing's, read with the aggregation's status
             c.enclose_pending = false;
             // redone without deferring
-            if (c.h_status->flags & (F_LEVEL_FIXUP | F_K_UNSORTED | F_R_UNSORTED | F_LEVELS_MANY)) continue;
+            if ((c.redo = c.h_status->flags & F_REDO)) continue;
             // the enclosure's error before the aggregation's (nesting is only
             // judged when the range records passed their checks)
             DevStatus H = *c.h_status;

@@ -33,6 +33,9 @@ enum FlagBit : unsigned {
     F_AGG_MISS = 32u,     // the owned-range aggregation missed kernels
     F_IDX_NOT_ID = 64u,   // some kernel's ncu row index is neither its own index nor -1
     F_LEVELS_MANY = 128u, // more range levels than the enclosure's common layout holds
+    F_TIMES_FAR = 256u,   // events too far apart for the enclosure's 32-bit times
+    // the enclosure has to run again
+    F_REDO = F_K_UNSORTED | F_R_UNSORTED | F_LEVEL_FIXUP | F_LEVELS_MANY | F_TIMES_FAR,
 };
 enum CountSlot {
     C_NAMES_MISMATCH = 0,
@@ -128,6 +131,7 @@ struct Ctx {
     // verdict is pending until then (enclose_pending; the aggregation keeps
     // the status block instead of resetting it)
     bool defer_status = false, enclose_pending = false;
+    unsigned redo = 0;               // why the enclosure's deferred run did not do (F_REDO bits)
     // within a join: the matching was the identity pairing (row k for kernel
     // k), so the aggregation need not read the row indices
     bool rows_identity = false;

@@ -453,14 +453,16 @@ __global__ void __launch_bounds__(1024) k_enc_carry(uint32_t *__restrict__ rows,
 // entries, E_NONE none.
 constexpr unsigned E_NONE = 0xFFFFu;
 constexpr unsigned D_DEPTH = 31u, D_MIXED = 32u;     // bits of `dep`
-template <int THREADS_, int BLOCKS_, bool JUMP_>
+template <int THREADS_, int BLOCKS_, bool JUMP_, typename Time_>
 struct EncTile {
+    using Time = Time_;                              // of a step, relative to its first event
     static constexpr int THREADS = THREADS_, BLOCKS = BLOCKS_;
     static constexpr bool JUMP = JUMP_;
     static constexpr int WORDS = 16;                 // ranges of a step, 32 to a group
     static constexpr int SR = 32 * WORDS;
     static constexpr int RPT = WORDS / (THREADS / 32);   // groups of a warp
-    uint32_t *ss, *se, *si;      // start, end (relative), position | kind << 30
+    Time *ss, *se;               // start, end (relative)
+    uint32_t *si;                // position | kind << 30
     uint32_t *amask;             // [ns] depths with an open range, per compact stream
     uint32_t *smask;             // [ns][WORDS] the stream's ranges among the tile's, one bit each
     uint32_t *sgroups;           // [ns] the groups that hold some
@@ -482,8 +484,8 @@ struct EncTile {
     __device__ __forceinline__ EncTile(unsigned char *p, int nl, int ns) {
         const int cap = SR + nl;
         auto take = [&](size_t n) { unsigned char *q = p; p += n; return q; };
-        ss = reinterpret_cast<uint32_t *>(take((size_t)cap * 4));
-        se = reinterpret_cast<uint32_t *>(take((size_t)cap * 4));
+        ss = reinterpret_cast<Time *>(take((size_t)cap * sizeof(Time)));
+        se = reinterpret_cast<Time *>(take((size_t)cap * sizeof(Time)));
         si = reinterpret_cast<uint32_t *>(take((size_t)cap * 4));
         amask = reinterpret_cast<uint32_t *>(take((size_t)ns * 4));
         smask = reinterpret_cast<uint32_t *>(take((size_t)ns * WORDS * 4));
@@ -507,11 +509,12 @@ struct EncTile {
         last = take((size_t)WORDS * nl);
     }
     static size_t smem(int nl, int ns) {
-        return (size_t)(SR + nl) * 26 + SR + (size_t)(WORDS + 2) * nl + (size_t)ns * (8 + 6 * WORDS + 1) + 1024 + 512;
+        return (size_t)(SR + nl) * (18 + 2 * sizeof(Time)) + SR + (size_t)(WORDS + 2) * nl + (size_t)ns * (8 + 6 * WORDS + 1) + 1024 + 512;
     }
 };
-using EncTileA = EncTile<256, 4, false>;
-using EncTileB = EncTile<512, 2, true>;
+using EncTileA = EncTile<256, 4, false, uint32_t>;
+using EncTileB = EncTile<512, 2, true, uint32_t>;
+using EncTileF = EncTile<256, 4, false, uint64_t>;       // the common layout for events far apart
 constexpr int EN_LEVELS_A = 512, EN_STREAMS_A = 64;      // levels and streams of the common layout
 constexpr int EN_LEVELS_B = 2048;                        // levels of the wide one
 // Groups of streams: past the wide layout's levels, and where a step of the whole
@@ -524,7 +527,13 @@ constexpr int EN_STREAMS_B = 160;
 constexpr int64_t EN_GROUP_EVENTS = 4 << 20;
 constexpr int64_t EN_TILE = 2048, EN_TILE_MIN = 512;     // events of a tile; of a part's one tile in small traces
 constexpr int64_t EN_EARLY = 1 << 20;                    // events from which a join looks at the checks before the end
-constexpr uint32_t EN_SPAN = 0xFFFFFFF0u;                // a step's times fit 32 bits relative to its first
+// Times of a step in 32 bits end it 4 s after its first event.  A block that has
+// taken more than EN_FAR steps, and one per tile, that ended so gives the trace up
+// (F_TIMES_FAR), and it is taken with times in 64 bits.  A join of 1M kernels on 8
+// streams with an event every 20 / 200 / 5,000 ms: 348 / 325 / 309 us, 336 / 1,157 /
+// 4,544 by 32-bit steps alone, 184 with events 0.3 ms apart.
+constexpr int EN_FAR = 8;
+constexpr size_t EN_SMEM_F = 74 * 1024;                  // of that layout: three blocks a multiprocessor at least, else groups
 
 // One block per part, tile by tile; a tile with more ranges than SR, or whose
 // times span 2^32 ns, is taken in steps.  A step's ranges, and the ranges open
@@ -585,6 +594,8 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
               uint8_t *__restrict__ out_nop, DevStatus *st) {
     pdl_wait();
     constexpr int THREADS = TL::THREADS, WARPS = THREADS / 32, RPT = TL::RPT, SR = TL::SR, WORDS = TL::WORDS;
+    using Time = typename TL::Time;
+    constexpr Time NEVER = ~(Time)0;                 // an end past a step's times
     static_assert(THREADS >= 256, "a thread per stream");
     static_assert(WORDS == 16 && RPT * WARPS == WORDS, "half a warp per stream, 16 bits per level");
     if ((st->err & (ERR_INVALID | ERR_DEPTH)) || (st->flags & leave_on)) return;
@@ -641,13 +652,13 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
         return t < a ? t : a;
     };
     long long base = first_time(k, r), first = base;      // times are relative to base; the step's first event
-    auto rel = [&](long long x) -> uint32_t {
+    auto rel = [&](long long x) -> Time {
         const unsigned long long v = (unsigned long long)x - (unsigned long long)base;
-        return x < base ? 0u : (v >= 0xFFFFFFFEull ? 0xFFFFFFFFu : (uint32_t)v + 1u);
+        return x < base ? (Time)0 : (v >= (unsigned long long)NEVER - 1 ? NEVER : (Time)(v + 1));
     };
     // What a warp writes of a stream's open ranges, lane by depth: the chain of
     // each is the run of open levels above it, read off four ballots.
-    auto open_ranges = [&](int q, uint32_t e0, bool live, uint32_t a, uint32_t z, uint32_t i) {
+    auto open_ranges = [&](int q, uint32_t e0, bool live, Time a, Time z, uint32_t i) {
         const uint32_t kind = i >> 30;
         const unsigned m = __ballot_sync(0xffffffffu, live), le = lt | 1u << lane;
         const unsigned ops = __ballot_sync(0xffffffffu, live && kind == KIND_OP);
@@ -675,7 +686,8 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
     };
     for (int q = (int)warp; q < ns; q += WARPS) {                                // a warp per stream, a lane per depth
         const unsigned s = S.slist[q], l = s * 32u + lane;
-        uint32_t v = 0, a = 0, z = 0, i = 0;
+        uint32_t v = 0, i = 0;
+        Time a = 0, z = 0;
         if (lane < S.ndep[s]) {
             if (carried) v = rows[b * LEVELS + l];
             else
@@ -696,6 +708,7 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
         open_ranges(q, (uint32_t)SR + S.cbase[s], live, a, z, i);
     }
     bool err = false, fix = false;
+    int far = 0;
     int64_t r_end_n = tile_r[b * tp + 1];           // the next step's end
     __syncthreads();
     for (int64_t t = b * tp + 1; t <= (b + 1) * tp; ++t) {
@@ -707,7 +720,7 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
             // ---- the step: the whole tile, or up to the first event that
             // must wait (a kernel that starts no earlier than a range not
             // loaded; 2^32 ns from base)
-            auto near = [&](long long x) { return (unsigned long long)x - (unsigned long long)base < EN_SPAN; };
+            auto near = [&](long long x) { return (unsigned long long)x - (unsigned long long)base < (unsigned long long)NEVER - 15; };
             const long long t_last = nk > 0 ? V.time<KEYS>(k + nk - 1) : first, a_last = nr > 0 ? V.r_start[r + nr - 1] : first;
             if (!(near(t_last) && near(a_last)) && base != first) {
                 // the open ranges relative to this step's first event (once in some 4 s of the trace)
@@ -716,19 +729,24 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                 for (int q = (int)warp; q < ns; q += WARPS) {
                     const unsigned s = S.slist[q];
                     const uint32_t e0 = (uint32_t)SR + S.cbase[s], e = e0 + lane;
-                    uint32_t a2 = 0, z2 = 0, i = 0;
+                    Time a2 = 0, z2 = 0;
+                    uint32_t i = 0;
                     if ((S.amask[q] >> lane) & 1u) {
-                        const uint32_t a = S.ss[e], z = S.se[e];
+                        const Time a = S.ss[e], z = S.se[e];
                         i = S.si[e];
-                        a2 = (unsigned long long)a > shift ? a - (uint32_t)shift : 0u;
-                        z2 = z == 0xFFFFFFFFu ? rel(V.r_end[i & POS_MASK])
-                                              : ((unsigned long long)z > shift ? z - (uint32_t)shift : 0u);
+                        a2 = (unsigned long long)a > shift ? a - (Time)shift : (Time)0;
+                        z2 = z == NEVER ? rel(V.r_end[i & POS_MASK])
+                                        : ((unsigned long long)z > shift ? z - (Time)shift : (Time)0);
                     }
                     open_ranges(q, e0, z2 > 0, a2, z2, i);
                 }
                 __syncthreads();
             }
-            bool whole = r1 - r <= SR && near(t_last) && near(a_last);
+            const bool close = near(t_last) && near(a_last), whole = r1 - r <= SR && close;
+            if (sizeof(Time) == 4 && !close && ++far > EN_FAR + tp) {
+                if (tid == 0) set_flag(st, F_TIMES_FAR);
+                return;
+            }
             if (!whole) {
                 // by two warps, 32 probes a round
                 if (warp < 2) {
@@ -765,8 +783,8 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
             }
             const bool more = r + nr < V.R;                              // ranges past this step's
             const long long next = more ? V.r_start[r + nr] : 0;
-            // times of this step as 32 bits: exact for its events
-            auto rel_near = [&](long long x) { return (uint32_t)x - (uint32_t)base + 1u; };
+            // exact for the step's events
+            auto rel_near = [&](long long x) { return (Time)x - (Time)base + 1u; };
             // ---- ranges, 32 at a time: the stream's and the level's earlier
             // ranges in the group by lane masks, before it by tables (links)
             uint32_t lk[RPT], pk[RPT];               // the level's range before | level << 16; parent | prev on stream << 16
@@ -823,7 +841,7 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
             }
             __syncthreads();
             // ---- links, and the laminar checks.  Relative times are exact
-            // below 2^32 - 1; two clamped ends are compared as they are.
+            // below NEVER; two clamped ends are compared as they are.
             auto last_of = [&](uint32_t l, unsigned below) -> uint32_t {                 // the level's, in groups below; + 1
                 const unsigned h = (S.lgroups[l / 2] >> (16 * (l & 1u))) & ((1u << below) - 1u);
                 const unsigned g = 31 - __clz(h);
@@ -836,7 +854,7 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                 if (c == 0xFFFFu) continue;
                 const uint32_t e = g * 32 + lane;
                 const unsigned q = S.sid[e], d = S.dep[e] & D_DEPTH, am = S.amask[q];
-                const uint32_t a = S.ss[e];
+                const Time a = S.ss[e];
                 auto earlier = [&](uint32_t u, uint32_t l, unsigned depth) -> uint32_t {
                     if (u == 0) u = last_of(l, g);
                     return u ? u - 1 : ((am >> depth) & 1u ? (uint32_t)SR + l : (uint32_t)E_NONE);
@@ -857,8 +875,8 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                 }
                 auto end_of = [&](uint32_t w) { return V.r_end[S.si[w] & POS_MASK]; };
                 auto ends_before = [&](uint32_t w, uint32_t v) {                     // entry w ends before entry v
-                    const uint32_t f = S.se[w], g = S.se[v];
-                    return f == 0xFFFFFFFFu && g == 0xFFFFFFFFu ? end_of(w) < end_of(v) : f < g;
+                    const Time f = S.se[w], g = S.se[v];
+                    return f == NEVER && g == NEVER ? end_of(w) < end_of(v) : f < g;
                 };
                 if (y != E_NONE) {
                     if (S.ss[y] == a && ends_before(e, y)) fix = true;               // starts with it, ends before it
@@ -904,7 +922,7 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                 while (e < SR && S.ss[e] >= S.se[e]) e = S.prev[e];                      // zero length
                 if (e >= SR) return e == E_NONE ? e : (uint32_t)S.best[e];
                 uint32_t w = e;
-                const uint32_t a = S.ss[e];
+                const Time a = S.ss[e];
                 for (uint32_t x = S.prev[e]; x != E_NONE && S.ss[x] == a; x = S.prev[x])
                     if (S.se[x] > a && (S.dep[x] & D_DEPTH) > (S.dep[w] & D_DEPTH)) w = x;
                 return w;
@@ -942,7 +960,7 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
             {
                 int q0 = 0;                                                              // ranges before the run
                 if (j0 < j1) {
-                    const uint32_t T0 = __shfl_sync(0xffffffffu, rel_near(t_n), 0);
+                    const Time T0 = __shfl_sync(0xffffffffu, rel_near(t_n), 0);
                     int hi = nr;
                     while (q0 < hi) {
                         const int m = (q0 + hi) >> 1;
@@ -951,7 +969,7 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                 }
                 for (int j = j0; j < j1; j += 32) {
                     const bool in = j + (int)lane < j1;
-                    const uint32_t T = rel_near(t_n);
+                    const Time T = rel_near(t_n);
                     const unsigned s = s_n;
                     const int64_t kk = k + j + (int)lane;
                     if (j + 32 + (int)lane < j1) {
@@ -961,10 +979,10 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                     // ranges that start by each kernel: those by the last one
                     // first, then each lane's share of them
                     const int top = j1 - j < 32 ? j1 - j - 1 : 31;
-                    const uint32_t Tm = __shfl_sync(0xffffffffu, T, top);
+                    const Time Tm = __shfl_sync(0xffffffffu, T, top);
                     int qn = q0;
                     for (;;) {
-                        const uint32_t v = q0 + (int)lane < nr ? S.ss[q0 + lane] : 0xFFFFFFFFu;
+                        const Time v = q0 + (int)lane < nr ? S.ss[q0 + lane] : NEVER;
                         const int c = __popc(__ballot_sync(0xffffffffu, v <= Tm));
                         int h = 0;
 #pragma unroll
@@ -974,7 +992,7 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                             qn += h;
                             break;
                         }
-                        const uint32_t v31 = __shfl_sync(0xffffffffu, v, 31);
+                        const Time v31 = __shfl_sync(0xffffffffu, v, 31);
                         qn += h + (v31 <= T ? 1 : 0);
                     }
                     if (!in) continue;
@@ -1041,7 +1059,8 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                 const int q = S.tlist[j];
                 const unsigned s = S.slist[q];
                 const uint32_t l = S.cbase[s] + lane;
-                uint32_t a = 0, z = 0, i = 0;
+                uint32_t i = 0;
+                Time a = 0, z = 0;
                 bool live = false;
                 if (lane < S.ndep[s]) {
                     const uint32_t u = last_of(l, WORDS), f = u ? u - 1 : (uint32_t)SR + l;
@@ -1049,7 +1068,7 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                         a = S.ss[f];
                         z = S.se[f];
                         i = S.si[f];
-                        live = z == 0xFFFFFFFFu ? V.r_end[i & POS_MASK] >= nbase : (unsigned long long)z > now;
+                        live = z == NEVER ? V.r_end[i & POS_MASK] >= nbase : (unsigned long long)z > now;
                     }
                     if (u) reinterpret_cast<uint16_t *>(S.lgroups)[l] = 0;
                 }
@@ -1325,7 +1344,10 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     const SmallCopy masks{c.h_small, B.lvlmask, 256 * sizeof(uint32_t)};
     if (early && (st = post_status(c, 1, &masks))) return st;
     launch_carry(c, B);
-    launch_tiles<EncTileA, false>(c, V, B, EN_LEVELS_A, EN_STREAMS_A, F_K_UNSORTED | F_R_UNSORTED, false, out_range, out_nop);
+    const bool run = !(c.redo & ~F_LEVEL_FIXUP);      // (else it would leave as it did before)
+    if (run)
+        launch_tiles<EncTileA, false>(c, V, B, EN_LEVELS_A, EN_STREAMS_A, F_K_UNSORTED | F_R_UNSORTED, false, out_range,
+                                      out_nop);
     if (c.defer_status) {
         bool usual = true;
         if (early) {
@@ -1346,14 +1368,19 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     c.enclose_k_sorted = k_sorted ? 1 : 0;
     const LevelCount present(c.h_small);
     const bool many = present.levels > EN_LEVELS_A || present.streams > EN_STREAMS_A;
-    const bool grouped = present.levels > EN_LEVELS_B || (present.streams > EN_STREAMS_B && K + R > EN_GROUP_EVENTS);
+    // (with tiles that span 8 s on average the 32-bit times need no try)
+    const uint64_t span = K > 0 ? (uint64_t)c.h_status->mm[MM_KSTART_MAX] - (uint64_t)c.h_status->mm[MM_KSTART_MIN] : 0;
+    bool far = ((c.h_status->flags | c.redo) & F_TIMES_FAR) != 0 || (span >> 33) > (uint64_t)tiles;
+    bool grouped = present.levels > EN_LEVELS_B || (present.streams > EN_STREAMS_B && K + R > EN_GROUP_EVENTS);
+    const bool far_fits = !many || EncTileF::smem(present.levels + 7, present.streams + 7) <= EN_SMEM_F;
     const bool fixup = (c.h_status->flags & F_LEVEL_FIXUP) != 0;
-    if ((st = enclose_verdict(*c.h_status, K)) && !(fixup && st == OPATTR_E_NOT_NESTED)) return st;
-    if (k_sorted && r_sorted && !many && !fixup) return OPATTR_OK;
+    if ((st = enclose_verdict(*c.h_status, K)) && !((fixup || far) && st == OPATTR_E_NOT_NESTED)) return st;
+    if (run && k_sorted && r_sorted && !many && !fixup && !far) return OPATTR_OK;
 
     // ---- records out of order, ranges of one level that share a start and are
-    // out of (start, end) order, or more levels than the common layout holds:
-    // the tiles again, on the sorted view, with room for every level or by groups
+    // out of (start, end) order, more levels than the common layout holds, or
+    // events far apart: the tiles again, on the sorted view, with room for every
+    // level or by groups, with wider times
     const unsigned names_differ = c.h_status->flags & F_NAMES_DIFFER;   // the pairing's verdict stays
     const long long rmin = c.h_status->mm[MM_RSTART_MIN], rmax = c.h_status->mm[MM_REND_MAX];
     const long long kmin = c.h_status->mm[MM_KSTART_MIN];
@@ -1374,7 +1401,7 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     }
     const int64_t g_parts = B.parts + N_GROUPS, g_tiles = (K + R) / EN_TILE + B.parts + 3 * N_GROUPS;
     const int64_t g_part = scan_scratch_elems(std::max(radix_hist_elems(K), radix_hist_elems(R)));
-    if (grouped) {
+    if (many) {
         Need n3;
         n3.add<int64_t>(K).add<uint8_t>(K).add<uint32_t>(K).add<uint32_t>(radix_hist_elems(K)).add<uint32_t>(g_part);
         n3.add<int64_t>(R).add<int64_t>(R).add<uint8_t>(R).add<uint8_t>(R).add<uint32_t>(R).add<uint32_t>(R);
@@ -1425,8 +1452,9 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     bool sort_ranges = !r_sorted || fixup, sorted = false;
     bool have_parts = k_sorted && !sort_ranges && !grouped;       // (too many levels only: the checking pass's parts stand)
     GroupArrays ga{};
-    if (grouped && !ga.take(a, K, R, g_part, g_tiles, g_parts)) return OPATTR_E_OOM;
-    for (int attempt = 0; attempt < 2; ++attempt) {
+    if (many && !ga.take(a, K, R, g_part, g_tiles, g_parts)) return OPATTR_E_OOM;
+    for (int attempt = 0; attempt < 3; ++attempt) {
+        grouped = grouped || (far && !far_fits);
         if (sort_ranges && R > 0) {
             uint64_t *ko = nullptr;
             uint32_t *perm = nullptr;
@@ -1453,7 +1481,8 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
                    EncCheck{}, BG.parts, BG.tp, BG.tile_r, BG.rows, BG.row_len, BG.lvlmask, (const EncGroup *)BG.groups,
                    c.d_status);
             launch_carry(c, BG);
-            launch_tiles<EncTileA, false, true>(c, VG, BG, EN_LEVELS_A, EN_STREAMS_A, 0u, sorted, out_range, out_nop);
+            (far ? launch_tiles<EncTileF, false, true> : launch_tiles<EncTileA, false, true>)(
+                c, VG, BG, EN_LEVELS_A, EN_STREAMS_A, 0u, sorted, out_range, out_nop);
         } else if (!have_parts) {
             launch(c, "enc_view", keys ? k_enc_parts<false, true> : k_enc_parts<false, false>, dim3((unsigned)B.parts),
                    dim3(EP_THREADS), 0, V, EncCheck{}, B.parts, B.tp, B.tile_r, B.rows, B.row_len, B.lvlmask,
@@ -1461,13 +1490,21 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
             launch_carry(c, B);
             have_parts = true;
         }
-        if (!grouped && !many)
+        if (!grouped && far)
+            (keys ? launch_tiles<EncTileF, true> : launch_tiles<EncTileF, false>)(
+                c, V, B, std::max(EN_LEVELS_A, present.levels), std::max(EN_STREAMS_A, present.streams), 0u, sorted, out_range,
+                out_nop);
+        else if (!grouped && !many)
             (keys ? launch_tiles<EncTileA, true> : launch_tiles<EncTileA, false>)(c, V, B, EN_LEVELS_A, EN_STREAMS_A, 0u, sorted,
                                                                                   out_range, out_nop);
         else if (!grouped)
             (keys ? launch_tiles<EncTileB, true> : launch_tiles<EncTileB, false>)(c, V, B, present.levels, present.streams, 0u,
                                                                                   sorted, out_range, out_nop);
         if ((st = read_status(c))) return st;
+        if (c.h_status->flags & F_TIMES_FAR) {
+            far = true;
+            continue;
+        }
         if ((c.h_status->flags & F_LEVEL_FIXUP) && !sorted) {
             sort_ranges = true;
             have_parts = false;

@@ -86,13 +86,37 @@ def test_ranges_without_kernels():
     _check(t)
 
 
-@pytest.mark.parametrize("streams,depth", [(3, 6), (66, 12)])
+def _stretch(t, bits):
+    t0 = min(int(t.k_start.min()), int(t.r_start.min()))
+    return dataclasses.replace(t, k_start=(t.k_start - t0) << bits, r_start=(t.r_start - t0) << bits,
+                               r_end=(t.r_end - t0) << bits)
+
+
+@pytest.mark.parametrize("streams,depth", [(3, 6), (66, 12), (200, 32)])
 @pytest.mark.parametrize("bits", [12, 17, 24])
-def test_long_traces(streams, depth, bits):
+@pytest.mark.parametrize("shuffle", [False, True])
+def test_long_traces(streams, depth, bits, shuffle):
     """Times stretched until a part, then a step, then the gap between two
     events is longer than the 32 bits that times in a step have: open ranges
-    are made relative to a later event, with ends past 32 bits among them."""
-    t = tracegen.generate("adversarial", n_kernels=20_000, n_streams=streams, max_depth=depth, seed=bits)
-    t0 = min(int(t.k_start.min()), int(t.r_start.min()))
-    _check(dataclasses.replace(t, k_start=(t.k_start - t0) << bits, r_start=(t.r_start - t0) << bits,
-                               r_end=(t.r_end - t0) << bits))
+    are made relative to a later event, with ends past 32 bits among them, or
+    the trace is taken again with wider times; by each call and by a join."""
+    import paper_2609_11938_gb300 as opa
+    t = _stretch(tracegen.generate("adversarial", n_kernels=20_000, n_streams=streams, max_depth=depth, seed=bits,
+                                   shuffle=shuffle), bits)
+    _check(t)
+    o = oracle.run(t, enclose_mode="indexed")
+    with opa.Context(0) as ctx:
+        _, out, ops, _, _ = ctx.join(opa.to_device(t))
+    np.testing.assert_array_equal(out["range_of_kernel"].cpu().numpy(), o["range_of_kernel"])
+    np.testing.assert_array_equal(out["n_op_enclosing"].cpu().numpy(), o["n_op_enclosing"])
+    np.testing.assert_array_equal(ops["kernel_count"].cpu().numpy(), o["ops"]["kernel_count"])
+
+
+@pytest.mark.parametrize("streams", [2, 80])
+@pytest.mark.parametrize("seed", range(4))
+def test_ties_far_apart(streams, seed):
+    """Few instants, 17 s apart, with many events each: in array order, and out
+    of (start, end) order within a level."""
+    t = tracegen.small_random(700 + seed, n_streams=streams, n_events=18_000 // streams, t_max=60, max_depth=5,
+                              shuffle=bool(seed & 1), n_names=7)
+    _check(_stretch(t, 34))
