@@ -109,10 +109,18 @@ void check_kernel_order(Ctx &c, const uint8_t *stream, const int64_t *start, int
 // 6M kernel records in no order: 16 us to count, 77 to scatter (bound by the
 // scattered 8-byte writes), 90 to sort the buckets (shared-memory latency),
 // against 115 us for each of five radix passes.
+//
+// An entry holds 32 bits of key, so the span of the keys sets how many buckets
+// there are at least, however few the records: 2^(bits - 32) of them.  A bucket
+// costs its block some 12 ns whatever it holds.  Up to BK_FEW buckets, or one to
+// BK_LEAST records, that is less than radix passes: 300,000 records whose keys span
+// 2^44 / 2^46 / 2^47 values 153 / 300 / 495 us by buckets and 206 by radix, 4M 298 /
+// 464 / 692 and 470; 3,000 with 4,096 buckets 126 and 170.
 constexpr int BK_THREADS = 512, BK_ITEMS = 16, BK_CAP = BK_THREADS * BK_ITEMS, BK_BIN_BITS = 12,
               BK_BINS = 1 << BK_BIN_BITS;
 constexpr int BK_TARGET = 3072;
 constexpr int BK_BIN_MAX = 64;
+constexpr int64_t BK_FEW = 4096, BK_LEAST = 256;
 constexpr int64_t BK_MAX = 32 * 1024;        // buckets: their counts fit a block's shared memory and one block's scan
 
 // Each block counts an equal share of the records in shared memory (global
@@ -287,7 +295,7 @@ static opattr_status time_sort(Ctx &c, Arena &a, Key key, int64_t n, uint64_t sp
     int shift = 32;
     while (shift > 0 && (int64_t)(top >> shift) + 1 < (n + BK_TARGET - 1) / BK_TARGET) --shift;
     const int64_t nb = (int64_t)(top >> shift) + 1;
-    if (c.host_mapped && nb <= BK_MAX) {
+    if (c.host_mapped && nb <= std::min(BK_MAX, std::max(BK_FEW, n / BK_LEAST))) {
         const int sms = sm_count(c);
         const size_t smem = sizeof(uint32_t) * nb, sort_smem = sizeof(uint64_t) * BK_CAP + sizeof(uint32_t) * BK_BINS;
         const dim3 g(grid_for(n, BK_THREADS * 8, (smem > 64 * 1024 ? 1 : 3) * sms));

@@ -16,13 +16,17 @@ def _times(case, n, rng):
         t = rng.integers(0, 50_000, n)
         t[0] = 1 << 40
         return t
+    if case in ("most buckets", "too many"):  # 4,096 buckets for few records, and one more
+        t = rng.integers(0, 4096 << 24, n)
+        t[0], t[-1] = (4096 << 24) - (case == "most buckets"), 0
+        return t
     if case == "long":                        # a span whose key needs more buckets than there may be
         return rng.integers(0, 1 << 52, n)
     assert case == "near"                     # nearly in order
     return np.arange(n) * 900 - rng.integers(0, 4000, n)
 
 
-@pytest.mark.parametrize("case", ["spread", "equal", "crowded", "long", "near"])
+@pytest.mark.parametrize("case", ["spread", "equal", "crowded", "most buckets", "too many", "long", "near"])
 @pytest.mark.parametrize("n", [2, 3073, 8193, 300_007])
 def test_time_order(case, n):
     import torch
