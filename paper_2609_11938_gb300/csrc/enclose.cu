@@ -1368,9 +1368,9 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     c.enclose_k_sorted = k_sorted ? 1 : 0;
     const LevelCount present(c.h_small);
     const bool many = present.levels > EN_LEVELS_A || present.streams > EN_STREAMS_A;
-    // (with tiles that span 8 s on average the 32-bit times need no try)
+    // (with tiles that span 8 s on average, 4 in the wide layout, the 32-bit times need no try)
     const uint64_t span = K > 0 ? (uint64_t)c.h_status->mm[MM_KSTART_MAX] - (uint64_t)c.h_status->mm[MM_KSTART_MIN] : 0;
-    bool far = ((c.h_status->flags | c.redo) & F_TIMES_FAR) != 0 || (span >> 33) > (uint64_t)tiles;
+    bool far = ((c.h_status->flags | c.redo) & F_TIMES_FAR) != 0 || (span >> (many ? 32 : 33)) > (uint64_t)tiles;
     bool grouped = present.levels > EN_LEVELS_B || (present.streams > EN_STREAMS_B && K + R > EN_GROUP_EVENTS);
     const bool far_fits = !many || EncTileF::smem(present.levels + 7, present.streams + 7) <= EN_SMEM_F;
     const bool fixup = (c.h_status->flags & F_LEVEL_FIXUP) != 0;
