@@ -1037,59 +1037,29 @@ __device__ __forceinline__ void acc_merge(Acc &a, const Acc &b) {
     for (int i = 0; i < N_MAX; ++i) a.mx[i] = fmaxf(a.mx[i], b.mx[i]);
 }
 
-// Piece offsets of the listed long ops, one block: poff[j] = pieces of the
-// ops listed before j (an op longer than `huge` has ceil(len / AG_PIECE)
-// pieces, a shorter one none); poff[nlong] = all pieces.
-// info (may be NULL) receives {listed ops, pieces, longest huge op, kernels
-// in huge ops, huge ops}; hop (with info) the huge ops in list order.
+// Piece offsets of the listed ops, one block: poff[j] = pieces of the ops listed
+// before j (ceil(kernels / AG_PIECE) each); poff[number of them] = all pieces.
 __global__ void __launch_bounds__(1024) k_agg_piece_offsets(const uint32_t *__restrict__ off,
                                                             const uint32_t *__restrict__ longs,
-                                                            const unsigned *__restrict__ nlong, uint32_t huge,
-                                                            uint32_t *__restrict__ poff, uint32_t *__restrict__ info,
-                                                            uint32_t *__restrict__ hop) {
+                                                            const unsigned *__restrict__ nlong,
+                                                            uint32_t *__restrict__ poff) {
     pdl_wait();
     __shared__ uint32_t wbuf[33];
     const int64_t n = *nlong;
-    uint32_t carry = 0, longest = 0, kern = 0, hcarry = 0;
+    uint32_t carry = 0;
     for (int64_t b = 0; b < n; b += 1024) {
         const int64_t j = b + threadIdx.x;
-        uint32_t np = 0, o = 0;
+        uint32_t np = 0;
         if (j < n) {
-            o = longs[j];
-            const uint32_t len = off[o + 1] - off[o];
-            np = len > huge ? (len + AG_PIECE - 1) / AG_PIECE : 0u;
-            if (np) {
-                longest = len > longest ? len : longest;
-                kern += len;
-            }
+            const uint32_t o = longs[j];
+            np = (off[o + 1] - off[o] + AG_PIECE - 1) / AG_PIECE;
         }
         uint32_t tot;
         const uint32_t ex = block_exclusive_scan<uint32_t>(np, wbuf, &tot);
         if (j < n) poff[j] = carry + ex;
         carry += tot;
-        if (info) {
-            uint32_t htot;
-            const uint32_t hx = block_exclusive_scan<uint32_t>(np ? 1u : 0u, wbuf, &htot);
-            if (np) hop[hcarry + hx] = o;
-            hcarry += htot;
-        }
     }
     if (threadIdx.x == 0) poff[n] = carry;
-    if (info) {
-        const uint32_t ksum = block_sum<uint32_t>(kern, wbuf);
-        __shared__ uint32_t lmax;
-        if (threadIdx.x == 0) lmax = 0;
-        __syncthreads();
-        atomicMax(&lmax, longest);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            info[0] = (uint32_t)n;
-            info[1] = carry;
-            info[2] = lmax;
-            info[3] = ksum;
-            info[4] = hcarry;
-        }
-    }
 }
 
 // Huge ops' segments in ascending kernel index without sorting: with at most
@@ -1333,7 +1303,7 @@ constexpr int FIN_THREADS = 256;
 __global__ void __launch_bounds__(FIN_THREADS) k_agg_long_ops(const uint32_t *__restrict__ longs,
                                                               const unsigned *__restrict__ nlong,
                                                               const uint32_t *__restrict__ poff,
-                                                              const Acc *__restrict__ part, int write_empty, AggIn A,
+                                                              const Acc *__restrict__ part, AggIn A,
                                                               DevStatus *st) {
     pdl_wait();
     __shared__ Acc wpart[FIN_THREADS / 32];
@@ -1341,7 +1311,6 @@ __global__ void __launch_bounds__(FIN_THREADS) k_agg_long_ops(const uint32_t *__
     const unsigned lane = lane_id(), w = threadIdx.x >> 5;
     int bad = 0;
     for (int64_t q = blockIdx.x; q < n; q += gridDim.x) {
-        if (poff[q + 1] == poff[q] && !write_empty) continue;   // not huge: the ops pass writes it
         const uint32_t o = longs[q];
         Acc acc;
         acc.init();
@@ -1391,8 +1360,7 @@ size_t aggregate_scratch(int64_t K, uint32_t n_ops) {
     nd.add<uint32_t>(mids_n).add<uint32_t>(mids_n).add<uint32_t>(O + 1);
     nd.add<uint32_t>(mids_n).add<Acc>(agg_partials(K));
     nd.add<uint32_t>(scan_scratch_elems(std::max<int64_t>(O + 1, radix_hist_elems(K))));
-    nd.add<uint32_t>(O + 1).add<uint32_t>(radix_hist_elems(K)).add<uint32_t>(8);   // huge-op index, histogram, info
-    nd.add<uint32_t>(mids_n);                                                        // huge ops
+    nd.add<uint32_t>(O + 1).add<uint32_t>(radix_hist_elems(K));       // huge-op index, histogram
     return nd.bytes + 4096;
 }
 
@@ -1440,8 +1408,7 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
     if (!npc || !partials) return OPATTR_E_OOM;
     uint32_t *part = a.take<uint32_t>(scan_scratch_elems(std::max<int64_t>(O + 1, radix_hist_elems(K))));
     uint32_t *hidx = a.take<uint32_t>(O + 1), *hhist = a.take<uint32_t>(radix_hist_elems(K));
-    uint32_t *info = a.take<uint32_t>(8), *hop = a.take<uint32_t>(mids_n);
-    if (!hidx || !hhist || !info || !hop) return OPATTR_E_OOM;
+    if (!hidx || !hhist) return OPATTR_E_OOM;
     if (!off || !list || !tmp || !mids || !longs || !part || !dirty) return OPATTR_E_OOM;
     // with the enclosure's or the matching's verdict pending (a join) the status
     // block keeps it: the enclosure's reset left the aggregation's slots at zero
@@ -1509,26 +1476,19 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
             launch(c, "agg_mid", k_agg_mid<512>, dim3(std::min<uint32_t>(n_mid, (unsigned)sms)), dim3(512), 0,
                    (const uint32_t *)off, (const uint32_t *)list, in, c.d_status);
         }
-        uint32_t pieces = 0, n_huge = 0;
         if (n_long > 0) {
             launch(c, "agg_piece_offsets", k_agg_piece_offsets, dim3(1), dim3(1024), 0, (const uint32_t *)off,
-                   (const uint32_t *)longs, (const unsigned *)nlong, 0u, npc, info, hop);
-            const SmallCopy pinfo{c.h_small, info, 5 * sizeof(uint32_t)};
-            if ((st = read_status(c, 1, &pinfo))) return st;
-            pieces = c.h_small[1];
-            n_huge = c.h_small[4];
-        }
-        if (pieces > 0) {
-            if (n_huge <= (uint32_t)RADIX_BINS && K > 0) {
+                   (const uint32_t *)longs, (const unsigned *)nlong, npc);
+            if (n_long <= (uint32_t)RADIX_BINS) {
                 // very long segments: placed in kernel order by one counting pass
                 cudaMemsetAsync(hidx, 0xFF, sizeof(uint32_t) * (O + 1), c.stream);
-                launch(c, "huge_index", k_huge_index, dim3(grid_for(n_huge, 256, 4096)), dim3(256), 0,
-                       (const uint32_t *)hop, (int64_t)n_huge, hidx);
+                launch(c, "huge_index", k_huge_index, dim3(grid_for(n_long, 256, 4096)), dim3(256), 0,
+                       (const uint32_t *)longs, (int64_t)n_long, hidx);
                 const HugeDigit dg{rok, rng->op_id, R, O, hidx};
                 const uint32_t *hoffs = digit_offsets(c, dg, K, hhist, part);
                 const int64_t ntiles = (K + RADIX_TILE - 1) / RADIX_TILE;
                 digit_rank(c, "huge_place", dg, K, hoffs,
-                           HugePlace{hoffs, ntiles, (const uint32_t *)hop, (const uint32_t *)off, list});
+                           HugePlace{hoffs, ntiles, (const uint32_t *)longs, (const uint32_t *)off, list});
             } else {
                 launch(c, "agg_sort_long", k_agg_sort_long, dim3(2 * std::max(1, sms)), dim3(SL_THREADS), 0,
                        (const uint32_t *)off, (const uint32_t *)longs, (const unsigned *)nlong, 2u,
@@ -1537,7 +1497,7 @@ opattr_status do_aggregate(Ctx &c, const opattr_kernels *kern, const opattr_rang
             launch_pieces(c, off, list, longs, nlong, npc, in, partials);
             launch(c, "agg_long_ops", k_agg_long_ops, dim3(2 * std::max(1, sms)), dim3(FIN_THREADS), 0,
                    (const uint32_t *)longs, (const unsigned *)nlong, (const uint32_t *)npc,
-                   (const Acc *)partials, 0, in, c.d_status);
+                   (const Acc *)partials, in, c.d_status);
         }
     }
     if (!status_fresh && (st = read_status(c))) return st;
@@ -1840,10 +1800,10 @@ opattr_status do_rollup(Ctx &c, const opattr_kernels *kern, const opattr_ranges 
         } else {
             launch(c, "class_iota", k_iota_u32, dim3(grid_for(C, 256, 4096)), dim3(256), 0, cls, C, ncls);
             launch(c, "agg_piece_offsets", k_agg_piece_offsets, dim3(1), dim3(1024), 0, (const uint32_t *)off,
-                   (const uint32_t *)cls, (const unsigned *)ncls, 0u, poff, (uint32_t *)nullptr, (uint32_t *)nullptr);
+                   (const uint32_t *)cls, (const unsigned *)ncls, poff);
             if (K > 0) launch_pieces(c, off, list, cls, ncls, poff, in, partials);
             launch(c, "class_records", k_agg_long_ops, dim3(2 * sms), dim3(FIN_THREADS), 0, (const uint32_t *)cls,
-                   (const unsigned *)ncls, (const uint32_t *)poff, (const Acc *)partials, 1, in, c.d_status);
+                   (const unsigned *)ncls, (const uint32_t *)poff, (const Acc *)partials, in, c.d_status);
         }
     }
     if ((st = read_status(c))) return st;
