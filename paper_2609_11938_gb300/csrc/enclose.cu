@@ -469,7 +469,7 @@ struct EncTile {
     uint16_t *par, *prev, *best; // parent; the entry before on the stream; where the climb begins (below)
     uint16_t *va;                // innermost operator of the entry's chain
     uint16_t *top;               // outermost ancestor
-    uint16_t *jump;              // ancestor four levels up, E_NONE none (where chains are long)
+    uint16_t *jump;              // with JUMP: ancestor four levels up, E_NONE none (where chains are long)
     uint16_t *before;            // [ns][WORDS] the stream's last entry before each group (before the first one
                                  // its deepest open range), E_NONE none
     uint32_t *lgroups;           // [nl / 2] the groups that hold ranges of a level, 16 bits each
@@ -496,7 +496,7 @@ struct EncTile {
         best = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
         va = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
         top = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
-        jump = reinterpret_cast<uint16_t *>(take((size_t)cap * 2));
+        jump = reinterpret_cast<uint16_t *>(take(JUMP ? (size_t)cap * 2 : 0));
         before = reinterpret_cast<uint16_t *>(take((size_t)ns * WORDS * 2));
         cbase = reinterpret_cast<uint16_t *>(take(512));
         scid = reinterpret_cast<uint16_t *>(take(512));
@@ -509,7 +509,7 @@ struct EncTile {
         last = take((size_t)WORDS * nl);
     }
     static size_t smem(int nl, int ns) {
-        return (size_t)(SR + nl) * (18 + 2 * sizeof(Time)) + SR + (size_t)(WORDS + 2) * nl + (size_t)ns * (8 + 6 * WORDS + 1) + 1024 + 512;
+        return (size_t)(SR + nl) * (16 + (JUMP ? 2 : 0) + 2 * sizeof(Time)) + SR + (size_t)(WORDS + 2) * nl + (size_t)ns * (8 + 6 * WORDS + 1) + 1024 + 512;
     }
 };
 using EncTileA = EncTile<256, 4, false, uint32_t>;
