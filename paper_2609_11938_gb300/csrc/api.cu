@@ -112,9 +112,9 @@ int sm_count(Ctx &c) {
     return c.sms;
 }
 
-// Up to SMALL_COPIES transfers in one launch, each between mapped pinned host
-// memory and device memory: words when both ends and the size are 4-byte
-// aligned (every caller's case), bytes otherwise.
+// Up to SMALL_COPIES transfers in one launch (blockIdx.y), each between mapped
+// pinned host memory and device memory: words when both ends and the size are
+// 4-byte aligned (every caller's case), bytes otherwise.
 constexpr int SMALL_COPIES = 4;
 struct SmallCopies {
     const unsigned char *src[SMALL_COPIES];
@@ -125,17 +125,15 @@ struct SmallCopies {
 __global__ void k_copy_small(SmallCopies cp) {
     pdl_wait();
     const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
-    for (int q = 0; q < cp.count; ++q) {
-        const unsigned char *src = cp.src[q];
-        unsigned char *dst = cp.dst[q];
-        const size_t n = cp.n[q];
-        if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst) | n) & 3u) == 0) {
-            const uint32_t *s = reinterpret_cast<const uint32_t *>(src);
-            uint32_t *d = reinterpret_cast<uint32_t *>(dst);
-            for (size_t i = t0; i < n / 4; i += step) d[i] = s[i];
-        } else {
-            for (size_t i = t0; i < n; i += step) dst[i] = src[i];
-        }
+    const unsigned char *src = cp.src[blockIdx.y];
+    unsigned char *dst = cp.dst[blockIdx.y];
+    const size_t n = cp.n[blockIdx.y];
+    if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst) | n) & 3u) == 0) {
+        const uint32_t *s = reinterpret_cast<const uint32_t *>(src);
+        uint32_t *d = reinterpret_cast<uint32_t *>(dst);
+        for (size_t i = t0; i < n / 4; i += step) d[i] = s[i];
+    } else {
+        for (size_t i = t0; i < n; i += step) dst[i] = src[i];
     }
 }
 
@@ -159,8 +157,8 @@ opattr_status copy_small_n(Ctx &c, int count, const SmallCopy *cp, cudaMemcpyKin
             most = std::max(most, cp[q].bytes);
             a.count++;
         }
-        launch(c, "small_copy", k_copy_small, dim3(grid_for((int64_t)std::max<size_t>(most, 1), 256 * 16, 8)),
-               dim3(256), 0, a);
+        launch(c, "small_copy", k_copy_small,
+               dim3(grid_for((int64_t)std::max<size_t>(most, 1), 256 * 16, 8), (unsigned)a.count), dim3(256), 0, a);
     }
     return c.last_error == cudaSuccess ? OPATTR_OK : cuda_status(c, c.last_error);
 }

@@ -412,12 +412,13 @@ __global__ void __launch_bounds__(EP_THREADS) k_enc_parts(EncView V, EncCheck C,
 // Rows of the parts' last ranges to rows of the last range before each part:
 // a running maximum down every column.  One block per stream: lane d of a
 // warp takes depth d, each of the 32 warps an equal run of the parts.
+template <bool GROUPS>
 __global__ void __launch_bounds__(1024) k_enc_carry(uint32_t *__restrict__ rows, const uint32_t *__restrict__ row_len,
                                                     int64_t parts, const uint32_t *__restrict__ lvlmask,
                                                     const EncGroup *__restrict__ G) {
     pdl_wait();
     if (lvlmask[blockIdx.x] == 0) return;
-    if (G) {                                     // the parts of the stream's group
+    if (GROUPS) {                                // the parts of the stream's group
         G += blockIdx.x >> GROUP_SHIFT;
         rows += (int64_t)G->part0 * LEVELS;
         row_len += G->part0;
@@ -742,12 +743,12 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
                 }
                 __syncthreads();
             }
-            const bool close = near(t_last) && near(a_last), whole = r1 - r <= SR && close;
-            if (sizeof(Time) == 4 && !close && ++far > EN_FAR + tp) {
-                if (tid == 0) set_flag(st, F_TIMES_FAR);
-                return;
-            }
+            bool whole = r1 - r <= SR && near(t_last) && near(a_last);
             if (!whole) {
+                if (sizeof(Time) == 4 && !(near(t_last) && near(a_last)) && ++far > EN_FAR + tp) {
+                    if (tid == 0) set_flag(st, F_TIMES_FAR);
+                    return;
+                }
                 // by two warps, 32 probes a round
                 if (warp < 2) {
                     const bool more = r + nr < r1;
@@ -1207,7 +1208,7 @@ static void launch_tiles(Ctx &c, const EncView &V, const EncBufs &B, int nl, int
 }
 static void launch_carry(Ctx &c, const EncBufs &B) {
     if (B.groups || B.parts > EN_DIRECT_PARTS)
-        launch(c, "enc_carry", k_enc_carry, dim3(256), dim3(1024), 0, B.rows, (const uint32_t *)B.row_len, B.parts,
+        launch(c, "enc_carry", B.groups ? k_enc_carry<true> : k_enc_carry<false>, dim3(256), dim3(1024), 0, B.rows, (const uint32_t *)B.row_len, B.parts,
                (const uint32_t *)B.lvlmask, (const EncGroup *)B.groups);
 }
 
