@@ -95,6 +95,12 @@ opattr_status ensure_arena(Ctx &c, size_t bytes) {
     return OPATTR_OK;
 }
 
+// Why the join's enclosure has to run again, if it has.
+static bool note_redo(Ctx &c) {
+    c.redo |= c.h_status->flags & F_REDO;
+    return (c.h_status->flags & F_REDO) != 0;
+}
+
 static opattr_status drop_arena(Ctx &c) {
     if (cudaStreamSynchronize(c.stream) != cudaSuccess) return cuda_status(c, cudaGetLastError());
     if (c.arena) cudaFree(c.arena);
@@ -461,7 +467,7 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
     const bool spec = same && !ncu->stream;
     const bool ahead = same || (full && dd && !ncu->stream && match_layers_ahead(dedup));
     bool lean = false;                   // each step asks for its own scratch
-    for (int pass = 0; pass < 2; ++pass) {
+    for (int pass = 0; pass < 3; ++pass) {
         c.enclose_k_sorted = -1;
         c.spec_k = 0;
         c.spec_ran = false;
@@ -486,7 +492,7 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
             c.spec_kind = match_kind;
             c.spec_k = kernels->n;
         }
-        c.defer_status = ahead && pass == 0;
+        c.defer_status = ahead && (pass == 0 || c.redo == F_TIMES_FAR);
         opattr_status st = finish(c, do_enclose(c, kernels, ranges, range_of_kernel, n_op_enclosing));
         c.defer_status = false;
         if (st == OPATTR_E_OOM && c.join_scratch > 0 && drop_arena(c) == OPATTR_OK) {
@@ -508,7 +514,7 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
             // the enclosure's error comes before the matching's
             if (!c.enclose_pending) return sm;
             if ((st = read_status(c)) < 0) return st;
-            if ((c.redo = c.h_status->flags & F_REDO)) continue;
+            if (note_redo(c)) continue;
             st = enclose_verdict(*c.h_status, kernels->n);
             return st < 0 ? st : sm;
         }
@@ -523,7 +529,7 @@ opattr_status opattr_join(opattr_ctx *ctx, const opattr_kernels *kernels, const 
             // the enclosure's verdict and the pairing's, read with the aggregation's status
             c.enclose_pending = false;
             // redone without deferring
-            if ((c.redo = c.h_status->flags & F_REDO)) continue;
+            if (note_redo(c)) continue;
             // the enclosure's error before the aggregation's (nesting is only
             // judged when the range records passed their checks)
             DevStatus H = *c.h_status;

@@ -528,12 +528,15 @@ constexpr int EN_STREAMS_B = 160;
 constexpr int64_t EN_GROUP_EVENTS = 4 << 20;
 constexpr int64_t EN_TILE = 2048, EN_TILE_MIN = 512;     // events of a tile; of a part's one tile in small traces
 constexpr int64_t EN_EARLY = 1 << 20;                    // events from which a join looks at the checks before the end
-// Times of a step in 32 bits end it 4 s after its first event.  A block that has
-// taken more than EN_FAR steps, and one per tile, that ended so gives the trace up
-// (F_TIMES_FAR), and it is taken with times in 64 bits.  A join of 1M kernels on 8
-// streams with an event every 20 / 200 / 5,000 ms: 348 / 325 / 309 us, 336 / 1,157 /
-// 4,544 by 32-bit steps alone, 184 with events 0.3 ms apart.
-constexpr int EN_FAR = 8;
+// Times of a step in 32 bits end it 4 s after its first event.  A block counts the
+// steps that ended so.  Where the trace's span alone makes as many of them on
+// average as a second run costs (a few us each: far_steps), a block with more than
+// EN_FAR gives the trace up (F_TIMES_FAR), and it is taken with times in 64 bits;
+// else (long gaps, a thin tail) one with four times that many does.  A join of 1M kernels
+// on 8 streams with an event every 5 / 20 / 200 / 5,000 ms: 223 / 279 / 265 / 260 us,
+// 221 / 331 / 1,152 / 4,516 by 32-bit steps alone; 182 with events 0.3 ms apart.
+constexpr int EN_FAR = 4;
+__host__ __device__ __forceinline__ int far_steps(int64_t events) { return 8 + (int)(events >> 20); }
 constexpr size_t EN_SMEM_F = 74 * 1024;                  // of that layout: three blocks a multiprocessor at least, else groups
 
 // One block per part, tile by tile; a tile with more ranges than SR, or whose
@@ -745,9 +748,13 @@ __global__ void __launch_bounds__(TL::THREADS, TL::BLOCKS)
             }
             bool whole = r1 - r <= SR && near(t_last) && near(a_last);
             if (!whole) {
-                if (sizeof(Time) == 4 && !(near(t_last) && near(a_last)) && ++far > EN_FAR + tp) {
-                    if (tid == 0) set_flag(st, F_TIMES_FAR);
-                    return;
+                if (sizeof(Time) == 4 && !(near(t_last) && near(a_last)) && ++far > EN_FAR) {
+                    const uint64_t span = V.K > 0 ? (uint64_t)st->mm[MM_KSTART_MAX] - (uint64_t)st->mm[MM_KSTART_MIN] : 0;
+                    const int most = far_steps(events);
+                    if ((span >> 32) > (uint64_t)(most * parts) || far > 4 * most) {
+                        if (tid == 0) set_flag(st, F_TIMES_FAR);
+                        return;
+                    }
                 }
                 // by two warps, 32 probes a round
                 if (warp < 2) {
@@ -1345,10 +1352,12 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     const SmallCopy masks{c.h_small, B.lvlmask, 256 * sizeof(uint32_t)};
     if (early && (st = post_status(c, 1, &masks))) return st;
     launch_carry(c, B);
-    const bool run = !(c.redo & ~F_LEVEL_FIXUP);      // (else it would leave as it did before)
+    // (the run of a join that is redone would leave as it did before, but for wider times)
+    const unsigned again = c.redo & ~F_LEVEL_FIXUP;
+    const bool run = again == 0 || again == F_TIMES_FAR;
     if (run)
-        launch_tiles<EncTileA, false>(c, V, B, EN_LEVELS_A, EN_STREAMS_A, F_K_UNSORTED | F_R_UNSORTED, false, out_range,
-                                      out_nop);
+        (again ? launch_tiles<EncTileF, false> : launch_tiles<EncTileA, false>)(
+            c, V, B, EN_LEVELS_A, EN_STREAMS_A, F_K_UNSORTED | F_R_UNSORTED, false, out_range, out_nop);
     if (c.defer_status) {
         bool usual = true;
         if (early) {
@@ -1369,14 +1378,18 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     c.enclose_k_sorted = k_sorted ? 1 : 0;
     const LevelCount present(c.h_small);
     const bool many = present.levels > EN_LEVELS_A || present.streams > EN_STREAMS_A;
-    // (with tiles that span 8 s on average, 4 in the wide layout, the 32-bit times need no try)
+    // (with a span of so many steps the 32-bit times need no try; nor in the wide
+    // layout, which is no faster than wider times in the common one, with a step of
+    // 4 s for every four tiles)
     const uint64_t span = K > 0 ? (uint64_t)c.h_status->mm[MM_KSTART_MAX] - (uint64_t)c.h_status->mm[MM_KSTART_MIN] : 0;
-    bool far = ((c.h_status->flags | c.redo) & F_TIMES_FAR) != 0 || (span >> (many ? 32 : 33)) > (uint64_t)tiles;
-    bool grouped = present.levels > EN_LEVELS_B || (present.streams > EN_STREAMS_B && K + R > EN_GROUP_EVENTS);
     const bool far_fits = !many || EncTileF::smem(present.levels + 7, present.streams + 7) <= EN_SMEM_F;
+    const bool gave_up = (c.h_status->flags & F_TIMES_FAR) != 0;
+    bool far = gave_up || (c.redo & F_TIMES_FAR) || (span >> 32) > (uint64_t)(far_steps(K + R) * B.parts) ||
+               (many && far_fits && (span >> 30) > (uint64_t)tiles);
+    bool grouped = present.levels > EN_LEVELS_B || (present.streams > EN_STREAMS_B && K + R > EN_GROUP_EVENTS);
     const bool fixup = (c.h_status->flags & F_LEVEL_FIXUP) != 0;
-    if ((st = enclose_verdict(*c.h_status, K)) && !((fixup || far) && st == OPATTR_E_NOT_NESTED)) return st;
-    if (run && k_sorted && r_sorted && !many && !fixup && !far) return OPATTR_OK;
+    if ((st = enclose_verdict(*c.h_status, K)) && !((fixup || gave_up) && st == OPATTR_E_NOT_NESTED)) return st;
+    if (run && k_sorted && r_sorted && !many && !fixup && !gave_up) return OPATTR_OK;
 
     // ---- records out of order, ranges of one level that share a start and are
     // out of (start, end) order, more levels than the common layout holds, or
