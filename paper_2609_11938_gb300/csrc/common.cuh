@@ -106,7 +106,6 @@ struct Ctx {
     bool in_join = false;
     uint32_t *join_korder = nullptr;
     size_t arena_keep = 0;
-    // launch accounting
     // within a join: the matching's identity pairing (rows equal to the
     // kernels in time order), done by the enclosure's checking pass when
     // spec_k > 0; spec_ran: it was, its verdict in the status the enclosure
@@ -144,6 +143,7 @@ struct Ctx {
     // records in order (beyond what is kept), so that the enclosure's request is
     // the join's only one
     size_t join_scratch = 0;
+    // launch accounting
     int64_t launches = 0;
     bool timing = false;
     std::string timing_only;         // with timing on: bracket only this kernel (empty = all)
