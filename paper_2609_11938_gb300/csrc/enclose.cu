@@ -1386,7 +1386,8 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     const bool gave_up = (c.h_status->flags & F_TIMES_FAR) != 0;
     bool far = gave_up || (c.redo & F_TIMES_FAR) || (span >> 32) > (uint64_t)(far_steps(K + R) * B.parts) ||
                (many && far_fits && (span >> 30) > (uint64_t)tiles);
-    bool grouped = present.levels > EN_LEVELS_B || (present.streams > EN_STREAMS_B && K + R > EN_GROUP_EVENTS);
+    const bool grouped = present.levels > EN_LEVELS_B || (present.streams > EN_STREAMS_B && K + R > EN_GROUP_EVENTS) ||
+                         (far && !far_fits);
     const bool fixup = (c.h_status->flags & F_LEVEL_FIXUP) != 0;
     if ((st = enclose_verdict(*c.h_status, K)) && !((fixup || gave_up) && st == OPATTR_E_NOT_NESTED)) return st;
     if (run && k_sorted && r_sorted && !many && !fixup && !gave_up) return OPATTR_OK;
@@ -1415,7 +1416,7 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     }
     const int64_t g_parts = B.parts + N_GROUPS, g_tiles = (K + R) / EN_TILE + B.parts + 3 * N_GROUPS;
     const int64_t g_part = scan_scratch_elems(std::max(radix_hist_elems(K), radix_hist_elems(R)));
-    if (many) {
+    if (grouped) {
         Need n3;
         n3.add<int64_t>(K).add<uint8_t>(K).add<uint32_t>(K).add<uint32_t>(radix_hist_elems(K)).add<uint32_t>(g_part);
         n3.add<int64_t>(R).add<int64_t>(R).add<uint8_t>(R).add<uint8_t>(R).add<uint32_t>(R).add<uint32_t>(R);
@@ -1466,9 +1467,8 @@ opattr_status do_enclose(Ctx &c, const opattr_kernels *kern, const opattr_ranges
     bool sort_ranges = !r_sorted || fixup, sorted = false;
     bool have_parts = k_sorted && !sort_ranges && !grouped;       // (too many levels only: the checking pass's parts stand)
     GroupArrays ga{};
-    if (many && !ga.take(a, K, R, g_part, g_tiles, g_parts)) return OPATTR_E_OOM;
+    if (grouped && !ga.take(a, K, R, g_part, g_tiles, g_parts)) return OPATTR_E_OOM;
     for (int attempt = 0; attempt < 3; ++attempt) {
-        grouped = grouped || (far && !far_fits);
         if (sort_ranges && R > 0) {
             uint64_t *ko = nullptr;
             uint32_t *perm = nullptr;
