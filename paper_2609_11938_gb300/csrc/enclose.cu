@@ -17,7 +17,8 @@
 // Nothing is regrouped in device memory: kernels and ranges are read where
 // they lie, in order, and results are written in order.  Records out of order
 // are found by enc_parts (the other two then leave at once), sorted, and the
-// last two run again on the sorted view.
+// last two run again on the sorted view; so they do with wider tables, by groups of
+// streams or with wider times where the levels, the streams or the times ask for it.
 #include <algorithm>
 #include <type_traits>
 
@@ -542,8 +543,8 @@ constexpr size_t EN_SMEM_F = 74 * 1024;                  // of that layout: thre
 // One block per part, tile by tile; a tile with more ranges than SR, or whose
 // times span 2^32 ns, is taken in steps.  A step's ranges, and the ranges open
 // when it begins, lie in shared memory (times relative to the part's first
-// event, or to the step's after 2^32 ns, in 32 bits), and once per range this
-// is worked out:
+// event, or to the step's after 2^32 ns, in 32 bits; in 64 with EncTileF), and
+// once per range this is worked out:
 //   parent  the last range of the level above that starts no later
 //   chain   Algorithm 2's result for the range and its ancestors: walking
 //           outward to the first structural range, the innermost operator
@@ -575,7 +576,7 @@ constexpr size_t EN_SMEM_F = 74 * 1024;                  // of that layout: thre
 // first open one, and a step's tables are cleared by the entries it made.
 //
 // Bound by issue (2.4 instructions a cycle) and by the shared-memory chains of
-// the links, not by HBM: 425 us for 20M kernels and 5.1M ranges on 16 streams
+// the links, not by HBM: 430 us for 20M kernels and 5.1M ranges on 16 streams
 // of 8 levels, 1,950 us for 50M and 14.5M on 64 streams of 32 (1,990 with climbs
 // of one level at a time), 14 us for 2,000.
 // With every open range's chain walked, and every level's tables cleared,

@@ -264,7 +264,8 @@ __global__ void __launch_bounds__(RADIX_THREADS) k_digit_rank(DigitFn digit, int
 
 // The same for an epi that moves wide elements: it is called in order of the
 // destinations, so that a tile's elements of one digit are written side by side
-// (and read from the 4,096 of the tile).
+// (and read from the 4,096 of the tile).  20M records of 9 bytes to 13 in 16 groups:
+// 150 us, 324 written in the order of the records.
 template <typename DigitFn, typename Epi>
 __global__ void __launch_bounds__(RADIX_THREADS) k_digit_move(DigitFn digit, int64_t n,
                                                               const uint32_t *__restrict__ offs, int64_t ntiles,
@@ -322,8 +323,8 @@ __global__ void __launch_bounds__(RADIX_THREADS) k_digit_move(DigitFn digit, int
     }
 }
 
-// nbins: digits used (every digit below it); only those rows of the matrix
-// are counted on and scanned.  The scan goes out of place, into the second
+// nbins: digits used: digit(i) is below it, or RADIX_BINS; only those rows of the
+// matrix are counted on and scanned, and others have no offsets.  The scan goes out of place, into the second
 // half of `hist` (radix_hist_elems(n) entries: one pass); the offsets'
 // address is returned for digit_rank.
 template <typename DigitFn>
